@@ -109,9 +109,15 @@ int64_t row_pad(int executor) { return executor == DMP_EXEC_TC ? 256 : kTileM; }
     if (e_ != cudaSuccess) return DMP_ERR_CUDA; \
   } while (0)
 
+// The tcgen05 executor's group sums in a workspace (empty for the other executors).
+size_t area_bytes(const Opts& o) {
+  return o.mode != DMP_FP64 && o.executor == DMP_EXEC_TC ? tc_area_bytes() : 0;
+}
+TcArea area_at(const Opts& o, void* ws, size_t off) { return TcArea{static_cast<char*>(ws) + off, area_bytes(o), 0}; }
+
 // ---------------------------------------------------------------- dm_purify layout
 struct PurifyLayout {
-  size_t state, partials, rowbuf, expsP, expsX, err, Palt, X2, planesP, planesX, scratch, split, total;
+  size_t state, partials, rowbuf, expsP, expsX, err, Palt, X2, planesP, planesX, area, total;
   int64_t n_pad, k_pad;
 };
 
@@ -130,28 +136,26 @@ PurifyLayout purify_layout(int64_t n, const Opts& o) {
   L.X2 = c.take(static_cast<size_t>(n) * n * sizeof(double));
   if (o.mode != DMP_FP64) {
     // room for the refinement step's slices too
-    const int smax = std::max(std::max(o.s, o.refine), o.late_s);
-    const size_t plane = static_cast<size_t>(smax) * L.n_pad * L.k_pad * elem_bytes(o);
+    const int planes = std::max(std::max(o.s, o.refine), o.late_s);
+    const size_t plane = static_cast<size_t>(planes) * L.n_pad * L.k_pad * elem_bytes(o);
     L.planesP = c.take(plane);
     L.planesX = c.take(plane);
   } else {
     L.planesP = L.planesX = 0;
   }
-  L.scratch = (o.mode != DMP_FP64 && o.executor == DMP_EXEC_TC) ? c.take(tc_scratch_bytes()) : 0;
-  L.split = (o.mode != DMP_FP64 && o.executor == DMP_EXEC_TC) ? c.take(tc_split_bytes()) : 0;
+  L.area = c.take(area_bytes(o));
   L.total = c.cur;
   return L;
 }
 
 // One Ozaki product from prepared digit planes on the chosen executor.
-// `split_ws` (nullable) is the tcgen05 executor's workspace for split launches (tc_split_bytes).
+// `area` holds the tcgen05 executor's group sums; k is the unpadded inner size.
 cudaError_t launch_product(const Opts& o, const void* pa, const void* pb, const int32_t* ea, const int32_t* eb,
-                           int64_t m, int64_t n, int64_t rows_a, int64_t rows_b, int64_t k_pad, int sym,
-                           const EpiArgs& epi, const int* done, int* err, double* scratch, void* split_ws,
-                           cudaStream_t st) {
+                           int64_t m, int64_t n, int64_t k, int64_t rows_a, int64_t rows_b, int64_t k_pad, int sym,
+                           const EpiArgs& epi, const int* done, int* err, TcArea& area, cudaStream_t st) {
   if (o.executor == DMP_EXEC_TC)
-    return launch_ozaki_tc(pa, pb, ea, eb, m, n, rows_a, rows_b, k_pad, o.s, o.beta, sym, epi, done, err, scratch,
-                           split_ws, st);
+    return launch_ozaki_tc(pa, pb, ea, eb, m, n, k, rows_a, rows_b, k_pad, o.s, o.beta,
+                           sym, epi, done, err, area, st);
   return launch_ozaki_imma(static_cast<const int8_t*>(pa), static_cast<const int8_t*>(pb), ea, eb, m, n, rows_a,
                            rows_b, k_pad, o.s, o.beta, sym, epi, done, st);
 }
@@ -187,7 +191,7 @@ inline char* at(void* base, size_t off) { return static_cast<char*>(base) + off;
 // buffers of one product.
 struct BackwardLayout {
   size_t state, scalars, p0, partials, err, expsP, expsA, G, Gn, Y, Z, YP, ZP, segP, segX, planesP, planesA,
-      scratch, split, total;
+      area, total;
   int64_t n_pad, k_pad;
 };
 
@@ -219,8 +223,7 @@ BackwardLayout backward_layout(int64_t n, const Opts& o) {
   } else {
     B.planesP = B.planesA = 0;
   }
-  B.scratch = (o.mode != DMP_FP64 && o.executor == DMP_EXEC_TC) ? c.take(tc_scratch_bytes()) : 0;
-  B.split = (o.mode != DMP_FP64 && o.executor == DMP_EXEC_TC) ? c.take(tc_split_bytes()) : 0;
+  B.area = c.take(area_bytes(o));
   B.total = c.cur;
   return B;
 }
@@ -241,7 +244,7 @@ constexpr int kFoeMaxQ = 128;  // ps_q(DMP_FOE_MAX_TERMS)
 // (split once), of the current right operand, and of y = T_q (scheme 1).
 struct FoeLayout {
   size_t state, rowbuf, scal, coeffs, traces, w, gx, fold, psw, ip, dots, partials, err, Hs, Ta, Tb, Y, Tps, expsH,
-      expsT, expsY, planesH, planesT, planesY, scratch, split, total;
+      expsT, expsY, planesH, planesT, planesY, area, total;
   int64_t n_pad, k_pad;
 };
 
@@ -285,8 +288,7 @@ FoeLayout foe_layout(int64_t n, const Opts& o, int scheme, int M) {
       F.planesY = c.take(plane);
     }
   }
-  F.scratch = (o.mode != DMP_FP64 && o.executor == DMP_EXEC_TC) ? c.take(tc_scratch_bytes()) : 0;
-  F.split = (o.mode != DMP_FP64 && o.executor == DMP_EXEC_TC) ? c.take(tc_split_bytes()) : 0;
+  F.area = c.take(area_bytes(o));
   F.total = c.cur;
   return F;
 }
@@ -385,8 +387,7 @@ int dm_purify(const double* H, int64_t n, int64_t ldh, int64_t n_occ, const dmp_
   void* planesP = o.mode != DMP_FP64 ? at(ws, L.planesP) : nullptr;
   void* planesX = o.mode != DMP_FP64 ? at(ws, L.planesX) : nullptr;
   int* err = reinterpret_cast<int*>(at(ws, L.err));
-  double* scratch = L.scratch ? reinterpret_cast<double*>(at(ws, L.scratch)) : nullptr;
-  void* split_ws = L.split ? at(ws, L.split) : nullptr;
+  TcArea area = area_at(o, ws, L.area);
   DMP_CUDA(cudaMemsetAsync(err, 0, sizeof(int), st));
 
   PurifyState init;
@@ -431,8 +432,8 @@ int dm_purify(const double* H, int64_t n, int64_t ldh, int64_t n_occ, const dmp_
     } else {
       DMP_CUDA(launch_split_rows(cur, n, n, ldcur, oi.s, oi.beta, expsP, planesP, L.n_pad, L.k_pad,
                                  elem_kind(o), nullptr, done, st));
-      DMP_CUDA(launch_product(oi, planesP, planesP, expsP, expsP, n, n, L.n_pad, L.n_pad, L.k_pad, 1, e2, done,
-                              err, scratch, split_ws, st));
+      DMP_CUDA(launch_product(oi, planesP, planesP, expsP, expsP, n, n, n, L.n_pad, L.n_pad, L.k_pad, 1, e2, done,
+                              err, area, st));
     }
     if (o.method == DMP_METHOD_PM) {
       DMP_CUDA(launch_measure(cur, ldcur, X2, n, H, ldh, n, partials, state, st));
@@ -469,8 +470,8 @@ int dm_purify(const double* H, int64_t n, int64_t ldh, int64_t n_occ, const dmp_
                                      elem_kind(o), nullptr, done, st));
           DMP_CUDA(launch_split_rows(alt, n, n, ldalt, oi.s, oi.beta, expsP, planesP, L.n_pad, L.k_pad,
                                      elem_kind(o), nullptr, done, st));
-          DMP_CUDA(launch_product(oi, planesX, planesP, expsX, expsP, n, n, L.n_pad, L.n_pad, L.k_pad, 1, ez, done,
-                                  err, scratch, split_ws, st));
+          DMP_CUDA(launch_product(oi, planesX, planesP, expsX, expsP, n, n, n, L.n_pad, L.n_pad, L.k_pad, 1, ez, done,
+                                  err, area, st));
         }
       }
       continue;
@@ -493,8 +494,8 @@ int dm_purify(const double* H, int64_t n, int64_t ldh, int64_t n_occ, const dmp_
     } else {
       DMP_CUDA(launch_split_rows(X2, n, n, n, oi.s, oi.beta, expsX, planesX, L.n_pad, L.k_pad,
                                  elem_kind(o), nullptr, done, st));
-      DMP_CUDA(launch_product(oi, planesP, planesX, expsP, expsX, n, n, L.n_pad, L.n_pad, L.k_pad, 1, e3, done,
-                              err, scratch, split_ws, st));
+      DMP_CUDA(launch_product(oi, planesP, planesX, expsP, expsX, n, n, n, L.n_pad, L.n_pad, L.k_pad, 1, e3, done,
+                              err, area, st));
     }
     std::swap(cur, alt);
     std::swap(ldcur, ldalt);
@@ -531,12 +532,12 @@ int dm_purify(const double* H, int64_t n, int64_t ldh, int64_t n_occ, const dmp_
         orr.s = o.refine;
         DMP_CUDA(launch_split_rows(cur, n, n, ldcur, orr.s, orr.beta, expsP, planesP, L.n_pad, L.k_pad,
                                    elem_kind(o), nullptr, nullptr, st));
-        DMP_CUDA(launch_product(orr, planesP, planesP, expsP, expsP, n, n, L.n_pad, L.n_pad, L.k_pad, 1, r2, nullptr,
-                                err, scratch, split_ws, st));
+        DMP_CUDA(launch_product(orr, planesP, planesP, expsP, expsP, n, n, n, L.n_pad, L.n_pad, L.k_pad, 1, r2, nullptr,
+                                err, area, st));
         DMP_CUDA(launch_split_rows(X2, n, n, n, orr.s, orr.beta, expsX, planesX, L.n_pad, L.k_pad,
                                    elem_kind(o), nullptr, nullptr, st));
-        DMP_CUDA(launch_product(orr, planesP, planesX, expsP, expsX, n, n, L.n_pad, L.n_pad, L.k_pad, 1, r3, nullptr,
-                                err, scratch, split_ws, st));
+        DMP_CUDA(launch_product(orr, planesP, planesX, expsP, expsX, n, n, n, L.n_pad, L.n_pad, L.k_pad, 1, r3, nullptr,
+                                err, area, st));
       }
       std::swap(cur, alt);
       std::swap(ldcur, ldalt);
@@ -614,10 +615,10 @@ int dm_purify_host(const double* H_host, int64_t n, int64_t ldh, int64_t n_occ, 
                    double* P_host, int64_t ldp, dmp_info* info, void* ws, size_t ws_bytes, void* stream) {
   if (H_host == nullptr || P_host == nullptr || ws == nullptr || opts == nullptr) return DMP_ERR_INVALID_ARG;
   if (n < 2 || ldh < n || ldp < n) return DMP_ERR_INVALID_ARG;
-  size_t need = 0;
-  const int rc = dmp_host_workspace_size(n, opts, &need);
+  Opts o;
+  const int rc = normalize(opts, o);
   if (rc != DMP_OK) return rc;
-  if (ws_bytes < need) return DMP_ERR_WORKSPACE;
+  if (ws_bytes < host_front_bytes(n) + purify_layout(n, o).total) return DMP_ERR_WORKSPACE;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const size_t front = host_front_bytes(n);
   double* Hd = reinterpret_cast<double*>(ws);
@@ -639,44 +640,61 @@ int dm_purify_host(const double* H_host, int64_t n, int64_t ldh, int64_t n_occ, 
   return status;
 }
 
-int ozaki_gemm_workspace_size(int64_t m, int64_t n, int64_t k, int32_t mode, int32_t slices,
-                              int32_t executor, size_t* bytes) {
+}  // extern "C"
+
+namespace dmp {
+namespace {
+// ozaki_gemm workspace: exponents, error flag, group sums, the operands' planes, B transposed.
+struct GemmLayout {
+  size_t ea, eb, err, area, pa, pb, Bt, total;
+  int64_t m_pad, n_pad, k_pad;
+};
+
+GemmLayout gemm_layout(int64_t m, int64_t n, int64_t k, const Opts& o) {
+  GemmLayout G;
+  Carver c;
+  G.m_pad = round_up(std::max<int64_t>(m, 1), row_pad(o.executor));
+  G.n_pad = round_up(std::max<int64_t>(n, 1), row_pad(o.executor));
+  G.k_pad = k_pad_of(o, k);
+  const size_t planes = static_cast<size_t>(o.s);
+  G.ea = c.take(G.m_pad * sizeof(int32_t));
+  G.eb = c.take(G.n_pad * sizeof(int32_t));
+  G.err = c.take(sizeof(int32_t));
+  G.pa = c.take(planes * G.m_pad * G.k_pad * elem_bytes(o));
+  G.pb = c.take(planes * G.n_pad * G.k_pad * elem_bytes(o));
+  G.Bt = c.take(static_cast<size_t>(n) * k * sizeof(double));
+  G.area = c.take(area_bytes(o));
+  G.total = c.cur;
+  return G;
+}
+
+int gemm_opts(int32_t mode, int32_t slices, int32_t executor, Opts& o) {
   dmp_opts d{};
   d.mode = mode;
   d.slices = slices;
   d.executor = executor;
+  return normalize(&d, o);
+}
+}  // namespace
+}  // namespace dmp
+
+extern "C" {
+
+int ozaki_gemm_workspace_size(int64_t m, int64_t n, int64_t k, int32_t mode, int32_t slices,
+                              int32_t executor, size_t* bytes) {
   Opts o;
-  const int rc = normalize(&d, o);
+  const int rc = gemm_opts(mode, slices, executor, o);
   if (rc != DMP_OK) return rc;
   if (m < 0 || n < 0 || k < 0 || bytes == nullptr) return DMP_ERR_INVALID_ARG;
-  if (o.mode == DMP_FP64) {
-    *bytes = 0;
-    return DMP_OK;
-  }
-  Carver c;
-  const int64_t m_pad = round_up(std::max<int64_t>(m, 1), row_pad(o.executor));
-  const int64_t n_pad = round_up(std::max<int64_t>(n, 1), row_pad(o.executor));
-  const int64_t k_pad = k_pad_of(o, k);
-  c.take(m_pad * sizeof(int32_t));
-  c.take(n_pad * sizeof(int32_t));
-  c.take(sizeof(int32_t));
-  c.take(o.executor == DMP_EXEC_TC ? tc_scratch_bytes() : 0);
-  c.take(static_cast<size_t>(o.s) * m_pad * k_pad * elem_bytes(o));
-  c.take(static_cast<size_t>(o.s) * n_pad * k_pad * elem_bytes(o));
-  c.take(static_cast<size_t>(n) * k * sizeof(double));
-  *bytes = c.cur;
+  *bytes = o.mode == DMP_FP64 ? 0 : gemm_layout(m, n, k, o).total;
   return DMP_OK;
 }
 
 static int ozaki_common(int64_t m, int64_t n, int64_t k, const double* A, int64_t lda, const double* B,
                         int64_t ldb, const EpiArgs& epi, int32_t mode, int32_t slices, int32_t executor,
                         void* ws, size_t ws_bytes, void* stream) {
-  dmp_opts d{};
-  d.mode = mode;
-  d.slices = slices;
-  d.executor = executor;
   Opts o;
-  const int rc = normalize(&d, o);
+  const int rc = gemm_opts(mode, slices, executor, o);
   if (rc != DMP_OK) return rc;
   if (m < 0 || n < 0 || k < 0) return DMP_ERR_INVALID_ARG;
   if (m == 0 || n == 0) return DMP_OK;
@@ -689,27 +707,22 @@ static int ozaki_common(int64_t m, int64_t n, int64_t k, const double* A, int64_
   }
   if (!levels_fit_int32(k, o.s, o.mode))
     return DMP_ERR_UNSUPPORTED;
-  size_t need = 0;
-  ozaki_gemm_workspace_size(m, n, k, mode, slices, executor, &need);
-  if (ws == nullptr || ws_bytes < need) return DMP_ERR_WORKSPACE;
-  Carver c;
-  const int64_t m_pad = round_up(m, row_pad(o.executor));
-  const int64_t n_pad = round_up(n, row_pad(o.executor));
-  const int64_t k_pad = k_pad_of(o, k);
-  int32_t* ea = reinterpret_cast<int32_t*>(at(ws, c.take(m_pad * sizeof(int32_t))));
-  int32_t* eb = reinterpret_cast<int32_t*>(at(ws, c.take(n_pad * sizeof(int32_t))));
-  int* err = reinterpret_cast<int*>(at(ws, c.take(sizeof(int32_t))));
-  double* scratch = reinterpret_cast<double*>(at(ws, c.take(o.executor == DMP_EXEC_TC ? tc_scratch_bytes() : 0)));
-  void* pa = at(ws, c.take(static_cast<size_t>(o.s) * m_pad * k_pad * elem_bytes(o)));
-  void* pb = at(ws, c.take(static_cast<size_t>(o.s) * n_pad * k_pad * elem_bytes(o)));
-  double* Bt = reinterpret_cast<double*>(at(ws, c.take(static_cast<size_t>(n) * k * sizeof(double))));
-  DMP_CUDA(launch_split_rows(A, m, k, lda, o.s, o.beta, ea, pa, m_pad, k_pad, elem_kind(o), nullptr,
+  const GemmLayout G = gemm_layout(m, n, k, o);
+  if (ws == nullptr || ws_bytes < G.total) return DMP_ERR_WORKSPACE;
+  int32_t* ea = reinterpret_cast<int32_t*>(at(ws, G.ea));
+  int32_t* eb = reinterpret_cast<int32_t*>(at(ws, G.eb));
+  int* err = reinterpret_cast<int*>(at(ws, G.err));
+  TcArea area = area_at(o, ws, G.area);
+  void* pa = at(ws, G.pa);
+  void* pb = at(ws, G.pb);
+  double* Bt = reinterpret_cast<double*>(at(ws, G.Bt));
+  DMP_CUDA(launch_split_rows(A, m, k, lda, o.s, o.beta, ea, pa, G.m_pad, G.k_pad, elem_kind(o), nullptr,
                              nullptr, st));
   DMP_CUDA(launch_transpose(B, k, n, ldb, Bt, st));
-  DMP_CUDA(launch_split_rows(Bt, n, k, k, o.s, o.beta, eb, pb, n_pad, k_pad, elem_kind(o), nullptr,
+  DMP_CUDA(launch_split_rows(Bt, n, k, k, o.s, o.beta, eb, pb, G.n_pad, G.k_pad, elem_kind(o), nullptr,
                              nullptr, st));
   if (o.executor == DMP_EXEC_TC) DMP_CUDA(cudaMemsetAsync(err, 0, sizeof(int), st));
-  DMP_CUDA(launch_product(o, pa, pb, ea, eb, m, n, m_pad, n_pad, k_pad, 0, epi, nullptr, err, scratch, nullptr, st));
+  DMP_CUDA(launch_product(o, pa, pb, ea, eb, m, n, k, G.m_pad, G.n_pad, G.k_pad, 0, epi, nullptr, err, area, st));
   if (o.executor == DMP_EXEC_TC) {
     // report an expired device wait; skipped while the stream is being captured
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
@@ -747,28 +760,19 @@ int ozaki_level_sums(int64_t m, int64_t n, int64_t k, const double* A, int64_t l
 
 int ozaki_split(int64_t m, int64_t k, const double* A, int64_t lda, int32_t mode, int32_t slices,
                 int32_t executor, int32_t* exps, void* digits, void* ws, size_t ws_bytes, void* stream) {
-  dmp_opts d{};
-  d.mode = mode;
-  d.slices = slices;
-  d.executor = executor;
   Opts o;
-  const int rc = normalize(&d, o);
+  const int rc = gemm_opts(mode, slices, executor, o);
   if (rc != DMP_OK) return rc;
   if (o.mode == DMP_FP64) return DMP_ERR_INVALID_ARG;
   if (m <= 0 || k <= 0 || A == nullptr || lda < k || exps == nullptr || digits == nullptr)
     return DMP_ERR_INVALID_ARG;
-  size_t need = 0;
-  ozaki_gemm_workspace_size(m, 1, k, mode, slices, executor, &need);
-  if (ws == nullptr || ws_bytes < need) return DMP_ERR_WORKSPACE;
+  const GemmLayout G = gemm_layout(m, 1, k, o);
+  if (ws == nullptr || ws_bytes < G.total) return DMP_ERR_WORKSPACE;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  Carver c;
-  const int64_t m_pad = round_up(m, row_pad(o.executor));
-  const int64_t k_pad = k_pad_of(o, k);
-  int32_t* ea = reinterpret_cast<int32_t*>(at(ws, c.take(m_pad * sizeof(int32_t))));
-  c.take(round_up(1, row_pad(o.executor)) * sizeof(int32_t));
-  c.take(sizeof(int32_t));
+  int32_t* ea = reinterpret_cast<int32_t*>(at(ws, G.ea));
   const int eb = elem_bytes(o);
-  char* pa = at(ws, c.take(static_cast<size_t>(o.s) * m_pad * k_pad * eb));
+  const int64_t m_pad = G.m_pad, k_pad = G.k_pad;
+  char* pa = at(ws, G.pa);
   DMP_CUDA(launch_split_rows(A, m, k, lda, o.s, o.beta, ea, pa, m_pad, k_pad, elem_kind(o), nullptr,
                              nullptr, st));
   DMP_CUDA(cudaMemcpyAsync(exps, ea, m * sizeof(int32_t), cudaMemcpyDeviceToDevice, st));
@@ -837,8 +841,7 @@ int dm_purify_backward(const double* H, int64_t n, int64_t n_occ, const dmp_opts
   int32_t* expsA = reinterpret_cast<int32_t*>(at(ws, B.expsA));
   void* planesP = o.mode != DMP_FP64 ? at(ws, B.planesP) : nullptr;
   void* planesA = o.mode != DMP_FP64 ? at(ws, B.planesA) : nullptr;
-  double* scratch = B.scratch ? reinterpret_cast<double*>(at(ws, B.scratch)) : nullptr;
-  void* split_ws = B.split ? at(ws, B.split) : nullptr;
+  TcArea area = area_at(o, ws, B.area);
   DMP_CUDA(cudaMemsetAsync(err, 0, sizeof(int), st));
   const int64_t npad = B.n_pad, kpad = B.k_pad;
 
@@ -852,13 +855,13 @@ int dm_purify_backward(const double* H, int64_t n, int64_t n_occ, const dmp_opts
     cudaError_t r = launch_split_rows(A, n, n, n, o.s, o.beta, expsA, planesA, npad, kpad, elem_kind(o),
                                       nullptr, nullptr, st);
     if (r != cudaSuccess) return r;
-    return launch_product(o, planesA, planesP, expsA, expsP, n, n, npad, npad, kpad, 0, e, nullptr,
-                          err, scratch, split_ws, st);
+    return launch_product(o, planesA, planesP, expsA, expsP, n, n, n, npad, npad, kpad, 0, e, nullptr,
+                          err, area, st);
   };
   auto split_P = [&](const double* Pk) -> cudaError_t {
     if (o.mode == DMP_FP64) return cudaSuccess;
-    return launch_split_rows(Pk, n, n, n, o.s, o.beta, expsP, planesP, npad, kpad, elem_kind(o), nullptr,
-                             nullptr, st);
+    return launch_split_rows(Pk, n, n, n, o.s, o.beta, expsP, planesP, npad, kpad, elem_kind(o),
+                             nullptr, nullptr, st);
   };
 
   // host copies of the per-step update weights (kept alive until the stream syncs)
@@ -896,8 +899,8 @@ int dm_purify_backward(const double* H, int64_t n, int64_t n_occ, const dmp_opts
         DMP_CUDA(launch_gemm_f64(Pk, n, Pk, n, n, n, n, 1, e2, nullptr, st));
       } else {
         DMP_CUDA(split_P(Pk));
-        DMP_CUDA(launch_product(o, planesP, planesP, expsP, expsP, n, n, npad, npad, kpad, 1, e2, nullptr,
-                                err, scratch, split_ws, st));
+        DMP_CUDA(launch_product(o, planesP, planesP, expsP, expsP, n, n, n, npad, npad, kpad, 1, e2, nullptr,
+                                err, area, st));
       }
       if (k + 1 < k1) {
         DMP_CUDA(cudaMemcpyAsync(&state->alpha, &wts[k].alpha, 3 * sizeof(double), cudaMemcpyHostToDevice, st));
@@ -915,8 +918,8 @@ int dm_purify_backward(const double* H, int64_t n, int64_t n_occ, const dmp_opts
         } else {
           DMP_CUDA(launch_split_rows(Xk, n, n, n, o.s, o.beta, expsA, planesA, npad, kpad, elem_kind(o),
                                      nullptr, nullptr, st));
-          DMP_CUDA(launch_product(o, planesP, planesA, expsP, expsA, n, n, npad, npad, kpad, 1, e3, nullptr,
-                                  err, scratch, split_ws, st));
+          DMP_CUDA(launch_product(o, planesP, planesA, expsP, expsA, n, n, n, npad, npad, kpad, 1, e3, nullptr,
+                                  err, area, st));
         }
       }
     }
@@ -1011,8 +1014,7 @@ int dm_foe(const double* H, int64_t n, int64_t ldh, const dmp_foe_params* params
   int32_t* expsT = oz ? reinterpret_cast<int32_t*>(at(ws, L.expsT)) : nullptr;
   void* planesH = oz ? at(ws, L.planesH) : nullptr;
   void* planesT = oz ? at(ws, L.planesT) : nullptr;
-  double* scratch = L.scratch ? dbl(L.scratch) : nullptr;
-  void* split_ws = L.split ? at(ws, L.split) : nullptr;
+  TcArea area = area_at(o, ws, L.area);
   DMP_CUDA(cudaMemsetAsync(err, 0, sizeof(int), st));
 
   PurifyState init;
@@ -1049,10 +1051,10 @@ int dm_foe(const double* H, int64_t n, int64_t ldh, const dmp_foe_params* params
     if (!oz) {
       DMP_CUDA(launch_gemm_f64(A, n, B, n, n, n, n, 1, e, nullptr, st));
     } else {
-      DMP_CUDA(launch_split_rows(B, n, n, n, o.s, o.beta, expsT, planesT, L.n_pad, L.k_pad, elem_kind(o), nullptr,
-                                 err, st));
-      DMP_CUDA(launch_product(o, pa, planesT, ea, expsT, n, n, L.n_pad, L.n_pad, L.k_pad, 1, e, err,
-                              err, scratch, split_ws, st));
+      DMP_CUDA(launch_split_rows(B, n, n, n, o.s, o.beta, expsT, planesT, L.n_pad, L.k_pad, elem_kind(o),
+                                 nullptr, err, st));
+      DMP_CUDA(launch_product(o, pa, planesT, ea, expsT, n, n, n, L.n_pad, L.n_pad, L.k_pad, 1, e, err,
+                              err, area, st));
     }
     ++products;
     if (oz && o.executor == DMP_EXEC_TC && products % kFoeCheckEvery == 0) {
@@ -1065,8 +1067,8 @@ int dm_foe(const double* H, int64_t n, int64_t ldh, const dmp_foe_params* params
   };
   auto split_a = [&](const double* A, void* planes, int32_t* exps) -> int {
     if (oz)
-      DMP_CUDA(launch_split_rows(A, n, n, n, o.s, o.beta, exps, planes, L.n_pad, L.k_pad, elem_kind(o), nullptr,
-                                 err, st));
+      DMP_CUDA(launch_split_rows(A, n, n, n, o.s, o.beta, exps, planes, L.n_pad, L.k_pad, elem_kind(o),
+                                 nullptr, err, st));
     return DMP_OK;
   };
 

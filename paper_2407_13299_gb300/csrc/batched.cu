@@ -201,7 +201,7 @@ __global__ void refine_end_kernel(const BatchMat* __restrict__ mats, int nmats, 
 
 // ---------------------------------------------------------------- host side
 struct BatchLayout {
-  size_t mats, tiles, row_start, partials, err, counter, active, scratch, tune_ws, total;
+  size_t mats, tiles, row_start, partials, err, counter, active, area, tune_ws, total;
   std::vector<size_t> state, rowbuf, expsP, expsX, buf1, X2, planesP, planesX;
   std::vector<int64_t> n_pad, k_pad;
   int ntiles;
@@ -239,7 +239,7 @@ BatchLayout batch_layout(int batch, const int64_t* n, int s_max, int beta) {
   L.err = c.take(sizeof(int));
   L.counter = c.take(sizeof(int));
   L.active = c.take(sizeof(int));
-  L.scratch = c.take(tc_scratch_bytes());
+  L.area = c.take(tc_area_bytes());
   int64_t nmax = 2;
   for (int b = 0; b < batch; ++b) {
     const int64_t np = round_up(n[b], 256), kp = round_up(n[b], kq);
@@ -361,8 +361,9 @@ int dm_purify_batched(int32_t batch, const double* const* H, const int64_t* n, c
   double* dpart = reinterpret_cast<double*>(at(ws, L.partials));
   int* derr = reinterpret_cast<int*>(at(ws, L.err));
   int* dcounter = reinterpret_cast<int*>(at(ws, L.counter));
-  double* scratch = reinterpret_cast<double*>(at(ws, L.scratch));
+  TcArea area{at(ws, L.area), tc_area_bytes(), 0};
   const int64_t nmax_idx = std::max_element(n, n + batch) - n;
+  const int64_t nmax = n[nmax_idx];
 
   // ---- autotune: slice count (accuracy) and tile width (speed), cached per shape
   TuneKey key{std::vector<int64_t>(n, n + batch),
@@ -497,6 +498,8 @@ int dm_purify_batched(int32_t batch, const double* const* H, const int64_t* n, c
   };
   const int tbeta = beta;
   std::vector<int4> htiles;
+  // cleared here, outside the graph: every product finds and leaves it zero
+  DMP_CUDA(tc_area_clear(area, area.bytes, st));
   DMP_CUDA(cudaMemcpyAsync(drow, hrow.data(), sizeof(int64_t) * (batch + 1), cudaMemcpyHostToDevice, st));
 
   if (!tile_tuned && forced == 0) {
@@ -519,8 +522,8 @@ int dm_purify_batched(int32_t batch, const double* const* H, const int64_t* n, c
       DMP_CUDA(cudaEventCreate(&e0));
       DMP_CUDA(cudaEventCreate(&e1));
       DMP_CUDA(cudaEventRecord(e0, st));
-      DMP_CUDA(launch_ozaki_tc_grouped(dmats, dtiles, static_cast<int>(htiles.size()), cfg_bn(cand), cfg_pair(cand),
-                                       tbeta, 0, 0, derr, scratch, dcounter, st));
+      DMP_CUDA(launch_ozaki_tc_grouped(dmats, dtiles, static_cast<int>(htiles.size()), nmax, cfg_bn(cand),
+                                       cfg_pair(cand), tbeta, s, 0, 0, derr, area, dcounter, st));
       DMP_CUDA(cudaEventRecord(e1, st));
       DMP_CUDA(cudaEventSynchronize(e1));
       float ms = 0.f;
@@ -583,11 +586,11 @@ int dm_purify_batched(int32_t batch, const double* const* H, const int64_t* n, c
     DMP_CUDA(cudaStreamBeginCaptureToGraph(cs, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed));
     for (int cur = 0; cur < 2; ++cur) {
       launch_split_grouped(dmats, drow, batch, hrow[batch], cur, tbeta, s, cs);
-      launch_ozaki_tc_grouped(dmats, dtiles, ntiles, cfg_bn(cfg), cfg_pair(cfg), tbeta, 0, cur, derr, scratch,
+      launch_ozaki_tc_grouped(dmats, dtiles, ntiles, nmax, cfg_bn(cfg), cfg_pair(cfg), tbeta, s, 0, cur, derr, area,
                               dcounter, cs);
       launch_measure_grouped(dmats, batch, cur, dpart, cond, 1, nullptr, cs);
       launch_split_grouped(dmats, drow, batch, hrow[batch], 2, tbeta, s, cs);
-      launch_ozaki_tc_grouped(dmats, dtiles, ntiles, cfg_bn(cfg), cfg_pair(cfg), tbeta, 1, cur, derr, scratch,
+      launch_ozaki_tc_grouped(dmats, dtiles, ntiles, nmax, cfg_bn(cfg), cfg_pair(cfg), tbeta, s, 1, cur, derr, area,
                               dcounter, cs);
     }
     cudaGraph_t captured = nullptr;
@@ -605,12 +608,12 @@ int dm_purify_batched(int32_t batch, const double* const* H, const int64_t* n, c
     for (int it = 0; it < max_iter; it += 2) {
       for (int cur = 0; cur < 2; ++cur) {
         DMP_CUDA(launch_split_grouped(dmats, drow, batch, hrow[batch], cur, tbeta, s, st));
-        DMP_CUDA(launch_ozaki_tc_grouped(dmats, dtiles, ntiles, cfg_bn(cfg), cfg_pair(cfg), tbeta, 0, cur, derr,
-                                         scratch, dcounter, st));
+        DMP_CUDA(launch_ozaki_tc_grouped(dmats, dtiles, ntiles, nmax, cfg_bn(cfg), cfg_pair(cfg), tbeta, s, 0, cur,
+                                         derr, area, dcounter, st));
         DMP_CUDA(launch_measure_grouped(dmats, batch, cur, dpart, cudaGraphConditionalHandle{}, 0, dactive, st));
         DMP_CUDA(launch_split_grouped(dmats, drow, batch, hrow[batch], 2, tbeta, s, st));
-        DMP_CUDA(launch_ozaki_tc_grouped(dmats, dtiles, ntiles, cfg_bn(cfg), cfg_pair(cfg), tbeta, 1, cur, derr,
-                                         scratch, dcounter, st));
+        DMP_CUDA(launch_ozaki_tc_grouped(dmats, dtiles, ntiles, nmax, cfg_bn(cfg), cfg_pair(cfg), tbeta, s, 1, cur,
+                                         derr, area, dcounter, st));
       }
       int active = 0;
       DMP_CUDA(cudaMemcpyAsync(&active, dactive, sizeof(int), cudaMemcpyDeviceToHost, st));
@@ -637,11 +640,11 @@ int dm_purify_batched(int32_t batch, const double* const* H, const int64_t* n, c
       DMP_CUDA(cudaGetLastError());
     }
     DMP_CUDA(launch_split_grouped(dmats, drow, batch, hrow[batch], 0, tbeta, refine, st));
-    DMP_CUDA(launch_ozaki_tc_grouped(dmats, dtiles, ntiles, cfg_bn(cfg), cfg_pair(cfg), tbeta, 0, 0, derr, scratch,
-                                     dcounter, st));
+    DMP_CUDA(launch_ozaki_tc_grouped(dmats, dtiles, ntiles, nmax, cfg_bn(cfg), cfg_pair(cfg), tbeta, refine, 0, 0, derr,
+                                     area, dcounter, st));
     DMP_CUDA(launch_split_grouped(dmats, drow, batch, hrow[batch], 2, tbeta, refine, st));
-    DMP_CUDA(launch_ozaki_tc_grouped(dmats, dtiles, ntiles, cfg_bn(cfg), cfg_pair(cfg), tbeta, 1, 0, derr, scratch,
-                                     dcounter, st));
+    DMP_CUDA(launch_ozaki_tc_grouped(dmats, dtiles, ntiles, nmax, cfg_bn(cfg), cfg_pair(cfg), tbeta, refine, 1, 0, derr,
+                                     area, dcounter, st));
     {
       // the grouped measures' partial sums of P' (buf[1]) give its P H sums
       // (no stopping rules: those would take P' for another iterate)

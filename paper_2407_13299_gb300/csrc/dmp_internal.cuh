@@ -118,16 +118,20 @@ cudaError_t launch_ozaki_imma(const int8_t* A, const int8_t* B, const int32_t* e
 // A planes [s][rows_a][k_pad], B planes [s][rows_b][k_pad] in bfloat16 (E4M3
 // bytes for beta 5); rows_a a multiple of 128, rows_b of 256, k_pad of 64
 // (128 for beta 5).
-// *err is set to 1 if a bounded device wait expired. `scratch` holds
-// tc_scratch_bytes() of per-CTA float64 partial sums (the kernel is persistent:
-// at most kTcMaxCtas CTAs, one per SM).
+// *err is set to 1 if a bounded device wait expired. k is the unpadded inner size.
 constexpr int kTcMaxCtas = 160;
-size_t tc_scratch_bytes();
-// workspace of the tcgen05 executor's split launches (the tiles' shared group sums and
-// counters); a launch given none runs whole tiles only
-size_t tc_split_bytes();
-// whether single-matrix tcgen05 products that fill at most half a wave of CTAs
-// are split into chunk units shared by every CTA; returns the previous setting
+// The tcgen05 executor's group sums (int64, per tile of a launch): `clean` bytes
+// from ptr on are zero between products (cleared at first use, then behind the
+// output step's reads); a new call starts with clean = 0.
+struct TcArea {
+  void* ptr;
+  size_t bytes, clean;
+};
+size_t tc_area_bytes();
+// zeroes the first `bytes` of the area as far as they are not known to be zero
+cudaError_t tc_area_clear(TcArea& a, size_t bytes, cudaStream_t st);
+// whether the last partial wave of a single-matrix tcgen05 product's tiles is cut
+// into chunk units shared by every CTA; returns the previous setting
 int set_tc_split_tiles(int enable);
 // beta = 7 single-matrix products on CTA pairs (2-SM MMA); returns the previous setting
 int set_tc_pairing(int enable);
@@ -138,9 +142,8 @@ bool tc_pairs_available();
 // bounds its waits by wait_limit_us (the bounded-wait test); one-shot.
 int set_stall_test(int wait_limit_us);
 cudaError_t launch_ozaki_tc(const void* A, const void* B, const int32_t* ea, const int32_t* eb, int64_t m,
-                            int64_t n, int64_t rows_a, int64_t rows_b, int64_t k_pad, int s, int beta, int sym,
-                            const EpiArgs& epi, const int* done, int* err, double* scratch, void* split_ws,
-                            cudaStream_t st);
+                            int64_t n, int64_t k, int64_t rows_a, int64_t rows_b, int64_t k_pad, int s, int beta,
+                            int sym, const EpiArgs& epi, const int* done, int* err, TcArea& area, cudaStream_t st);
 
 // FP64 executor: C = A B (A m x k, B k x n row-major) with the same epilogues.
 cudaError_t launch_gemm_f64(const double* A, int64_t lda, const double* B, int64_t ldb, int64_t m,
@@ -324,13 +327,15 @@ cudaError_t launch_measure_grouped(const BatchMat* mats, int nmats, int cur, dou
                                    cudaGraphConditionalHandle cond, int set_cond, int* active,
                                    cudaStream_t st);
 cudaError_t launch_finish_grouped(const BatchMat* mats, int nmats, cudaStream_t st);
-// phase 0: X2 = P P from buf[cur]; phase 1: update buf[cur] -> buf[1 - cur].
-// `counter` (one int of device memory) is zeroed on the stream before a
-// single-CTA launch; its CTAs take tiles from it in list order.
+// phase 0: X2 = P P from buf[cur]; phase 1: update buf[cur] -> buf[1 - cur], with
+// s-slice planes of matrices of at most nmax rows. `counter` (one int of device
+// memory) is zeroed on the stream before a single-CTA launch; its CTAs take
+// tiles from it in list order.
 // `pair`: CTA pairs on 256-row tiles (bn 256; the tiles' row blocks are 256
 // rows and the B maps have bn / 2-row boxes), else single CTAs on 128-row tiles.
-cudaError_t launch_ozaki_tc_grouped(const BatchMat* mats, const int4* tiles, int ntiles, int bn, bool pair, int beta,
-                                    int phase, int cur, int* err, double* scratch, int* counter, cudaStream_t st);
+cudaError_t launch_ozaki_tc_grouped(const BatchMat* mats, const int4* tiles, int ntiles, int64_t nmax, int bn,
+                                    bool pair, int beta, int s, int phase, int cur, int* err, TcArea& area,
+                                    int* counter, cudaStream_t st);
 
 }  // namespace dmp
 

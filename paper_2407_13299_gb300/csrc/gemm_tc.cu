@@ -12,22 +12,39 @@
 // 1024 * 128^2 = 2^24) or 65536 (beta = 5: 65536 * 16^2 = 2^24, so a whole
 // level is one chunk) K elements. Each chunk lands in one of two TMEM
 // accumulators; while the tensor core fills the other, eight epilogue warps
-// drain the finished one into exact int32 level sums in registers. Up to G
-// consecutive levels (G = 4 for beta 7 and 5, 3 for beta 8) are combined
-// exactly in int64 and the groups are added in float64 from L = s+1 down to 2
-// -- the same operation sequence as the definition, so the float64 result is
-// bit-for-bit the one the IMMA executor and the oracle produce.
+// drain the finished one into exact int32 sums in registers.
 //
-// CTA layout (320 threads, one CTA per SM):
-//   warp 0      TMA producer: A tile 128 x 64 and B tile BN x 64 bf16 per stage,
-//               128-byte swizzle, into a 4- or 6-stage shared-memory ring
+// A product runs as two kernels:
+//   ozaki_tc_kernel      the integer part. A program of slice-pair steps, cut
+//                        into segments, is run for every output tile; the
+//                        exact sum of a segment is added, times the segment's
+//                        power-of-two weights, to the tile's int64 group sums
+//                        in an L2-resident area (red.global.add.u64: nothing
+//                        comes back). Integer adds commute, so a tile's work
+//                        may be shared by any number of CTAs.
+//   ozaki_finish_kernel  the float64 part, spread over the whole GPU: the
+//                        group sums rounded to float64 in the order of the
+//                        definition, unscaled, the update applied and both
+//                        triangles written in full lines; the area is zeroed
+//                        behind the reads for the next product.
+// The output step used to run in the product kernel's epilogue, where one CTA
+// wrote its 128 x 256 part of a tile alone in 60-75 us while its tensor core
+// waited: at n = 256 (one tile) a product took 95 us, 85 of them in that step.
+// Up to G consecutive levels (G = 4 for beta 7 and 5, 3 for beta 8) form an
+// exact group; one or two groups are one exact integer, rounded once, and
+// three or more are added in float64 from L = s+1 down to 2 -- the operation
+// sequence of the definition, so the float64 result is bit-for-bit the one the
+// IMMA executor and the oracle produce.
+//
+// CTA layout of the product kernel (320 threads, one CTA per SM):
+//   warp 0      TMA producer: A tile 128 x 64 and B tile BN x 64 bf16 per K
+//               atom, 128-byte swizzle, into a shared-memory ring
 //   warp 1      TMEM owner and MMA issuer (one thread): 4 MMAs of K = 16 per
-//               stage, commits free the stage and publish finished chunks
+//               atom, commits free the stage and publish finished chunks
 //   warps 2..9  epilogue: warp w reads TMEM lanes 32 (w % 4) .. +31 (one output
 //               row per thread) and half of the BN columns
-// Output tile 128 x BN (BN = 256; 128 or 256 in the batched path). In
-// symmetric mode only tiles holding some element with row <= column run; each
-// element with row <= column is accumulated and written once, and mirrored.
+// In symmetric mode only tiles holding some element with row <= column run;
+// each element with row <= column is computed and written once, and mirrored.
 //
 // Every mbarrier wait is bounded by a %globaltimer deadline; on expiry the CTA
 // raises an error flag, drains what it has in flight (bounded again), frees
@@ -36,9 +53,11 @@
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
+#include <algorithm>
 #include <atomic>
 #include <cmath>
 #include <cstring>
+#include <vector>
 
 #include "dmp_internal.cuh"
 
@@ -57,36 +76,66 @@ constexpr int kTileRing = 4;  // WALK 2: tile indices the producer may announce 
 // PAIR: a cluster of two CTAs computes a 256 x BN tile with tcgen05.mma.cta_group::2;
 // each CTA stages its own 128 rows of A and half of the BN rows of B, and its
 // TMEM receives its 128 output rows with all BN columns.
-// A PAIR stage holds two 64-element K atoms of each operand (8 MMAs per stage
-// barrier round: with 4 the per-stage wait and commit left the tensor pipe
-// idle about a third of the time).
+// A stage holds one K atom (a 128-byte row) of each operand. The copies into the
+// SM bound the kernel: an atom of the pair kernel takes 646 clocks (51 bytes per
+// clock and SM, at any size and hit rate) against 512 of its MMAs. The ring is
+// cut fine so that most of it is in flight (with two atoms per stage and three
+// stages a product of n = 8192, s = 5 took 3.88 ms, now 3.69). Sharing the A
+// rows of two pairs by TMA multicast (a quarter fewer bytes from L2, the same
+// into the SMs) left the clocks per atom as they are.
 template <int BN, bool PAIR = false, bool F8 = false>
 struct TcCfg {
-  static constexpr int KSUB = PAIR ? 2 : 1;  // K atoms (128-byte rows) per stage
   static constexpr int ATOM_K = F8 ? 128 : TC_BK;  // K elements per atom
-  static constexpr int A_ATOM = TC_BM * TC_ROW_BYTES;
-  static constexpr int B_ATOM = (PAIR ? BN / 2 : BN) * TC_ROW_BYTES;
-  static constexpr int A_BYTES = KSUB * A_ATOM;
-  static constexpr int B_BYTES = KSUB * B_ATOM;
+  static constexpr int A_BYTES = TC_BM * TC_ROW_BYTES;
+  static constexpr int B_BYTES = (PAIR ? BN / 2 : BN) * TC_ROW_BYTES;
   static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
-  static constexpr int STAGES = PAIR ? 3 : (BN == 128 ? 6 : 4);
+  static constexpr int STAGES = PAIR ? 7 : (BN <= 128 ? 6 : 4);
   static constexpr int TMEM_COLS = 2 * BN;      // two fp32 chunk accumulators
   static constexpr int COLS = BN / 2;           // columns per epilogue thread
   static constexpr int BAR_BYTES = 256;
   static constexpr int SMEM = STAGES * STAGE_BYTES + BAR_BYTES + 1024;  // + alignment slack
+  static constexpr int BM = PAIR ? 2 * TC_BM : TC_BM;  // rows of a (pair) tile
+  static constexpr int RANKS = PAIR ? 2 : 1;
+  static constexpr int PART = TC_BM * BN;       // elements of one CTA's part of a tile
+};
+
+// The program of one output tile: steps (the product of plane a of A with
+// plane b of B over the whole K) in segments. A segment's exact sum goes, times
+// w[i], into the group sums g0 + i; consecutive segments with fold = 0 share
+// the weights of the next one and are folded together.
+constexpr int kMaxSegs = 32;
+constexpr int kMaxSteps = 96;
+constexpr int kMaxLaunchTiles = 160;  // single-matrix launches
+
+struct TcSeg {
+  int step0, nsteps;
+  int fold;  // the segment's sum (and those of the unfolded ones before it) is added to the groups
+  int g0;
+  long long w[3];
+};
+
+struct TcProgram {
+  int nsegs;
+  int ng;       // group sums per element
+  TcSeg seg[kMaxSegs];
+  unsigned char pa[kMaxSteps], pb[kMaxSteps];  // plane indices of the steps
+};
+
+struct TileAt {
+  unsigned short bi, bj;
 };
 
 struct TcParams {
-  int s, beta, KT, CH, ntiles;
+  int s, beta, KT, CH;
+  int tile0, ntiles;  // this launch's tiles: tile0 .. tile0 + ntiles - 1
+  int nwhole;         // tiles (of ntiles) walked whole, round robin; the rest are split over all CTAs (CTA pairs)
+  int units;          // fp32 chunks per tile (split launches: one matrix, every tile alike)
+  int parts;          // each split tile in this many equal ranges; 0: all split tiles' units in one sequence
   int group;        // levels combined exactly per int64 group: 4 (beta 7, 5) or 3 (beta 8)
-  double* scratch;  // per-CTA float64 partial sums, TC_BM * BN doubles per CTA
+  long long* area;  // group sums of the launch's tiles: [tile][CTA rank][group][PART]
   int64_t m, n;
   int64_t rows_a, rows_b;  // padded rows per digit plane
-  int sym, tiles_m, tiles_n;
-  // tile order: bands of band_w column blocks, each cut into groups of group_h
-  // row blocks, so the tiles in flight together form a near-square block and
-  // share their operand panels in L2 (band_w = 0: column-major order)
-  int band_w, group_h;
+  int sym;
   const int32_t* ea;
   const int32_t* eb;
   EpiArgs epi;
@@ -94,23 +143,28 @@ struct TcParams {
   int* err;
   unsigned long long timeout_ns;
   int stall_test;  // withhold each CTA's first stage (the bounded-wait test; see dmp_test_stall_next_product)
-  // split launches (fewer tiles than CTAs or CTA pairs): every tile is cut
-  // into split_unit_count units of one fp32 chunk, shared out in contiguous
-  // ranges over all CTAs (CTA pairs)
-  int split_unit_count;
   int* tile_counter;  // WALK 2: next tile to take (zeroed before the launch)
-  long long* split_area;  // per (tile, CTA rank in the pair): two TC_BM x BN int64 group sums
-  int* split_cnt;         // per (tile, rank, epilogue warp): contributors counted in
   // grouped mode (batched purification): tiles of many matrices in one launch
   const BatchMat* mats;  // nullptr: the single matrix above
   const int4* tiles;     // {matrix, bi, bj, 0}
   int phase;             // 0: X2 = P P;  1: P' = update(P, X2, P X2)
   int cur;               // the iterate is mats[.].buf[cur]
+  TcProgram prog;
+  // single-matrix launches: row and column block of each of the launch's tiles
+  // (a table: finding a tile's place in the order by counting took the finish
+  // kernel a thousand instructions per warp)
+  TileAt at[kMaxLaunchTiles];
 };
 
 // ---------------------------------------------------------------- PTX wrappers
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
+}
+// one lane of the (converged) warp, always the same
+__device__ __forceinline__ bool elect_one() {
+  uint32_t ok;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(ok));
+  return ok != 0;
 }
 __device__ __forceinline__ uint64_t globaltimer() {
   uint64_t t;
@@ -266,28 +320,12 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&v)[16]) {
 }
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
-// Scratch accesses with an L2 evict-last policy: the fold buffers are touched
-// once per level while gigabytes of operand tiles stream through L2.
+// L2 evict-last policy for the group sums: touched once per segment while
+// gigabytes of operand tiles stream through L2
 __device__ __forceinline__ uint64_t policy_evict_last() {
   uint64_t pol;
   asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(pol));
   return pol;
-}
-__device__ __forceinline__ void st_keep(void* p, long long v, uint64_t pol) {
-  asm volatile("st.global.L2::cache_hint.b64 [%0], %1, %2;" ::"l"(p), "l"(v), "l"(pol) : "memory");
-}
-// 64-bit load from L2 (.cg: not through this SM's L1, which may hold a line
-// from before a reduction at L2)
-__device__ __forceinline__ long long ld_l2(const void* p, uint64_t pol) {
-  long long v;
-  asm volatile("ld.global.cg.L2::cache_hint.b64 %0, [%1], %2;" : "=l"(v) : "l"(p), "l"(pol) : "memory");
-  return v;
-}
-__device__ __forceinline__ void prefetch_l1(const void* p) {
-  asm volatile("prefetch.global.L1 [%0];" ::"l"(p));
-}
-__device__ __forceinline__ void prefetch_l2(const void* p) {
-  asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
 }
 // 64-bit integer add performed at L2 (no value returned, so no round trip):
 // two's complement, so it adds signed values exactly
@@ -295,58 +333,78 @@ __device__ __forceinline__ void red_add_keep(void* p, long long v, uint64_t pol)
   asm volatile("red.global.add.L2::cache_hint.u64 [%0], %1, %2;" ::"l"(p), "l"(v), "l"(pol) : "memory");
 }
 
-// RN(h 2^sh + l) 2^e2 as a double, for integers |h|, |l| < 2^53, 0 <= sh < 64
-// and a normal result, by integer arithmetic alone: the exact sum is formed in
-// 128 bits, its leading 53 bits are rounded to nearest-even, and the exponent
-// and sign are set directly. This is the value float64 arithmetic gives for
-// double(h) 2^(sh + e2) + double(l) 2^e2 (both products exact, one rounding),
-// without the int64-to-double conversions and multiplies, which on this GPU
-// run on the narrow FP64 pipe.
-__device__ __forceinline__ double round_exact(long long h, int sh, long long l, int e2) {
-  // x = h 2^sh + l in two's complement (xh:xl)
-  const unsigned long long hl = static_cast<unsigned long long>(h) << sh;
-  unsigned long long xh = sh == 0 ? static_cast<unsigned long long>(h >> 63)
-                                  : static_cast<unsigned long long>(h >> (64 - sh));
-  const unsigned long long xl = hl + static_cast<unsigned long long>(l);
-  xh += static_cast<unsigned long long>(l >> 63) + (xl < hl ? 1ull : 0ull);
-  const bool neg = static_cast<long long>(xh) < 0;
-  // magnitude (mh:ml)
-  const unsigned long long ml = neg ? ~xl + 1ull : xl;
-  const unsigned long long mh = neg ? ~xh + (ml == 0 ? 1ull : 0ull) : xh;
-  if ((mh | ml) == 0) return 0.0;
-  int msb = mh != 0 ? 127 - __clzll(static_cast<long long>(mh)) : 63 - __clzll(static_cast<long long>(ml));
-  unsigned long long mant;
-  if (msb <= 52) {
-    mant = ml << (52 - msb);  // exact (mh is zero)
-  } else {
-    const int r = msb - 52;  // 1 .. 63: the dropped bits all lie in ml
-    mant = (ml >> r) | (r == 0 ? 0ull : mh << (64 - r));
-    const unsigned long long rem = ml & ((1ull << r) - 1ull);
-    const unsigned long long half = 1ull << (r - 1);
-    if (rem > half || (rem == half && (mant & 1ull))) {
-      ++mant;
-      if (mant >> 53) {
-        mant >>= 1;
-        ++msb;
-      }
+// RN(x) 2^e as a double for the signed 96-bit integer x = (w2:w1:w0), rounded to
+// nearest even: the value of the float64 expression in which x is the exact sum
+// of its groups. Integer operations only: float64 conversions, multiplies and
+// adds run on this GPU's narrow FP64 pipe (two lanes per clock and SM), which
+// bound the finish kernel at 83 % of its issue rate when it used them.
+__device__ __forceinline__ double round_words(uint32_t w0, uint32_t w1, uint32_t w2, int e) {
+  const uint32_t neg = static_cast<uint32_t>(static_cast<int32_t>(w2) >> 31);  // all ones when negative
+  // magnitude: (x ^ neg) - neg
+  uint32_t a0 = w0 ^ neg, a1 = w1 ^ neg, a2 = w2 ^ neg;
+  asm("add.cc.u32 %0, %0, %3;\n\taddc.cc.u32 %1, %1, 0;\n\taddc.u32 %2, %2, 0;"
+      : "+r"(a0), "+r"(a1), "+r"(a2)
+      : "r"(neg & 1u));
+  // leading zeros, then the magnitude shifted so that its top bit is bit 95
+  int lz = 0;
+  if (a2 == 0) {
+    a2 = a1;
+    a1 = a0;
+    a0 = 0;
+    lz = 32;
+    if (a2 == 0) {
+      a2 = a1;
+      a1 = 0;
+      lz = 64;
+      if (a2 == 0) return 0.0;
     }
   }
-  const unsigned long long bits = (neg ? (1ull << 63) : 0ull) |
-                                  (static_cast<unsigned long long>(msb + e2 + 1023) << 52) |
-                                  (mant & ((1ull << 52) - 1ull));
-  return __longlong_as_double(static_cast<long long>(bits));
+  const int z = __clz(static_cast<int>(a2));
+  lz += z;
+  a2 = __funnelshift_l(a1, a2, z);
+  a1 = __funnelshift_l(a0, a1, z);
+  a0 <<= z;
+  // 53 bits: a2 and the top 21 bits of a1; the rest rounds to nearest even
+  const uint32_t rest = (a1 << 21) | (a0 != 0 ? 1u : 0u);
+  uint32_t lo = (a2 << 21) | (a1 >> 11), hi = a2 >> 11;
+  const uint32_t up = (rest > 0x80000000u || (rest == 0x80000000u && (lo & 1u))) ? 1u : 0u;
+  const int E = 95 - lz + e + 1023;  // biased exponent before rounding
+  // the leading one (bit 20 of hi) adds one to the exponent field, and so does a carry out of the fraction
+  hi += static_cast<uint32_t>(E - 1) << 20;
+  asm("add.cc.u32 %0, %0, %2;\n\taddc.u32 %1, %1, 0;" : "+r"(lo), "+r"(hi) : "r"(up));
+  if (E < 1 || E > 2045) {
+    // outside the normal range: the rounded integer scaled by ldexp
+    uint32_t l0 = (a2 << 21) | (a1 >> 11), h0 = (a2 >> 11) + (static_cast<uint32_t>(95 - lz + 1022) << 20);
+    asm("add.cc.u32 %0, %0, %2;\n\taddc.u32 %1, %1, 0;" : "+r"(l0), "+r"(h0) : "r"(up));
+    const double v = ldexp(__hiloint2double(static_cast<int>(h0), static_cast<int>(l0)), e);
+    return neg ? -v : v;
+  }
+  return __hiloint2double(static_cast<int>(hi | (neg & 0x80000000u)), static_cast<int>(lo));
 }
 
-// RN(h 2^sh + l) as a double (unscaled), for integers |h|, |l| < 2^53 and
-// 0 <= sh < 64: when the exact sum fits in 63 bits (|h| < 2^(62 - sh), always
-// so for a last group of one level) it is formed in int64 and converted with
-// one correctly rounded conversion; otherwise round_exact forms it in 128 bits.
-// Either way the value is that of the float64 expression.
-__device__ __forceinline__ double round_sum(long long h, int sh, long long l) {
-  const long long lim = 1ll << (62 - sh);
-  if (h > -lim && h < lim)
-    return __ll2double_rn(static_cast<long long>(static_cast<unsigned long long>(h) << sh) + l);
-  return round_exact(h, sh, l, 0);
+// The same for a signed 64-bit integer x = (w1:w0), without branches, so that
+// the elements of a thread overlap. `slow` is raised (and the value to be taken
+// from round_words) when the result is not a normal number.
+__device__ __forceinline__ double round_fast2(uint32_t w0, uint32_t w1, int e, bool& slow) {
+  const uint32_t neg = static_cast<uint32_t>(static_cast<int32_t>(w1) >> 31);
+  uint32_t a0 = w0 ^ neg, a1 = w1 ^ neg;
+  asm("add.cc.u32 %0, %0, %2;\n\taddc.u32 %1, %1, 0;" : "+r"(a0), "+r"(a1) : "r"(neg & 1u));
+  const bool small = a1 == 0;
+  a1 = small ? a0 : a1;
+  a0 = small ? 0u : a0;
+  const int z = __clz(static_cast<int>(a1));  // 32 for zero
+  const bool zero = a1 == 0;
+  a1 = __funnelshift_l(a0, a1, z);
+  a0 <<= z & 31;
+  uint32_t lo = (a1 << 21) | (a0 >> 11), hi = a1 >> 11;
+  // up on more than half, or on half with an odd last bit
+  const uint32_t up = ((a0 & 0x7ffu) + (lo & 1u)) > 0x400u ? 1u : 0u;
+  const int E = (small ? 31 : 63) - z + e + 1023;  // biased exponent before rounding
+  slow |= !zero && static_cast<uint32_t>(E - 1) > 2044u;
+  hi += static_cast<uint32_t>(E - 1) << 20;
+  asm("add.cc.u32 %0, %0, %2;\n\taddc.u32 %1, %1, 0;" : "+r"(lo), "+r"(hi) : "r"(up));
+  hi |= neg & 0x80000000u;
+  return __hiloint2double(zero ? 0 : static_cast<int>(hi), zero ? 0 : static_cast<int>(lo));
 }
 
 // x 2^e for a finite double: exponent arithmetic when the result stays normal,
@@ -400,137 +458,317 @@ __device__ __forceinline__ bool wait_bar(uint32_t bar, uint32_t parity, volatile
     }
   }
 }
-
-__device__ __forceinline__ int npairs_of(int L, int s) { return min(s, L - 1) - max(1, L - s) + 1; }
-
-// Row blocks of column block c that hold tiles (symmetric: some element with row <= column).
-template <int BN, int BM>
-__device__ __forceinline__ int rows_of_col(const TcParams& p, int c) {
-  return p.sym ? min(p.tiles_m, (BN * (c + 1)) / BM) : p.tiles_m;
-}
-
-// Row block bi (BM rows: 128, or 256 for a CTA pair) and column block bj of tile idx.
-template <int BN, int BM>
-__device__ __forceinline__ void tile_of(const TcParams& p, int idx, int& bi, int& bj) {
-  if (p.band_w > 0) {
-    const int W = p.band_w, H = p.group_h;
-    for (int c0 = 0; c0 < p.tiles_n; c0 += W) {
-      const int c1 = min(p.tiles_n, c0 + W);
-      const int rmax = rows_of_col<BN, BM>(p, c1 - 1);  // nondecreasing in the column
-      for (int r0 = 0; r0 < rmax; r0 += H) {
-        const int r1 = min(rmax, r0 + H);
-        for (int c = c0; c < c1; ++c) {
-          const int k = max(0, min(rows_of_col<BN, BM>(p, c), r1) - r0);
-          if (idx < k) {
-            bi = r0 + idx;
-            bj = c;
-            return;
-          }
-          idx -= k;
-        }
-      }
-    }
-    bi = bj = 0;  // not reached for idx < ntiles
-    return;
-  }
-  if (!p.sym) {
-    bj = idx / p.tiles_m;  // column-block major: CTAs running together share B blocks
-    bi = idx % p.tiles_m;
-    return;
-  }
-  bj = 0;
-  for (;;) {
-    const int cnt = min(p.tiles_m, (BN * (bj + 1)) / BM);
-    if (idx < cnt) break;
-    idx -= cnt;
-    ++bj;
-  }
-  bi = idx;
-}
-
-// Everything one output tile needs: operands, sizes and the output step.
+// Where one CTA's part of an output tile lies and what feeds it.
 struct Job {
   const CUtensorMap* ta;
   const CUtensorMap* tb;
-  int64_t m0, n0, rows_a, rows_b, m, n;
-  int s, KT;
-  const int32_t* ea;
-  const int32_t* eb;
-  bool skip, sym;
-  EpiArgs epi;
+  int64_t m0, n0, rows_a, rows_b;
+  int KT;
+  bool skip;
 };
 
+// tile: counted from the launch's first (tile0).
 // PAIR: tile is a 256-row pair tile and this CTA (rank 0 or 1) takes rows
 // 128 rank .. 128 rank + 127 of it.
-template <int BN, bool PAIR = false>
+template <int BN, bool PAIR>
 __device__ __forceinline__ Job job_of(const TcParams& p, const CUtensorMap* tmA, const CUtensorMap* tmB, int tile,
-                                      uint32_t rank = 0) {
+                                      uint32_t rank) {
+  constexpr int BM = TcCfg<BN, PAIR>::BM;
   Job j;
   if (p.mats == nullptr) {
-    int bi, bj;
-    tile_of<BN, PAIR ? 2 * TC_BM : TC_BM>(p, tile, bi, bj);
     j.ta = tmA;
     j.tb = tmB;
-    j.m0 = static_cast<int64_t>(bi) * (PAIR ? 2 * TC_BM : TC_BM) + TC_BM * static_cast<int64_t>(rank);
-    j.n0 = static_cast<int64_t>(bj) * BN;
+    j.m0 = static_cast<int64_t>(p.at[tile].bi) * BM + TC_BM * static_cast<int64_t>(rank);
+    j.n0 = static_cast<int64_t>(p.at[tile].bj) * BN;
     j.rows_a = p.rows_a;
     j.rows_b = p.rows_b;
-    j.m = p.m;
-    j.n = p.n;
-    j.s = p.s;
     j.KT = p.KT;
-    j.ea = p.ea;
-    j.eb = p.eb;
     j.skip = false;
-    j.sym = p.sym != 0;
-    j.epi = p.epi;
     return j;
   }
-  const int4 t = p.tiles[tile];
+  const int4 t = p.tiles[p.tile0 + tile];
   const BatchMat& M = p.mats[t.x];
-  // row block t.y of 128 rows, or of 256 for a CTA pair (this CTA: half `rank`)
-  j.m0 = static_cast<int64_t>(t.y) * (PAIR ? 2 * TC_BM : TC_BM) + TC_BM * static_cast<int64_t>(rank);
+  j.m0 = static_cast<int64_t>(t.y) * BM + TC_BM * static_cast<int64_t>(rank);
   j.n0 = static_cast<int64_t>(t.z) * BN;
   j.rows_a = M.n_pad;
   j.rows_b = M.n_pad;
-  j.m = M.n;
-  j.n = M.n;
-  j.s = M.s;
   j.KT = static_cast<int>(M.k_pad / (p.beta == 5 ? 128 : TC_BK));  // K atoms of 128 bytes
   j.skip = M.state->done != 0;
-  j.sym = true;
   j.ta = &M.tmPa;
-  j.ea = M.expsP;
-  j.epi.state = M.state;
-  j.epi.levels = nullptr;
-  j.epi.round32 = 0;
-  if (p.phase == 0) {
-    j.tb = &M.tmPb;
-    j.eb = M.expsP;
-    j.epi.kind = EPI_SYM_STORE;
-    j.epi.C = M.X2;
-    j.epi.ldc = M.n;
-    j.epi.P = nullptr;
-    j.epi.X2 = nullptr;
-    j.epi.ldp = M.n;
-    j.epi.ldx = M.n;
-  } else {
-    j.tb = &M.tmXb;
-    j.eb = M.expsX;
-    j.epi.kind = EPI_PM_UPDATE;
-    j.epi.P = M.buf[p.cur];
-    j.epi.ldp = p.cur == 0 ? M.ldp : M.n;
-    j.epi.X2 = M.X2;
-    j.epi.ldx = M.n;
-    j.epi.C = M.buf[1 - p.cur];
-    j.epi.ldc = p.cur == 0 ? M.n : M.ldp;
-  }
+  j.tb = p.phase == 0 ? &M.tmPb : &M.tmXb;
   return j;
 }
 
-// Persistent: one CTA per SM walks tiles blockIdx.x, blockIdx.x + gridDim.x, ...
-// The three roles keep their ring and buffer phases across tiles, so the next
-// tile's loads and MMAs overlap the current tile's last fold and output.
+// Three groups: scaled and added in float64 from the smallest up. Not inlined:
+// the compiler would compute it for every element and drop it (six FP64
+// operations, which bound the finish kernel at one group per element).
+__device__ __noinline__ double add_groups(long long t0, long long t1, long long t2, int e_sum, int step, int e) {
+  const double d0 = static_cast<double>(t0) * ldexp(1.0, e_sum);
+  const double d1 = d0 + static_cast<double>(t1) * ldexp(1.0, e_sum + step);
+  const double d2 = d1 + static_cast<double>(t2) * ldexp(1.0, e_sum + 2 * step);
+  return scale_pow2(d2, e);
+}
+
+// Four consecutive doubles or int64 group sums, in 16-byte pieces when the
+// address allows (`vec`), else one by one at immediate offsets.
+__device__ __forceinline__ void load4(double (&v)[4], const double* __restrict__ a, bool vec) {
+  if (vec) {
+    const double2 x = reinterpret_cast<const double2*>(a)[0], y = reinterpret_cast<const double2*>(a)[1];
+    v[0] = x.x, v[1] = x.y, v[2] = y.x, v[3] = y.y;
+  } else {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) v[i] = a[i];
+  }
+}
+__device__ __forceinline__ void store4(double* a, const double (&v)[4], bool vec) {
+  if (vec) {
+    reinterpret_cast<double2*>(a)[0] = make_double2(v[0], v[1]);
+    reinterpret_cast<double2*>(a)[1] = make_double2(v[2], v[3]);
+  } else {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) a[i] = v[i];
+  }
+}
+
+// The float64 part of a product, one CTA per 32 x 32 block of a tile, four rows
+// of a column per thread and pass. The group sums lie as [column][row], P and
+// P^2 are exactly symmetric (read at (column, row)) and the mirrored elements
+// are four in a row too, so every array costs a thread one address and 16-byte
+// accesses; the row-major elements go through shared memory for the same
+// reason. n = 4096: 0.06 ms beside 0.5 ms of products, n = 1024: 6 beside 29 us.
+// (Done instead by two further warps of the next wave's product kernel it cost
+// 3 % of the whole: 200 us per wave of 76 tiles on so few threads, and the
+// shared memory of a seventh stage.)
+// UPD: the PM update (EPI_PM_UPDATE). NG: group sums per element (0: EPI_LEVELS).
+constexpr int FIN_THREADS = 128;
+
+template <int BN, bool PAIR, bool UPD, int NG>
+__global__ void __launch_bounds__(FIN_THREADS)
+ozaki_finish_kernel(const __grid_constant__ TcParams p) {
+  if (p.done != nullptr && *p.done) return;
+  __shared__ double trans[32][33];
+  using Cfg = TcCfg<BN, PAIR>;
+  constexpr int SR = Cfg::BM / 32, SC = BN / 32;
+  constexpr int LINES = FIN_THREADS / 8, PASSES = 32 / LINES;  // lines of a block per pass
+  const int q4 = 4 * (threadIdx.x & 7), line0 = threadIdx.x >> 3;  // four entries of lines line0, line0 + LINES, ..
+  const bool sym = p.sym != 0;
+  const int e_sum = -p.beta * (p.s + 1);
+
+  const int tile = blockIdx.x / (SR * SC);
+  const int sub = blockIdx.x % (SR * SC);
+  const int sr = sub % SR, sc = sub / SR;
+  const int rank = sr / 4;
+  const int h = 32 * sc / Cfg::COLS;
+  const int e = 4 * h + ((sr + 2) & 3);  // the epilogue warp that owns these rows and columns
+
+  // the tile's place and its output step
+  int m0, n0, m = static_cast<int>(p.m), n = static_cast<int>(p.n);
+  const int32_t* ea = p.ea;
+  const int32_t* eb = p.eb;
+  EpiArgs epi = p.epi;
+  if (p.mats == nullptr) {
+    m0 = p.at[tile].bi * Cfg::BM;
+    n0 = p.at[tile].bj * BN;
+  } else {
+    const int4 t = p.tiles[p.tile0 + tile];
+    const BatchMat& M = p.mats[t.x];
+    if (M.state->done) return;
+    m0 = t.y * Cfg::BM;
+    n0 = t.z * BN;
+    m = n = static_cast<int>(M.n);
+    ea = M.expsP;
+    epi.state = M.state;
+    if (!UPD) {
+      eb = M.expsP;
+      epi.C = M.X2;
+      epi.ldc = M.n;
+    } else {
+      eb = M.expsX;
+      epi.P = M.buf[p.cur];
+      epi.ldp = p.cur == 0 ? M.ldp : M.n;
+      epi.X2 = M.X2;
+      epi.ldx = M.n;
+      epi.C = M.buf[1 - p.cur];
+      epi.ldc = p.cur == 0 ? M.n : M.ldp;
+    }
+  }
+  const int r0 = m0 + 32 * sr, c0 = n0 + 32 * sc;
+  const int r = r0 + q4;  // this thread's first row
+  // nothing of this block is written: outside the matrix, or below the diagonal
+  const bool none = r0 >= m || c0 >= n || (sym && r0 > c0 + 31);
+  long long* part0 = p.area + (static_cast<int64_t>(tile) * Cfg::RANKS + rank) * (NG == 0 ? p.prog.ng : NG) * Cfg::PART +
+                     (e * (Cfg::COLS * 32) + (32 * sc - h * Cfg::COLS + line0) * 32 + q4);
+  const bool vec = (epi.ldc & 1) == 0 && (reinterpret_cast<uintptr_t>(epi.C) & 15) == 0;
+
+  if constexpr (NG == 0) {
+    // test hook: group g holds the exact sum of level g + 2
+    for (int pass = 0; pass < PASSES; ++pass) {
+      const int c = c0 + line0 + LINES * pass;
+      for (int g = 0; g < p.prog.ng; ++g) {
+        long long* part = part0 + g * Cfg::PART + pass * (LINES * 32);
+        for (int t = 0; t < 4; ++t) {
+          if (r + t < m && c < n)
+            epi.levels[(static_cast<int64_t>(g) * m + r + t) * n + c] = static_cast<int32_t>(part[t]);
+          part[t] = 0;
+        }
+      }
+    }
+    return;
+  }
+
+  const double wa = UPD ? epi.state->alpha : 0.0;
+  const double w2 = UPD ? epi.state->b2 : 0.0;
+  const double w3 = UPD ? epi.state->b3 : 0.0;
+  // every load of the block before the first store, so that a thread waits
+  // for one round of latencies per block
+  constexpr int G = NG == 0 ? 1 : NG;
+  long long T[PASSES][G][4];
+  double pv[PASSES][4], xv[PASSES][4];
+  int32_t ec[PASSES];
+  int4 er4 = make_int4(0, 0, 0, 0);
+  if (r < m) er4 = *reinterpret_cast<const int4*>(ea + r);  // (the exponent arrays are padded to 256 rows)
+  const int32_t er[4] = {er4.x, er4.y, er4.z, er4.w};
+  const double* pp = UPD ? epi.P + (c0 + line0) * epi.ldp + r : nullptr;
+  const double* xp = UPD ? epi.X2 + (c0 + line0) * epi.ldx + r : nullptr;
+  const bool vecp = UPD && (epi.ldp & 1) == 0 && (reinterpret_cast<uintptr_t>(epi.P) & 15) == 0;
+  const bool vecx = UPD && (epi.ldx & 1) == 0 && (reinterpret_cast<uintptr_t>(epi.X2) & 15) == 0;
+#pragma unroll
+  for (int pass = 0; pass < PASSES; ++pass) {
+    const int c = c0 + line0 + LINES * pass;
+#pragma unroll
+    for (int g = 0; g < NG; ++g) {
+      const longlong2* a = reinterpret_cast<const longlong2*>(part0 + g * Cfg::PART + pass * (LINES * 32));
+      const longlong2 x = a[0], y = a[1];
+      T[pass][g][0] = x.x, T[pass][g][1] = x.y, T[pass][g][2] = y.x, T[pass][g][3] = y.y;
+    }
+    ec[pass] = c < n ? eb[c] : 0;
+    if (UPD) {
+      // the rows of this column that are written: inside the matrix, and not below the diagonal
+      const int rows = c < n ? min(sym ? c + 1 : m, m) - r : 0;
+      const double* pc = pp + static_cast<int64_t>(LINES * pass) * epi.ldp;
+      const double* xc = xp + static_cast<int64_t>(LINES * pass) * epi.ldx;
+#pragma unroll
+      for (int t = 0; t < 4; ++t) pv[pass][t] = xv[pass][t] = 0.0;
+      if (rows >= 4) {
+        load4(pv[pass], pc, vecp);
+        load4(xv[pass], xc, vecx);
+      } else {
+#pragma unroll
+        for (int t = 0; t < 3; ++t) {
+          if (t < rows) {
+            pv[pass][t] = pc[t];
+            xv[pass][t] = xc[t];
+          }
+        }
+      }
+    }
+  }
+#pragma unroll
+  for (int pass = 0; pass < PASSES; ++pass) {
+#pragma unroll
+    for (int g = 0; g < NG; ++g) {
+      longlong2* a = reinterpret_cast<longlong2*>(part0 + g * Cfg::PART + pass * (LINES * 32));
+      a[0] = a[1] = make_longlong2(0, 0);
+    }
+  }
+  if (none) return;
+#pragma unroll
+  for (int pass = 0; pass < PASSES; ++pass) {
+    const int line = line0 + LINES * pass;
+    const int c = c0 + line;
+    const int rows = c < n ? min(sym ? c + 1 : m, m) - r : 0;  // t < rows
+    double v[4];
+    // one or two groups: the exact integer T_1 2^(beta G) + T_0 rounded once and
+    // scaled by 2^(-beta (s+1)) (exact); three: the groups scaled and added in
+    // float64 from the smallest up
+    bool slow = ec[pass] == kBadExp;
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      slow |= er[t] == kBadExp;
+      if (NG == 1) {
+        v[t] = round_fast2(static_cast<uint32_t>(T[pass][0][t]), static_cast<uint32_t>(T[pass][0][t] >> 32),
+                           er[t] + ec[pass] + e_sum, slow);
+      } else {
+        slow = true;
+      }
+    }
+    if (NG != 1 || slow) {
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        const int ee = er[t] + ec[pass];
+        const long long t0 = T[pass][0][t], t1 = T[pass][NG > 1 ? 1 : 0][t], t2 = T[pass][NG > 2 ? 2 : 0][t];
+        const uint32_t l0 = static_cast<uint32_t>(t0), h0 = static_cast<uint32_t>(t0 >> 32);
+        const uint32_t x0 = static_cast<uint32_t>(static_cast<int32_t>(h0) >> 31);
+        if (NG == 1) {
+          v[t] = round_words(l0, h0, x0, ee + e_sum);
+        } else if (NG == 2) {
+          // T_1 shifted by beta G = 20 .. 28 bits, plus T_0 (|T| < 2^53 each)
+          const int sh = p.beta * p.group;
+          const uint32_t l1 = static_cast<uint32_t>(t1), h1 = static_cast<uint32_t>(t1 >> 32);
+          const uint32_t x1 = static_cast<uint32_t>(static_cast<int32_t>(h1) >> 31);
+          uint32_t w0 = l1 << sh, w1 = __funnelshift_l(l1, h1, sh), w2s = __funnelshift_l(h1, x1, sh);
+          asm("add.cc.u32 %0, %0, %3;\n\taddc.cc.u32 %1, %1, %4;\n\taddc.u32 %2, %2, %5;"
+              : "+r"(w0), "+r"(w1), "+r"(w2s)
+              : "r"(l0), "r"(h0), "r"(x0));
+          v[t] = round_words(w0, w1, w2s, ee + e_sum);
+        } else {
+          v[t] = add_groups(t0, t1, t2, e_sum, p.beta * p.group, ee);
+        }
+        if (er[t] == kBadExp || ec[pass] == kBadExp) v[t] = __longlong_as_double(0x7ff8000000000000ll);
+      }
+    }
+    if (UPD) {
+#pragma unroll
+      for (int t = 0; t < 4; ++t) v[t] = wa * pv[pass][t] + w2 * xv[pass][t] + w3 * v[t];
+    }
+    if (epi.round32 != 0) {
+      // stored_value; volatile, so that without the flag the two conversions
+      // (FP64 pipe) are branched over instead of being computed and dropped
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        float f;
+        asm volatile("cvt.rn.f32.f64 %0, %1;" : "=f"(f) : "d"(v[t]));
+        asm volatile("cvt.f64.f32 %0, %1;" : "=d"(v[t]) : "f"(f));
+      }
+    }
+#pragma unroll
+    for (int t = 0; t < 4; ++t) trans[line][q4 + t] = v[t];
+    if (sym && rows > 0) {
+      double* mirror = epi.C + c * epi.ldc + r;
+      if (rows >= 4) {
+        store4(mirror, v, vec);
+      } else {
+#pragma unroll
+        for (int t = 0; t < 3; ++t)
+          if (t < rows) mirror[t] = v[t];
+      }
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int pass = 0; pass < PASSES; ++pass) {
+    // row r0 + line, columns c0 + q4 .. + 3 (symmetric: right of the diagonal)
+    const int line = line0 + LINES * pass;
+    const int rr = r0 + line, cc = c0 + q4;
+    if (rr >= m) continue;
+    const int first = sym ? rr + 1 - cc : 0;  // first column of the four that is written
+    double* out = epi.C + rr * epi.ldc + cc;
+    double v[4];
+#pragma unroll
+    for (int t = 0; t < 4; ++t) v[t] = trans[q4 + t][line];
+    if (first <= 0 && cc + 4 <= n) {
+      store4(out, v, vec);
+    } else {
+#pragma unroll
+      for (int t = 0; t < 4; ++t)
+        if (t >= first && cc + t < n) out[t] = v[t];
+    }
+  }
+}
+
+// Persistent: each CTA (CTA pair) walks its share of the launch's tiles. The
+// three roles keep their ring and buffer phases across tiles, so the next
+// tile's loads and MMAs overlap the current tile's last adds.
 //
 // PAIR (launched as clusters of two CTAs): the cluster walks 256-row pair
 // tiles. Each CTA loads its A rows and its half of the B rows, signalling the
@@ -539,22 +777,20 @@ __device__ __forceinline__ Job job_of(const TcParams& p, const CUtensorMap* tmA,
 // CTAs; both epilogues release a TMEM buffer on the leader's barrier.
 //
 // WALK: how the CTAs share the launch's tiles.
-//   0  each CTA (pair) takes tiles cta, cta + #CTAs, ... (the single-matrix products)
+//   0  the first p.nwhole tiles whole, round robin; the others (less than one
+//      per CTA or CTA pair) are cut into units of one exact fp32 chunk and
+//      shared out evenly, in contiguous ranges, over every CTA, so that no
+//      last wave is left half empty. The group sums are integers: the result
+//      does not depend on the split.
 //   2  each CTA takes the next tile from a counter in global memory (the
 //      grouped launches of the batched purification, whose tiles differ in
 //      work: listed largest first, taken as CTAs free up); the producer takes
 //      the tile and passes its index to the MMA and epilogue warps through a
 //      small ring in shared memory
-//   1  (split) the launch's tiles fill at most half a wave of CTAs (CTA pairs), so
-// they are all cut into units of one exact fp32 chunk and shared out evenly in
-// contiguous ranges over every CTA; each range's partial level sums are added
-// at L2 into the tiles' shared group sums, and the last contributor to a tile
-// writes its output. Integer sums do not depend on the split: the result is
-// bit-for-bit that of whole tiles.
 template <int BN, bool PAIR, bool F8 = false, int WALK = 0>
 __global__ void __launch_bounds__(TC_THREADS, 1)
 ozaki_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-                const TcParams p) {
+                const __grid_constant__ TcParams p) {
   using Cfg = TcCfg<BN, PAIR, F8>;
   if (p.done != nullptr && *p.done) return;  // uniform: the whole CTA leaves before any setup
   extern __shared__ uint8_t smem_raw[];
@@ -620,28 +856,39 @@ ozaki_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
 
-  const int CH = p.CH;
+  const int CHS = p.CH;  // stages per fp32 chunk
 
-  // WALK 1: this CTA's contiguous range [u_begin, u_end) of the launch's chunk
-  // units (p.split_unit_count per tile, all tiles split)
-  const int KTS_ = p.KT / Cfg::KSUB;  // stages per slice pair (single-matrix launches)
-  const int CHS_ = CH / Cfg::KSUB;    // stages per fp32 chunk
-  const int64_t split_units = WALK == 1 ? static_cast<int64_t>(p.ntiles) * p.split_unit_count : 0;
-  const int64_t u_begin = split_units * cta_id / cta_stride;
-  const int64_t u_end = split_units * (cta_id + 1) / cta_stride;
-  // unit u: its tile tt, level L and stage range [kb0, kb1)
-  auto split_unit = [&](int64_t u, int& tt, int& L, int& kb0, int& kb1) __attribute__((always_inline)) {
-    tt = static_cast<int>(u / p.split_unit_count);
-    int w = static_cast<int>(u % p.split_unit_count);
-    for (L = p.s + 1; L > 2; --L) {
-      const int nkb = npairs_of(L, p.s) * KTS_;
-      const int nch = (nkb + CHS_ - 1) / CHS_;
-      if (w < nch) break;
-      w -= nch;
+  // WALK 0: this CTA's items. Items 0 .. nfull - 1 are whole tiles; after them
+  // come the tiles its range [u_begin, u_end) of the split tiles' units meets.
+  const int nfull = p.nwhole > cta_id ? (p.nwhole - cta_id - 1) / cta_stride + 1 : 0;
+  const int nsplit = p.ntiles - p.nwhole;
+  int64_t u_begin, u_end;
+  if (p.parts > 0) {
+    const int part = cta_id / max(nsplit, 1);
+    const int64_t base = static_cast<int64_t>(cta_id - part * nsplit) * p.units;
+    u_begin = base + p.units * min(part, p.parts) / p.parts;
+    u_end = base + p.units * min(part + 1, p.parts) / p.parts;
+  } else {
+    const int64_t split_units = static_cast<int64_t>(nsplit) * p.units;
+    u_begin = split_units * cta_id / cta_stride;
+    u_end = split_units * (cta_id + 1) / cta_stride;
+  }
+  const int split_lo = u_begin < u_end ? static_cast<int>(u_begin / p.units) : 0;
+  // item `it`: its tile (counted from tile0) and unit range [u0, u1); false past the last
+  auto static_item = [&](int it, int& tile, int& u0, int& u1) __attribute__((always_inline)) -> bool {
+    if (it < nfull) {
+      tile = cta_id + it * cta_stride;
+      u0 = 0;
+      u1 = 0x7fffffff;
+      return true;
     }
-    const int nkb = npairs_of(L, p.s) * KTS_;
-    kb0 = w * CHS_;
-    kb1 = min(kb0 + CHS_, nkb);
+    const int tt = split_lo + (it - nfull);
+    const int64_t base = static_cast<int64_t>(tt) * p.units;
+    if (u_begin >= u_end || base >= u_end) return false;
+    tile = p.nwhole + tt;
+    u0 = static_cast<int>(u_begin > base ? u_begin - base : 0);
+    u1 = static_cast<int>(u_end - base < p.units ? u_end - base : p.units);
+    return true;
   };
 
   if (warp == 0) {
@@ -658,11 +905,11 @@ ozaki_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
       const uint32_t full_target0 = PAIR ? map_to_cta(full_bar(0), 0) : full_bar(0);
       const uint32_t expect_bytes = PAIR ? 2u * Cfg::STAGE_BYTES : static_cast<uint32_t>(Cfg::STAGE_BYTES);
       const int b_off = PAIR ? static_cast<int>(rank) * (BN / 2) : 0;  // this CTA's half of the B rows
-      // one stage: slice pair (i, j), K atoms kt .. kt + KSUB - 1
-      auto put_stage = [&](const Job& jb, int i, int j, int kt) __attribute__((always_inline)) -> bool {
+      // one stage: K atom kt of planes pa of A and pb of B
+      auto put_stage = [&](const Job& jb, int pa, int pb, int kt) __attribute__((always_inline)) -> bool {
         if (!wait_bar<PAIR>(empty_bar(stage), phase ^ 1u, abort_flag, p)) return false;
-        const int ya = static_cast<int>((i - 1) * jb.rows_a + jb.m0);
-        const int yb = static_cast<int>((j - 1) * jb.rows_b + jb.n0) + b_off;
+        const int ya = static_cast<int>(pa * jb.rows_a + jb.m0);
+        const int yb = static_cast<int>(pb * jb.rows_b + jb.n0) + b_off;
         const uint32_t sa = sbase + stage * Cfg::STAGE_BYTES;
         if (p.stall_test && !withheld) {
           // stall test: neither the expected bytes nor the copies of this CTA's
@@ -674,11 +921,8 @@ ozaki_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
           if (PAIR) {
             const uint32_t fb = full_target0 + 8u * stage;
             if (leader) mbar_arrive_expect_tx(full_bar(stage), expect_bytes);
-#pragma unroll
-            for (int u = 0; u < Cfg::KSUB; ++u) {
-              tma_load_2d_pair(sa + u * Cfg::A_ATOM, jb.ta, fb, (kt + u) * Cfg::ATOM_K, ya);
-              tma_load_2d_pair(sa + Cfg::A_BYTES + u * Cfg::B_ATOM, jb.tb, fb, (kt + u) * Cfg::ATOM_K, yb);
-            }
+            tma_load_2d_pair(sa, jb.ta, fb, kt * Cfg::ATOM_K, ya);
+            tma_load_2d_pair(sa + Cfg::A_BYTES, jb.tb, fb, kt * Cfg::ATOM_K, yb);
           } else {
             mbar_arrive_expect_tx(full_bar(stage), expect_bytes);
             tma_load_2d(sa, jb.ta, full_bar(stage), kt * Cfg::ATOM_K, ya);
@@ -693,29 +937,16 @@ ozaki_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
         }
         return true;
       };
-      // every stage of one whole tile
-      auto put_tile = [&](const Job& jb) __attribute__((always_inline)) {
-        const int s = jb.s;
-        for (int L = s + 1; L >= 2 && ok; --L) {
-          const int i_lo = max(1, L - s), i_hi = min(s, L - 1);
-          for (int i = i_lo; i <= i_hi && ok; ++i)
-            for (int kt = 0; kt < jb.KT && ok; kt += Cfg::KSUB) ok = put_stage(jb, i, L - i, kt);
-        }
-      };
-      if constexpr (WALK == 0) {
-        for (int tile = cta_id; tile < p.ntiles && ok; tile += cta_stride) {
-          const Job jb = job_of<BN, PAIR>(p, &tmA, &tmB, tile, rank);
-          if (jb.skip) continue;
-          put_tile(jb);
-        }
-      } else if constexpr (WALK == 2) {
-        // take tiles from the global counter (skipping finished matrices) and
-        // announce each, then -1, to the other warps through the ring
-        int rslot = 0;
-        uint32_t rph = 0;
-        while (ok) {
-          int tile = atomicAdd(p.tile_counter, 1);
-          while (tile < p.ntiles && job_of<BN, PAIR>(p, &tmA, &tmB, tile, rank).skip) tile = atomicAdd(p.tile_counter, 1);
+      int rslot = 0;
+      uint32_t rph = 0;
+      for (int it = 0; ok; ++it) {
+        int tile = 0, u0 = 0, u1 = 0x7fffffff;
+        if constexpr (WALK == 2) {
+          // take the next tile from the global counter (skipping finished
+          // matrices) and announce it, or -1, to the other warps through the ring
+          tile = atomicAdd(p.tile_counter, 1);
+          while (tile < p.ntiles && job_of<BN, PAIR>(p, &tmA, &tmB, tile, rank).skip)
+            tile = atomicAdd(p.tile_counter, 1);
           if (tile >= p.ntiles) tile = -1;
           if (!wait_bar<false>(ring_empty(rslot), rph ^ 1u, abort_flag, p)) {
             ok = false;
@@ -728,17 +959,28 @@ ozaki_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
             rph ^= 1u;
           }
           if (tile < 0) break;
-          put_tile(job_of<BN, PAIR>(p, &tmA, &tmB, tile, rank));
+        } else {
+          if (!static_item(it, tile, u0, u1)) break;
         }
-      } else {
-        for (int64_t u = u_begin; u < u_end && ok; ++u) {
-          int tt, L, kb0, kb1;
-          split_unit(u, tt, L, kb0, kb1);
-          const Job jb = job_of<BN, PAIR>(p, &tmA, &tmB, tt, rank);
-          const int i_lo = max(1, L - p.s);
-          for (int kb = kb0; kb < kb1 && ok; ++kb) {
-            const int i = i_lo + kb / KTS_;
-            ok = put_stage(jb, i, L - i, (kb % KTS_) * Cfg::KSUB);
+        const Job jb = job_of<BN, PAIR>(p, &tmA, &tmB, tile, rank);
+        if (jb.skip) continue;
+        const int KTS = jb.KT;
+        int base = 0;
+        for (int g = 0; g < p.prog.nsegs && ok; ++g) {
+          const int nkb = p.prog.seg[g].nsteps * KTS;
+          const int nch = (nkb + CHS - 1) / CHS;
+          const int lo = max(u0 - base, 0), hi = min(u1 - base, nch);
+          base += nch;
+          if (lo >= hi) continue;
+          const int kb1 = min(hi * CHS, nkb);
+          int step = p.prog.seg[g].step0 + lo * CHS / KTS;
+          int kt = lo * CHS % KTS;
+          for (int kb = lo * CHS; kb < kb1 && ok; ++kb) {
+            ok = put_stage(jb, p.prog.pa[step], p.prog.pb[step], kt);
+            if (++kt == KTS) {
+              kt = 0;
+              ++step;
+            }
           }
         }
       }
@@ -768,34 +1010,37 @@ ozaki_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
-    if (lane == 0 && leader) {
-      constexpr uint32_t idesc =
-          F8 ? idesc_e4m3(PAIR ? 2 * TC_BM : TC_BM, BN) : idesc_bf16(PAIR ? 2 * TC_BM : TC_BM, BN);
+    // The whole warp walks the loops and an elected lane issues: descriptors and
+    // barrier addresses are then the same for all lanes, and the compiler keeps
+    // them in the uniform registers that the tensor instructions take.
+    if (leader) {
+      constexpr uint32_t idesc = F8 ? idesc_e4m3(Cfg::BM, BN) : idesc_bf16(Cfg::BM, BN);
       int stage = 0;
       uint32_t phase = 0;
       int buf = 0;
-      uint32_t aph[2] = {0u, 0u};
+      uint32_t aph0 = 0, aph1 = 0;  // phases of the two accumulators
       bool ok = true;
       bool issued = false;
+      auto wait_all = [&](uint32_t bar, uint32_t parity) __attribute__((always_inline)) -> bool {
+        return __all_sync(0xffffffffu, wait_bar<PAIR>(bar, parity, abort_flag, p)) != 0;
+      };
       // one stage of MMAs; `first` starts a chunk (waits for a free TMEM buffer
       // and overwrites it), `last` ends it (publishes the buffer)
       auto mma_stage = [&](bool first, bool last) __attribute__((always_inline)) -> bool {
         if (first) {
-          if (!wait_bar<PAIR>(accempty_bar(buf), aph[buf] ^ 1u, abort_flag, p)) return false;
-          tc_fence_after();
+          if (!wait_all(accempty_bar(buf), (buf ? aph1 : aph0) ^ 1u)) return false;
         }
-        if (!wait_bar<PAIR>(full_bar(stage), phase, abort_flag, p)) return false;
+        if (!wait_all(full_bar(stage), phase)) return false;
         tc_fence_after();
-        const uint32_t sa = sbase + stage * Cfg::STAGE_BYTES;
-        const uint32_t d = tmem + static_cast<uint32_t>(buf * BN);
-#pragma unroll
-        for (int u = 0; u < Cfg::KSUB; ++u) {
-          const uint64_t ad = sdesc_sw128(sa + u * Cfg::A_ATOM);
-          const uint64_t bd = sdesc_sw128(sa + Cfg::A_BYTES + u * Cfg::B_ATOM);
+        if (elect_one()) {
+          const uint32_t sa = sbase + stage * Cfg::STAGE_BYTES;
+          const uint32_t d = tmem + static_cast<uint32_t>(buf * BN);
+          const uint64_t ad = sdesc_sw128(sa);
+          const uint64_t bd = sdesc_sw128(sa + Cfg::A_BYTES);
 #pragma unroll
           for (int ks = 0; ks < TC_MMA_PER_ATOM; ++ks) {
             // advance 32 bytes (16 bf16 or 32 e4m3) along K inside the swizzled row
-            const uint32_t acc = (first && u == 0 && ks == 0) ? 0u : 1u;
+            const uint32_t acc = (first && ks == 0) ? 0u : 1u;
             if (F8) {
               if (PAIR) {
                 umma_e4m3_pair(d, ad + 2ull * ks, bd + 2ull * ks, idesc, acc);
@@ -808,20 +1053,27 @@ ozaki_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
               umma_bf16(d, ad + 2ull * ks, bd + 2ull * ks, idesc, acc);
             }
           }
-        }
-        issued = true;
-        if (PAIR) {
-          umma_commit_pair_both(empty_bar(stage));
-        } else {
-          umma_commit(empty_bar(stage));
-        }
-        if (last) {
           if (PAIR) {
-            umma_commit_pair_both(accfull_bar(buf));
+            umma_commit_pair_both(empty_bar(stage));
           } else {
-            umma_commit(accfull_bar(buf));
+            umma_commit(empty_bar(stage));
           }
-          aph[buf] ^= 1u;
+          if (last) {
+            if (PAIR) {
+              umma_commit_pair_both(accfull_bar(buf));
+            } else {
+              umma_commit(accfull_bar(buf));
+            }
+          }
+        }
+        __syncwarp();
+        issued = true;
+        if (last) {
+          if (buf) {
+            aph1 ^= 1u;
+          } else {
+            aph0 ^= 1u;
+          }
           buf ^= 1;
         }
         if (++stage == Cfg::STAGES) {
@@ -830,50 +1082,49 @@ ozaki_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
         }
         return true;
       };
-      // every stage of one whole tile
-      auto mma_tile = [&](const Job& jb) __attribute__((always_inline)) {
-        const int s = jb.s;
-        // stages per level and per fp32 chunk (KT and CH are multiples of KSUB)
-        const int CHS = CH / Cfg::KSUB;
-        for (int L = s + 1; L >= 2 && ok; --L) {
-          const int nkb = npairs_of(L, s) * (jb.KT / Cfg::KSUB);
-          for (int kb = 0; kb < nkb && ok; ++kb) {
-            const int kc = kb % CHS;
-            ok = mma_stage(kc == 0, (kc == CHS - 1) || (kb == nkb - 1));
-          }
-        }
-      };
-      if constexpr (WALK == 0) {
-        for (int tile = cta_id; tile < p.ntiles && ok; tile += cta_stride) {
-          const Job jb = job_of<BN, PAIR>(p, &tmA, &tmB, tile, rank);
-          if (jb.skip) continue;
-          mma_tile(jb);
-        }
-      } else if constexpr (WALK == 2) {
-        int rslot = 0;
-        uint32_t rph = 0;
-        while (ok) {
-          if (!wait_bar<false>(ring_full(rslot), rph, abort_flag, p)) {
+      int rslot = 0;
+      uint32_t rph = 0;
+      for (int it = 0; ok; ++it) {
+        int tile = 0, u0 = 0, u1 = 0x7fffffff;
+        if constexpr (WALK == 2) {
+          if (!wait_all(ring_full(rslot), rph)) {
             ok = false;
             break;
           }
-          const int tile = ring_tile[rslot];
-          mbar_arrive(ring_empty(rslot));
+          tile = ring_tile[rslot];
+          __syncwarp();
+          if (lane == 0) mbar_arrive(ring_empty(rslot));
           if (++rslot == kTileRing) {
             rslot = 0;
             rph ^= 1u;
           }
           if (tile < 0) break;
-          mma_tile(job_of<BN, PAIR>(p, &tmA, &tmB, tile, rank));
+        } else {
+          if (!static_item(it, tile, u0, u1)) break;
         }
-      } else {
-        for (int64_t u = u_begin; u < u_end && ok; ++u) {
-          int tt, L, kb0, kb1;
-          split_unit(u, tt, L, kb0, kb1);
-          for (int kb = kb0; kb < kb1 && ok; ++kb) ok = mma_stage(kb == kb0, kb == kb1 - 1);
+        int KT = p.KT;
+        if (p.mats != nullptr) {
+          const Job jb = job_of<BN, PAIR>(p, &tmA, &tmB, tile, rank);
+          if (jb.skip) continue;
+          KT = jb.KT;
+        }
+        const int KTS = KT;  // stages per step
+        int base = 0;
+        for (int g = 0; g < p.prog.nsegs && ok; ++g) {
+          const int nkb = p.prog.seg[g].nsteps * KTS;
+          const int nch = (nkb + CHS - 1) / CHS;
+          const int lo = max(u0 - base, 0), hi = min(u1 - base, nch);
+          base += nch;
+          if (lo >= hi) continue;
+          const int kb1 = min(hi * CHS, nkb);
+          int kc = 0;
+          for (int kb = lo * CHS; kb < kb1 && ok; ++kb) {
+            ok = mma_stage(kc == 0, kc == CHS - 1 || kb == kb1 - 1);
+            if (++kc == CHS) kc = 0;
+          }
         }
       }
-      if (!ok && issued) {
+      if (!ok && issued && elect_one()) {
         // wait for the MMAs in flight before TMEM is released
         if (PAIR) {
           umma_commit_pair_self(drain_bar);
@@ -887,7 +1138,7 @@ ozaki_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
       if (PAIR && ok) {
         // both epilogues arrive on this CTA's accumulator barriers: wait for
         // their last releases, so no arrival is left in flight at exit
-        for (int b = 0; b < 2 && ok; ++b) ok = wait_bar<PAIR>(accempty_bar(b), aph[b] ^ 1u, abort_flag, p);
+        ok = wait_all(accempty_bar(0), aph0 ^ 1u) && wait_all(accempty_bar(1), aph1 ^ 1u);
       }
     }
   } else {
@@ -896,21 +1147,8 @@ ozaki_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     const int e = warp - 2;
     const int q = warp & 3;   // TMEM lane quadrant this warp may access
     const int h = e >> 2;     // which half of the BN columns
-    const int row = 32 * q + lane;
     const int cbase = h * COLS;
     const uint32_t taddr_row = tmem + (static_cast<uint32_t>(32 * q) << 16);
-    // fold buffers of this thread (whole tiles): the int64 group sums, or the
-    // running group and the float64 sum D; element c at [32 c] (a warp touches
-    // 256 contiguous bytes per column), private to this CTA and L2-resident
-    long long* scr_i = reinterpret_cast<long long*>(p.scratch) +
-                       static_cast<int64_t>(blockIdx.x) * (2 * TC_BM * BN) + e * (COLS * 32) + lane;
-    long long* scr_d = scr_i + TC_BM * BN;
-    // WALK 1: the group sums of (tile tt, this CTA's row half), shared by the
-    // CTAs that contribute to the tile; same element layout
-    auto split_area_of = [&](int tt, int gidx) __attribute__((always_inline)) -> long long* {
-      return p.split_area + ((static_cast<int64_t>(tt) * (PAIR ? 2 : 1) + rank) * 2 + gidx) * (TC_BM * BN) +
-             e * (COLS * 32) + lane;
-    };
 
     int32_t S[COLS];
     int buf = 0;
@@ -919,9 +1157,7 @@ ozaki_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     // PAIR: TMEM buffers are released on the leader's barrier
     const uint32_t accempty_target0 = PAIR ? map_to_cta(accempty_bar(0), 0) : accempty_bar(0);
 
-    // one finished chunk from TMEM added into the level sum S (one call site
-    // per kernel: a second, specialised copy costs the register allocator far
-    // more than zeroing S)
+    // one finished chunk from TMEM added into the segment's sum S
     auto drain_chunk = [&]() __attribute__((always_inline)) -> bool {
       // one lane polls the barrier (32 pollers per warp would crowd the
       // barrier word the MMA issuer and the copies also use); the warp then
@@ -954,273 +1190,69 @@ ozaki_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
       return true;
     };
 
-    // the output step of a finished tile: unscale the group sums in a0 (group 0)
-    // and a1 (group 1, or D with three or more groups) and write C (or the
-    // update). The group sums are read from L2 (.cg): reductions at L2, and for
-    // the split those of other CTAs, never pass through this SM's L1.
-    auto output_tile = [&](const Job& jb, int64_t m0, int64_t n0, int s, const long long* a0,
-                           const long long* a1) __attribute__((always_inline)) {
-      const int64_t r = m0 + row;
-      if (r >= jb.m) return;
-      const int32_t er = jb.ea[r];
-      const bool upd = jb.epi.kind == EPI_PM_UPDATE;
-      const double wa = upd ? jb.epi.state->alpha : 0.0;
-      const double w2 = upd ? jb.epi.state->b2 : 0.0;
-      const double w3 = upd ? jb.epi.state->b3 : 0.0;
-      // last group (levels 2 .. L_a, L_a = 2 + (s - 1) mod G) in a0, or in a1
-      // for two groups (then a0 holds group 0, weight 2^(-beta (s+1))); with
-      // three or more groups the earlier ones are summed in D (a1)
-      const double lscale = ldexp(1.0, -p.beta * (2 + (s - 1) % p.group));
-      const bool has_d = s > p.group;
-      const bool two_groups = has_d && s <= 2 * p.group;
-      // weight of the rounded sum: 2^(-beta (s+1)) for two groups, 2^(-beta L_a)
-      // for one, none with D (already scaled)
-      const int e_acc = two_groups ? -p.beta * (s + 1) : (has_d ? 0 : -p.beta * (2 + (s - 1) % p.group));
-      const uint64_t pol = policy_evict_last();
-      double* Cout = jb.epi.C;
-      const int64_t ldc = jb.epi.ldc;
-      // batches of 8 columns: issue every load of the batch, then compute and
-      // store; the next batch's P and P^2 lines are requested into L1 meanwhile
-      auto prefetch_batch = [&](int gb) __attribute__((always_inline)) {
-        const int64_t c0 = n0 + cbase + 8 * gb;
-        if (!upd || gb >= COLS / 8 || c0 >= jb.n) return;
 #pragma unroll
-        for (int t = 0; t < 8; ++t) {
-          if (c0 + t < jb.n) {
-            prefetch_l1(jb.epi.P + (c0 + t) * jb.epi.ldp + r);
-            prefetch_l1(jb.epi.X2 + (c0 + t) * jb.epi.ldx + r);
-          }
-        }
-      };
-      for (int g = 0; g < COLS / 8; ++g) {
-        const int64_t col0 = n0 + cbase + 8 * g;
-        if (col0 >= jb.n) break;
-        long long ti[8], td[8];
-        double pv[8], xv[8];
-        int32_t ecv[8];
-#pragma unroll
-        for (int t = 0; t < 8; ++t) {
-          const int c = 8 * g + t;
-          const int64_t col = col0 + t;
-          const bool ok = col < jb.n;
-          ti[t] = ld_l2(a0 + 32 * c, pol);
-          td[t] = has_d ? ld_l2(a1 + 32 * c, pol) : 0ll;
-          ecv[t] = ok ? jb.eb[col] : 0;
-          // P and P^2 are exactly symmetric: read them at (col, r), coalesced across the warp
-          pv[t] = (upd && ok) ? jb.epi.P[col * jb.epi.ldp + r] : 0.0;
-          xv[t] = (upd && ok) ? jb.epi.X2[col * jb.epi.ldx + r] : 0.0;
-        }
-        prefetch_batch(g + 1);
-#pragma unroll
-        for (int t = 0; t < 8; ++t) {
-          const int64_t col = col0 + t;
-          if (col >= jb.n) break;
-          if (jb.sym && r > col) continue;  // the (col, r) element's mirror covers it
-          // one or two groups: the exact integer combination rounded once and
-          // scaled by 2^e_acc (exact); three or more: the float64 sum D of the
-          // earlier groups plus the last
-          const double acc = two_groups ? round_sum(td[t], p.beta * p.group, ti[t])
-                                        : (has_d ? __longlong_as_double(td[t]) + static_cast<double>(ti[t]) * lscale
-                                                 : static_cast<double>(ti[t]));
-          double v = (er == kBadExp || ecv[t] == kBadExp) ? __longlong_as_double(0x7ff8000000000000ll)
-                                                          : scale_pow2(acc, er + ecv[t] + e_acc);
-          if (upd) v = wa * pv[t] + w2 * xv[t] + w3 * v;
-          v = stored_value(v, jb.epi.round32 != 0);
-          Cout[r * ldc + col] = v;
-          if (jb.sym && r < col) Cout[col * ldc + r] = v;
-        }
-      }
-    };
-
-    if constexpr (WALK != 1) {
-      // ---- whole tiles: cta, cta + #CTAs, ... (WALK 0) or as the producer
-      // announces them through the ring (WALK 2)
-      int rslot = 0;
-      uint32_t rph = 0;
-      for (int tile = cta_id - cta_stride; ok;) {
-        if constexpr (WALK == 0) {
-          tile += cta_stride;
-          if (tile >= p.ntiles) break;
-        } else {
-          int got = 0, t = 0;
-          if (lane == 0) {
-            got = wait_bar<false>(ring_full(rslot), rph, abort_flag, p) ? 1 : 0;
-            if (got) {
-              t = ring_tile[rslot];
-              mbar_arrive(ring_empty(rslot));
-            }
-          }
-          got = __shfl_sync(0xffffffffu, got, 0);
-          t = __shfl_sync(0xffffffffu, t, 0);
-          if (++rslot == kTileRing) {
-            rslot = 0;
-            rph ^= 1u;
-          }
-          if (!got) {
-            ok = false;
-            break;
-          }
-          if (t < 0) break;
-          tile = t;
-        }
-        int64_t m0, n0;
-        int s, KT;
-        bool skip;
-        {
-          const Job jb = job_of<BN, PAIR>(p, &tmA, &tmB, tile, rank);
-          m0 = jb.m0;
-          n0 = jb.n0;
-          s = jb.s;
-          KT = jb.KT;
-          skip = jb.skip;
-        }
-        if (skip) continue;
-        for (int L = s + 1; L >= 2 && ok; --L) {
-#pragma unroll
-          for (int c = 0; c < COLS; ++c) S[c] = 0;
-          if (L == 2 && p.epi.kind == EPI_PM_UPDATE && p.mats == nullptr && m0 + row < p.m) {
-            // the update reads P and P^2 in the output pass: ask L2 for this
-            // thread's elements while the last level's chunks are still running
-            for (int c = 0; c < COLS; ++c) {
-              const int64_t col = n0 + cbase + c;
-              if (col >= p.n) break;
-              prefetch_l2(p.epi.P + col * p.epi.ldp + m0 + row);
-              prefetch_l2(p.epi.X2 + col * p.epi.ldx + m0 + row);
-            }
-          }
-          const int nkb = npairs_of(L, s) * KT;
-          const int nch = (nkb + CH - 1) / CH;
-          for (int ch = 0; ch < nch && ok; ++ch) ok = drain_chunk();
-          if (!ok) break;
-          if (p.epi.kind == EPI_LEVELS && p.mats == nullptr) {
-            // test hook: write the exact level sum itself
-            const int64_t r = m0 + row;
-            if (r < p.m) {
-#pragma unroll
-              for (int c = 0; c < COLS; ++c) {
-                const int64_t col = n0 + cbase + c;
-                if (col < p.n) p.epi.levels[static_cast<int64_t>(L - 2) * p.m * p.n + r * p.n + col] = S[c];
-              }
-            }
-            continue;
-          }
-          // ---- fold the exact level sum (groups of levels, smallest first; see the header)
-          {
-            const uint64_t pol = policy_evict_last();
-            // up to G consecutive levels (G = 4 for beta 7 and 5, 3 for beta 8)
-            // combine exactly in int64, T = sum S_L 2^(beta (L_a - L)) < 2^53; the
-            // first level of a group stores its sum, the others add theirs at L2
-            // (red: nothing comes back, so the fold costs no round trip). With at
-            // most two groups each has its own area (group 0 in scr_i, group 1 in
-            // scr_d) and both are finished by the output pass. With three or more,
-            // scr_i holds the running group: at the end of a group (other than the
-            // last) its exact value T 2^(-beta L_a) is read back and added to D
-            // (scr_d) in float64.
-            const int G = p.group;
-            const int gpos = (s + 1 - L) % G;
-            const int gidx = (s + 1 - L) / G;
-            const bool two_areas = s <= 2 * G;
-            long long* area = (two_areas && gidx == 1) ? scr_d : scr_i;
-            const bool gend = !two_areas && (gpos == G - 1) && (L != 2);
-            const int La = L + gpos;
-            const bool first_group = gidx == 0;
-            const double gscale = ldexp(1.0, -p.beta * La);
-            const long long wgt = 1ll << (p.beta * gpos);
-            if (!gend) {
-#pragma unroll
-              for (int c = 0; c < COLS; ++c) {
-                const long long v = static_cast<long long>(S[c]) * wgt;
-                if (gpos == 0) {
-                  st_keep(area + 32 * c, v, pol);
-                } else {
-                  red_add_keep(area + 32 * c, v, pol);
-                }
-              }
-            } else {
-#pragma unroll
-              for (int g = 0; g < COLS / 8; ++g) {
-                long long told[8];
-#pragma unroll
-                for (int t = 0; t < 8; ++t) told[t] = ld_l2(scr_i + 32 * (8 * g + t), pol);
-#pragma unroll
-                for (int t = 0; t < 8; ++t) {
-                  const int c = 8 * g + t;
-                  const long long T = told[t] + static_cast<long long>(S[c]) * wgt;
-                  const double gv = static_cast<double>(T) * gscale;
-                  const double d = first_group ? gv : __longlong_as_double(ld_l2(scr_d + 32 * c, pol)) + gv;
-                  st_keep(scr_d + 32 * c, __double_as_longlong(d), pol);
-                }
-              }
-            }
-          }
-          if (L != 2) continue;
-          // ---- last level: unscale and apply the output step
-          const Job jb = job_of<BN, PAIR>(p, &tmA, &tmB, tile, rank);
-          output_tile(jb, m0, n0, s, scr_i, scr_d);
-        }
-      }
-    } else if (u_begin < u_end) {
-      // ---- the split: (tile, level) runs of this CTA's range, each drained
-      // into S and added at L2 to the tile's group sums (at most two groups,
-      // areas zeroed before the launch); leaving a tile counts this warp in
-      // for it, and the last of the tile's contributors writes this warp's
-      // part of the output
-      const uint64_t pol = policy_evict_last();
-      const int s = p.s;
-      const int G = p.group;
-      const int64_t units_per_tile = p.split_unit_count;
-      // CTA (pair) that owns unit u
-      auto owner = [&](int64_t u) __attribute__((always_inline)) -> int64_t {
-        return ((u + 1) * cta_stride + split_units - 1) / split_units - 1;
-      };
-      // tiles whose output this warp writes, after its whole range (a range
-      // shorter than a tile meets at most two tiles)
-      int out_tiles[2] = {-1, -1};
-      int n_out = 0;
-      // the tiles this range meets, level by level as whole tiles are walked;
-      // level L of tile tt holds units [base, base + nch_L) of the launch
-      const int tt_lo = static_cast<int>(u_begin / units_per_tile);
-      const int tt_hi = static_cast<int>((u_end - 1) / units_per_tile);
-      for (int tt = tt_lo; tt <= tt_hi && ok; ++tt) {
-        int base = static_cast<int>(static_cast<int64_t>(tt) * units_per_tile);
-        for (int L = s + 1; L >= 2 && ok; --L) {
-          const int nch_l = (npairs_of(L, s) * KTS_ + CHS_ - 1) / CHS_;
-          const int lo = max(base, static_cast<int>(u_begin));
-          const int hi = min(base + nch_l, static_cast<int>(u_end));
-          base += nch_l;
-          if (lo >= hi) continue;
-#pragma unroll
-          for (int c = 0; c < COLS; ++c) S[c] = 0;
-          for (int ch = lo; ch < hi && ok; ++ch) ok = drain_chunk();
-          if (!ok) break;
-          const int gpos = (s + 1 - L) % G;
-          long long* area = split_area_of(tt, (s + 1 - L) / G);
-          const long long wgt = 1ll << (p.beta * gpos);
-#pragma unroll
-          for (int c = 0; c < COLS; ++c) red_add_keep(area + 32 * c, static_cast<long long>(S[c]) * wgt, pol);
-        }
-        if (!ok) break;
-        __threadfence();  // this lane's reductions before the count
-        __syncwarp();
-        int last = 0;
+    for (int c = 0; c < COLS; ++c) S[c] = 0;
+    const uint64_t pol = policy_evict_last();
+    int rslot = 0;
+    uint32_t rph = 0;
+    for (int it = 0; ok; ++it) {
+      int tile = 0, u0 = 0, u1 = 0x7fffffff;
+      if constexpr (WALK == 2) {
+        int got = 0, t = 0;
         if (lane == 0) {
-          // the CTAs (pairs) whose non-empty ranges meet this tile (with fewer
-          // units than CTAs some ranges are empty)
-          const int64_t u0 = static_cast<int64_t>(tt) * units_per_tile;
-          int contributors = 0;
-          for (int64_t c = owner(u0); c <= owner(u0 + units_per_tile - 1); ++c)
-            contributors += (split_units * (c + 1) / cta_stride > split_units * c / cta_stride) ? 1 : 0;
-          int* cnt = p.split_cnt + (static_cast<int64_t>(tt) * (PAIR ? 2 : 1) + rank) * TC_EPI_WARPS + e;
-          last = atomicAdd(cnt, 1) == contributors - 1 ? 1 : 0;
+          got = wait_bar<false>(ring_full(rslot), rph, abort_flag, p) ? 1 : 0;
+          if (got) {
+            t = ring_tile[rslot];
+            mbar_arrive(ring_empty(rslot));
+          }
         }
-        if (__shfl_sync(0xffffffffu, last, 0) != 0 && n_out < 2) out_tiles[n_out++] = tt;
+        got = __shfl_sync(0xffffffffu, got, 0);
+        t = __shfl_sync(0xffffffffu, t, 0);
+        if (++rslot == kTileRing) {
+          rslot = 0;
+          rph ^= 1u;
+        }
+        if (!got) {
+          ok = false;
+          break;
+        }
+        if (t < 0) break;
+        tile = t;
+      } else {
+        if (!static_item(it, tile, u0, u1)) break;
       }
-      if (ok && n_out > 0) {
-        __threadfence();  // every contributor's reductions before the reads
-        for (int k = 0; k < n_out; ++k) {
-          const Job jb = job_of<BN, PAIR>(p, &tmA, &tmB, out_tiles[k], rank);
-          output_tile(jb, jb.m0, jb.n0, s, split_area_of(out_tiles[k], 0), split_area_of(out_tiles[k], 1));
+      int KT = p.KT;
+      if (p.mats != nullptr) {
+        const Job jb = job_of<BN, PAIR>(p, &tmA, &tmB, tile, rank);
+        if (jb.skip) continue;
+        KT = jb.KT;
+      }
+      const int KTS = KT;
+      // the group sums of this CTA's part of the tile; element c of this thread
+      // at [32 c] (a warp touches 256 contiguous bytes per column)
+      long long* part = p.area + (static_cast<int64_t>(tile) * Cfg::RANKS + rank) * p.prog.ng * Cfg::PART +
+                        e * (COLS * 32) + lane;
+      int base = 0;
+      for (int g = 0; g < p.prog.nsegs && ok; ++g) {
+        const TcSeg& seg = p.prog.seg[g];
+        const int nch = (seg.nsteps * KTS + CHS - 1) / CHS;
+        const int lo = max(u0 - base, 0), hi = min(u1 - base, nch);
+        base += nch;
+        if (lo >= hi) continue;
+        for (int ch = lo; ch < hi && ok; ++ch) ok = drain_chunk();
+        if (!ok) break;
+        if (!seg.fold && u1 > base) continue;  // folded with the next segment
+        // ---- add the exact sum to the tile's groups at L2 (red: nothing comes
+        // back, so the adds cost no round trip)
+        for (int i = 0; i < 3; ++i) {
+          const long long w = seg.w[i];
+          if (w == 0) continue;
+          long long* area = part + (seg.g0 + i) * Cfg::PART;
+#pragma unroll
+          for (int c = 0; c < COLS; ++c) red_add_keep(area + 32 * c, static_cast<long long>(S[c]) * w, pol);
         }
+#pragma unroll
+        for (int c = 0; c < COLS; ++c) S[c] = 0;
       }
     }
   }
@@ -1278,6 +1310,44 @@ bool make_plane_map_ext(CUtensorMap* tm, const void* planes, int64_t k_pad, int6
 }
 
 namespace {
+// Exact bound of a product's combined integer sum_L S_L 2^(beta (s+1-L)): whether
+// it fits a signed 64-bit word (then one group sum per element is enough).
+bool one_word(int s, int beta, int64_t k) {
+  const double dmax = beta == 7 ? 127.0 : (beta == 8 ? 128.0 : 16.0);
+  double t = 0.0;
+  for (int L = 2; L <= s + 1; ++L) t += (L - 1) * std::ldexp(1.0, beta * (s + 1 - L));
+  return t * dmax * dmax * static_cast<double>(k) < 9.0e18;
+}
+
+// Levels s+1 .. 2, one segment each: the pairs (i, j) with i + j = L.
+void direct_program(int s, int beta, int group, int64_t k, bool levels, TcProgram& pr) {
+  std::memset(&pr, 0, sizeof(pr));
+  const int groups = (s + group - 1) / group;
+  const bool one = groups <= 2 && one_word(s, beta, k);
+  pr.ng = levels ? s : (one ? 1 : groups);
+  int step = 0;
+  for (int L = s + 1; L >= 2; --L) {
+    TcSeg& g = pr.seg[pr.nsegs++];
+    const int pos = s + 1 - L;
+    g.step0 = step;
+    for (int i = std::max(1, L - s); i <= std::min(s, L - 1); ++i) {
+      pr.pa[step] = static_cast<unsigned char>(i - 1);
+      pr.pb[step] = static_cast<unsigned char>(L - i - 1);
+      ++step;
+    }
+    g.nsteps = step - g.step0;
+    g.fold = 1;
+    g.g0 = levels ? L - 2 : (one ? 0 : pos / group);
+    g.w[0] = levels ? 1 : 1ll << (beta * (one ? pos : pos % group));
+  }
+}
+
+// fp32 chunks of one tile (split launches)
+int chunk_count(const TcProgram& pr, int kts, int chs) {
+  int cnt = 0;
+  for (int g = 0; g < pr.nsegs; ++g) cnt += (pr.seg[g].nsteps * kts + chs - 1) / chs;
+  return cnt;
+}
 
 // Set before every launch rather than once per process: the attribute belongs
 // to the kernel as loaded in the current context, and a context created anew
@@ -1289,32 +1359,56 @@ cudaError_t set_smem_attr() {
                               TcCfg<BN, PAIR, F8>::SMEM);
 }
 
-template <int BN, bool PAIR = false, bool F8 = false, int WALK = 0>
-cudaError_t launch_tc_impl(const CUtensorMap& ta, const CUtensorMap& tb, const TcParams& p, int grid,
-                           cudaStream_t st) {
-  using Cfg = TcCfg<BN, PAIR, F8>;
-  cudaError_t e = set_smem_attr<BN, PAIR, F8, WALK>();
-  if (e != cudaSuccess) return e;
-  if (PAIR) {
-    cudaLaunchConfig_t cfg;
+// The launch configuration of the product kernel (clusters of two CTAs for PAIR).
+template <int BN, bool PAIR, bool F8>
+struct TcLaunch {
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute at[1];
+  TcLaunch(int grid, cudaStream_t st) {
     std::memset(&cfg, 0, sizeof(cfg));
+    std::memset(at, 0, sizeof(at));
     cfg.gridDim = dim3(static_cast<unsigned>(grid));
     cfg.blockDim = dim3(TC_THREADS);
-    cfg.dynamicSmemBytes = Cfg::SMEM;
+    cfg.dynamicSmemBytes = TcCfg<BN, PAIR, F8>::SMEM;
     cfg.stream = st;
-    cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = 2;
+    at[0].val.clusterDim.x = PAIR ? 2 : 1;
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    e = cudaLaunchKernelEx(&cfg, ozaki_tc_kernel<BN, PAIR, F8, WALK>, ta, tb, p);
-    if (e != cudaSuccess) return e;
-  } else {
-    ozaki_tc_kernel<BN, PAIR, F8, WALK><<<grid, TC_THREADS, Cfg::SMEM, st>>>(ta, tb, p);
   }
-  count_launch();
+};
+
+template <int BN, bool PAIR, bool UPD>
+void launch_finish(const TcParams& p, cudaStream_t st) {
+  const int grid = p.ntiles * (TcCfg<BN, PAIR>::BM / 32) * (BN / 32);
+  if (p.mats == nullptr && p.epi.kind == EPI_LEVELS) {
+    ozaki_finish_kernel<BN, PAIR, UPD, 0><<<grid, FIN_THREADS, 0, st>>>(p);
+  } else if (p.prog.ng == 1) {
+    ozaki_finish_kernel<BN, PAIR, UPD, 1><<<grid, FIN_THREADS, 0, st>>>(p);
+  } else if (p.prog.ng == 2) {
+    ozaki_finish_kernel<BN, PAIR, UPD, 2><<<grid, FIN_THREADS, 0, st>>>(p);
+  } else {
+    ozaki_finish_kernel<BN, PAIR, UPD, 3><<<grid, FIN_THREADS, 0, st>>>(p);
+  }
+}
+
+// The product kernel on `grid` CTAs, then the finish kernel over its tiles.
+template <int BN, bool PAIR = false, bool F8 = false, int WALK = 0>
+cudaError_t launch_tc_impl(const CUtensorMap& ta, const CUtensorMap& tb, const TcParams& p, int grid, cudaStream_t st) {
+  cudaError_t e = set_smem_attr<BN, PAIR, F8, WALK>();
+  if (e != cudaSuccess) return e;
+  TcLaunch<BN, PAIR, F8> l(grid, st);
+  e = cudaLaunchKernelEx(&l.cfg, ozaki_tc_kernel<BN, PAIR, F8, WALK>, ta, tb, p);
+  if (e != cudaSuccess) return e;
+  const bool upd = p.mats != nullptr ? p.phase != 0 : p.epi.kind == EPI_PM_UPDATE;
+  if (upd) {
+    launch_finish<BN, PAIR, true>(p, st);
+  } else {
+    launch_finish<BN, PAIR, false>(p, st);
+  }
+  count_launch(2);
   return cudaGetLastError();
 }
 
@@ -1324,30 +1418,18 @@ bool g_pairing = true;
 // for the next tcgen05 product launch, 0 = off.
 std::atomic<int> g_stall_us{0};
 
-// CTA pairs of the PAIR kernel that can be resident at once (0: none)
+// CTA pairs of the pair kernel that can be resident at once (0: none)
 int tc_max_pairs() {
-  static int pairs = -1;
-  if (pairs < 0) {
-    pairs = 0;
+  static const int pairs = [] {
+    int found = 0;
     if (set_smem_attr<256, true>() == cudaSuccess) {
-      cudaLaunchConfig_t cfg;
-      std::memset(&cfg, 0, sizeof(cfg));
-      cfg.gridDim = dim3(2);
-      cfg.blockDim = dim3(TC_THREADS);
-      cfg.dynamicSmemBytes = TcCfg<256, true>::SMEM;
-      cudaLaunchAttribute at[1];
-      at[0].id = cudaLaunchAttributeClusterDimension;
-      at[0].val.clusterDim.x = 2;
-      at[0].val.clusterDim.y = 1;
-      at[0].val.clusterDim.z = 1;
-      cfg.attrs = at;
-      cfg.numAttrs = 1;
+      TcLaunch<256, true, false> l(2, nullptr);
       int c = 0;
-      if (cudaOccupancyMaxActiveClusters(&c, ozaki_tc_kernel<256, true>, &cfg) == cudaSuccess) pairs = c;
+      if (cudaOccupancyMaxActiveClusters(&c, ozaki_tc_kernel<256, true>, &l.cfg) == cudaSuccess) found = c;
     }
     (void)cudaGetLastError();
-    pairs = std::min(pairs, kTcMaxCtas / 2);
-  }
+    return std::min(found, kTcMaxCtas / 2);
+  }();
   return pairs;
 }
 
@@ -1378,17 +1460,9 @@ int tc_max_ctas() {
   return std::min(sms, kTcMaxCtas);
 }
 
-size_t tc_scratch_bytes() { return static_cast<size_t>(kTcMaxCtas) * 2 * TC_BM * 256 * sizeof(double); }
-
-// Split launches: fewer than kTcMaxCtas / 2 tiles of one CTA (or kTcMaxCtas / 4
-// of a CTA pair, two row halves each), each with two TC_BM x 256 int64 group
-// sums per CTA, then one counter per (tile, CTA, epilogue warp).
-static size_t tc_split_area_bytes() {
-  return static_cast<size_t>(kTcMaxCtas / 2) * 2 * TC_BM * 256 * sizeof(long long);
-}
-size_t tc_split_bytes() {
-  return tc_split_area_bytes() + static_cast<size_t>(kTcMaxCtas / 2) * TC_EPI_WARPS * sizeof(int);
-}
+// 80 MiB: 160 pair tiles of one group sum per element, two waves of the pair
+// kernel, which stay in the 129 MB L2 between the product and its output step.
+size_t tc_area_bytes() { return static_cast<size_t>(kTcMaxCtas) * 2 * TC_BM * 256 * sizeof(long long); }
 
 bool g_split_tiles = true;
 
@@ -1398,27 +1472,101 @@ int set_tc_split_tiles(int enable) {
   return prev;
 }
 
+// The group sums of the next `bytes` of the area are zero before a launch adds
+// to them: cleared here once per call, by the finish kernel after that.
+cudaError_t tc_area_clear(TcArea& a, size_t bytes, cudaStream_t st) {
+  if (bytes <= a.clean) return cudaSuccess;
+  const cudaError_t e = cudaMemsetAsync(static_cast<char*>(a.ptr) + a.clean, 0, bytes - a.clean, st);
+  if (e == cudaSuccess) a.clean = bytes;
+  return e;
+}
+
+namespace {
+
+// The output tiles of an m x n product in the order they are walked: bands of
+// column blocks, each cut into groups of row blocks, about as many tiles per
+// block as run at once (`units`) and near-square in elements, so that the tiles
+// in flight together share their operand panels in L2.
+template <int BN, int BM>
+std::vector<TileAt> tile_order(int64_t m, int64_t n, int sym, int units) {
+  const int tm = static_cast<int>((m + BM - 1) / BM), tn = static_cast<int>((n + BN - 1) / BN);
+  const int w = std::max(1, std::min(static_cast<int>(std::lround(std::sqrt(static_cast<double>(units) * BM / BN))), tn));
+  const int hgt = std::max(1, units / w);
+  // row blocks of column block c that hold tiles (symmetric: some element with row <= column)
+  auto rows_of = [&](int c) { return sym ? std::min(tm, (BN * (c + 1) + BM - 1) / BM) : tm; };
+  std::vector<TileAt> t;
+  for (int c0 = 0; c0 < tn; c0 += w) {
+    const int c1 = std::min(tn, c0 + w);
+    for (int r0 = 0; r0 < rows_of(c1 - 1); r0 += hgt)
+      for (int c = c0; c < c1; ++c)
+        for (int r = r0; r < std::min(rows_of(c), r0 + hgt); ++r)
+          t.push_back({static_cast<unsigned short>(r), static_cast<unsigned short>(c)});
+  }
+  return t;
+}
+
+// Operand planes up to this size stay in L2 while a product runs.
+constexpr double kL2Planes = 70e6;
+
+// One single-matrix product on tiles of BM x BN.
+template <int BN, bool PAIR, bool F8>
+cudaError_t run_product(const void* A, const void* B, int64_t k_pad, int planes, TcParams& p,
+                        TcArea& area, cudaStream_t st) {
+  using Cfg = TcCfg<BN, PAIR, F8>;
+  CUtensorMap ta, tb;
+  if (!make_plane_map(&ta, A, k_pad, planes * p.rows_a, TC_BM, F8)) return cudaErrorInvalidValue;
+  if (!make_plane_map(&tb, B, k_pad, planes * p.rows_b, PAIR ? BN / 2 : BN, F8)) return cudaErrorInvalidValue;
+  const int units = PAIR ? tc_max_pairs() : tc_max_ctas();
+  const std::vector<TileAt> tiles = tile_order<BN, Cfg::BM>(p.m, p.n, p.sym, units);
+  const int ntiles = static_cast<int>(tiles.size());
+  p.units = chunk_count(p.prog, p.KT, p.CH);
+  const double plane_bytes = static_cast<double>(k_pad) * (F8 ? 1 : 2) * planes * (p.m + (A == B ? 0 : p.n));
+
+  // rounds of as many tiles as the area holds group sums for, in whole waves
+  const size_t tile_bytes = static_cast<size_t>(Cfg::RANKS) * p.prog.ng * Cfg::PART * sizeof(long long);
+  int per = static_cast<int>(std::min<size_t>(std::min(ntiles, kMaxLaunchTiles), area.bytes / tile_bytes));
+  if (per <= 0) return cudaErrorInvalidValue;
+  if (per < ntiles && per > units) per = per / units * units;
+  cudaError_t e = tc_area_clear(area, per * tile_bytes, st);
+  for (int t0 = 0; t0 < ntiles && e == cudaSuccess; t0 += per) {
+    p.tile0 = t0;
+    p.ntiles = std::min(per, ntiles - t0);
+    std::copy(tiles.begin() + t0, tiles.begin() + t0 + p.ntiles, p.at);
+    p.nwhole = g_split_tiles ? p.ntiles / units * units : p.ntiles;
+    const int nsplit = p.ntiles - p.nwhole;
+    // The tiles of a partial wave are shared by all CTAs. While the planes stay
+    // in L2, all their units in one sequence, evenly cut (n = 1792: 98 us per
+    // product against 105). Otherwise every tile in the same number of parts, so
+    // that the CTAs of a part walk the same planes at the same K and share their
+    // panels: out of step they stream them from HBM (n = 4096: 633 us against
+    // 754, n = 2048: 117 against 130).
+    p.parts = 0;
+    if (nsplit > 0 && plane_bytes > kL2Planes) p.parts = std::max(1, std::min(p.units, units / nsplit));
+    const int64_t split_units = static_cast<int64_t>(nsplit) * p.units;
+    int grid = units;
+    if (p.nwhole == 0) {
+      grid = p.parts > 0 ? nsplit * p.parts : static_cast<int>(std::min<int64_t>(units, split_units));
+    } else if (!g_split_tiles) {
+      grid = std::min(units, p.nwhole);
+    }
+    e = launch_tc_impl<BN, PAIR, F8>(ta, tb, p, (PAIR ? 2 : 1) * grid, st);
+  }
+  return e;
+}
+
+}  // namespace
+
 cudaError_t launch_ozaki_tc(const void* A, const void* B, const int32_t* ea, const int32_t* eb, int64_t m,
-                            int64_t n, int64_t rows_a, int64_t rows_b, int64_t k_pad, int s, int beta, int sym,
-                            const EpiArgs& epi, const int* done, int* err, double* scratch, void* split_ws,
-                            cudaStream_t st) {
+                            int64_t n, int64_t k, int64_t rows_a, int64_t rows_b, int64_t k_pad, int s, int beta,
+                            int sym, const EpiArgs& epi, const int* done, int* err, TcArea& area, cudaStream_t st) {
   if (m <= 0 || n <= 0) return cudaSuccess;
   const bool f8 = beta == 5;  // E4M3 nearest digits
-  const int BN = 256;
   const int atom_k = f8 ? 128 : TC_BK;
-  if (rows_a % TC_BM != 0 || rows_b % BN != 0 || k_pad % atom_k != 0) return cudaErrorInvalidValue;
+  if (rows_a % TC_BM != 0 || rows_b % 256 != 0 || k_pad % atom_k != 0) return cudaErrorInvalidValue;
   // products run on CTA pairs (256 x 256 tiles, 2-SM MMA) when rows allow
   const bool pair = g_pairing && rows_a % (2 * TC_BM) == 0 && k_pad % (2 * atom_k) == 0 && tc_max_pairs() > 0;
-  const int BM = pair ? 2 * TC_BM : TC_BM;
-  CUtensorMap ta, tb;
-  if (!make_plane_map(&ta, A, k_pad, static_cast<int64_t>(s) * rows_a, TC_BM, f8)) return cudaErrorInvalidValue;
-  if (!make_plane_map(&tb, B, k_pad, static_cast<int64_t>(s) * rows_b, pair ? BN / 2 : BN, f8))
-    return cudaErrorInvalidValue;
   TcParams p;
-  p.mats = nullptr;
-  p.tiles = nullptr;
-  p.phase = 0;
-  p.cur = 0;
+  std::memset(&p, 0, sizeof(p));
   p.s = s;
   p.beta = beta;
   p.KT = static_cast<int>(k_pad / atom_k);
@@ -1431,23 +1579,13 @@ cudaError_t launch_ozaki_tc(const void* A, const void* B, const int32_t* ea, con
   p.rows_a = rows_a;
   p.rows_b = rows_b;
   p.sym = sym;
-  p.tiles_m = static_cast<int>(rows_a / BM);
-  p.tiles_n = static_cast<int>(rows_b / BN);
-  {
-    // blocks of about as many tiles as run at once, near-square in elements
-    const int units = pair ? tc_max_pairs() : tc_max_ctas();
-    int w = static_cast<int>(std::lround(std::sqrt(static_cast<double>(units) * BM / BN)));
-    w = std::max(1, std::min(w, p.tiles_n));
-    p.band_w = w;
-    p.group_h = std::max(1, units / w);
-  }
   p.ea = ea;
   p.eb = eb;
   p.epi = epi;
   p.done = done;
   p.err = err;
+  p.area = static_cast<long long*>(area.ptr);
   p.timeout_ns = 5000000000ull;
-  p.stall_test = 0;
   // the stall test is taken by a launch that runs now, never by one being
   // captured into a graph (every replay would stall)
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
@@ -1457,105 +1595,71 @@ cudaError_t launch_ozaki_tc(const void* A, const void* B, const int32_t* ea, con
       p.timeout_ns = 1000ull * static_cast<unsigned long long>(us);
     }
   }
-  int ntiles = 0;
-  if (sym) {
-    for (int bj = 0; bj < p.tiles_n; ++bj) ntiles += std::min(p.tiles_m, (BN * (bj + 1)) / BM);
-  } else {
-    ntiles = p.tiles_m * p.tiles_n;
-  }
-  p.ntiles = ntiles;
-  p.scratch = scratch;
-  // split: when the tiles fill at most half a wave of CTAs (CTA pairs), they
-  // are all cut into fp32-chunk units shared out evenly over every CTA, so the
-  // idle part of the wave works too. Needs at most two level groups (their
-  // sums are then finished in the output pass) and the caller's split
-  // workspace. Measured on GB300 (INT8, s = 5 with an 8-slice refinement):
-  // 10 pair tiles (n = 1024) 0.197 -> 0.117 ms per product, 36 (n = 2048) 0.273
-  // -> 0.204 ms, but 66 of 74 pairs (n = 2816) 0.339 -> 0.443 ms: the units'
-  // L2 reductions then cost more than the few idle pairs; sharing out only the
-  // last partial wave of a larger launch measured slower as well (n >= 4096).
-  const int units = pair ? tc_max_pairs() : tc_max_ctas();
-  p.split_unit_count = 0;
-  p.split_area = nullptr;
-  p.split_cnt = nullptr;
-  p.tile_counter = nullptr;
-  const bool split =
-      g_split_tiles && split_ws != nullptr && 2 * ntiles <= units && s <= 2 * p.group && epi.kind != EPI_LEVELS;
-  if (split) {
-    const int ranks = pair ? 2 : 1;
-    const int KSUB = pair ? 2 : 1;
-    const int kts = p.KT / KSUB, chs = p.CH / KSUB;
-    int cnt = 0;
-    for (int L = s + 1; L >= 2; --L) {
-      const int np = std::min(s, L - 1) - std::max(1, L - s) + 1;
-      cnt += (np * kts + chs - 1) / chs;
-    }
-    p.split_unit_count = cnt;
-    p.split_area = static_cast<long long*>(split_ws);
-    p.split_cnt = reinterpret_cast<int*>(static_cast<char*>(split_ws) + tc_split_area_bytes());
-    // the tiles' group sums and counters start from zero
-    const size_t area = static_cast<size_t>(ntiles) * ranks * 2 * TC_BM * 256 * sizeof(long long);
-    cudaError_t e = cudaMemsetAsync(split_ws, 0, area, st);
-    if (e == cudaSuccess)
-      e = cudaMemsetAsync(p.split_cnt, 0, static_cast<size_t>(ntiles) * ranks * TC_EPI_WARPS * sizeof(int), st);
-    if (e != cudaSuccess) return e;
-  }
+  direct_program(s, beta, p.group, k, epi.kind == EPI_LEVELS, p.prog);
   ProfScope prof(DMP_PROF_PRODUCT, st);
-  const int grid_units = split ? units : std::min(ntiles, units);
-  if (pair) {
-    const int grid = 2 * grid_units;
-    if (split)
-      return f8 ? launch_tc_impl<256, true, true, 1>(ta, tb, p, grid, st)
-                : launch_tc_impl<256, true, false, 1>(ta, tb, p, grid, st);
-    return f8 ? launch_tc_impl<256, true, true>(ta, tb, p, grid, st) : launch_tc_impl<256, true>(ta, tb, p, grid, st);
-  }
-  const int grid = grid_units;
-  if (split)
-    return f8 ? launch_tc_impl<256, false, true, 1>(ta, tb, p, grid, st)
-              : launch_tc_impl<256, false, false, 1>(ta, tb, p, grid, st);
-  return f8 ? launch_tc_impl<256, false, true>(ta, tb, p, grid, st) : launch_tc_impl<256, false>(ta, tb, p, grid, st);
+  if (pair)
+    return f8 ? run_product<256, true, true>(A, B, k_pad, s, p, area, st)
+              : run_product<256, true, false>(A, B, k_pad, s, p, area, st);
+  return f8 ? run_product<256, false, true>(A, B, k_pad, s, p, area, st)
+            : run_product<256, false, false>(A, B, k_pad, s, p, area, st);
 }
 
-cudaError_t launch_ozaki_tc_grouped(const BatchMat* mats, const int4* tiles, int ntiles, int bn, bool pair, int beta,
-                                    int phase, int cur, int* err, double* scratch, int* counter, cudaStream_t st) {
+cudaError_t launch_ozaki_tc_grouped(const BatchMat* mats, const int4* tiles, int ntiles, int64_t nmax, int bn,
+                                    bool pair, int beta, int s, int phase, int cur, int* err, TcArea& area,
+                                    int* counter, cudaStream_t st) {
   if (ntiles <= 0) return cudaSuccess;
+  if (pair && (bn != 256 || tc_max_pairs() <= 0)) return cudaErrorInvalidValue;
+  if (beta == 5 && bn != 256) return cudaErrorInvalidValue;  // E4M3 digits: 256-column tiles
   TcParams p;
   std::memset(&p, 0, sizeof(p));
+  p.s = s;
   p.beta = beta;
   p.CH = beta == 5 ? 512 : 16;
   p.group = beta == 8 ? 3 : 4;
-  p.ntiles = ntiles;
-  p.scratch = scratch;
   p.sym = 1;
+  p.units = 1;
   p.mats = mats;
   p.tiles = tiles;
   p.phase = phase;
   p.cur = cur;
   p.err = err;
-  p.done = nullptr;
+  p.area = static_cast<long long*>(area.ptr);
   p.timeout_ns = 5000000000ull;
+  p.tile_counter = counter;
+  direct_program(s, beta, p.group, nmax, false, p.prog);
   CUtensorMap unused;
   std::memset(&unused, 0, sizeof(unused));
-  if (pair) {
-    // CTA pairs (256-row tiles, 256 columns): the pairs walk the list (largest
-    // matrices first) round robin
-    if (bn != 256 || tc_max_pairs() <= 0) return cudaErrorInvalidValue;
-    const int grid = 2 * std::min(ntiles, tc_max_pairs());
-    ProfScope prof(DMP_PROF_PRODUCT, st);
-    return beta == 5 ? launch_tc_impl<256, true, true>(unused, unused, p, grid, st)
-                     : launch_tc_impl<256, true, false>(unused, unused, p, grid, st);
-  }
-  // single CTAs take tiles from a counter as they free up (the tiles differ in
-  // work: the list holds the largest matrices' tiles first)
-  p.tile_counter = counter;
-  cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(int), st);
-  if (e != cudaSuccess) return e;
-  const int grid = std::min(ntiles, tc_max_ctas());
+  const int units = pair ? tc_max_pairs() : tc_max_ctas();
+  const size_t tile_bytes = static_cast<size_t>(pair ? 2 : 1) * p.prog.ng * TC_BM * bn * sizeof(long long);
+  int per = static_cast<int>(std::min<size_t>(ntiles, area.bytes / tile_bytes));
+  if (per <= 0) return cudaErrorInvalidValue;
+  if (pair && per < ntiles && per > units) per = per / units * units;
   ProfScope prof(DMP_PROF_PRODUCT, st);
-  if (beta == 5) return bn == 256 ? launch_tc_impl<256, false, true, 2>(unused, unused, p, grid, st)
-                                  : cudaErrorInvalidValue;  // E4M3 digits: 256-column tiles
-  if (bn == 128) return launch_tc_impl<128, false, false, 2>(unused, unused, p, grid, st);
-  return launch_tc_impl<256, false, false, 2>(unused, unused, p, grid, st);
+  cudaError_t e = tc_area_clear(area, per * tile_bytes, st);
+  for (int t0 = 0; t0 < ntiles && e == cudaSuccess; t0 += per) {
+    p.tile0 = t0;
+    p.ntiles = p.nwhole = std::min(per, ntiles - t0);
+    const int grid = std::min(p.ntiles, units);
+    if (pair) {
+      // CTA pairs (256-row tiles, 256 columns): the pairs walk the list (largest
+      // matrices first) round robin
+      e = beta == 5 ? launch_tc_impl<256, true, true>(unused, unused, p, 2 * grid, st)
+                    : launch_tc_impl<256, true, false>(unused, unused, p, 2 * grid, st);
+      continue;
+    }
+    // single CTAs take tiles from a counter as they free up (the tiles differ in
+    // work: the list holds the largest matrices' tiles first)
+    e = cudaMemsetAsync(counter, 0, sizeof(int), st);
+    if (e != cudaSuccess) return e;
+    if (beta == 5) {
+      e = launch_tc_impl<256, false, true, 2>(unused, unused, p, grid, st);
+    } else if (bn == 128) {
+      e = launch_tc_impl<128, false, false, 2>(unused, unused, p, grid, st);
+    } else {
+      e = launch_tc_impl<256, false, false, 2>(unused, unused, p, grid, st);
+    }
+  }
+  return e;
 }
 
 }  // namespace dmp
