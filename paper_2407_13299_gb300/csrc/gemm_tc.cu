@@ -130,7 +130,9 @@ struct TcParams {
   int tile0, ntiles;  // this launch's tiles: tile0 .. tile0 + ntiles - 1
   int nwhole;         // tiles (of ntiles) walked whole, round robin; the rest are split over all CTAs (CTA pairs)
   int units;          // fp32 chunks per tile (split launches: one matrix, every tile alike)
-  int parts;          // each split tile in this many equal ranges; 0: all split tiles' units in one sequence
+  // the first heads * head_len units of each split tile in `heads` equal ranges, one CTA (CTA pair) each; the
+  // other units of all split tiles in one sequence, evenly cut over the other CTAs
+  int heads, head_len;
   int group;        // levels combined exactly per int64 group: 4 (beta 7, 5) or 3 (beta 8)
   long long* area;  // group sums of the launch's tiles: [tile][CTA rank][group][PART]
   int64_t m, n;
@@ -861,19 +863,24 @@ ozaki_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
   // WALK 0: this CTA's items. Items 0 .. nfull - 1 are whole tiles; after them
   // come the tiles its range [u_begin, u_end) of the split tiles' units meets.
   const int nfull = p.nwhole > cta_id ? (p.nwhole - cta_id - 1) / cta_stride + 1 : 0;
+  // (u_end - u_begin units of the sequence of the tiles' units seg_off .. seg_off + seg_len - 1)
   const int nsplit = p.ntiles - p.nwhole;
+  const int heads = nsplit * p.heads;
   int64_t u_begin, u_end;
-  if (p.parts > 0) {
-    const int part = cta_id / max(nsplit, 1);
-    const int64_t base = static_cast<int64_t>(cta_id - part * nsplit) * p.units;
-    u_begin = base + p.units * min(part, p.parts) / p.parts;
-    u_end = base + p.units * min(part + 1, p.parts) / p.parts;
+  int seg_off = 0, seg_len = p.units;
+  if (cta_id < heads) {
+    const int part = cta_id / nsplit;
+    seg_off = part * p.head_len;
+    seg_len = max(min(p.head_len, p.units - seg_off), 0);
+    u_begin = static_cast<int64_t>(cta_id - part * nsplit) * seg_len;
+    u_end = u_begin + seg_len;
   } else {
-    const int64_t split_units = static_cast<int64_t>(nsplit) * p.units;
-    u_begin = split_units * cta_id / cta_stride;
-    u_end = split_units * (cta_id + 1) / cta_stride;
+    seg_off = p.heads * p.head_len;
+    seg_len = max(p.units - seg_off, 0);
+    const int64_t all = static_cast<int64_t>(nsplit) * seg_len;
+    u_begin = all * (cta_id - heads) / max(cta_stride - heads, 1);
+    u_end = all * (cta_id - heads + 1) / max(cta_stride - heads, 1);
   }
-  const int split_lo = u_begin < u_end ? static_cast<int>(u_begin / p.units) : 0;
   // item `it`: its tile (counted from tile0) and unit range [u0, u1); false past the last
   auto static_item = [&](int it, int& tile, int& u0, int& u1) __attribute__((always_inline)) -> bool {
     if (it < nfull) {
@@ -882,12 +889,13 @@ ozaki_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
       u1 = 0x7fffffff;
       return true;
     }
-    const int tt = split_lo + (it - nfull);
-    const int64_t base = static_cast<int64_t>(tt) * p.units;
-    if (u_begin >= u_end || base >= u_end) return false;
+    if (u_begin >= u_end) return false;
+    const int tt = static_cast<int>(u_begin / seg_len) + (it - nfull);
+    const int64_t base = static_cast<int64_t>(tt) * seg_len;
+    if (base >= u_end) return false;
     tile = p.nwhole + tt;
-    u0 = static_cast<int>(u_begin > base ? u_begin - base : 0);
-    u1 = static_cast<int>(u_end - base < p.units ? u_end - base : p.units);
+    u0 = seg_off + static_cast<int>(u_begin > base ? u_begin - base : 0);
+    u1 = seg_off + static_cast<int>(u_end - base < seg_len ? u_end - base : seg_len);
     return true;
   };
 
@@ -1505,6 +1513,24 @@ std::vector<TileAt> tile_order(int64_t m, int64_t n, int sym, int units) {
   return t;
 }
 
+// Length of the equal parts of a split tile's `units` (TcParams::head_len): the
+// one for which the longest share is shortest, the rest of the nsplit tiles
+// going to `extra` CTAs (none: the parts cover the tile).
+int head_length(int units, int nsplit, int heads, int extra) {
+  const int most = (units + heads - 1) / heads;
+  if (extra <= 0) return most;
+  int best = most, best_share = most;
+  for (int h = 1; h < most; ++h) {
+    const int64_t rest = static_cast<int64_t>(nsplit) * (units - heads * h);
+    const int share = std::max(h, static_cast<int>((rest + extra - 1) / extra));
+    if (share < best_share) {
+      best = h;
+      best_share = share;
+    }
+  }
+  return best;
+}
+
 // Operand planes up to this size stay in L2 while a product runs.
 constexpr double kL2Planes = 70e6;
 
@@ -1535,17 +1561,21 @@ cudaError_t run_product(const void* A, const void* B, int64_t k_pad, int planes,
     p.nwhole = g_split_tiles ? p.ntiles / units * units : p.ntiles;
     const int nsplit = p.ntiles - p.nwhole;
     // The tiles of a partial wave are shared by all CTAs. While the planes stay
-    // in L2, all their units in one sequence, evenly cut (n = 1792: 98 us per
-    // product against 105). Otherwise every tile in the same number of parts, so
-    // that the CTAs of a part walk the same planes at the same K and share their
-    // panels: out of step they stream them from HBM (n = 4096: 633 us against
-    // 754, n = 2048: 117 against 130).
-    p.parts = 0;
-    if (nsplit > 0 && plane_bytes > kL2Planes) p.parts = std::max(1, std::min(p.units, units / nsplit));
+    // in L2, all their units are one sequence, evenly cut (n = 1792: 98 us per
+    // product against 105 for two CTAs per tile). Otherwise a CTA takes the same
+    // part of its tile as the others, so that they walk the same planes at the
+    // same K and share their panels (out of step they stream them from HBM: n =
+    // 4096 754 us against 633 for one CTA per tile), and what that leaves of
+    // each tile goes to the CTAs that are left.
+    p.heads = p.head_len = 0;
     const int64_t split_units = static_cast<int64_t>(nsplit) * p.units;
+    if (nsplit > 0 && plane_bytes > kL2Planes) {
+      p.heads = std::min(p.units, units / nsplit);
+      p.head_len = head_length(p.units, nsplit, p.heads, units - nsplit * p.heads);
+    }
     int grid = units;
     if (p.nwhole == 0) {
-      grid = p.parts > 0 ? nsplit * p.parts : static_cast<int>(std::min<int64_t>(units, split_units));
+      grid = static_cast<int>(std::min<int64_t>(units, split_units));
     } else if (!g_split_tiles) {
       grid = std::min(units, p.nwhole);
     }

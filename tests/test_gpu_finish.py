@@ -56,8 +56,8 @@ def test_results_outside_the_normal_range(dmp, s):
     """Rows scaled so that products are subnormal, zero or near the largest
     double, in one matrix with ordinary rows."""
     rng = np.random.default_rng(40 + s)
-    A = rng.standard_normal((64, 40)) * (2.0 ** rng.integers(-520, 500, size=(64, 1)).astype(float))
-    B = rng.standard_normal((40, 48)) * (2.0 ** rng.integers(-540, 500, size=(1, 48)).astype(float))
+    A = rng.standard_normal((64, 40)) * (2.0 ** np.linspace(-540, 500, 64).round())[:, None]
+    B = rng.standard_normal((40, 48)) * (2.0 ** np.linspace(-540, 500, 48).round())[None, :]
     A[5] = 0.0
     want = _want(A, B, "int8", s)
     assert np.any((want != 0) & (np.abs(want) < 2.0 ** -1022)) and np.any(np.abs(want) > 1e200)
