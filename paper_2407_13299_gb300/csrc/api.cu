@@ -38,6 +38,7 @@ struct Opts {
   bool store32;  // DMP_FLAG_FP32_STORAGE
   int late_s;    // late-slice schedule: 0 off, else the slice count after the switch
   double late_idem;
+  int64_t diff_n;  // the size that decides on difference products (they take more planes); 0: none
 };
 
 int normalize(const dmp_opts* o, Opts& out) {
@@ -74,6 +75,7 @@ int normalize(const dmp_opts* o, Opts& out) {
   out.refine = o->refine_slices;
   if (out.refine != 0 && out.mode == DMP_FP64) out.refine = -1;
   if (out.refine < -1 || out.refine > smax) return DMP_ERR_INVALID_ARG;
+  out.diff_n = 0;
   out.late_s = out.mode == DMP_FP64 ? 0 : o->late_slices;
   out.late_idem = o->late_idem;
   if (out.late_s < 0 || out.late_s > smax || !(out.late_idem >= 0.0)) return DMP_ERR_INVALID_ARG;
@@ -87,6 +89,26 @@ bool levels_fit_int32(int64_t k, int s, int mode) {
   const double dmax = digit_max(mode);
   const double bound = static_cast<double>(s) * static_cast<double>(k) * dmax * dmax;
   return bound < 2147483648.0;
+}
+
+// Difference products pay from these sizes on (the smallest dimension): they
+// save products, n^3, for more planes to split, n^2, and about twice the adds to
+// the group sums, which bound the product kernel below. Split and product in us,
+// with differences / without: s = 5, n = 1792 115 / 114, 2048 138 / 143, 3000
+// 320 / 341, 4096 671 / 722; s = 8 (two group sums), n = 2304 370 / 342, 2560
+// 448 / 456, 3000 629 / 684, 4096 1354 / 1552.
+constexpr int64_t kDiffMin = 1920;     // s <= 6: one group sum per element
+constexpr int64_t kDiffMinTwo = 2560;  // s >= 7
+
+bool has_diff(const Opts& o, int s) {
+  return s >= kDiffSlicesMin && s <= kDiffSlicesMax && o.diff_n >= (s <= 6 ? kDiffMin : kDiffMinTwo);
+}
+// planes of an operand at s slices
+int64_t planes_of(const Opts& o, int s) { return s + (has_diff(o, s) ? diff_planes(s) : 0); }
+// The size that decides for an m x n product with inner size k; 0 for digits
+// other than INT8's held in bfloat16 (the tcgen05 executor).
+int64_t diff_size(const Opts& o, int64_t m, int64_t n, int64_t k) {
+  return o.mode == DMP_OZAKI_INT8 && o.executor == DMP_EXEC_TC ? std::min(m, std::min(n, k)) : 0;
 }
 
 // digit plane element: int8 (IMMA), bfloat16 (tcgen05) or E4M3 bytes (E4M3 mode)
@@ -136,7 +158,7 @@ PurifyLayout purify_layout(int64_t n, const Opts& o) {
   L.X2 = c.take(static_cast<size_t>(n) * n * sizeof(double));
   if (o.mode != DMP_FP64) {
     // room for the refinement step's slices too
-    const int planes = std::max(std::max(o.s, o.refine), o.late_s);
+    const int64_t planes = std::max(planes_of(o, o.s), std::max(planes_of(o, o.refine), planes_of(o, o.late_s)));
     const size_t plane = static_cast<size_t>(planes) * L.n_pad * L.k_pad * elem_bytes(o);
     L.planesP = c.take(plane);
     L.planesX = c.take(plane);
@@ -155,7 +177,7 @@ cudaError_t launch_product(const Opts& o, const void* pa, const void* pb, const 
                            const EpiArgs& epi, const int* done, int* err, TcArea& area, cudaStream_t st) {
   if (o.executor == DMP_EXEC_TC)
     return launch_ozaki_tc(pa, pb, ea, eb, m, n, k, rows_a, rows_b, k_pad, o.s, o.beta,
-                           sym, epi, done, err, area, st);
+                           has_diff(o, o.s), sym, epi, done, err, area, st);
   return launch_ozaki_imma(static_cast<const int8_t*>(pa), static_cast<const int8_t*>(pb), ea, eb, m, n, rows_a,
                            rows_b, k_pad, o.s, o.beta, sym, epi, done, st);
 }
@@ -217,7 +239,7 @@ BackwardLayout backward_layout(int64_t n, const Opts& o) {
   B.segP = c.take(nn * o.every);
   B.segX = c.take(nn * o.every);
   if (o.mode != DMP_FP64) {
-    const size_t plane = static_cast<size_t>(o.s) * B.n_pad * B.k_pad * elem_bytes(o);
+    const size_t plane = static_cast<size_t>(planes_of(o, o.s)) * B.n_pad * B.k_pad * elem_bytes(o);
     B.planesP = c.take(plane);
     B.planesA = c.take(plane);
   } else {
@@ -278,7 +300,7 @@ FoeLayout foe_layout(int64_t n, const Opts& o, int scheme, int M) {
   F.Tb = c.take(nn);
   F.Y = c.take(nn);
   if (o.mode != DMP_FP64) {
-    const size_t plane = static_cast<size_t>(o.s) * F.n_pad * F.k_pad * elem_bytes(o);
+    const size_t plane = static_cast<size_t>(planes_of(o, o.s)) * F.n_pad * F.k_pad * elem_bytes(o);
     F.expsH = c.take(static_cast<size_t>(F.n_pad) * sizeof(int32_t));
     F.expsT = c.take(static_cast<size_t>(F.n_pad) * sizeof(int32_t));
     F.planesH = c.take(plane);
@@ -339,6 +361,7 @@ int dmp_workspace_size(int64_t n, const dmp_opts* opts, size_t* bytes) {
   const int rc = normalize(opts, o);
   if (rc != DMP_OK) return rc;
   if (n < 2 || bytes == nullptr) return DMP_ERR_INVALID_ARG;
+  o.diff_n = diff_size(o, n, n, n);
   *bytes = purify_layout(n, o).total;
   return DMP_OK;
 }
@@ -368,6 +391,9 @@ int dm_purify(const double* H, int64_t n, int64_t ldh, int64_t n_occ, const dmp_
     return DMP_ERR_UNSUPPORTED;
   if ((o.refine != 0 || o.method != DMP_METHOD_PM || o.store32 || o.late_s > 0) && tape != nullptr)
     return DMP_ERR_UNSUPPORTED;
+  // a workspace without room for the difference planes runs the pairs one by one
+  o.diff_n = diff_size(o, n, n, n);
+  if (ws_bytes < purify_layout(n, o).total) o.diff_n = 0;
   const PurifyLayout L = purify_layout(n, o);
   if (ws_bytes < L.total) return DMP_ERR_WORKSPACE;
   TapeLayout TL{};
@@ -431,7 +457,7 @@ int dm_purify(const double* H, int64_t n, int64_t ldh, int64_t n_occ, const dmp_
       DMP_CUDA(launch_gemm_f64(cur, ldcur, cur, ldcur, n, n, n, 1, e2, done, st));
     } else {
       DMP_CUDA(launch_split_rows(cur, n, n, ldcur, oi.s, oi.beta, expsP, planesP, L.n_pad, L.k_pad,
-                                 elem_kind(o), nullptr, done, st));
+                                 elem_kind(o), has_diff(oi, oi.s), nullptr, done, st));
       DMP_CUDA(launch_product(oi, planesP, planesP, expsP, expsP, n, n, n, L.n_pad, L.n_pad, L.k_pad, 1, e2, done,
                               err, area, st));
     }
@@ -467,9 +493,9 @@ int dm_purify(const double* H, int64_t n, int64_t ldh, int64_t n_occ, const dmp_
           DMP_CUDA(launch_gemm_f64(X2, n, alt, ldalt, n, n, n, 1, ez, done, st));
         } else {
           DMP_CUDA(launch_split_rows(X2, n, n, n, oi.s, oi.beta, expsX, planesX, L.n_pad, L.k_pad,
-                                     elem_kind(o), nullptr, done, st));
+                                     elem_kind(o), has_diff(oi, oi.s), nullptr, done, st));
           DMP_CUDA(launch_split_rows(alt, n, n, ldalt, oi.s, oi.beta, expsP, planesP, L.n_pad, L.k_pad,
-                                     elem_kind(o), nullptr, done, st));
+                                     elem_kind(o), has_diff(oi, oi.s), nullptr, done, st));
           DMP_CUDA(launch_product(oi, planesX, planesP, expsX, expsP, n, n, n, L.n_pad, L.n_pad, L.k_pad, 1, ez, done,
                                   err, area, st));
         }
@@ -493,7 +519,7 @@ int dm_purify(const double* H, int64_t n, int64_t ldh, int64_t n_occ, const dmp_
       DMP_CUDA(launch_gemm_f64(cur, ldcur, X2, n, n, n, n, 1, e3, done, st));
     } else {
       DMP_CUDA(launch_split_rows(X2, n, n, n, oi.s, oi.beta, expsX, planesX, L.n_pad, L.k_pad,
-                                 elem_kind(o), nullptr, done, st));
+                                 elem_kind(o), has_diff(oi, oi.s), nullptr, done, st));
       DMP_CUDA(launch_product(oi, planesP, planesX, expsP, expsX, n, n, n, L.n_pad, L.n_pad, L.k_pad, 1, e3, done,
                               err, area, st));
     }
@@ -531,11 +557,11 @@ int dm_purify(const double* H, int64_t n, int64_t ldh, int64_t n_occ, const dmp_
         Opts orr = o;
         orr.s = o.refine;
         DMP_CUDA(launch_split_rows(cur, n, n, ldcur, orr.s, orr.beta, expsP, planesP, L.n_pad, L.k_pad,
-                                   elem_kind(o), nullptr, nullptr, st));
+                                   elem_kind(o), has_diff(orr, orr.s), nullptr, nullptr, st));
         DMP_CUDA(launch_product(orr, planesP, planesP, expsP, expsP, n, n, n, L.n_pad, L.n_pad, L.k_pad, 1, r2, nullptr,
                                 err, area, st));
         DMP_CUDA(launch_split_rows(X2, n, n, n, orr.s, orr.beta, expsX, planesX, L.n_pad, L.k_pad,
-                                   elem_kind(o), nullptr, nullptr, st));
+                                   elem_kind(o), has_diff(orr, orr.s), nullptr, nullptr, st));
         DMP_CUDA(launch_product(orr, planesP, planesX, expsP, expsX, n, n, n, L.n_pad, L.n_pad, L.k_pad, 1, r3, nullptr,
                                 err, area, st));
       }
@@ -656,7 +682,7 @@ GemmLayout gemm_layout(int64_t m, int64_t n, int64_t k, const Opts& o) {
   G.m_pad = round_up(std::max<int64_t>(m, 1), row_pad(o.executor));
   G.n_pad = round_up(std::max<int64_t>(n, 1), row_pad(o.executor));
   G.k_pad = k_pad_of(o, k);
-  const size_t planes = static_cast<size_t>(o.s);
+  const size_t planes = static_cast<size_t>(planes_of(o, o.s));
   G.ea = c.take(G.m_pad * sizeof(int32_t));
   G.eb = c.take(G.n_pad * sizeof(int32_t));
   G.err = c.take(sizeof(int32_t));
@@ -676,6 +702,17 @@ int gemm_opts(int32_t mode, int32_t slices, int32_t executor, Opts& o) {
   return normalize(&d, o);
 }
 }  // namespace
+
+int gemm_least_bytes(int64_t m, int64_t n, int64_t k, int32_t mode, int32_t slices, int32_t executor,
+                     size_t* bytes) {
+  Opts o;
+  const int rc = gemm_opts(mode, slices, executor, o);
+  if (rc != DMP_OK) return rc;
+  if (m < 0 || n < 0 || k < 0 || bytes == nullptr) return DMP_ERR_INVALID_ARG;
+  *bytes = o.mode == DMP_FP64 ? 0 : gemm_layout(m, n, k, o).total;
+  return DMP_OK;
+}
+
 }  // namespace dmp
 
 extern "C" {
@@ -686,6 +723,7 @@ int ozaki_gemm_workspace_size(int64_t m, int64_t n, int64_t k, int32_t mode, int
   const int rc = gemm_opts(mode, slices, executor, o);
   if (rc != DMP_OK) return rc;
   if (m < 0 || n < 0 || k < 0 || bytes == nullptr) return DMP_ERR_INVALID_ARG;
+  o.diff_n = diff_size(o, m, n, k);
   *bytes = o.mode == DMP_FP64 ? 0 : gemm_layout(m, n, k, o).total;
   return DMP_OK;
 }
@@ -707,8 +745,11 @@ static int ozaki_common(int64_t m, int64_t n, int64_t k, const double* A, int64_
   }
   if (!levels_fit_int32(k, o.s, o.mode))
     return DMP_ERR_UNSUPPORTED;
+  if (epi.kind != EPI_LEVELS) o.diff_n = diff_size(o, m, n, k);
+  if (ws_bytes < gemm_layout(m, n, k, o).total) o.diff_n = 0;
   const GemmLayout G = gemm_layout(m, n, k, o);
   if (ws == nullptr || ws_bytes < G.total) return DMP_ERR_WORKSPACE;
+  const bool diff = has_diff(o, o.s);
   int32_t* ea = reinterpret_cast<int32_t*>(at(ws, G.ea));
   int32_t* eb = reinterpret_cast<int32_t*>(at(ws, G.eb));
   int* err = reinterpret_cast<int*>(at(ws, G.err));
@@ -716,10 +757,10 @@ static int ozaki_common(int64_t m, int64_t n, int64_t k, const double* A, int64_
   void* pa = at(ws, G.pa);
   void* pb = at(ws, G.pb);
   double* Bt = reinterpret_cast<double*>(at(ws, G.Bt));
-  DMP_CUDA(launch_split_rows(A, m, k, lda, o.s, o.beta, ea, pa, G.m_pad, G.k_pad, elem_kind(o), nullptr,
+  DMP_CUDA(launch_split_rows(A, m, k, lda, o.s, o.beta, ea, pa, G.m_pad, G.k_pad, elem_kind(o), diff, nullptr,
                              nullptr, st));
   DMP_CUDA(launch_transpose(B, k, n, ldb, Bt, st));
-  DMP_CUDA(launch_split_rows(Bt, n, k, k, o.s, o.beta, eb, pb, G.n_pad, G.k_pad, elem_kind(o), nullptr,
+  DMP_CUDA(launch_split_rows(Bt, n, k, k, o.s, o.beta, eb, pb, G.n_pad, G.k_pad, elem_kind(o), diff, nullptr,
                              nullptr, st));
   if (o.executor == DMP_EXEC_TC) DMP_CUDA(cudaMemsetAsync(err, 0, sizeof(int), st));
   DMP_CUDA(launch_product(o, pa, pb, ea, eb, m, n, k, G.m_pad, G.n_pad, G.k_pad, 0, epi, nullptr, err, area, st));
@@ -773,7 +814,7 @@ int ozaki_split(int64_t m, int64_t k, const double* A, int64_t lda, int32_t mode
   const int eb = elem_bytes(o);
   const int64_t m_pad = G.m_pad, k_pad = G.k_pad;
   char* pa = at(ws, G.pa);
-  DMP_CUDA(launch_split_rows(A, m, k, lda, o.s, o.beta, ea, pa, m_pad, k_pad, elem_kind(o), nullptr,
+  DMP_CUDA(launch_split_rows(A, m, k, lda, o.s, o.beta, ea, pa, m_pad, k_pad, elem_kind(o), false, nullptr,
                              nullptr, st));
   DMP_CUDA(cudaMemcpyAsync(exps, ea, m * sizeof(int32_t), cudaMemcpyDeviceToDevice, st));
   for (int i = 0; i < o.s; ++i) {
@@ -789,6 +830,7 @@ int dmp_backward_workspace_size(int64_t n, const dmp_opts* opts, size_t* bytes) 
   const int rc = normalize(opts, o);
   if (rc != DMP_OK) return rc;
   if (n < 2 || bytes == nullptr) return DMP_ERR_INVALID_ARG;
+  o.diff_n = diff_size(o, n, n, n);
   *bytes = backward_layout(n, o).total;
   return DMP_OK;
 }
@@ -805,6 +847,8 @@ int dm_purify_backward(const double* H, int64_t n, int64_t n_occ, const dmp_opts
   if (n < 2 || n_occ <= 0 || n_occ >= n) return DMP_ERR_INVALID_ARG;
   const TapeLayout TL = tape_layout(n, o);
   if (tape_bytes < TL.total) return DMP_ERR_WORKSPACE;
+  o.diff_n = diff_size(o, n, n, n);
+  if (ws_bytes < backward_layout(n, o).total) o.diff_n = 0;
   const BackwardLayout B = backward_layout(n, o);
   if (ws_bytes < B.total) return DMP_ERR_WORKSPACE;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
@@ -853,7 +897,7 @@ int dm_purify_backward(const double* H, int64_t n, int64_t n_occ, const dmp_opts
     e.ldc = n;
     if (o.mode == DMP_FP64) return launch_gemm_f64(A, n, Pk, n, n, n, n, 0, e, nullptr, st);
     cudaError_t r = launch_split_rows(A, n, n, n, o.s, o.beta, expsA, planesA, npad, kpad, elem_kind(o),
-                                      nullptr, nullptr, st);
+                                      has_diff(o, o.s), nullptr, nullptr, st);
     if (r != cudaSuccess) return r;
     return launch_product(o, planesA, planesP, expsA, expsP, n, n, n, npad, npad, kpad, 0, e, nullptr,
                           err, area, st);
@@ -861,7 +905,7 @@ int dm_purify_backward(const double* H, int64_t n, int64_t n_occ, const dmp_opts
   auto split_P = [&](const double* Pk) -> cudaError_t {
     if (o.mode == DMP_FP64) return cudaSuccess;
     return launch_split_rows(Pk, n, n, n, o.s, o.beta, expsP, planesP, npad, kpad, elem_kind(o),
-                             nullptr, nullptr, st);
+                             has_diff(o, o.s), nullptr, nullptr, st);
   };
 
   // host copies of the per-step update weights (kept alive until the stream syncs)
@@ -917,7 +961,7 @@ int dm_purify_backward(const double* H, int64_t n, int64_t n_occ, const dmp_opts
           DMP_CUDA(launch_gemm_f64(Pk, n, Xk, n, n, n, n, 1, e3, nullptr, st));
         } else {
           DMP_CUDA(launch_split_rows(Xk, n, n, n, o.s, o.beta, expsA, planesA, npad, kpad, elem_kind(o),
-                                     nullptr, nullptr, st));
+                                     has_diff(o, o.s), nullptr, nullptr, st));
           DMP_CUDA(launch_product(o, planesP, planesA, expsP, expsA, n, n, n, npad, npad, kpad, 1, e3, nullptr,
                                   err, area, st));
         }
@@ -969,6 +1013,7 @@ int dm_foe_workspace_size(int64_t n, const dmp_foe_params* params, const dmp_opt
   const int scheme = params->scheme;
   if (M < 2 || M > kFoeMaxTerms) return DMP_ERR_INVALID_ARG;
   if (scheme != DMP_FOE_RECURRENCE && scheme != DMP_FOE_PATERSON_STOCKMEYER) return DMP_ERR_INVALID_ARG;
+  o.diff_n = diff_size(o, n, n, n);
   *bytes = foe_layout(n, o, scheme, M).total;
   return DMP_OK;
 }
@@ -991,6 +1036,8 @@ int dm_foe(const double* H, int64_t n, int64_t ldh, const dmp_foe_params* params
   if (fp.scheme != DMP_FOE_RECURRENCE && !ps) return DMP_ERR_INVALID_ARG;
   if (!std::isfinite(fp.e_min) || !std::isfinite(fp.e_max)) return DMP_ERR_INVALID_ARG;
   if (o.mode != DMP_FP64 && !levels_fit_int32(n, o.s, o.mode)) return DMP_ERR_UNSUPPORTED;
+  o.diff_n = diff_size(o, n, n, n);
+  if (ws_bytes < foe_layout(n, o, fp.scheme, M).total) o.diff_n = 0;
   const FoeLayout L = foe_layout(n, o, fp.scheme, M);
   if (ws_bytes < L.total) return DMP_ERR_WORKSPACE;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
@@ -1052,7 +1099,7 @@ int dm_foe(const double* H, int64_t n, int64_t ldh, const dmp_foe_params* params
       DMP_CUDA(launch_gemm_f64(A, n, B, n, n, n, n, 1, e, nullptr, st));
     } else {
       DMP_CUDA(launch_split_rows(B, n, n, n, o.s, o.beta, expsT, planesT, L.n_pad, L.k_pad, elem_kind(o),
-                                 nullptr, err, st));
+                                 has_diff(o, o.s), nullptr, err, st));
       DMP_CUDA(launch_product(o, pa, planesT, ea, expsT, n, n, n, L.n_pad, L.n_pad, L.k_pad, 1, e, err,
                               err, area, st));
     }
@@ -1068,7 +1115,7 @@ int dm_foe(const double* H, int64_t n, int64_t ldh, const dmp_foe_params* params
   auto split_a = [&](const double* A, void* planes, int32_t* exps) -> int {
     if (oz)
       DMP_CUDA(launch_split_rows(A, n, n, n, o.s, o.beta, exps, planes, L.n_pad, L.k_pad, elem_kind(o),
-                                 nullptr, err, st));
+                                 has_diff(o, o.s), nullptr, err, st));
     return DMP_OK;
   };
 

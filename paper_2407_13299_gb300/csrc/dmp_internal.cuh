@@ -30,6 +30,32 @@ inline int digit_max(int mode) {
 inline int max_slices(int mode) { return mode == DMP_OZAKI_E4M3 ? 12 : (mode == DMP_OZAKI_BF16 ? 9 : 10); }
 inline int64_t round_up(int64_t x, int64_t m) { return (x + m - 1) / m * m; }
 
+// ---------------------------------------------------------------- difference products
+// The pairs (i, j) and (j, i) of a level together cost one product instead of
+// two: A_i B_j + A_j B_i = A_i B_i + A_j B_j - (A_i - A_j)(B_i - B_j), where the
+// A_i B_i are shared by all levels. The truncated beta = 7 digits of an entry
+// have its sign, so the differences stay within +-127 and the products are as
+// exact as the digits' own. Digit pairs i < j <= s - 1 with i + j <= s + 1 are
+// taken this way (for j = s the extra A_s B_s would cost what it saves), in the
+// order (1,2), (1,3), ..; their planes follow the s digit planes. Products per
+// output tile: s = 4: 8 instead of 10, 5: 11 / 15, 6: 15 / 21, 7: 19 / 28,
+// 8: 24 / 36, 9: 29 / 45.
+constexpr int kDiffSlicesMin = 4, kDiffSlicesMax = 9;
+// difference planes of s digit slices
+__host__ __device__ constexpr int diff_planes(int s) {
+  int c = 0;
+  for (int i = 1; i < s; ++i)
+    for (int j = i + 1; j < s && i + j <= s + 1; ++j) ++c;
+  return c;
+}
+// plane index of the difference of digits i < j
+__host__ __device__ constexpr int diff_plane(int s, int i, int j) {
+  int c = s;
+  for (int a = 1; a < i; ++a)
+    for (int b = a + 1; b < s && a + b <= s + 1; ++b) ++c;
+  return c + (j - i - 1);
+}
+
 // ---------------------------------------------------------------- launch accounting
 extern std::atomic<long long> g_launches;
 inline void count_launch(long long k = 1) { g_launches.fetch_add(k, std::memory_order_relaxed); }
@@ -82,10 +108,14 @@ __device__ __forceinline__ double stored_value(double v, bool round32) {
 // (int8 truncated digits), 3 (bfloat16: the beta 7 truncated digits, or the
 // beta 8 nearest digits) or 4 (beta 5 nearest digits as E4M3 bytes). Nearest
 // digits take a row exponent one larger. Padding rows/columns are zero. Sets
-// *flag to 1 if A holds a NaN/Inf.
+// *flag to 1 if A holds a NaN/Inf. diff: the difference planes follow the digit
+// planes (kind 3 with beta 7, kDiffSlicesMin <= s <= kDiffSlicesMax).
 cudaError_t launch_split_rows(const double* A, int64_t m, int64_t k, int64_t lda, int s, int beta,
                               int32_t* exps, void* planes, int64_t m_pad, int64_t k_pad,
-                              int elem_kind, int* flag, const int* done, cudaStream_t st);
+                              int elem_kind, bool diff, int* flag, const int* done, cudaStream_t st);
+
+// The smallest workspace ozaki_gemm accepts (without difference planes).
+int gemm_least_bytes(int64_t m, int64_t n, int64_t k, int32_t mode, int32_t slices, int32_t executor, size_t* bytes);
 
 // Out-of-place transpose (m x n, lda) -> (n x m, leading dimension m).
 cudaError_t launch_transpose(const double* A, int64_t m, int64_t n, int64_t lda, double* At,
@@ -118,6 +148,7 @@ cudaError_t launch_ozaki_imma(const int8_t* A, const int8_t* B, const int32_t* e
 // A planes [s][rows_a][k_pad], B planes [s][rows_b][k_pad] in bfloat16 (E4M3
 // bytes for beta 5); rows_a a multiple of 128, rows_b of 256, k_pad of 64
 // (128 for beta 5).
+// diff: both operands hold their difference planes.
 // *err is set to 1 if a bounded device wait expired. k is the unpadded inner size.
 constexpr int kTcMaxCtas = 160;
 // The tcgen05 executor's group sums (int64, per tile of a launch): `clean` bytes
@@ -143,7 +174,7 @@ bool tc_pairs_available();
 int set_stall_test(int wait_limit_us);
 cudaError_t launch_ozaki_tc(const void* A, const void* B, const int32_t* ea, const int32_t* eb, int64_t m,
                             int64_t n, int64_t k, int64_t rows_a, int64_t rows_b, int64_t k_pad, int s, int beta,
-                            int sym, const EpiArgs& epi, const int* done, int* err, TcArea& area, cudaStream_t st);
+                            bool diff, int sym, const EpiArgs& epi, const int* done, int* err, TcArea& area, cudaStream_t st);
 
 // FP64 executor: C = A B (A m x k, B k x n row-major) with the same epilogues.
 cudaError_t launch_gemm_f64(const double* A, int64_t lda, const double* B, int64_t ldb, int64_t m,

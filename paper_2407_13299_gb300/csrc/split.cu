@@ -79,12 +79,12 @@ __device__ __forceinline__ uint32_t field(uint32_t w0, uint32_t w1, uint32_t w2)
   }
 }
 
-// bfloat16 bits of sign * v for 0 <= v <= 255, in the upper half of a float:
-// g = 1.5 2^23 + v is exact, and sg g - sg 1.5 2^23 is exactly +v, -v or +0
+// bfloat16 bits of sign * v for -255 <= v <= 255 (two's complement), in the upper
+// half of a float: g = 1.5 2^23 + v is exact, and sg g - sg 1.5 2^23 is exactly +v, -v or +0
 // (an exact zero sum rounds to +0), so the float holds sign * v exactly, and
 // sign * v has at most 8 significant bits, so its float bits end in 16 zeros.
 __device__ __forceinline__ uint32_t digit_float_bits(uint32_t v, float sg) {
-  const float g = __uint_as_float(0x4B400000u | v);
+  const float g = __uint_as_float(0x4B400000u + v);
   return __float_as_uint(fmaf(sg, g, -sg * 12582912.0f));
 }
 
@@ -223,6 +223,24 @@ __device__ __forceinline__ void store_digits(int s, uint32_t a0, uint32_t a1, ui
   }
 }
 
+// Difference planes of an entry pair (diff_planes below): sign * (v_i - v_j) for
+// the pairs in the order of diff_plane. The digits of an entry share its sign,
+// so |d_i - d_j| <= 127 like the digits themselves.
+template <int S, int I, int J, int BETA>
+__device__ __forceinline__ void store_diffs(uint32_t a0, uint32_t a1, uint32_t a2, bool na, uint32_t b0, uint32_t b1,
+                                            uint32_t b2, bool nb, char* base, int pair_off, int64_t plane_bytes) {
+  if constexpr (I + J > S + 1 || J >= S) {
+    if constexpr (2 * (I + 1) + 1 <= S + 1)
+      store_diffs<S, I + 1, I + 2, BETA>(a0, a1, a2, na, b0, b1, b2, nb, base, pair_off, plane_bytes);
+  } else {
+    constexpr int PI = 96 - BETA * I, PJ = 96 - BETA * J;
+    const uint32_t fa = digit_float_bits(field<PI, BETA>(a0, a1, a2) - field<PJ, BETA>(a0, a1, a2), na ? -1.0f : 1.0f);
+    const uint32_t fb = digit_float_bits(field<PI, BETA>(b0, b1, b2) - field<PJ, BETA>(b0, b1, b2), nb ? -1.0f : 1.0f);
+    reinterpret_cast<uint32_t*>(base + diff_plane(S, I, J) * plane_bytes)[pair_off] = __byte_perm(fa, fb, 0x7632);
+    store_diffs<S, I, J + 1, BETA>(a0, a1, a2, na, b0, b1, b2, nb, base, pair_off, plane_bytes);
+  }
+}
+
 // frexp exponent of the row maximum from the maxima of the high words (sign
 // cleared) and of the low words of its entries (0 for a zero row): a normal
 // value 1.f 2^(E-1023) is 0.1f 2^(E-1022); a subnormal frac 2^-1074 with frac of
@@ -263,7 +281,8 @@ __device__ __forceinline__ void max_bits(double a, uint32_t& mxh, uint32_t& mxl,
 // S > 0: the slice count is the compile-time constant S (s is ignored), so the
 // per-digit slice test folds away. THREADS threads share the row (kPairs entry
 // pairs each per sweep of 2 kPairs THREADS entries).
-template <int KIND, int BETA, int S = 0, int THREADS = kSplitThreads>
+// DIFF (S > 0, bf16-held beta 7 digits): the difference planes too.
+template <int KIND, int BETA, int S = 0, int THREADS = kSplitThreads, bool DIFF = false>
 __device__ __forceinline__ void split_one_row(const double* __restrict__ A, int64_t r, int64_t m, int k,
                                               int64_t lda, int s_arg, int32_t* __restrict__ exps,
                                               void* __restrict__ planes, int k_pad, int64_t plane_stride,
@@ -341,6 +360,7 @@ __device__ __forceinline__ void split_one_row(const double* __restrict__ A, int6
           fix96(v[q].x, c_row, a0, a1, a2, na);
           fix96(v[q].y, c_row, b0, b1, b2, nb);
           store_digits<0, KIND, BETA>(s, a0, a1, a2, na, b0, b1, b2, nb, base, j >> 1, plane_bytes);
+          if constexpr (DIFF) store_diffs<S, 1, 2, BETA>(a0, a1, a2, na, b0, b1, b2, nb, base, j >> 1, plane_bytes);
         }
       }
     }
@@ -351,36 +371,36 @@ __device__ __forceinline__ void split_one_row(const double* __restrict__ A, int6
   }
 }
 
-template <int KIND, int BETA, int S = 0>
+template <int KIND, int BETA, int S = 0, bool DIFF = false>
 __global__ void __launch_bounds__(kSplitThreads, 2)
 split_rows_kernel(const double* __restrict__ A, int64_t m, int64_t k, int64_t lda, int s,
                   int32_t* __restrict__ exps, void* __restrict__ planes, int64_t k_pad,
                   int64_t plane_stride, int* flag, const int* done) {
   if (done != nullptr && *done) return;
-  split_one_row<KIND, BETA, S>(A, blockIdx.x, m, static_cast<int>(k), lda, s, exps, planes,
-                               static_cast<int>(k_pad), plane_stride, flag);
+  split_one_row<KIND, BETA, S, kSplitThreads, DIFF>(A, blockIdx.x, m, static_cast<int>(k), lda, s, exps, planes,
+                                                    static_cast<int>(k_pad), plane_stride, flag);
 }
 
 // The split with a compile-time slice count for the counts the purification
 // uses most (INT8 digits in bf16, BF16 nearest digits, E4M3 digits), else the
 // runtime count.
-template <int KIND, int BETA, int S>
+template <int KIND, int BETA, int S, bool DIFF = false>
 void launch_split_s(dim3 grid, cudaStream_t st, const double* A, int64_t m, int64_t k, int64_t lda, int s,
                     int32_t* exps, void* planes, int64_t k_pad, int64_t plane_stride, int* flag, const int* done) {
-  split_rows_kernel<KIND, BETA, S><<<grid, kSplitThreads, 0, st>>>(A, m, k, lda, s, exps, planes, k_pad,
-                                                                   plane_stride, flag, done);
+  split_rows_kernel<KIND, BETA, S, DIFF><<<grid, kSplitThreads, 0, st>>>(A, m, k, lda, s, exps, planes, k_pad,
+                                                                         plane_stride, flag, done);
 }
-template <int KIND, int BETA, int S_LO, int S_HI>
+template <int KIND, int BETA, int S_LO, int S_HI, bool DIFF = false>
 void launch_split_any(dim3 grid, cudaStream_t st, const double* A, int64_t m, int64_t k, int64_t lda, int s,
                       int32_t* exps, void* planes, int64_t k_pad, int64_t plane_stride, int* flag, const int* done) {
   if constexpr (S_LO <= S_HI) {
     if (s == S_LO) {
-      launch_split_s<KIND, BETA, S_LO>(grid, st, A, m, k, lda, s, exps, planes, k_pad, plane_stride, flag, done);
+      launch_split_s<KIND, BETA, S_LO, DIFF>(grid, st, A, m, k, lda, s, exps, planes, k_pad, plane_stride, flag, done);
       return;
     }
-    launch_split_any<KIND, BETA, S_LO + 1, S_HI>(grid, st, A, m, k, lda, s, exps, planes, k_pad, plane_stride, flag,
-                                                 done);
-  } else {
+    launch_split_any<KIND, BETA, S_LO + 1, S_HI, DIFF>(grid, st, A, m, k, lda, s, exps, planes, k_pad, plane_stride,
+                                                       flag, done);
+  } else if constexpr (!DIFF) {
     launch_split_s<KIND, BETA, 0>(grid, st, A, m, k, lda, s, exps, planes, k_pad, plane_stride, flag, done);
   }
 }
@@ -434,13 +454,17 @@ __global__ void transpose_kernel(const double* __restrict__ A, int64_t m, int64_
 
 cudaError_t launch_split_rows(const double* A, int64_t m, int64_t k, int64_t lda, int s, int beta,
                               int32_t* exps, void* planes, int64_t m_pad, int64_t k_pad,
-                              int elem_kind, int* flag, const int* done, cudaStream_t st) {
+                              int elem_kind, bool diff, int* flag, const int* done, cudaStream_t st) {
   if (m_pad <= 0 || k_pad <= 0) return cudaSuccess;
   if (k > k_pad || k_pad > kMaxRow) return cudaErrorInvalidValue;
   const int64_t plane_stride = m_pad * k_pad;
   dim3 grid(static_cast<unsigned>(m_pad));
   ProfScope prof(DMP_PROF_SPLIT, st);
-  if (elem_kind == 1 && beta == 7) {
+  if (diff) {
+    if (elem_kind != 3 || beta != 7 || s < kDiffSlicesMin || s > kDiffSlicesMax) return cudaErrorInvalidValue;
+    launch_split_any<3, 7, kDiffSlicesMin, kDiffSlicesMax, true>(grid, st, A, m, k, lda, s, exps, planes, k_pad,
+                                                                 plane_stride, flag, done);
+  } else if (elem_kind == 1 && beta == 7) {
     split_rows_kernel<1, 7><<<grid, kSplitThreads, 0, st>>>(A, m, k, lda, s, exps, planes, k_pad, plane_stride,
                                                             flag, done);
   } else if (elem_kind == 3 && beta == 7) {
