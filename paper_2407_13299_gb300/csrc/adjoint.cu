@@ -23,12 +23,6 @@ namespace dmp {
 
 namespace {
 
-__device__ __forceinline__ double warp_sum(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
 // Partial sums over all elements, rows i = blockIdx.x + k gridDim.x:
 //   0: tr P   1: tr X2   2: <G, P>   3: <G, X2>   4: <Z, X2>
 __global__ void __launch_bounds__(256)

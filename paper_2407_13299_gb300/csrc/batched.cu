@@ -39,12 +39,6 @@ namespace {
 
 constexpr int kMeasBlk = 32;  // measure CTAs per matrix
 
-__device__ __forceinline__ double warp_sum(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
 // Per-matrix partial measures over the upper triangle (the quantities of the
 // single path's measure kernel). Batch rows are short (at most a few thousand
 // entries), so each warp takes whole rows: rows blockIdx.x 8 + w, + 8 kMeasBlk,
@@ -52,7 +46,8 @@ __device__ __forceinline__ double warp_sum(double v) {
 // accumulator sets per lane, combined in a fixed order (reproducible sums).
 __global__ void __launch_bounds__(256)
 measure_grouped_kernel(const BatchMat* __restrict__ mats, int cur, double* __restrict__ part) {
-  const BatchMat& M = mats[blockIdx.y];
+  const int b = mats[blockIdx.y].by_size;  // the largest matrices first, so that the launch ends evenly
+  const BatchMat& M = mats[b];
   if (M.state->done) return;
   const int64_t n = M.n;
   const double* P = M.buf[cur];
@@ -102,43 +97,42 @@ measure_grouped_kernel(const BatchMat* __restrict__ mats, int cur, double* __res
   const double u_id = (a_id[0] + a_id[1]) + (a_id[2] + a_id[3]);
   const double u_ph = (a_ph[0] + a_ph[1]) + (a_ph[2] + a_ph[3]);
   __shared__ double red[8][8];
-  double v[8] = {d_p, d_x, d_px, u_px, d_id, u_id, d_ph, u_ph};
-#pragma unroll
-  for (int q = 0; q < 8; ++q) v[q] = warp_sum(v[q]);
-  if (lane == 0)
-#pragma unroll
-    for (int q = 0; q < 8; ++q) red[w][q] = v[q];
-  __syncthreads();
-  if (threadIdx.x < 8) {
-    double t = 0.0;
-    for (int ww = 0; ww < 8; ++ww) t += red[ww][threadIdx.x];
-    part[(static_cast<int64_t>(blockIdx.y) * kMeasBlk + blockIdx.x) * 8 + threadIdx.x] = t;
-  }
+  __shared__ double tot[8];
+  const double v[8] = {d_p, d_x, d_px, u_px, d_id, u_id, d_ph, u_ph};
+  block_totals<8>(v, red, tot);
+  if (threadIdx.x < 8) part[(static_cast<int64_t>(b) * kMeasBlk + blockIdx.x) * 8 + threadIdx.x] = tot[threadIdx.x];
 }
 
-// One thread per matrix applies the stopping rules; the block then tells the
-// graph (or, in stream mode, the host through *active) whether any matrix
-// still runs.
-__global__ void measure_grouped_final_kernel(const BatchMat* __restrict__ mats, int nmats,
-                                             const double* __restrict__ part, cudaGraphConditionalHandle cond,
-                                             int set_cond, int* __restrict__ active) {
+// Eight threads per matrix sum its partials (a measure each, in block order) and
+// the first applies the stopping rules; the block then tells the graph (or, in
+// stream mode, the host through *active) whether any matrix still runs.
+constexpr int kFinalThreads = 512;
+
+__global__ void __launch_bounds__(kFinalThreads)
+measure_grouped_final_kernel(const BatchMat* __restrict__ mats, int nmats, const double* __restrict__ part,
+                             cudaGraphConditionalHandle cond, int set_cond, int* __restrict__ active) {
   __shared__ int any_active;
+  __shared__ double tot[kFinalThreads];
   if (threadIdx.x == 0) any_active = 0;
-  __syncthreads();
-  for (int b = threadIdx.x; b < nmats; b += blockDim.x) {
-    PurifyState* st = mats[b].state;
-    if (!st->done) {
-      double tot[8];
-      for (int q = 0; q < 8; ++q) {
-        double t = 0.0;
-        for (int k = 0; k < kMeasBlk; ++k) t += part[(static_cast<int64_t>(b) * kMeasBlk + k) * 8 + q];
-        tot[q] = t;
-      }
-      pm_decide(st, tot);
+  const int q = threadIdx.x & 7, sub = threadIdx.x >> 3;
+  for (int b0 = 0; b0 < nmats; b0 += kFinalThreads / 8) {
+    const int b = b0 + sub;
+    PurifyState* st = b < nmats ? mats[b].state : nullptr;
+    const bool runs = st != nullptr && !st->done;
+    double t = 0.0;
+    if (runs) {
+      const double* p = part + static_cast<int64_t>(b) * kMeasBlk * 8 + q;
+#pragma unroll
+      for (int k = 0; k < kMeasBlk; ++k) t += p[k * 8];
     }
-    if (!st->done) atomicOr(&any_active, 1);
+    tot[threadIdx.x] = t;
+    __syncthreads();
+    if (runs && q == 0) {
+      pm_decide(st, tot + threadIdx.x);
+      if (!st->done) atomicOr(&any_active, 1);
+    }
+    __syncthreads();
   }
-  __syncthreads();
   if (threadIdx.x == 0 && set_cond) cudaGraphSetConditional(cond, any_active ? 1u : 0u);
   if (threadIdx.x == 0 && active != nullptr) *active = any_active;
 }
@@ -469,6 +463,7 @@ int dm_purify_batched(int32_t batch, const double* const* H, const int64_t* n, c
   std::vector<int> by_size(batch);
   for (int b = 0; b < batch; ++b) by_size[b] = b;
   std::stable_sort(by_size.begin(), by_size.end(), [&](int x, int y) { return n[x] > n[y]; });
+  for (int b = 0; b < batch; ++b) hm[b].by_size = by_size[b];
   auto build_tiles = [&](int cfg, std::vector<int4>& out) {
     out.clear();
     const int tile_n = cfg_bn(cfg), bm = cfg_pair(cfg) ? 256 : 128;
@@ -705,7 +700,7 @@ cudaError_t launch_measure_grouped(const BatchMat* mats, int nmats, int cur, dou
                                    cudaStream_t st) {
   ProfScope prof(DMP_PROF_MEASURE, st);
   measure_grouped_kernel<<<dim3(kMeasBlk, nmats), 256, 0, st>>>(mats, cur, partials);
-  measure_grouped_final_kernel<<<1, 256, 0, st>>>(mats, nmats, partials, cond, set_cond, active);
+  measure_grouped_final_kernel<<<1, kFinalThreads, 0, st>>>(mats, nmats, partials, cond, set_cond, active);
   count_launch(2);
   return cudaGetLastError();
 }

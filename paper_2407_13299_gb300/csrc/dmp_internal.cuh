@@ -92,6 +92,7 @@ struct PurifyState {
   double tol, energy_tol;
   int32_t max_iter;
   int32_t store32;  // DMP_FLAG_FP32_STORAGE: stored matrices rounded to FP32 values
+  int32_t ticket;   // blocks of a running measure that have finished; 0 between kernels
 };
 
 // A matrix element as it is stored: rounded to the nearest FP32 value under
@@ -253,6 +254,64 @@ cudaError_t launch_foe_fold(const double* coeffs, int M, int q, int r, double* a
 
 namespace dmp {
 
+// ---------------------------------------------------------------- reductions
+__device__ __forceinline__ double warp_sum(double v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// warp_sum of eight values at once: at each of the first three steps a lane hands
+// half of its values to its partner and keeps the partner's part of the others,
+// so a warp adds 4 + 2 + 1 + 1 + 1 times instead of 40. The sums are warp_sum's
+// bit for bit (the same pairs, addition being commutative). The total of value
+// lane >> 2 is returned.
+__device__ __forceinline__ double warp_sum8(const double* v) {
+  const int lane = threadIdx.x & 31;
+  double a[4], b[2];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const bool up = (lane & 16) != 0;
+    a[i] = (up ? v[i + 4] : v[i]) + __shfl_xor_sync(0xffffffffu, up ? v[i] : v[i + 4], 16);
+  }
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const bool up = (lane & 8) != 0;
+    b[i] = (up ? a[i + 2] : a[i]) + __shfl_xor_sync(0xffffffffu, up ? a[i] : a[i + 2], 8);
+  }
+  const bool up = (lane & 4) != 0;
+  double c = (up ? b[1] : b[0]) + __shfl_xor_sync(0xffffffffu, up ? b[0] : b[1], 4);
+  c += __shfl_xor_sync(0xffffffffu, c, 2);
+  c += __shfl_xor_sync(0xffffffffu, c, 1);
+  return c;
+}
+
+// tot[q] = sum of v[q] over the block (256 threads): warp trees, then the eight
+// warps in order. All threads see tot afterwards.
+template <int NQ>
+__device__ __forceinline__ void block_totals(const double (&v)[NQ], double (*red)[NQ], double* tot) {
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const double c = warp_sum8(v);
+  if ((lane & 3) == 0) red[w][lane >> 2] = c;
+#pragma unroll
+  for (int q = 8; q < NQ; ++q) {
+    const double x = warp_sum(v[q]);
+    if (lane == 0) red[w][q] = x;
+  }
+  __syncthreads();
+  if (threadIdx.x < NQ) {
+    double t = 0.0;
+#pragma unroll
+    for (int ww = 0; ww < 8; ++ww) t += red[ww][threadIdx.x];
+    tot[threadIdx.x] = t;
+  }
+  __syncthreads();
+}
+
+}  // namespace dmp
+
+namespace dmp {
+
 // ---------------------------------------------------------------- shared epilogue
 // Applies one output element v = C[r][c] of a product. `mirror` writes the
 // transposed element as well (off-diagonal tiles of a symmetric product).
@@ -342,7 +401,8 @@ struct alignas(128) BatchMat {
   int32_t* expsX;
   PurifyState* state;
   int64_t n, n_occ, ldh, ldp, n_pad, k_pad;
-  int32_t s, pad_;
+  int32_t s;
+  int32_t by_size;  // entry i of the array: the i-th largest matrix of the batch
 };
 
 // 2-D TMA map over s stacked bf16 digit planes (k_pad contiguous, rows_total

