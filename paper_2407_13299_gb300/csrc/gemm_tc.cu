@@ -9,9 +9,8 @@
 // bytes (a 128-byte swizzle row holds 128 of them instead of 64). An fp32 sum
 // of such products is exact while every partial sum stays at most 2^24 in
 // magnitude; the K loop is therefore cut into chunks of 1024 (beta = 7 and 8:
-// 1024 * 128^2 = 2^24) or 65536 (beta = 5: 65536 * 16^2 = 2^24, so a whole
-// level is one chunk) K elements. Each chunk lands in one of two TMEM
-// accumulators; while the tensor core fills the other, eight epilogue warps
+// 1024 * 128^2 = 2^24) or 8192 (beta = 5, where 65536 * 16^2 = 2^24 would do) K
+// elements. Each chunk lands in one of two TMEM accumulators; while the tensor core fills the other, eight epilogue warps
 // drain the finished one into exact int32 sums in registers.
 //
 // A product runs as two kernels:
@@ -134,6 +133,7 @@ struct TcParams {
   // other units of all split tiles in one sequence, evenly cut over the other CTAs
   int heads, head_len;
   int group;        // levels combined exactly per int64 group: 4 (beta 7, 5) or 3 (beta 8)
+  double gscale[3];   // three groups: the weights 2^(-beta (s + 1 - group g)) of their sums
   long long* area;  // group sums of the launch's tiles: [tile][CTA rank][group][PART]
   int64_t m, n;
   int64_t rows_a, rows_b;  // padded rows per digit plane
@@ -501,16 +501,6 @@ __device__ __forceinline__ Job job_of(const TcParams& p, const CUtensorMap* tmA,
   return j;
 }
 
-// Three groups: scaled and added in float64 from the smallest up. Not inlined:
-// the compiler would compute it for every element and drop it (six FP64
-// operations, which bound the finish kernel at one group per element).
-__device__ __noinline__ double add_groups(long long t0, long long t1, long long t2, int e_sum, int step, int e) {
-  const double d0 = static_cast<double>(t0) * ldexp(1.0, e_sum);
-  const double d1 = d0 + static_cast<double>(t1) * ldexp(1.0, e_sum + step);
-  const double d2 = d1 + static_cast<double>(t2) * ldexp(1.0, e_sum + 2 * step);
-  return scale_pow2(d2, e);
-}
-
 // Four consecutive doubles or int64 group sums, in 16-byte pieces when the
 // address allows (`vec`), else one by one at immediate offsets.
 __device__ __forceinline__ void load4(double (&v)[4], const double* __restrict__ a, bool vec) {
@@ -714,7 +704,9 @@ ozaki_finish_kernel(const __grid_constant__ TcParams p) {
               : "r"(l0), "r"(h0), "r"(x0));
           v[t] = round_words(w0, w1, w2s, ee + e_sum);
         } else {
-          v[t] = add_groups(t0, t1, t2, e_sum, p.beta * p.group, ee);
+          const double d0 = static_cast<double>(t0) * p.gscale[0];
+          const double d1 = d0 + static_cast<double>(t1) * p.gscale[1];
+          v[t] = scale_pow2(d1 + static_cast<double>(t2) * p.gscale[2], ee);
         }
         if (er[t] == kBadExp || ec[pass] == kBadExp) v[t] = __longlong_as_double(0x7ff8000000000000ll);
       }
@@ -1400,6 +1392,12 @@ void diff_program(int s, int beta, int group, int64_t k, TcProgram& pr) {
   }
 }
 
+int chunk_atoms(int beta) { return beta == 5 ? 64 : 16; }
+
+void group_scales(TcParams& p) {
+  for (int g = 0; g < 3; ++g) p.gscale[g] = std::ldexp(1.0, -p.beta * (p.s + 1 - p.group * g));
+}
+
 // fp32 chunks of one tile (split launches)
 int chunk_count(const TcProgram& pr, int kts, int chs) {
   int cnt = 0;
@@ -1595,6 +1593,16 @@ cudaError_t run_product(const void* A, const void* B, int64_t k_pad, int planes,
   const int units = PAIR ? tc_max_pairs() : tc_max_ctas();
   const std::vector<TileAt> tiles = tile_order<BN, Cfg::BM>(p.m, p.n, p.sym, units);
   const int ntiles = static_cast<int>(tiles.size());
+  // While there are fewer tiles than CTAs, chunks no longer than a CTA's share of
+  // the K atoms (half of it on 256-column tiles, where an added chunk costs less
+  // than an uneven share: n = 1024, E4M3, s = 9 62 -> 58 us).
+  if (g_split_tiles && ntiles < units) {
+    int steps = 0;
+    for (int g = 0; g < p.prog.nsegs; ++g) steps += p.prog.seg[g].nsteps;
+    const int64_t atoms = static_cast<int64_t>(steps) * p.KT * ntiles;
+    const int cut = (BN < 256 ? 1 : 2) * units;
+    p.CH = static_cast<int>(std::min<int64_t>(p.CH, std::max<int64_t>(BN < 256 ? 1 : 2, (atoms + cut - 1) / cut)));
+  }
   p.units = chunk_count(p.prog, p.KT, p.CH);
   const double plane_bytes = static_cast<double>(k_pad) * (F8 ? 1 : 2) * planes * (p.m + (A == B ? 0 : p.n));
 
@@ -1650,10 +1658,12 @@ cudaError_t launch_ozaki_tc(const void* A, const void* B, const int32_t* ea, con
   p.s = s;
   p.beta = beta;
   p.KT = static_cast<int>(k_pad / atom_k);
-  // K chunk in atoms: 1024 (beta 7: 127^2; beta 8 nearest: 128^2) or 65536
-  // (beta 5 nearest: 16^2) K elements keep every fp32 partial sum at most 2^24
-  p.CH = f8 ? 512 : 16;
+  // K chunk in atoms: 1024 (beta 7: 127^2; beta 8 nearest: 128^2) K elements, of
+  // up to 65536 (beta 5 nearest: 16^2) 8192 so that tiles can be shared in fine
+  // parts, keep every fp32 partial sum at most 2^24
+  p.CH = chunk_atoms(beta);
   p.group = beta == 8 ? 3 : 4;
+  group_scales(p);
   p.m = m;
   p.n = n;
   p.rows_a = rows_a;
@@ -1684,6 +1694,20 @@ cudaError_t launch_ozaki_tc(const void* A, const void* B, const int32_t* ea, con
   }
   const int planes = s + (diff ? diff_planes(s) : 0);
   ProfScope prof(DMP_PROF_PRODUCT, st);
+  // Few tiles: smaller ones, whose group sums a CTA adds in proportion faster
+  // (a 128 x 256 part takes it 6 us, 128 x 64 1.5 us) and whose operands more CTAs
+  // share; larger outputs want the pair kernel's fewer bytes per product. Per
+  // product, INT8 s = 5, pair / 128 x 128 / 128 x 64 tiles: n = 256 22.9 / 18.1 /
+  // 16.1 us, n = 384 25.1 / 19.5 / 19.0, n = 512 27.7 / 21.5 / 25.5, n = 768 34.5 /
+  // 30.4 / 34.4, n = 1024 41.0 / 42.7 / 52.2; the other modes alike.
+  const int64_t tm = (m + 255) / 256, tn = (n + 255) / 256;
+  const int64_t big_tiles = sym ? tn * (tn + 1) / 2 : tm * tn;
+  if (pair && big_tiles <= 1)
+    return f8 ? run_product<64, false, true>(A, B, k_pad, planes, p, area, st)
+              : run_product<64, false, false>(A, B, k_pad, planes, p, area, st);
+  if (pair && big_tiles <= 6)
+    return f8 ? run_product<128, false, true>(A, B, k_pad, planes, p, area, st)
+              : run_product<128, false, false>(A, B, k_pad, planes, p, area, st);
   if (pair)
     return f8 ? run_product<256, true, true>(A, B, k_pad, planes, p, area, st)
               : run_product<256, true, false>(A, B, k_pad, planes, p, area, st);
@@ -1701,8 +1725,9 @@ cudaError_t launch_ozaki_tc_grouped(const BatchMat* mats, const int4* tiles, int
   std::memset(&p, 0, sizeof(p));
   p.s = s;
   p.beta = beta;
-  p.CH = beta == 5 ? 512 : 16;
+  p.CH = chunk_atoms(beta);
   p.group = beta == 8 ? 3 : 4;
+  group_scales(p);
   p.sym = 1;
   p.units = 1;
   p.mats = mats;
