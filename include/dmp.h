@@ -453,7 +453,7 @@ int dm_foe_workspace_size(int64_t n, const dmp_foe_params* params, const dmp_opt
  *   H_s (and y = T_q) is split once per call.
  * With params->n_occ > 0, the traces tr T_k come first (a first pass of the
  * recurrence, or the giant steps of the Paterson-Stockmeyer scheme) and mu
- * solves sum_k c_k(mu) tr T_k = n_occ by 100 bisection halvings of
+ * solves sum_k c_k(mu) tr T_k = n_occ by bisection, at least 100 halvings of
  * [e_min - 40 kT, e_max + 40 kT]; then P is formed.
  * The truncation error falls roughly like exp(-M pi kT / b): M must grow with
  * b / kT, so a tight enclosure matters (Gershgorin bounds of a dense H can be

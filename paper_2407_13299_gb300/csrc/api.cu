@@ -1090,11 +1090,8 @@ int dm_foe(const double* H, int64_t n, int64_t ldh, const dmp_foe_params* params
   // word), and every kFoeCheckEvery products the host reads the flag and
   // stops enqueueing with DMP_ERR_TIMEOUT.
   constexpr int kFoeCheckEvery = 8;
-  auto product = [&](const double* A, const void* pa, const int32_t* ea, const double* B) -> int {
-    EpiArgs e{};
-    e.kind = EPI_SYM_STORE;
-    e.C = Y;
-    e.ldc = n;
+  auto product_with = [&](const double* A, const void* pa, const int32_t* ea, const double* B,
+                          const EpiArgs& e) -> int {
     if (!oz) {
       DMP_CUDA(launch_gemm_f64(A, n, B, n, n, n, n, 1, e, nullptr, st));
     } else {
@@ -1111,6 +1108,28 @@ int dm_foe(const double* H, int64_t n, int64_t ldh, const dmp_foe_params* params
       if (flag) return DMP_ERR_TIMEOUT;
     }
     return DMP_OK;
+  };
+  auto product = [&](const double* A, const void* pa, const int32_t* ea, const double* B) -> int {
+    EpiArgs e{};
+    e.kind = EPI_SYM_STORE;
+    e.C = Y;
+    e.ldc = n;
+    return product_with(A, pa, ea, B, e);
+  };
+  // out = 2 A B - prev (prev null: the identity; out may be prev), formed in the
+  // product's output step; with a coefficient also P += *coef out
+  auto next_term = [&](const double* A, const void* pa, const int32_t* ea, const double* B, const double* prev,
+                       double* out, const double* coef) -> int {
+    EpiArgs e{};
+    e.kind = EPI_CHEB;
+    e.C = out;
+    e.ldc = n;
+    e.P = prev;
+    e.ldp = n;
+    e.acc = coef ? P : nullptr;
+    e.ldacc = ldp;
+    e.coef = coef;
+    return product_with(A, pa, ea, B, e);
   };
   auto split_a = [&](const double* A, void* planes, int32_t* exps) -> int {
     if (oz)
@@ -1137,9 +1156,8 @@ int dm_foe(const double* H, int64_t n, int64_t ldh, const dmp_foe_params* params
       double* prev = Ta;
       double* cur = Tb;
       for (int k = 1; k <= M - 2; ++k) {
-        const int prc = product(Hs, planesH, expsH, cur);
+        const int prc = next_term(Hs, planesH, expsH, cur, prev, prev, acc ? coeffs + k + 1 : nullptr);
         if (prc != DMP_OK) return prc;
-        DMP_CUDA(launch_foe_step(Y, prev, acc ? P : nullptr, ldp, coeffs + k + 1, n, st));
         if (!acc) DMP_CUDA(launch_foe_trace(prev, n, n, traces + k + 1, st));
         std::swap(prev, cur);
       }
@@ -1170,30 +1188,27 @@ int dm_foe(const double* H, int64_t n, int64_t ldh, const dmp_foe_params* params
     DMP_CUDA(launch_foe_init(H, ldh, n, sc, nullptr, slot(1), nullptr, nullptr, P, ldp, st));
     if (nb >= 2 && split_a(slot(1), planesH, expsH) != DMP_OK) return DMP_ERR_CUDA;
     for (int j = 1; j < nb; ++j) {
-      rc = product(slot(1), planesH, expsH, slot(j));
+      rc = next_term(slot(1), planesH, expsH, slot(j), j == 1 ? nullptr : slot(j - 1), slot(j + 1), nullptr);
       if (rc != DMP_OK) return rc;
-      DMP_CUDA(launch_foe_next(Y, j == 1 ? nullptr : slot(j - 1), slot(j + 1), n, st));
     }
     double* yq = r > 1 ? slot(q) : nullptr;
     if (r > 1 && split_a(yq, planesY, expsY) != DMP_OK) return DMP_ERR_CUDA;
     if (canonical) {
       // traces: T_1 .. T_{q-1} directly; T_{qm} = T_m(y) by the recurrence in y
-      // (T_q for m = 1), with <T_{qm}, T_j> for the rest
-      for (int k = 1; k < q && k < M; ++k) DMP_CUDA(launch_foe_trace(slot(k), n, n, traces + k, st));
+      // (T_q for m = 1), with <T_{qm}, T_j> for the rest (j = 0: the trace itself)
+      DMP_CUDA(launch_foe_traces(Tps, std::min(q, M) - 1, n, traces + 1, st));
       double* g_prev = nullptr;  // T_0 = I
       double* g_cur = yq;
       for (int m = 1; q * m < M; ++m) {
         if (m >= 2) {
-          rc = product(yq, planesY, expsY, g_cur);
-          if (rc != DMP_OK) return rc;
           // G_2 and G_3 take the two free buffers; later terms overwrite G_{m-2} in place
           double* out = m == 2 ? Ta : (m == 3 ? Tb : g_prev);
-          DMP_CUDA(launch_foe_next(Y, g_prev, out, n, st));
+          rc = next_term(yq, planesY, expsY, g_cur, g_prev, out, nullptr);
+          if (rc != DMP_OK) return rc;
           g_prev = g_cur;
           g_cur = out;
         }
-        DMP_CUDA(launch_foe_trace(g_cur, n, n, traces + q * m, st));
-        DMP_CUDA(launch_foe_dots(g_cur, Tps, q, n, dots, ip + static_cast<size_t>(m) * q + 1, st));
+        DMP_CUDA(launch_foe_dots(g_cur, Tps, q, n, dots, ip + static_cast<size_t>(m) * q, sc, st));
       }
       DMP_CUDA(launch_foe_ps_traces(traces, ip, q, M, n, st));
       DMP_CUDA(launch_foe_coefficients(sc, fp.kT, 0.0, static_cast<double>(fp.n_occ), traces, M, w, gx, coeffs, st));

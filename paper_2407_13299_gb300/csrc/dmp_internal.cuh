@@ -122,19 +122,24 @@ int gemm_least_bytes(int64_t m, int64_t n, int64_t k, int32_t mode, int32_t slic
 cudaError_t launch_transpose(const double* A, int64_t m, int64_t n, int64_t lda, double* At,
                              cudaStream_t st);
 
-enum EpiKind { EPI_STORE = 0, EPI_SYM_STORE = 1, EPI_PM_UPDATE = 2, EPI_LEVELS = 3 };
+// EPI_CHEB: the next Chebyshev term, C = 2 v - P of a symmetric product v (P null:
+// the identity; C may be P), and acc += *coef C when acc is given.
+enum EpiKind { EPI_STORE = 0, EPI_SYM_STORE = 1, EPI_PM_UPDATE = 2, EPI_LEVELS = 3, EPI_CHEB = 4 };
 
 struct EpiArgs {
   int kind;
   double* C;          // output (EPI_STORE / EPI_SYM_STORE / EPI_PM_UPDATE: P_next)
   int64_t ldc;
-  const double* P;    // EPI_PM_UPDATE: current iterate
+  const double* P;    // EPI_PM_UPDATE: current iterate; EPI_CHEB: the term before
   const double* X2;   // EPI_PM_UPDATE: P^2
   int64_t ldp;        // leading dimension of P
   int64_t ldx;        // leading dimension of X2
   const PurifyState* state;  // EPI_PM_UPDATE weights
   int32_t* levels;    // EPI_LEVELS: [s][m][n]
   int round32;        // round every stored element to an FP32 value (DMP_FLAG_FP32_STORAGE)
+  double* acc;        // EPI_CHEB: the running sum (nullable), its leading dimension and the term's coefficient
+  int64_t ldacc;
+  const double* coef;
 };
 
 // IMMA executor: level sums of int8 planes with fused FP64 recombination.
@@ -215,37 +220,37 @@ constexpr int kMeasureBlocks = 608;  // 4 x 152 SMs; fixed so sums are reproduci
 struct FoeScalars {
   double a, b, mu, e_min, e_max, trace;
   int32_t nonfinite;  // H held a NaN/Inf (copied from the Gershgorin pass)
+  int32_t ticket;     // blocks of a running reduction that have finished; 0 between kernels
 };
 constexpr int kFoeMaxTerms = 16384;  // DMP_FOE_MAX_TERMS
 // Enclosure: the given one when use_given, else the Gershgorin bounds in `state`.
 cudaError_t launch_foe_scale(const PurifyState* state, double e_min, double e_max, int use_given, FoeScalars* sc,
                              cudaStream_t st);
 // mu (solved from n_occ and the traces tr T_k when `traces` is non-null, else
-// the given mu), then the M coefficients. w and gx hold 2M doubles each.
+// the given mu), then the M coefficients. w, gx and coeffs hold 2M doubles each,
+// at least 512.
 cudaError_t launch_foe_coefficients(FoeScalars* sc, double kT, double mu, double n_occ, const double* traces, int M,
                                     double* w, double* gx, double* coeffs, cudaStream_t st);
 // H_s, T_0 = I, T_1 = H_s (leading dimension n) and, with coeffs, P = c_0/2 I + c_1 H_s.
 cudaError_t launch_foe_init(const double* H, int64_t ldh, int64_t n, const FoeScalars* sc, const double* coeffs,
                             double* Hs, double* T0, double* T1, double* P, int64_t ldp, cudaStream_t st);
-// Tprev <- 2 Y - Tprev; with P non-null, P += (*coeff) Tprev.
-cudaError_t launch_foe_step(const double* Y, double* Tprev, double* P, int64_t ldp, const double* coeff, int64_t n,
-                            cudaStream_t st);
 // *out = tr A (fixed order).
 cudaError_t launch_foe_trace(const double* A, int64_t lda, int64_t n, double* out, cudaStream_t st);
+// out[t] = tr of the t-th of `count` matrices n x n, one after the other.
+cudaError_t launch_foe_traces(const double* T, int count, int64_t n, double* out, cudaStream_t st);
 // Paterson-Stockmeyer scheme. Baby steps T_1 .. T_q are kept in consecutive
 // n x n slots (T_t at T + (t - 1) n^2; T_0 = I implicit).
 constexpr int kFoeDotBlocks = 304;  // 2 x 152 SMs; fixed so sums are reproducible
-// Tout = 2 Y - Tprev (Tprev = I when null; Tout may be Tprev).
-cudaError_t launch_foe_next(const double* Y, const double* Tprev, double* Tout, int64_t n, cudaStream_t st);
 // out = ((w_0 I + sum_{t=1}^{nt-1} w_t T_t) + alpha Y) - Bm2 (Y, Bm2 nullable; out
 // of leading dimension ldo may be Bm2).
 cudaError_t launch_foe_combine(const double* T, int nt, const double* w, const double* Y, double alpha,
                                const double* Bm2, double* out, int64_t ldo, int64_t n, cudaStream_t st);
-// out[t - 1] = <G, T_t>_F for t = 1 .. nt - 1; partials holds kFoeDotBlocks (nt - 1) doubles.
+// out[t] = <G, T_t>_F for t = 0 .. nt - 1 (symmetric matrices; T_0 = I: tr G);
+// partials holds kFoeDotBlocks nt doubles.
 cudaError_t launch_foe_dots(const double* G, const double* T, int nt, int64_t n, double* partials, double* out,
-                            cudaStream_t st);
-// tr T_k, k < M, from the baby- and giant-step traces already in `traces` and the
-// Frobenius products ip[m q + j] = <T_{qm}, T_j>.
+                            FoeScalars* sc, cudaStream_t st);
+// tr T_k, k < M, from the baby-step traces already in `traces` and the Frobenius
+// products ip[m q + j] = <T_{qm}, T_j> (j = 0: tr T_{qm}).
 cudaError_t launch_foe_ps_traces(double* traces, const double* ip, int q, int M, int64_t n, cudaStream_t st);
 // Block weights w[r][q] from the M coefficients (a: scratch of r q doubles).
 cudaError_t launch_foe_fold(const double* coeffs, int M, int q, int r, double* a, double* w, cudaStream_t st);
@@ -321,6 +326,13 @@ __device__ __forceinline__ void epi_apply(const EpiArgs& e, int64_t r, int64_t c
     const double p = e.P[r * e.ldp + c];
     const double x2 = e.X2[r * e.ldx + c];
     v = e.state->alpha * p + e.state->b2 * x2 + e.state->b3 * v;
+  } else if (e.kind == EPI_CHEB) {
+    v = 2.0 * v - (e.P ? e.P[r * e.ldp + c] : (r == c ? 1.0 : 0.0));
+    if (e.acc) {
+      const double a = e.acc[r * e.ldacc + c] + *e.coef * v;
+      e.acc[r * e.ldacc + c] = a;
+      if (mirror) e.acc[c * e.ldacc + r] = a;
+    }
   }
   v = stored_value(v, e.round32 != 0);
   e.C[r * e.ldc + c] = v;

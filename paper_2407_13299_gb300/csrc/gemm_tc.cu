@@ -531,12 +531,14 @@ __device__ __forceinline__ void store4(double* a, const double (&v)[4], bool vec
 // (Done instead by two further warps of the next wave's product kernel it cost
 // 3 % of the whole: 200 us per wave of 76 tiles on so few threads, and the
 // shared memory of a seventh stage.)
-// UPD: the PM update (EPI_PM_UPDATE). NG: group sums per element (0: EPI_LEVELS).
+// OUT: what becomes of an element. NG: group sums per element (0: EPI_LEVELS).
 constexpr int FIN_THREADS = 128;
+enum { OUT_STORE = 0, OUT_UPDATE = 1, OUT_CHEB = 2 };  // EPI_STORE and EPI_SYM_STORE, EPI_PM_UPDATE, EPI_CHEB
 
-template <int BN, bool PAIR, bool UPD, int NG>
+template <int BN, bool PAIR, int OUT, int NG>
 __global__ void __launch_bounds__(FIN_THREADS)
 ozaki_finish_kernel(const __grid_constant__ TcParams p) {
+  constexpr bool UPD = OUT == OUT_UPDATE, CHEB = OUT == OUT_CHEB;
   if (p.done != nullptr && *p.done) return;
   __shared__ double trans[32][33];
   using Cfg = TcCfg<BN, PAIR>;
@@ -611,6 +613,7 @@ ozaki_finish_kernel(const __grid_constant__ TcParams p) {
   const double wa = UPD ? epi.state->alpha : 0.0;
   const double w2 = UPD ? epi.state->b2 : 0.0;
   const double w3 = UPD ? epi.state->b3 : 0.0;
+  const double coef = CHEB && epi.acc != nullptr ? *epi.coef : 0.0;
   // every load of the block before the first store, so that a thread waits
   // for one round of latencies per block
   constexpr int G = NG == 0 ? 1 : NG;
@@ -620,10 +623,14 @@ ozaki_finish_kernel(const __grid_constant__ TcParams p) {
   int4 er4 = make_int4(0, 0, 0, 0);
   if (r < m) er4 = *reinterpret_cast<const int4*>(ea + r);  // (the exponent arrays are padded to 256 rows)
   const int32_t er[4] = {er4.x, er4.y, er4.z, er4.w};
-  const double* pp = UPD ? epi.P + (c0 + line0) * epi.ldp + r : nullptr;
-  const double* xp = UPD ? epi.X2 + (c0 + line0) * epi.ldx + r : nullptr;
-  const bool vecp = UPD && (epi.ldp & 1) == 0 && (reinterpret_cast<uintptr_t>(epi.P) & 15) == 0;
-  const bool vecx = UPD && (epi.ldx & 1) == 0 && (reinterpret_cast<uintptr_t>(epi.X2) & 15) == 0;
+  // the update's P and P^2; the recurrence's term before and its running sum
+  const bool two = UPD || (CHEB && epi.acc != nullptr), one = UPD || (CHEB && epi.P != nullptr);
+  const double* xbase = CHEB ? epi.acc : epi.X2;
+  const int64_t ldx = CHEB ? epi.ldacc : epi.ldx;
+  const double* pp = one ? epi.P + (c0 + line0) * epi.ldp + r : nullptr;
+  const double* xp = two ? xbase + (c0 + line0) * ldx + r : nullptr;
+  const bool vecp = one && (epi.ldp & 1) == 0 && (reinterpret_cast<uintptr_t>(epi.P) & 15) == 0;
+  const bool vecx = two && (ldx & 1) == 0 && (reinterpret_cast<uintptr_t>(xbase) & 15) == 0;
 #pragma unroll
   for (int pass = 0; pass < PASSES; ++pass) {
     const int c = c0 + line0 + LINES * pass;
@@ -634,22 +641,26 @@ ozaki_finish_kernel(const __grid_constant__ TcParams p) {
       T[pass][g][0] = x.x, T[pass][g][1] = x.y, T[pass][g][2] = y.x, T[pass][g][3] = y.y;
     }
     ec[pass] = c < n ? eb[c] : 0;
-    if (UPD) {
+    if (UPD || CHEB) {
       // the rows of this column that are written: inside the matrix, and not below the diagonal
       const int rows = c < n ? min(sym ? c + 1 : m, m) - r : 0;
       const double* pc = pp + static_cast<int64_t>(LINES * pass) * epi.ldp;
-      const double* xc = xp + static_cast<int64_t>(LINES * pass) * epi.ldx;
+      const double* xc = xp + static_cast<int64_t>(LINES * pass) * ldx;
 #pragma unroll
-      for (int t = 0; t < 4; ++t) pv[pass][t] = xv[pass][t] = 0.0;
+      for (int t = 0; t < 4; ++t) {
+        // no term before: the identity
+        pv[pass][t] = CHEB && epi.P == nullptr && r + t == c ? 1.0 : 0.0;
+        xv[pass][t] = 0.0;
+      }
       if (rows >= 4) {
-        load4(pv[pass], pc, vecp);
-        load4(xv[pass], xc, vecx);
+        if (one) load4(pv[pass], pc, vecp);
+        if (two) load4(xv[pass], xc, vecx);
       } else {
 #pragma unroll
         for (int t = 0; t < 3; ++t) {
           if (t < rows) {
-            pv[pass][t] = pc[t];
-            xv[pass][t] = xc[t];
+            if (one) pv[pass][t] = pc[t];
+            if (two) xv[pass][t] = xc[t];
           }
         }
       }
@@ -714,6 +725,23 @@ ozaki_finish_kernel(const __grid_constant__ TcParams p) {
     if (UPD) {
 #pragma unroll
       for (int t = 0; t < 4; ++t) v[t] = wa * pv[pass][t] + w2 * xv[pass][t] + w3 * v[t];
+    }
+    if (CHEB) {
+#pragma unroll
+      for (int t = 0; t < 4; ++t) v[t] = 2.0 * v[t] - pv[pass][t];
+      if (epi.acc != nullptr && rows > 0) {
+        // both triangles of the running sum (no other thread reads or writes these elements)
+        double* a = epi.acc + c * epi.ldacc + r;
+        double* am = epi.acc + r * epi.ldacc + c;
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+          if (t < rows) {
+            const double x = xv[pass][t] + coef * v[t];
+            a[t] = x;
+            am[t * epi.ldacc] = x;
+          }
+        }
+      }
     }
     if (epi.round32 != 0) {
       // stored_value; volatile, so that without the flag the two conversions
@@ -1436,17 +1464,17 @@ struct TcLaunch {
   }
 };
 
-template <int BN, bool PAIR, bool UPD>
+template <int BN, bool PAIR, int OUT>
 void launch_finish(const TcParams& p, cudaStream_t st) {
   const int grid = p.ntiles * (TcCfg<BN, PAIR>::BM / 32) * (BN / 32);
-  if (p.mats == nullptr && p.epi.kind == EPI_LEVELS) {
-    ozaki_finish_kernel<BN, PAIR, UPD, 0><<<grid, FIN_THREADS, 0, st>>>(p);
+  if (OUT == OUT_STORE && p.mats == nullptr && p.epi.kind == EPI_LEVELS) {
+    ozaki_finish_kernel<BN, PAIR, OUT_STORE, 0><<<grid, FIN_THREADS, 0, st>>>(p);
   } else if (p.prog.ng == 1) {
-    ozaki_finish_kernel<BN, PAIR, UPD, 1><<<grid, FIN_THREADS, 0, st>>>(p);
+    ozaki_finish_kernel<BN, PAIR, OUT, 1><<<grid, FIN_THREADS, 0, st>>>(p);
   } else if (p.prog.ng == 2) {
-    ozaki_finish_kernel<BN, PAIR, UPD, 2><<<grid, FIN_THREADS, 0, st>>>(p);
+    ozaki_finish_kernel<BN, PAIR, OUT, 2><<<grid, FIN_THREADS, 0, st>>>(p);
   } else {
-    ozaki_finish_kernel<BN, PAIR, UPD, 3><<<grid, FIN_THREADS, 0, st>>>(p);
+    ozaki_finish_kernel<BN, PAIR, OUT, 3><<<grid, FIN_THREADS, 0, st>>>(p);
   }
 }
 
@@ -1458,11 +1486,13 @@ cudaError_t launch_tc_impl(const CUtensorMap& ta, const CUtensorMap& tb, const T
   TcLaunch<BN, PAIR, F8> l(grid, st);
   e = cudaLaunchKernelEx(&l.cfg, ozaki_tc_kernel<BN, PAIR, F8, WALK>, ta, tb, p);
   if (e != cudaSuccess) return e;
-  const bool upd = p.mats != nullptr ? p.phase != 0 : p.epi.kind == EPI_PM_UPDATE;
-  if (upd) {
-    launch_finish<BN, PAIR, true>(p, st);
+  const int kind = p.mats != nullptr ? (p.phase != 0 ? EPI_PM_UPDATE : EPI_SYM_STORE) : p.epi.kind;
+  if (kind == EPI_PM_UPDATE) {
+    launch_finish<BN, PAIR, OUT_UPDATE>(p, st);
+  } else if (kind == EPI_CHEB) {
+    launch_finish<BN, PAIR, OUT_CHEB>(p, st);
   } else {
-    launch_finish<BN, PAIR, false>(p, st);
+    launch_finish<BN, PAIR, OUT_STORE>(p, st);
   }
   count_launch(2);
   return cudaGetLastError();
