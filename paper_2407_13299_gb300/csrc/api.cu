@@ -212,7 +212,7 @@ inline char* at(void* base, size_t off) { return static_cast<char*>(base) + off;
 // recomputed iterates and squares of one checkpoint segment, and the split
 // buffers of one product.
 struct BackwardLayout {
-  size_t state, scalars, p0, partials, err, expsP, expsA, G, Gn, Y, Z, YP, ZP, segP, segX, planesP, planesA,
+  size_t state, scalars, p0, partials, err, expsP, expsA, G, Gn, Y, W, V, U, segP, segX, planesP, planesA,
       area, total;
   int64_t n_pad, k_pad;
 };
@@ -227,15 +227,15 @@ BackwardLayout backward_layout(int64_t n, const Opts& o) {
   B.scalars = c.take(sizeof(AdjScalars));
   B.p0 = c.take(sizeof(P0Adjoint));
   B.partials = c.take(304 * 5 * sizeof(double));
-  B.err = c.take(sizeof(int32_t));
+  B.err = c.take(2 * sizeof(int32_t));  // the error flag and the reductions' ticket
   B.expsP = c.take(static_cast<size_t>(B.n_pad) * sizeof(int32_t));
   B.expsA = c.take(static_cast<size_t>(B.n_pad) * sizeof(int32_t));
   B.G = c.take(nn);
   B.Gn = c.take(nn);
   B.Y = c.take(nn);
-  B.Z = c.take(nn);
-  B.YP = c.take(nn);
-  B.ZP = c.take(nn);
+  B.W = c.take(nn);
+  B.V = c.take(nn);
+  B.U = c.take(nn);
   B.segP = c.take(nn * o.every);
   B.segX = c.take(nn * o.every);
   if (o.mode != DMP_FP64) {
@@ -871,9 +871,9 @@ int dm_purify_backward(const double* H, int64_t n, int64_t n_occ, const dmp_opts
   double* G = reinterpret_cast<double*>(at(ws, B.G));
   double* Gn = reinterpret_cast<double*>(at(ws, B.Gn));
   double* Y = reinterpret_cast<double*>(at(ws, B.Y));
-  double* Z = reinterpret_cast<double*>(at(ws, B.Z));
-  double* YP = reinterpret_cast<double*>(at(ws, B.YP));
-  double* ZP = reinterpret_cast<double*>(at(ws, B.ZP));
+  double* W = reinterpret_cast<double*>(at(ws, B.W));
+  double* V = reinterpret_cast<double*>(at(ws, B.V));
+  double* U = reinterpret_cast<double*>(at(ws, B.U));
   double* segP = reinterpret_cast<double*>(at(ws, B.segP));
   double* segX = reinterpret_cast<double*>(at(ws, B.segX));
   PurifyState* state = reinterpret_cast<PurifyState*>(at(ws, B.state));
@@ -881,12 +881,13 @@ int dm_purify_backward(const double* H, int64_t n, int64_t n_occ, const dmp_opts
   P0Adjoint* p0s = reinterpret_cast<P0Adjoint*>(at(ws, B.p0));
   double* part = reinterpret_cast<double*>(at(ws, B.partials));
   int* err = reinterpret_cast<int*>(at(ws, B.err));
+  int32_t* ticket = err + 1;
   int32_t* expsP = reinterpret_cast<int32_t*>(at(ws, B.expsP));
   int32_t* expsA = reinterpret_cast<int32_t*>(at(ws, B.expsA));
   void* planesP = o.mode != DMP_FP64 ? at(ws, B.planesP) : nullptr;
   void* planesA = o.mode != DMP_FP64 ? at(ws, B.planesA) : nullptr;
   TcArea area = area_at(o, ws, B.area);
-  DMP_CUDA(cudaMemsetAsync(err, 0, sizeof(int), st));
+  DMP_CUDA(cudaMemsetAsync(err, 0, 2 * sizeof(int), st));
   const int64_t npad = B.n_pad, kpad = B.k_pad;
 
   // C = A P (P symmetric; its planes are already in planesP for the Ozaki modes)
@@ -923,6 +924,9 @@ int dm_purify_backward(const double* H, int64_t n, int64_t n_occ, const dmp_opts
       wts[k].b3 = -1.0 / (1.0 - c);
     }
   }
+
+  // one product for G P^2 and P G P where the digits leave its change of rounding below 1e-9 (adjoint.cu)
+  const bool merged = o.mode == DMP_FP64 || o.beta * o.s >= 42;
 
   DMP_CUDA(launch_sym_part(dLdP, n, n, G, st));
   const int E = o.every;
@@ -971,13 +975,18 @@ int dm_purify_backward(const double* H, int64_t n, int64_t n_occ, const dmp_opts
     for (int k = k1 - 1; k >= k0; --k) {
       const double* Pk = segP + static_cast<size_t>(k - k0) * nn;
       const double* Xk = segX + static_cast<size_t>(k - k0) * nn;
-      DMP_CUDA(split_P(Pk));
-      DMP_CUDA(times_P(G, Pk, Y));    // Y = G P
-      DMP_CUDA(launch_transpose(Y, n, n, n, Z, st));  // Z = Y^T = P G
-      DMP_CUDA(times_P(Y, Pk, YP));   // G P^2
-      DMP_CUDA(times_P(Z, Pk, ZP));   // P G P
-      DMP_CUDA(launch_adj_reduce(Pk, Xk, G, Z, n, part, cs[k], sc, st));
-      DMP_CUDA(launch_adj_step(G, Y, YP, ZP, Pk, Xk, n, sc, Gn, st));
+      if (k != k1 - 1) DMP_CUDA(split_P(Pk));  // (the last one's planes are there: its square came last)
+      DMP_CUDA(times_P(G, Pk, Y));
+      if (merged) {
+        DMP_CUDA(launch_adj_half(Y, n, W, st));
+        DMP_CUDA(times_P(W, Pk, V));
+      } else {
+        DMP_CUDA(times_P(Y, Pk, V));
+        DMP_CUDA(launch_transpose(Y, n, n, n, W, st));
+        DMP_CUDA(times_P(W, Pk, U));
+      }
+      DMP_CUDA(launch_adj_reduce(Pk, Xk, G, Y, n, part, ticket, cs[k], sc, st));
+      DMP_CUDA(launch_adj_step(G, Y, V, merged ? nullptr : U, Pk, Xk, n, sc, Gn, st));
       std::swap(G, Gn);
     }
     int flag = 0;
@@ -999,7 +1008,7 @@ int dm_purify_backward(const double* H, int64_t n, int64_t n_occ, const dmp_opts
   h0.row_max = hd.row_max;
   h0.bounds_grad = (opts->flags & DMP_FLAG_BOUNDS_CONSTANT) ? 0 : 1;
   DMP_CUDA(cudaMemcpyAsync(p0s, &h0, sizeof(h0), cudaMemcpyHostToDevice, st));
-  DMP_CUDA(launch_p0_adjoint(G, H, n, n, part, p0s, dLdH, n, st));
+  DMP_CUDA(launch_p0_adjoint(G, H, n, n, part, ticket, p0s, dLdH, n, st));
   DMP_CUDA(cudaStreamSynchronize(st));
   return DMP_OK;
 }
