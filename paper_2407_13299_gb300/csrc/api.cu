@@ -30,6 +30,36 @@ struct Carver {
   }
 };
 
+// Reads device words at a marked point of a stream on a stream of its own, so
+// that what was enqueued after the mark runs meanwhile.
+class StateReader {
+ public:
+  explicit StateReader(cudaStream_t st) : st_(st) {}
+  StateReader(const StateReader&) = delete;
+  StateReader& operator=(const StateReader&) = delete;
+  ~StateReader() {
+    if (marked_ != nullptr) cudaEventDestroy(marked_);
+    if (side_ != nullptr) cudaStreamDestroy(side_);
+  }
+  cudaError_t mark() {
+    cudaError_t e = cudaSuccess;
+    if (side_ == nullptr) e = cudaStreamCreateWithFlags(&side_, cudaStreamNonBlocking);
+    if (e == cudaSuccess && marked_ == nullptr) e = cudaEventCreateWithFlags(&marked_, cudaEventDisableTiming);
+    return e == cudaSuccess ? cudaEventRecord(marked_, st_) : e;
+  }
+  // Returns when the words, as they were at the mark, are in dst (what runs
+  // after the mark must not write them, or the reader bear either value).
+  cudaError_t read(void* dst, const void* src, size_t bytes) {
+    cudaError_t e = cudaStreamWaitEvent(side_, marked_, 0);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, side_);
+    return e == cudaSuccess ? cudaStreamSynchronize(side_) : e;
+  }
+
+ private:
+  cudaStream_t st_, side_ = nullptr;
+  cudaEvent_t marked_ = nullptr;
+};
+
 struct Opts {
   int mode, s, beta, executor, max_iter, every;
   double tol, energy_tol;
@@ -139,7 +169,7 @@ TcArea area_at(const Opts& o, void* ws, size_t off) { return TcArea{static_cast<
 
 // ---------------------------------------------------------------- dm_purify layout
 struct PurifyLayout {
-  size_t state, partials, rowbuf, expsP, expsX, err, Palt, X2, planesP, planesX, area, total;
+  size_t state, partials, rowbuf, expsP, expsX, Palt, X2, planesP, planesX, area, total;
   int64_t n_pad, k_pad;
 };
 
@@ -153,7 +183,6 @@ PurifyLayout purify_layout(int64_t n, const Opts& o) {
   L.rowbuf = c.take(gershgorin_rowbuf_bytes(n));
   L.expsP = c.take(static_cast<size_t>(L.n_pad) * sizeof(int32_t));
   L.expsX = c.take(static_cast<size_t>(L.n_pad) * sizeof(int32_t));
-  L.err = c.take(sizeof(int32_t));
   L.Palt = c.take(static_cast<size_t>(n) * n * sizeof(double));
   L.X2 = c.take(static_cast<size_t>(n) * n * sizeof(double));
   if (o.mode != DMP_FP64) {
@@ -412,9 +441,8 @@ int dm_purify(const double* H, int64_t n, int64_t ldh, int64_t n_occ, const dmp_
   double* X2 = reinterpret_cast<double*>(at(ws, L.X2));
   void* planesP = o.mode != DMP_FP64 ? at(ws, L.planesP) : nullptr;
   void* planesX = o.mode != DMP_FP64 ? at(ws, L.planesX) : nullptr;
-  int* err = reinterpret_cast<int*>(at(ws, L.err));
+  int* err = &state->timeout;
   TcArea area = area_at(o, ws, L.area);
-  DMP_CUDA(cudaMemsetAsync(err, 0, sizeof(int), st));
 
   PurifyState init;
   std::memset(&init, 0, sizeof(init));
@@ -435,6 +463,7 @@ int dm_purify(const double* H, int64_t n, int64_t ldh, int64_t n_occ, const dmp_
   double* alt = Palt;
   int64_t ldalt = n;
   const int* done = &state->done;
+  StateReader reader(st);
   bool late = false;  // the late-slice schedule has switched
   int late_iters = 0;
   for (int k = 0; k <= o.max_iter; ++k) {
@@ -466,44 +495,41 @@ int dm_purify(const double* H, int64_t n, int64_t ldh, int64_t n_occ, const dmp_
     } else {
       DMP_CUDA(launch_measure_variant(cur, ldcur, X2, n, H, ldh, n, partials, state, st));
     }
-    int32_t flags[3] = {0, 0, 0};
-    double idem2 = 0.0;
-    DMP_CUDA(cudaMemcpyAsync(&flags[0], &state->done, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-    DMP_CUDA(cudaMemcpyAsync(&flags[1], err, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-    DMP_CUDA(cudaMemcpyAsync(&flags[2], &state->step_kind, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-    if (o.late_s > 0) DMP_CUDA(cudaMemcpyAsync(&idem2, &state->idem2, sizeof(double), cudaMemcpyDeviceToHost, st));
-    DMP_CUDA(cudaStreamSynchronize(st));
-    if (flags[1]) return DMP_ERR_TIMEOUT;
-    if (flags[0]) break;
+    // The step is enqueued before the measured state is read: the device goes on
+    // with it meanwhile (its kernels return at once where a stopping rule has
+    // fired), and the next iteration's launches are in the queue when it ends.
+    DMP_CUDA(reader.mark());
+    PurifyState now;
     if (o.method != DMP_METHOD_PM) {
-      // SP2 / TRS4 step (the weights are on the device)
-      if (flags[2] == 0) {
-        DMP_CUDA(launch_axpby(cur, ldcur, X2, n, alt, ldalt, n, state, st));
-        std::swap(cur, alt);
-        std::swap(ldcur, ldalt);
-      } else {
-        // X' = X2 Z: Z into alt, then the symmetric product written over X
+      // SP2 / TRS4 (the step's kind and weights are on the device): elementwise, in place
+      DMP_CUDA(launch_axpby(cur, ldcur, X2, n, n, state, st));
+      if (o.method == DMP_METHOD_TRS4) {
+        // or X' = X2 Z: Z into alt, then the symmetric product written over X
         DMP_CUDA(launch_trs4_z(cur, ldcur, X2, n, alt, ldalt, n, state, st));
+        const int* skip = &state->no_product;
         EpiArgs ez{};
         ez.kind = EPI_SYM_STORE;
         ez.C = cur;
         ez.ldc = ldcur;
         ez.round32 = o.store32 ? 1 : 0;
         if (o.mode == DMP_FP64) {
-          DMP_CUDA(launch_gemm_f64(X2, n, alt, ldalt, n, n, n, 1, ez, done, st));
+          DMP_CUDA(launch_gemm_f64(X2, n, alt, ldalt, n, n, n, 1, ez, skip, st));
         } else {
           DMP_CUDA(launch_split_rows(X2, n, n, n, oi.s, oi.beta, expsX, planesX, L.n_pad, L.k_pad,
-                                     elem_kind(o), has_diff(oi, oi.s), nullptr, done, st));
+                                     elem_kind(o), has_diff(oi, oi.s), nullptr, skip, st));
           DMP_CUDA(launch_split_rows(alt, n, n, ldalt, oi.s, oi.beta, expsP, planesP, L.n_pad, L.k_pad,
-                                     elem_kind(o), has_diff(oi, oi.s), nullptr, done, st));
-          DMP_CUDA(launch_product(oi, planesX, planesP, expsX, expsP, n, n, n, L.n_pad, L.n_pad, L.k_pad, 1, ez, done,
+                                     elem_kind(o), has_diff(oi, oi.s), nullptr, skip, st));
+          DMP_CUDA(launch_product(oi, planesX, planesP, expsX, expsP, n, n, n, L.n_pad, L.n_pad, L.k_pad, 1, ez, skip,
                                   err, area, st));
         }
       }
+      DMP_CUDA(reader.read(&now, state, sizeof(now)));
+      if (now.timeout) {
+        DMP_CUDA(cudaStreamSynchronize(st));
+        return DMP_ERR_TIMEOUT;
+      }
+      if (now.done) break;
       continue;
-    }
-    if (tape != nullptr) {
-      DMP_CUDA(cudaMemcpyAsync(tape_c + k, &state->c, sizeof(double), cudaMemcpyDeviceToDevice, st));
     }
     EpiArgs e3{};
     e3.kind = EPI_PM_UPDATE;
@@ -523,10 +549,19 @@ int dm_purify(const double* H, int64_t n, int64_t ldh, int64_t n_occ, const dmp_
       DMP_CUDA(launch_product(oi, planesP, planesX, expsP, expsX, n, n, n, L.n_pad, L.n_pad, L.k_pad, 1, e3, done,
                               err, area, st));
     }
+    DMP_CUDA(reader.read(&now, state, sizeof(now)));
+    if (now.timeout) {
+      DMP_CUDA(cudaStreamSynchronize(st));
+      return DMP_ERR_TIMEOUT;
+    }
+    if (now.done) break;
+    if (tape != nullptr) {
+      DMP_CUDA(cudaMemcpyAsync(tape_c + k, &state->c, sizeof(double), cudaMemcpyDeviceToDevice, st));
+    }
     std::swap(cur, alt);
     std::swap(ldcur, ldalt);
     // the late-slice schedule switches after an update whose iterate was within late_idem of idempotency
-    if (o.late_s > 0 && std::sqrt(idem2) < o.late_idem) late = true;
+    if (o.late_s > 0 && std::sqrt(now.idem2) < o.late_idem) late = true;
   }
   // ---- refinement (Sec. "Precision Requirements Sweep"): one McWeeny step in
   // full precision, P' = 3 P^2 - 2 P^3, run as the update with the weights of c = 1/2
@@ -576,11 +611,9 @@ int dm_purify(const double* H, int64_t n, int64_t ldh, int64_t n_occ, const dmp_
                                cudaMemcpyDeviceToDevice, st));
   }
   PurifyState fin;
-  int32_t err_end = 0;
   DMP_CUDA(cudaMemcpyAsync(&fin, state, sizeof(fin), cudaMemcpyDeviceToHost, st));
-  DMP_CUDA(cudaMemcpyAsync(&err_end, err, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
   DMP_CUDA(cudaStreamSynchronize(st));
-  if (err_end) return DMP_ERR_TIMEOUT;
+  if (fin.timeout) return DMP_ERR_TIMEOUT;
   if (tape != nullptr) {
     TapeHeader h;
     std::memset(&h, 0, sizeof(h));

@@ -93,6 +93,8 @@ struct PurifyState {
   int32_t max_iter;
   int32_t store32;  // DMP_FLAG_FP32_STORAGE: stored matrices rounded to FP32 values
   int32_t ticket;   // blocks of a running measure that have finished; 0 between kernels
+  int32_t timeout;  // dm_purify: a product's bounded device wait ran out
+  int32_t no_product;  // SP2 / TRS4: this step has no product (done, or step_kind 0)
 };
 
 // A matrix element as it is stored: rounded to the nearest FP32 value under
@@ -198,12 +200,13 @@ cudaError_t launch_refine_weights(PurifyState* state, cudaStream_t st);
 cudaError_t launch_energy(const double* P, int64_t ldp, const double* H, int64_t ldh, int64_t n, double* partials,
                           PurifyState* state, cudaStream_t st);
 // SP2 / TRS4: measures with tr X^4 and variant_decide; the elementwise step
-// Out = alpha X + b2 X2; the TRS4 factor Z = zd I + zx X + zx2 X2 (weights from
-// the state; full n x n, so the results are exactly symmetric as X and X2 are).
+// X <- alpha X + b2 X2 (a step of kind 0, else nothing); the TRS4 factor
+// Z = zd I + zx X + zx2 X2 (a step of kind 1, else nothing); weights from the
+// state; full n x n, so the results are exactly symmetric as X and X2 are).
 cudaError_t launch_measure_variant(const double* X, int64_t ldx, const double* X2, int64_t ldx2, const double* H,
                                    int64_t ldh, int64_t n, double* partials, PurifyState* state, cudaStream_t st);
-cudaError_t launch_axpby(const double* X, int64_t ldx, const double* X2, int64_t ldx2, double* out, int64_t ldo,
-                         int64_t n, const PurifyState* state, cudaStream_t st);
+cudaError_t launch_axpby(double* X, int64_t ldx, const double* X2, int64_t ldx2, int64_t n, const PurifyState* state,
+                         cudaStream_t st);
 cudaError_t launch_trs4_z(const double* X, int64_t ldx, const double* X2, int64_t ldx2, double* out, int64_t ldo,
                           int64_t n, const PurifyState* state, cudaStream_t st);
 cudaError_t launch_measure(const double* P, int64_t ldp, const double* X2, int64_t ldx,

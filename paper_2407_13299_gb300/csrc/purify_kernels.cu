@@ -272,32 +272,64 @@ measure_kernel(const double* __restrict__ P, int64_t ldp, const double* __restri
       pm_decide(st, tot);
     } else {
       variant_decide(st, tot);
+      st->no_product = st->done != 0 || st->step_kind == 0;
     }
   }
 }
 
-// Out = alpha X + b2 X2 (SP2 steps), over the full n x n (grid-stride, rows of 256 threads)
+// The elementwise steps below return at once unless the measured state asks for
+// them: both are enqueued before the host knows which it is. A block holds up to
+// 1024 entries of a row, four per thread, whose loads do not wait for one another.
+constexpr int kElemCols = 1024;
+
+dim3 elem_grid(int64_t n) {
+  return dim3(static_cast<unsigned>((n + kElemCols - 1) / kElemCols), static_cast<unsigned>(std::min<int64_t>(n, 65535)));
+}
+
+// X <- alpha X + b2 X2 (step_kind 0), over the full n x n
 __global__ void __launch_bounds__(256)
-axpby_kernel(const double* __restrict__ X, int64_t ldx, const double* __restrict__ X2, int64_t ldx2,
-             double* __restrict__ out, int64_t ldo, int64_t n, const PurifyState* st) {
+axpby_kernel(double* X, int64_t ldx, const double* __restrict__ X2, int64_t ldx2, int64_t n, const PurifyState* st) {
+  if (st->done != 0 || st->step_kind != 0) return;
   const double a = st->alpha, b = st->b2;
   const bool r32 = st->store32 != 0;
-  for (int64_t i = blockIdx.x; i < n; i += gridDim.x) {
-    for (int64_t j = threadIdx.x; j < n; j += blockDim.x)
-      out[i * ldo + j] = stored_value(a * X[i * ldx + j] + b * X2[i * ldx2 + j], r32);
+  const int64_t j0 = static_cast<int64_t>(blockIdx.x) * kElemCols + threadIdx.x;
+  for (int64_t i = blockIdx.y; i < n; i += gridDim.y) {
+    double x[4], y[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int64_t j = j0 + 256 * u;
+      x[u] = j < n ? X[i * ldx + j] : 0.0;
+      y[u] = j < n ? X2[i * ldx2 + j] : 0.0;
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int64_t j = j0 + 256 * u;
+      if (j < n) X[i * ldx + j] = stored_value(a * x[u] + b * y[u], r32);
+    }
   }
 }
 
-// Z = zd I + zx X + zx2 X2 (the TRS4 factor with F + gamma G = X2 Z)
+// Z = zd I + zx X + zx2 X2 (the TRS4 factor with F + gamma G = X2 Z; step_kind 1)
 __global__ void __launch_bounds__(256)
 trs4_z_kernel(const double* __restrict__ X, int64_t ldx, const double* __restrict__ X2, int64_t ldx2,
               double* __restrict__ out, int64_t ldo, int64_t n, const PurifyState* st) {
+  if (st->no_product != 0) return;
   const double zd = st->zd, zx = st->zx, zx2 = st->zx2;
   const bool r32 = st->store32 != 0;
-  for (int64_t i = blockIdx.x; i < n; i += gridDim.x) {
-    for (int64_t j = threadIdx.x; j < n; j += blockDim.x) {
-      const double v = zx * X[i * ldx + j] + zx2 * X2[i * ldx2 + j];
-      out[i * ldo + j] = stored_value(j == i ? v + zd : v, r32);
+  const int64_t j0 = static_cast<int64_t>(blockIdx.x) * kElemCols + threadIdx.x;
+  for (int64_t i = blockIdx.y; i < n; i += gridDim.y) {
+    double x[4], y[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int64_t j = j0 + 256 * u;
+      x[u] = j < n ? X[i * ldx + j] : 0.0;
+      y[u] = j < n ? X2[i * ldx2 + j] : 0.0;
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int64_t j = j0 + 256 * u;
+      const double v = zx * x[u] + zx2 * y[u];
+      if (j < n) out[i * ldo + j] = stored_value(j == i ? v + zd : v, r32);
     }
   }
 }
@@ -373,11 +405,10 @@ cudaError_t launch_measure_variant(const double* X, int64_t ldx, const double* X
   return cudaGetLastError();
 }
 
-cudaError_t launch_axpby(const double* X, int64_t ldx, const double* X2, int64_t ldx2, double* out, int64_t ldo,
-                         int64_t n, const PurifyState* state, cudaStream_t st) {
+cudaError_t launch_axpby(double* X, int64_t ldx, const double* X2, int64_t ldx2, int64_t n, const PurifyState* state,
+                         cudaStream_t st) {
   ProfScope prof(DMP_PROF_OTHER, st);
-  axpby_kernel<<<static_cast<unsigned>(std::min<int64_t>(n, 4 * 152)), 256, 0, st>>>(X, ldx, X2, ldx2, out, ldo, n,
-                                                                                     state);
+  axpby_kernel<<<elem_grid(n), 256, 0, st>>>(X, ldx, X2, ldx2, n, state);
   count_launch();
   return cudaGetLastError();
 }
@@ -385,8 +416,7 @@ cudaError_t launch_axpby(const double* X, int64_t ldx, const double* X2, int64_t
 cudaError_t launch_trs4_z(const double* X, int64_t ldx, const double* X2, int64_t ldx2, double* out, int64_t ldo,
                           int64_t n, const PurifyState* state, cudaStream_t st) {
   ProfScope prof(DMP_PROF_OTHER, st);
-  trs4_z_kernel<<<static_cast<unsigned>(std::min<int64_t>(n, 4 * 152)), 256, 0, st>>>(X, ldx, X2, ldx2, out, ldo,
-                                                                                      n, state);
+  trs4_z_kernel<<<elem_grid(n), 256, 0, st>>>(X, ldx, X2, ldx2, out, ldo, n, state);
   count_launch();
   return cudaGetLastError();
 }
