@@ -269,28 +269,29 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
-// warp_sum of eight values at once: at each of the first three steps a lane hands
-// half of its values to its partner and keeps the partner's part of the others,
-// so a warp adds 4 + 2 + 1 + 1 + 1 times instead of 40. The sums are warp_sum's
-// bit for bit (the same pairs, addition being commutative). The total of value
-// lane >> 2 is returned.
-__device__ __forceinline__ double warp_sum8(const double* v) {
+// warp_sum of NV = 2, 4 or 8 values at once: at each of the first log2 NV steps a
+// lane hands half of its values to its partner and keeps the partner's part of
+// the others, so a warp adds 4 + 2 + 1 + 1 + 1 times for eight values instead of
+// 40. The sums are warp_sum's bit for bit (the same pairs, addition being
+// commutative). The total of value lane / (32 / NV) is returned.
+template <int NV>
+__device__ __forceinline__ double warp_sums(const double* v) {
+  static_assert(NV == 2 || NV == 4 || NV == 8, "");
   const int lane = threadIdx.x & 31;
-  double a[4], b[2];
+  double a[NV];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const bool up = (lane & 16) != 0;
-    a[i] = (up ? v[i + 4] : v[i]) + __shfl_xor_sync(0xffffffffu, up ? v[i] : v[i + 4], 16);
-  }
+  for (int i = 0; i < NV; ++i) a[i] = v[i];
+  int o = 16;
 #pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    const bool up = (lane & 8) != 0;
-    b[i] = (up ? a[i + 2] : a[i]) + __shfl_xor_sync(0xffffffffu, up ? a[i] : a[i + 2], 8);
+  for (int half = NV / 2; half > 0; half >>= 1, o >>= 1) {
+    const bool up = (lane & o) != 0;
+#pragma unroll
+    for (int i = 0; i < half; ++i)
+      a[i] = (up ? a[i + half] : a[i]) + __shfl_xor_sync(0xffffffffu, up ? a[i] : a[i + half], o);
   }
-  const bool up = (lane & 4) != 0;
-  double c = (up ? b[1] : b[0]) + __shfl_xor_sync(0xffffffffu, up ? b[0] : b[1], 4);
-  c += __shfl_xor_sync(0xffffffffu, c, 2);
-  c += __shfl_xor_sync(0xffffffffu, c, 1);
+  double c = a[0];
+#pragma unroll
+  for (int p = 16 / NV; p > 0; p >>= 1) c += __shfl_xor_sync(0xffffffffu, c, p);
   return c;
 }
 
@@ -299,12 +300,12 @@ __device__ __forceinline__ double warp_sum8(const double* v) {
 template <int NQ>
 __device__ __forceinline__ void block_totals(const double (&v)[NQ], double (*red)[NQ], double* tot) {
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const double c = warp_sum8(v);
+  static_assert(NQ == 8 || NQ == 10, "");
+  const double c = warp_sums<8>(v);
   if ((lane & 3) == 0) red[w][lane >> 2] = c;
-#pragma unroll
-  for (int q = 8; q < NQ; ++q) {
-    const double x = warp_sum(v[q]);
-    if (lane == 0) red[w][q] = x;
+  if (NQ == 10) {
+    const double x = warp_sums<2>(v + NQ - 2);
+    if ((lane & 15) == 0) red[w][8 + (lane >> 4)] = x;
   }
   __syncthreads();
   if (threadIdx.x < NQ) {

@@ -190,13 +190,17 @@ __global__ void p0_kernel(const double* __restrict__ H, int64_t n, int64_t ldh, 
 // stopping rules: NQ = 8 canonical purification (pm_decide), NQ = 10 SP2 / TRS4
 // (variant_decide). At large sizes bound by the FP64 pipe, four operations per
 // upper element (n = 8192: 0.30 ms, 0.22 ms for the operations alone); at small
-// ones by the block sums, whose adds warp_sum8 cuts from 40 to 9 per warp, and by
-// launches (n = 256: 31 us for two kernels before, now 11).
+// ones by the block sums: an add takes the pipe as long for one lane as for 32,
+// so warp_sums adds 6 times for the sums that every thread has a part of, and
+// those that only thread 0 has are not summed at all (n = 256: 31 us for two
+// kernels before, 12.7 with all ten summed by 9 adds a warp, 11.4 now; n = 999,
+// SP2 / TRS4: 30 to 24).
 template <int NQ>
 __global__ void __launch_bounds__(256)
 measure_kernel(const double* __restrict__ P, int64_t ldp, const double* __restrict__ X2, int64_t ldx,
                const double* __restrict__ H, int64_t ldh, int64_t n, double* __restrict__ part, PurifyState* st) {
   if (st->done) return;
+  bool four = false;
   double d_xx = 0.0, a_xx[4] = {0.0, 0.0, 0.0, 0.0};
   // four independent accumulator sets (entries j, j + 256, j + 512, j + 768 of
   // a step) keep twelve loads in flight per thread; combined in order below
@@ -218,6 +222,7 @@ measure_kernel(const double* __restrict__ P, int64_t ldp, const double* __restri
     }
     int64_t j = i + 1 + threadIdx.x;
     for (; j + 3 * B < n; j += 4 * B) {
+      four = true;
       double p[4], x[4], h[4];
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
@@ -241,27 +246,48 @@ measure_kernel(const double* __restrict__ P, int64_t ldp, const double* __restri
       if (NQ == 10) a_xx[0] += x * x;
     }
   }
-  const double u_px = (a_px[0] + a_px[1]) + (a_px[2] + a_px[3]);
-  const double u_id = (a_id[0] + a_id[1]) + (a_id[2] + a_id[3]);
-  const double u_ph = (a_ph[0] + a_ph[1]) + (a_ph[2] + a_ph[3]);
-  const double u_xx = (a_xx[0] + a_xx[1]) + (a_xx[2] + a_xx[3]);
-  double v[NQ];
-  v[0] = d_p, v[1] = d_x, v[2] = d_px, v[3] = u_px, v[4] = d_id, v[5] = u_id, v[6] = d_ph, v[7] = u_ph;
-  if (NQ == 10) v[NQ - 2] = d_xx, v[NQ - 1] = u_xx;
+  // the block's sums: the diagonal's from thread 0, which alone has any (the adds
+  // of zeros to them are left out; + 0.0 is what is left of them), and three or
+  // four from every thread. Sets that stayed zero in the whole warp are not added.
+  double u[4] = {a_px[0], a_id[0], a_ph[0], a_xx[0]};
+  if (__any_sync(0xffffffffu, four)) {
+    u[0] = (a_px[0] + a_px[1]) + (a_px[2] + a_px[3]);
+    u[1] = (a_id[0] + a_id[1]) + (a_id[2] + a_id[3]);
+    u[2] = (a_ph[0] + a_ph[1]) + (a_ph[2] + a_ph[3]);
+    u[3] = (a_xx[0] + a_xx[1]) + (a_xx[2] + a_xx[3]);
+  }
   __shared__ double red[8][NQ];
   __shared__ double tot[NQ];
   __shared__ bool last;
-  block_totals<NQ>(v, red, tot);
-  if (threadIdx.x < NQ) part[static_cast<int64_t>(blockIdx.x) * NQ + threadIdx.x] = tot[threadIdx.x];
+  double* mine = part + static_cast<int64_t>(blockIdx.x) * NQ;
+  const double c = warp_sums<4>(u);
+  if ((threadIdx.x & 7) == 0) red[threadIdx.x >> 5][(threadIdx.x >> 3) & 3] = c;
+  if (threadIdx.x == 0) {
+    mine[0] = d_p + 0.0;
+    mine[1] = d_x + 0.0;
+    mine[2] = d_px + 0.0;
+    mine[4] = d_id + 0.0;
+    mine[6] = d_ph + 0.0;
+    if (NQ == 10) mine[NQ - 2] = d_xx + 0.0;
+  }
+  __syncthreads();
+  if (threadIdx.x < (NQ - 2) / 2) {
+    double t = 0.0;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) t += red[w][threadIdx.x];
+    mine[3 + 2 * threadIdx.x] = t;
+  }
   __threadfence();  // the partials before the count
   __syncthreads();
   if (threadIdx.x == 0) last = atomicAdd(&st->ticket, 1) == static_cast<int>(gridDim.x) - 1;
   __syncthreads();
   if (!last) return;
   __threadfence();  // every block's partials before the reads
+  double v[NQ];
 #pragma unroll
-  for (int q = 0; q < NQ; ++q) v[q] = 0.0;
-  for (int b = threadIdx.x; b < static_cast<int>(gridDim.x); b += blockDim.x) {
+  for (int q = 0; q < NQ; ++q)
+    v[q] = threadIdx.x < gridDim.x ? __ldcg(part + static_cast<int64_t>(threadIdx.x) * NQ + q) : 0.0;
+  for (int b = threadIdx.x + blockDim.x; b < static_cast<int>(gridDim.x); b += blockDim.x) {
 #pragma unroll
     for (int q = 0; q < NQ; ++q) v[q] += __ldcg(part + static_cast<int64_t>(b) * NQ + q);
   }
