@@ -527,7 +527,8 @@ __device__ __forceinline__ void store4(double* a, const double (&v)[4], bool vec
 // P^2 are exactly symmetric (read at (column, row)) and the mirrored elements
 // are four in a row too, so every array costs a thread one address and 16-byte
 // accesses; the row-major elements go through shared memory for the same
-// reason. n = 4096: 0.06 ms beside 0.5 ms of products, n = 1024: 6 beside 29 us.
+// reason. n = 4096: 40 us (with the update 60, 45 of them the FP64 pipe's)
+// beside 470 of products, n = 1024: 6 (9) beside 29.
 // (Done instead by two further warps of the next wave's product kernel it cost
 // 3 % of the whole: 200 us per wave of 76 tiles on so few threads, and the
 // shared memory of a seventh stage.)
@@ -539,7 +540,6 @@ template <int BN, bool PAIR, int OUT, int NG>
 __global__ void __launch_bounds__(FIN_THREADS)
 ozaki_finish_kernel(const __grid_constant__ TcParams p) {
   constexpr bool UPD = OUT == OUT_UPDATE, CHEB = OUT == OUT_CHEB;
-  if (p.done != nullptr && *p.done) return;
   __shared__ double trans[32][33];
   using Cfg = TcCfg<BN, PAIR>;
   constexpr int SR = Cfg::BM / 32, SC = BN / 32;
@@ -555,7 +555,26 @@ ozaki_finish_kernel(const __grid_constant__ TcParams p) {
   const int h = 32 * sc / Cfg::COLS;
   const int e = 4 * h + ((sr + 2) & 3);  // the epilogue warp that owns these rows and columns
 
+  // The group sums first: their place follows from the block alone, so they are
+  // on their way while the batch's tile, matrix and state are looked up one after
+  // the other, and so does the check of the done flag (152 tiles of a batch: 42 us,
+  // with the update 65; 107 and 123 with the loads after the check).
+  constexpr int G = NG == 0 ? 1 : NG;
+  long long* part0 = p.area + (static_cast<int64_t>(tile) * Cfg::RANKS + rank) * (NG == 0 ? p.prog.ng : NG) * Cfg::PART +
+                     (e * (Cfg::COLS * 32) + (32 * sc - h * Cfg::COLS + line0) * 32 + q4);
+  long long T[PASSES][G][4];
+#pragma unroll
+  for (int pass = 0; pass < PASSES; ++pass) {
+#pragma unroll
+    for (int g = 0; g < NG; ++g) {
+      const longlong2* a = reinterpret_cast<const longlong2*>(part0 + g * Cfg::PART + pass * (LINES * 32));
+      const longlong2 x = a[0], y = a[1];
+      T[pass][g][0] = x.x, T[pass][g][1] = x.y, T[pass][g][2] = y.x, T[pass][g][3] = y.y;
+    }
+  }
+
   // the tile's place and its output step
+  int done = p.done != nullptr ? *p.done : 0;
   int m0, n0, m = static_cast<int>(p.m), n = static_cast<int>(p.n);
   const int32_t* ea = p.ea;
   const int32_t* eb = p.eb;
@@ -566,7 +585,7 @@ ozaki_finish_kernel(const __grid_constant__ TcParams p) {
   } else {
     const int4 t = p.tiles[p.tile0 + tile];
     const BatchMat& M = p.mats[t.x];
-    if (M.state->done) return;
+    done = M.state->done;
     m0 = t.y * Cfg::BM;
     n0 = t.z * BN;
     m = n = static_cast<int>(M.n);
@@ -590,11 +609,10 @@ ozaki_finish_kernel(const __grid_constant__ TcParams p) {
   const int r = r0 + q4;  // this thread's first row
   // nothing of this block is written: outside the matrix, or below the diagonal
   const bool none = r0 >= m || c0 >= n || (sym && r0 > c0 + 31);
-  long long* part0 = p.area + (static_cast<int64_t>(tile) * Cfg::RANKS + rank) * (NG == 0 ? p.prog.ng : NG) * Cfg::PART +
-                     (e * (Cfg::COLS * 32) + (32 * sc - h * Cfg::COLS + line0) * 32 + q4);
   const bool vec = (epi.ldc & 1) == 0 && (reinterpret_cast<uintptr_t>(epi.C) & 15) == 0;
 
   if constexpr (NG == 0) {
+    if (done) return;
     // test hook: group g holds the exact sum of level g + 2
     for (int pass = 0; pass < PASSES; ++pass) {
       const int c = c0 + line0 + LINES * pass;
@@ -610,19 +628,23 @@ ozaki_finish_kernel(const __grid_constant__ TcParams p) {
     return;
   }
 
-  const double wa = UPD ? epi.state->alpha : 0.0;
-  const double w2 = UPD ? epi.state->b2 : 0.0;
-  const double w3 = UPD ? epi.state->b3 : 0.0;
-  const double coef = CHEB && epi.acc != nullptr ? *epi.coef : 0.0;
-  // every load of the block before the first store, so that a thread waits
-  // for one round of latencies per block
-  constexpr int G = NG == 0 ? 1 : NG;
-  long long T[PASSES][G][4];
+  // the exponents beside the check, the rest after it; every load of the block
+  // before the first store, so that a thread waits for few rounds of latencies
   double pv[PASSES][4], xv[PASSES][4];
   int32_t ec[PASSES];
   int4 er4 = make_int4(0, 0, 0, 0);
   if (r < m) er4 = *reinterpret_cast<const int4*>(ea + r);  // (the exponent arrays are padded to 256 rows)
   const int32_t er[4] = {er4.x, er4.y, er4.z, er4.w};
+#pragma unroll
+  for (int pass = 0; pass < PASSES; ++pass) {
+    const int c = c0 + line0 + LINES * pass;
+    ec[pass] = c < n ? eb[c] : 0;
+  }
+  const double wa = UPD ? epi.state->alpha : 0.0;
+  const double w2 = UPD ? epi.state->b2 : 0.0;
+  const double w3 = UPD ? epi.state->b3 : 0.0;
+  const double coef = CHEB && epi.acc != nullptr ? *epi.coef : 0.0;
+  if (done) return;
   // the update's P and P^2; the recurrence's term before and its running sum
   const bool two = UPD || (CHEB && epi.acc != nullptr), one = UPD || (CHEB && epi.P != nullptr);
   const double* xbase = CHEB ? epi.acc : epi.X2;
@@ -634,13 +656,6 @@ ozaki_finish_kernel(const __grid_constant__ TcParams p) {
 #pragma unroll
   for (int pass = 0; pass < PASSES; ++pass) {
     const int c = c0 + line0 + LINES * pass;
-#pragma unroll
-    for (int g = 0; g < NG; ++g) {
-      const longlong2* a = reinterpret_cast<const longlong2*>(part0 + g * Cfg::PART + pass * (LINES * 32));
-      const longlong2 x = a[0], y = a[1];
-      T[pass][g][0] = x.x, T[pass][g][1] = x.y, T[pass][g][2] = y.x, T[pass][g][3] = y.y;
-    }
-    ec[pass] = c < n ? eb[c] : 0;
     if (UPD || CHEB) {
       // the rows of this column that are written: inside the matrix, and not below the diagonal
       const int rows = c < n ? min(sym ? c + 1 : m, m) - r : 0;
