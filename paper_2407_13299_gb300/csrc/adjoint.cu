@@ -87,9 +87,11 @@ __device__ __forceinline__ bool last_block_sums(double* part, int32_t* ticket, d
 // matrix in flight per thread; n = 1024: 5 us of the FP64 pipe, 20 in all (27 with
 // one element in flight, 63 with a single thread's final sums in their own kernel).
 __global__ void __launch_bounds__(256)
-adj_reduce_kernel(const double* __restrict__ P, const double* __restrict__ X2, const double* __restrict__ G,
-                  const double* __restrict__ Y, int64_t n, double* __restrict__ part, int32_t* ticket, double c,
+adj_reduce_kernel(const double* P, const double* X2, const double* G,
+                  const double* Y, int64_t n, double* part, int32_t* ticket, double c,
                   AdjScalars* out) {
+  chain_wait();
+  chain_next();
   __shared__ double red[8][8];
   __shared__ double tot[8];
   double v[8] = {0, 0, 0, 0, 0, 0, 0, 0};
@@ -124,7 +126,9 @@ adj_reduce_kernel(const double* __restrict__ P, const double* __restrict__ X2, c
 
 // W = Y + Y^T / 2, 32 x 32 block pairs (upper_tile), transposed through shared memory.
 __global__ void __launch_bounds__(256)
-adj_half_kernel(const double* __restrict__ Y, int64_t n, double* __restrict__ W, int T) {
+adj_half_kernel(const double* Y, int64_t n, double* W, int T) {
+  chain_wait();
+  chain_next();
   __shared__ double a[32][33], b[32][33];
   int bi, bj;
   upper_tile(blockIdx.x, T, bi, bj);
@@ -148,9 +152,11 @@ adj_half_kernel(const double* __restrict__ Y, int64_t n, double* __restrict__ W,
 // element pair read and wrote the lower side with a stride of n). (dL/dc) dc/dP
 // is cp P + cx X2 + ci I. n = 1024: 20 us.
 __global__ void __launch_bounds__(256)
-adj_step_kernel(const double* __restrict__ G, const double* __restrict__ Y, const double* __restrict__ V,
-                const double* __restrict__ U, const double* __restrict__ P, const double* __restrict__ X2, int64_t n,
-                const AdjScalars* __restrict__ sc, double* __restrict__ Gn, int T) {
+adj_step_kernel(const double* G, const double* Y, const double* V,
+                const double* U, const double* P, const double* X2, int64_t n,
+                const AdjScalars* sc, double* Gn, int T) {
+  chain_wait();
+  chain_next();
   __shared__ double low[32][33];  // b2 Y + b3 V of the lower block, then G_new of the upper
   int bi, bj;
   upper_tile(blockIdx.x, T, bi, bj);
@@ -276,7 +282,7 @@ constexpr int kAdjBlocks = 304;
 cudaError_t launch_adj_half(const double* Y, int64_t n, double* W, cudaStream_t st) {
   ProfScope prof(DMP_PROF_OTHER, st);
   const int T = static_cast<int>((n + 31) / 32);
-  adj_half_kernel<<<T * (T + 1) / 2, 256, 0, st>>>(Y, n, W, T);
+  launch_chained(adj_half_kernel, T * (T + 1) / 2, 256, st, Y, n, W, T);
   count_launch();
   return cudaGetLastError();
 }
@@ -284,7 +290,7 @@ cudaError_t launch_adj_half(const double* Y, int64_t n, double* W, cudaStream_t 
 cudaError_t launch_adj_reduce(const double* P, const double* X2, const double* G, const double* Y, int64_t n,
                               double* part, int32_t* ticket, double c, AdjScalars* sc, cudaStream_t st) {
   ProfScope prof(DMP_PROF_MEASURE, st);
-  adj_reduce_kernel<<<kAdjBlocks, 256, 0, st>>>(P, X2, G, Y, n, part, ticket, c, sc);
+  launch_chained(adj_reduce_kernel, kAdjBlocks, 256, st, P, X2, G, Y, n, part, ticket, c, sc);
   count_launch();
   return cudaGetLastError();
 }
@@ -293,7 +299,7 @@ cudaError_t launch_adj_step(const double* G, const double* Y, const double* V, c
                             const double* X2, int64_t n, const AdjScalars* sc, double* Gn, cudaStream_t st) {
   ProfScope prof(DMP_PROF_OTHER, st);
   const int T = static_cast<int>((n + 31) / 32);
-  adj_step_kernel<<<T * (T + 1) / 2, 256, 0, st>>>(G, Y, V, U, P, X2, n, sc, Gn, T);
+  launch_chained(adj_step_kernel, T * (T + 1) / 2, 256, st, G, Y, V, U, P, X2, n, sc, Gn, T);
   count_launch();
   return cudaGetLastError();
 }

@@ -60,6 +60,39 @@ __host__ __device__ constexpr int diff_plane(int s, int i, int j) {
 extern std::atomic<long long> g_launches;
 inline void count_launch(long long k = 1) { g_launches.fetch_add(k, std::memory_order_relaxed); }
 
+// ---------------------------------------------------------------- chained launches
+// The kernels of an iteration follow one another on one stream. Launched with
+// launch_chained, a kernel's CTAs are placed as soon as every CTA of the one
+// before has called chain_next, instead of after its end; chain_wait, before a
+// kernel's first access to device memory, then waits until the one before has
+// completed with its writes visible. A kernel calls chain_next after chain_wait,
+// so at most one waits behind the one that runs. (Launched any other way both
+// calls do nothing, and a kernel launched normally after a chained one waits for
+// its end as ever.) A canonical purification has seven such launches an iteration:
+// n = 256, 27 iterations 1.69 -> 1.54 ms; n = 2048, 39 iterations 11.65 -> 11.1.
+// Their pointers are not __restrict__: what they read is written while they may
+// already be resident, which the non-coherent loads of read-only data forbid.
+// Two product kernels are never on an SM together: each takes over half of its
+// shared memory, so neither waits for TMEM that the other holds.
+#ifdef __CUDACC__
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <typename... P, typename... A>
+inline void launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t st, A... args) {
+  cudaLaunchAttribute at[1] = {};
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.stream = st;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+#endif
+
 // ---------------------------------------------------------------- device-side run state
 // One per purification. Written by the measurement kernel, read by the update
 // epilogue and the host.

@@ -114,8 +114,10 @@ __device__ __forceinline__ double block_sum256(double v, double* red) {
 // node's energy e_j = a + b x_j. (A thread per node walked its M cosines one
 // after the other: 367 us at M = 200, 9 now.)
 __global__ void __launch_bounds__(kSumThreads)
-foe_weights_kernel(const FoeScalars* sc, const double* __restrict__ traces, int M, double* __restrict__ w,
-                   double* __restrict__ e) {
+foe_weights_kernel(const FoeScalars* sc, const double* traces, int M, double* w,
+                   double* e) {
+  chain_wait();
+  chain_next();
   __shared__ double red[kSumThreads / 32];
   const int64_t N = 2 * static_cast<int64_t>(M);
   const int64_t j = blockIdx.x;
@@ -163,8 +165,10 @@ __device__ __forceinline__ void mu_interval(const FoeScalars* sc, double kT, dou
 }
 
 __global__ void __launch_bounds__(kSumThreads)
-foe_mu_round_kernel(const FoeScalars* sc, double kT, double n_occ, int M, const double* __restrict__ w,
-                    const double* __restrict__ e, int round, MuRound* ws) {
+foe_mu_round_kernel(const FoeScalars* sc, double kT, double n_occ, int M, const double* w,
+                    const double* e, int round, MuRound* ws) {
+  chain_wait();
+  chain_next();
   __shared__ double tr[kMuNodes];
   __shared__ double red[kSumThreads / 32];
   double lo, hi;
@@ -196,6 +200,8 @@ foe_mu_round_kernel(const FoeScalars* sc, double kT, double n_occ, int M, const 
 __global__ void __launch_bounds__(kSumThreads)
 foe_occupation_kernel(FoeScalars* sc, double kT, double mu_given, double n_occ, int rounds, int M, const MuRound* ws,
                       const double* e, double* gx) {
+  chain_wait();
+  chain_next();
   __shared__ double tr[kMuNodes];
   double mu = mu_given;
   if (rounds > 0) {
@@ -212,7 +218,9 @@ foe_occupation_kernel(FoeScalars* sc, double kT, double mu_given, double n_occ, 
 // One CTA per k: c_k = (2 / N) sum_j g(x_j) cos(k theta_j). (A thread per k:
 // 621 us at M = 200, 9 now.)
 __global__ void __launch_bounds__(kSumThreads)
-foe_coeff_kernel(const double* __restrict__ gx, int M, double* __restrict__ coeffs) {
+foe_coeff_kernel(const double* gx, int M, double* coeffs) {
+  chain_wait();
+  chain_next();
   __shared__ double red[kSumThreads / 32];
   const int64_t N = 2 * static_cast<int64_t>(M);
   const int k = blockIdx.x;
@@ -228,9 +236,11 @@ foe_coeff_kernel(const double* __restrict__ gx, int M, double* __restrict__ coef
 // and P (ldp). 32 x 32 blocks on and above the diagonal, mirrored through
 // shared memory.
 __global__ void __launch_bounds__(256)
-foe_init_kernel(const double* __restrict__ H, int64_t ldh, int64_t n, const FoeScalars* sc,
-                const double* __restrict__ coeffs, double* __restrict__ Hs, double* __restrict__ T0,
-                double* __restrict__ T1, double* __restrict__ P, int64_t ldp, int T) {
+foe_init_kernel(const double* H, int64_t ldh, int64_t n, const FoeScalars* sc,
+                const double* coeffs, double* Hs, double* T0,
+                double* T1, double* P, int64_t ldp, int T) {
+  chain_wait();
+  chain_next();
   __shared__ double tile[32][33];
   int bi, bj;
   upper_tile(blockIdx.x, T, bi, bj);
@@ -264,7 +274,9 @@ foe_init_kernel(const double* __restrict__ H, int64_t ldh, int64_t n, const FoeS
 // out = sum_i A_ii in a fixed order (one CTA).
 // out[blockIdx.x] for the blockIdx.x-th matrix, `stride` doubles apart.
 __global__ void __launch_bounds__(kReduceThreads)
-foe_trace_kernel(const double* __restrict__ A, int64_t lda, int64_t stride, int64_t n, double* __restrict__ out) {
+foe_trace_kernel(const double* A, int64_t lda, int64_t stride, int64_t n, double* out) {
+  chain_wait();
+  chain_next();
   __shared__ double red[kReduceThreads];
   A += blockIdx.x * stride;
   double part = 0.0;
@@ -283,9 +295,11 @@ foe_trace_kernel(const double* __restrict__ A, int64_t lda, int64_t stride, int6
 // the FP64 operations that bound the kernel (nt + 1 per element; n = 2048, nt =
 // 15: 115 us over the full matrix, 66 now).
 __global__ void __launch_bounds__(256)
-foe_combine_kernel(const double* __restrict__ Tm, int64_t tstride, int nt, const double* __restrict__ w,
-                   const double* __restrict__ Y, double alpha, const double* Bm2, double* out, int64_t ldo, int64_t n,
+foe_combine_kernel(const double* Tm, int64_t tstride, int nt, const double* w,
+                   const double* Y, double alpha, const double* Bm2, double* out, int64_t ldo, int64_t n,
                    int T) {
+  chain_wait();
+  chain_next();
   __shared__ double tile[32][33];
   int bi, bj;
   upper_tile(blockIdx.x, T, bi, bj);
@@ -330,8 +344,10 @@ foe_combine_kernel(const double* __restrict__ Tm, int64_t tstride, int nt, const
 constexpr int kDotTerms = 7;
 
 __global__ void __launch_bounds__(256)
-foe_dots_kernel(const double* __restrict__ G, const double* __restrict__ T, int64_t tstride, int nt, int64_t n,
-                double* __restrict__ partials, double* __restrict__ out, FoeScalars* sc) {
+foe_dots_kernel(const double* G, const double* T, int64_t tstride, int nt, int64_t n,
+                double* partials, double* out, FoeScalars* sc) {
+  chain_wait();
+  chain_next();
   __shared__ double red[8][8];
   __shared__ double tot[8];
   __shared__ bool last;
@@ -381,7 +397,9 @@ foe_dots_kernel(const double* __restrict__ G, const double* __restrict__ T, int6
 // Frobenius products ip[m q + j] = <T_{qm}, T_j> (j = 0: tr T_{qm}):
 // tr T_{qm+j} = 2 ip[m q + j] - tr T_{qm-j}. One CTA; a block m needs block m - 1.
 __global__ void __launch_bounds__(128)
-foe_ps_traces_kernel(double* traces, const double* __restrict__ ip, int q, int M, int64_t n) {
+foe_ps_traces_kernel(double* traces, const double* ip, int q, int M, int64_t n) {
+  chain_wait();
+  chain_next();
   if (threadIdx.x == 0) traces[0] = static_cast<double>(n);
   __syncthreads();
   for (int m = 1; q * m < M; ++m) {
@@ -395,7 +413,9 @@ foe_ps_traces_kernel(double* traces, const double* __restrict__ ip, int q, int M
 // a_k = c_k (a_0 = c_0 / 2, zero past M), folded from the top block down
 // (T_{qm+j} = 2 T_m(y) T_j - T_{qm-j}). One CTA; a holds r q doubles.
 __global__ void __launch_bounds__(128)
-foe_fold_kernel(const double* __restrict__ coeffs, int M, int q, int r, double* a, double* __restrict__ w) {
+foe_fold_kernel(const double* coeffs, int M, int q, int r, double* a, double* w) {
+  chain_wait();
+  chain_next();
   for (int k = threadIdx.x; k < r * q; k += blockDim.x) a[k] = k == 0 ? 0.5 * coeffs[0] : (k < M ? coeffs[k] : 0.0);
   __syncthreads();
   for (int m = r - 1; m > 0; --m) {
@@ -433,14 +453,14 @@ cudaError_t launch_foe_coefficients(FoeScalars* sc, double kT, double mu, double
   const int rounds = canonical ? (kMuHalvings + kMuLevels - 1) / kMuLevels : 0;
   MuRound* ws = reinterpret_cast<MuRound*>(coeffs);  // written by the last kernel only
   if (canonical) {
-    foe_weights_kernel<<<static_cast<unsigned>(N), kSumThreads, 0, st>>>(sc, traces, M, w, gx);
+    launch_chained(foe_weights_kernel, static_cast<unsigned>(N), kSumThreads, st, sc, traces, M, w, gx);
     for (int r = 0; r < rounds; ++r)
-      foe_mu_round_kernel<<<kMuNodes, kSumThreads, 0, st>>>(sc, kT, n_occ, M, w, gx, r, ws);
+      launch_chained(foe_mu_round_kernel, kMuNodes, kSumThreads, st, sc, kT, n_occ, M, w, gx, r, ws);
     count_launch(1 + rounds);
   }
-  foe_occupation_kernel<<<static_cast<unsigned>((N + kSumThreads - 1) / kSumThreads), kSumThreads, 0, st>>>(
+  launch_chained(foe_occupation_kernel, static_cast<unsigned>((N + kSumThreads - 1) / kSumThreads), kSumThreads, st,
       sc, kT, mu, n_occ, rounds, M, ws, gx, gx);
-  foe_coeff_kernel<<<static_cast<unsigned>(M), kSumThreads, 0, st>>>(gx, M, coeffs);
+  launch_chained(foe_coeff_kernel, static_cast<unsigned>(M), kSumThreads, st, gx, M, coeffs);
   count_launch(2);
   return cudaGetLastError();
 }
@@ -450,7 +470,7 @@ cudaError_t launch_foe_init(const double* H, int64_t ldh, int64_t n, const FoeSc
   ProfScope prof(DMP_PROF_OTHER, st);
   int T;
   const int blocks = upper_blocks(n, T);
-  foe_init_kernel<<<blocks, 256, 0, st>>>(H, ldh, n, sc, coeffs, Hs, T0, T1, P, ldp, T);
+  launch_chained(foe_init_kernel, blocks, 256, st, H, ldh, n, sc, coeffs, Hs, T0, T1, P, ldp, T);
   count_launch();
   return cudaGetLastError();
 }
@@ -460,7 +480,7 @@ cudaError_t launch_foe_combine(const double* T, int nt, const double* w, const d
   ProfScope prof(DMP_PROF_OTHER, st);
   int blocks_T;
   const int blocks = upper_blocks(n, blocks_T);
-  foe_combine_kernel<<<blocks, 256, 0, st>>>(T, n * n, nt, w, Y, alpha, Bm2, out, ldo, n, blocks_T);
+  launch_chained(foe_combine_kernel, blocks, 256, st, T, n * n, nt, w, Y, alpha, Bm2, out, ldo, n, blocks_T);
   count_launch();
   return cudaGetLastError();
 }
@@ -470,28 +490,28 @@ cudaError_t launch_foe_dots(const double* G, const double* T, int nt, int64_t n,
   if (nt < 1) return cudaSuccess;
   ProfScope prof(DMP_PROF_MEASURE, st);
   const dim3 grid(kFoeDotBlocks, static_cast<unsigned>(std::max(1, (nt - 1 + kDotTerms - 1) / kDotTerms)));
-  foe_dots_kernel<<<grid, 256, 0, st>>>(G, T, n * n, nt, n, partials, out, sc);
+  launch_chained(foe_dots_kernel, grid, 256, st, G, T, n * n, nt, n, partials, out, sc);
   count_launch();
   return cudaGetLastError();
 }
 
 cudaError_t launch_foe_ps_traces(double* traces, const double* ip, int q, int M, int64_t n, cudaStream_t st) {
   ProfScope prof(DMP_PROF_MEASURE, st);
-  foe_ps_traces_kernel<<<1, 128, 0, st>>>(traces, ip, q, M, n);
+  launch_chained(foe_ps_traces_kernel, 1, 128, st, traces, ip, q, M, n);
   count_launch();
   return cudaGetLastError();
 }
 
 cudaError_t launch_foe_fold(const double* coeffs, int M, int q, int r, double* a, double* w, cudaStream_t st) {
   ProfScope prof(DMP_PROF_INIT, st);
-  foe_fold_kernel<<<1, 128, 0, st>>>(coeffs, M, q, r, a, w);
+  launch_chained(foe_fold_kernel, 1, 128, st, coeffs, M, q, r, a, w);
   count_launch();
   return cudaGetLastError();
 }
 
 cudaError_t launch_foe_trace(const double* A, int64_t lda, int64_t n, double* out, cudaStream_t st) {
   ProfScope prof(DMP_PROF_MEASURE, st);
-  foe_trace_kernel<<<1, kReduceThreads, 0, st>>>(A, lda, 0, n, out);
+  launch_chained(foe_trace_kernel, 1, kReduceThreads, st, A, lda, 0, n, out);
   count_launch();
   return cudaGetLastError();
 }
@@ -499,7 +519,7 @@ cudaError_t launch_foe_trace(const double* A, int64_t lda, int64_t n, double* ou
 cudaError_t launch_foe_traces(const double* T, int count, int64_t n, double* out, cudaStream_t st) {
   if (count <= 0) return cudaSuccess;
   ProfScope prof(DMP_PROF_MEASURE, st);
-  foe_trace_kernel<<<static_cast<unsigned>(count), kReduceThreads, 0, st>>>(T, n, n * n, n, out);
+  launch_chained(foe_trace_kernel, static_cast<unsigned>(count), kReduceThreads, st, T, n, n * n, n, out);
   count_launch();
   return cudaGetLastError();
 }

@@ -503,7 +503,7 @@ __device__ __forceinline__ Job job_of(const TcParams& p, const CUtensorMap* tmA,
 
 // Four consecutive doubles or int64 group sums, in 16-byte pieces when the
 // address allows (`vec`), else one by one at immediate offsets.
-__device__ __forceinline__ void load4(double (&v)[4], const double* __restrict__ a, bool vec) {
+__device__ __forceinline__ void load4(double (&v)[4], const double* a, bool vec) {
   if (vec) {
     const double2 x = reinterpret_cast<const double2*>(a)[0], y = reinterpret_cast<const double2*>(a)[1];
     v[0] = x.x, v[1] = x.y, v[2] = y.x, v[3] = y.y;
@@ -539,6 +539,8 @@ enum { OUT_STORE = 0, OUT_UPDATE = 1, OUT_CHEB = 2 };  // EPI_STORE and EPI_SYM_
 template <int BN, bool PAIR, int OUT, int NG>
 __global__ void __launch_bounds__(FIN_THREADS)
 ozaki_finish_kernel(const __grid_constant__ TcParams p) {
+  chain_wait();
+  chain_next();
   constexpr bool UPD = OUT == OUT_UPDATE, CHEB = OUT == OUT_CHEB;
   __shared__ double trans[32][33];
   using Cfg = TcCfg<BN, PAIR>;
@@ -829,7 +831,6 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
 ozaki_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                 const __grid_constant__ TcParams p) {
   using Cfg = TcCfg<BN, PAIR, F8>;
-  if (p.done != nullptr && *p.done) return;  // uniform: the whole CTA leaves before any setup
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const uint32_t sbase = smem_u32(smem);
@@ -892,12 +893,17 @@ ozaki_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
   if (PAIR) cluster_sync();  // barriers of both CTAs initialised before any remote use
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  // the setup above touches no device memory; a set done flag leaves the CTA without tiles
+  // (the grouped walk looks at each matrix's own flag)
+  chain_wait();
+  chain_next();
+  const int done = p.done != nullptr ? *p.done : 0;
 
   const int CHS = p.CH;  // stages per fp32 chunk
 
   // WALK 0: this CTA's items. Items 0 .. nfull - 1 are whole tiles; after them
   // come the tiles its range [u_begin, u_end) of the split tiles' units meets.
-  const int nfull = p.nwhole > cta_id ? (p.nwhole - cta_id - 1) / cta_stride + 1 : 0;
+  const int nfull = !done && p.nwhole > cta_id ? (p.nwhole - cta_id - 1) / cta_stride + 1 : 0;
   // (u_end - u_begin units of the sequence of the tiles' units seg_off .. seg_off + seg_len - 1)
   const int nsplit = p.ntiles - p.nwhole;
   const int heads = nsplit * p.heads;
@@ -916,6 +922,7 @@ ozaki_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     u_begin = all * (cta_id - heads) / max(cta_stride - heads, 1);
     u_end = all * (cta_id - heads + 1) / max(cta_stride - heads, 1);
   }
+  if (done) u_end = u_begin;
   // item `it`: its tile (counted from tile0) and unit range [u0, u1); false past the last
   auto static_item = [&](int it, int& tile, int& u0, int& u1) __attribute__((always_inline)) -> bool {
     if (it < nfull) {
@@ -1462,8 +1469,8 @@ cudaError_t set_smem_attr() {
 template <int BN, bool PAIR, bool F8>
 struct TcLaunch {
   cudaLaunchConfig_t cfg;
-  cudaLaunchAttribute at[1];
-  TcLaunch(int grid, cudaStream_t st) {
+  cudaLaunchAttribute at[2];
+  TcLaunch(int grid, cudaStream_t st, bool chained = false) {
     std::memset(&cfg, 0, sizeof(cfg));
     std::memset(at, 0, sizeof(at));
     cfg.gridDim = dim3(static_cast<unsigned>(grid));
@@ -1474,22 +1481,31 @@ struct TcLaunch {
     at[0].val.clusterDim.x = PAIR ? 2 : 1;
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = chained ? 2 : 1;
   }
 };
 
 template <int BN, bool PAIR, int OUT>
 void launch_finish(const TcParams& p, cudaStream_t st) {
   const int grid = p.ntiles * (TcCfg<BN, PAIR>::BM / 32) * (BN / 32);
+  auto launch = [&](void (*kernel)(TcParams)) {
+    if (p.mats == nullptr) {
+      launch_chained(kernel, grid, FIN_THREADS, st, p);
+    } else {
+      kernel<<<grid, FIN_THREADS, 0, st>>>(p);
+    }
+  };
   if (OUT == OUT_STORE && p.mats == nullptr && p.epi.kind == EPI_LEVELS) {
-    ozaki_finish_kernel<BN, PAIR, OUT_STORE, 0><<<grid, FIN_THREADS, 0, st>>>(p);
+    launch(ozaki_finish_kernel<BN, PAIR, OUT_STORE, 0>);
   } else if (p.prog.ng == 1) {
-    ozaki_finish_kernel<BN, PAIR, OUT, 1><<<grid, FIN_THREADS, 0, st>>>(p);
+    launch(ozaki_finish_kernel<BN, PAIR, OUT, 1>);
   } else if (p.prog.ng == 2) {
-    ozaki_finish_kernel<BN, PAIR, OUT, 2><<<grid, FIN_THREADS, 0, st>>>(p);
+    launch(ozaki_finish_kernel<BN, PAIR, OUT, 2>);
   } else {
-    ozaki_finish_kernel<BN, PAIR, OUT, 3><<<grid, FIN_THREADS, 0, st>>>(p);
+    launch(ozaki_finish_kernel<BN, PAIR, OUT, 3>);
   }
 }
 
@@ -1498,7 +1514,7 @@ template <int BN, bool PAIR = false, bool F8 = false, int WALK = 0>
 cudaError_t launch_tc_impl(const CUtensorMap& ta, const CUtensorMap& tb, const TcParams& p, int grid, cudaStream_t st) {
   cudaError_t e = set_smem_attr<BN, PAIR, F8, WALK>();
   if (e != cudaSuccess) return e;
-  TcLaunch<BN, PAIR, F8> l(grid, st);
+  TcLaunch<BN, PAIR, F8> l(grid, st, p.mats == nullptr);  // (a batch's products are captured in a graph's loop)
   e = cudaLaunchKernelEx(&l.cfg, ozaki_tc_kernel<BN, PAIR, F8, WALK>, ta, tb, p);
   if (e != cudaSuccess) return e;
   const int kind = p.mats != nullptr ? (p.phase != 0 ? EPI_PM_UPDATE : EPI_SYM_STORE) : p.epi.kind;

@@ -197,8 +197,10 @@ __global__ void p0_kernel(const double* __restrict__ H, int64_t n, int64_t ldh, 
 // SP2 / TRS4: 30 to 24).
 template <int NQ>
 __global__ void __launch_bounds__(256)
-measure_kernel(const double* __restrict__ P, int64_t ldp, const double* __restrict__ X2, int64_t ldx,
-               const double* __restrict__ H, int64_t ldh, int64_t n, double* __restrict__ part, PurifyState* st) {
+measure_kernel(const double* P, int64_t ldp, const double* X2, int64_t ldx,
+               const double* H, int64_t ldh, int64_t n, double* part, PurifyState* st) {
+  chain_wait();
+  chain_next();
   if (st->done) return;
   bool four = false;
   double d_xx = 0.0, a_xx[4] = {0.0, 0.0, 0.0, 0.0};
@@ -314,7 +316,9 @@ dim3 elem_grid(int64_t n) {
 
 // X <- alpha X + b2 X2 (step_kind 0), over the full n x n
 __global__ void __launch_bounds__(256)
-axpby_kernel(double* X, int64_t ldx, const double* __restrict__ X2, int64_t ldx2, int64_t n, const PurifyState* st) {
+axpby_kernel(double* X, int64_t ldx, const double* X2, int64_t ldx2, int64_t n, const PurifyState* st) {
+  chain_wait();
+  chain_next();
   if (st->done != 0 || st->step_kind != 0) return;
   const double a = st->alpha, b = st->b2;
   const bool r32 = st->store32 != 0;
@@ -337,8 +341,10 @@ axpby_kernel(double* X, int64_t ldx, const double* __restrict__ X2, int64_t ldx2
 
 // Z = zd I + zx X + zx2 X2 (the TRS4 factor with F + gamma G = X2 Z; step_kind 1)
 __global__ void __launch_bounds__(256)
-trs4_z_kernel(const double* __restrict__ X, int64_t ldx, const double* __restrict__ X2, int64_t ldx2,
-              double* __restrict__ out, int64_t ldo, int64_t n, const PurifyState* st) {
+trs4_z_kernel(const double* X, int64_t ldx, const double* X2, int64_t ldx2,
+              double* out, int64_t ldo, int64_t n, const PurifyState* st) {
+  chain_wait();
+  chain_next();
   if (st->no_product != 0) return;
   const double zd = st->zd, zx = st->zx, zx2 = st->zx2;
   const bool r32 = st->store32 != 0;
@@ -426,7 +432,7 @@ unsigned measure_blocks(int64_t n) { return static_cast<unsigned>(std::min<int64
 cudaError_t launch_measure_variant(const double* X, int64_t ldx, const double* X2, int64_t ldx2, const double* H,
                                    int64_t ldh, int64_t n, double* partials, PurifyState* state, cudaStream_t st) {
   ProfScope prof(DMP_PROF_MEASURE, st);
-  measure_kernel<10><<<measure_blocks(n), 256, 0, st>>>(X, ldx, X2, ldx2, H, ldh, n, partials, state);
+  launch_chained(measure_kernel<10>, measure_blocks(n), 256, st, X, ldx, X2, ldx2, H, ldh, n, partials, state);
   count_launch();
   return cudaGetLastError();
 }
@@ -434,7 +440,7 @@ cudaError_t launch_measure_variant(const double* X, int64_t ldx, const double* X
 cudaError_t launch_axpby(double* X, int64_t ldx, const double* X2, int64_t ldx2, int64_t n, const PurifyState* state,
                          cudaStream_t st) {
   ProfScope prof(DMP_PROF_OTHER, st);
-  axpby_kernel<<<elem_grid(n), 256, 0, st>>>(X, ldx, X2, ldx2, n, state);
+  launch_chained(axpby_kernel, elem_grid(n), 256, st, X, ldx, X2, ldx2, n, state);
   count_launch();
   return cudaGetLastError();
 }
@@ -442,7 +448,7 @@ cudaError_t launch_axpby(double* X, int64_t ldx, const double* X2, int64_t ldx2,
 cudaError_t launch_trs4_z(const double* X, int64_t ldx, const double* X2, int64_t ldx2, double* out, int64_t ldo,
                           int64_t n, const PurifyState* state, cudaStream_t st) {
   ProfScope prof(DMP_PROF_OTHER, st);
-  trs4_z_kernel<<<elem_grid(n), 256, 0, st>>>(X, ldx, X2, ldx2, out, ldo, n, state);
+  launch_chained(trs4_z_kernel, elem_grid(n), 256, st, X, ldx, X2, ldx2, out, ldo, n, state);
   count_launch();
   return cudaGetLastError();
 }
@@ -491,7 +497,7 @@ cudaError_t launch_measure(const double* P, int64_t ldp, const double* X2, int64
                            const double* H, int64_t ldh, int64_t n, double* partials,
                            PurifyState* state, cudaStream_t st) {
   ProfScope prof(DMP_PROF_MEASURE, st);
-  measure_kernel<8><<<measure_blocks(n), 256, 0, st>>>(P, ldp, X2, ldx, H, ldh, n, partials, state);
+  launch_chained(measure_kernel<8>, measure_blocks(n), 256, st, P, ldp, X2, ldx, H, ldh, n, partials, state);
   count_launch();
   return cudaGetLastError();
 }

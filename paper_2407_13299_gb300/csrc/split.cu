@@ -260,7 +260,7 @@ __device__ __forceinline__ int row_exponent(uint32_t mxh, uint32_t mxl) {
 }
 
 // Entries j, j + 1 of the row (zero past k or for a padding row).
-__device__ __forceinline__ double2 load_pair(const double* __restrict__ row, int j, int k, bool live, bool vec) {
+__device__ __forceinline__ double2 load_pair(const double* row, int j, int k, bool live, bool vec) {
   if (live && vec && j + 1 < k) return *reinterpret_cast<const double2*>(row + j);
   double2 v;
   v.x = (live && j < k) ? row[j] : 0.0;
@@ -285,9 +285,9 @@ __device__ __forceinline__ void max_bits(double a, uint32_t& mxh, uint32_t& mxl,
 // pairs each per sweep of 2 kPairs THREADS entries).
 // DIFF (S > 0, bf16-held beta 7 digits): the difference planes too.
 template <int KIND, int BETA, int S = 0, int THREADS = kSplitThreads, bool DIFF = false>
-__device__ __forceinline__ void split_one_row(const double* __restrict__ A, int64_t r, int64_t m, int k,
-                                              int64_t lda, int s_arg, int32_t* __restrict__ exps,
-                                              void* __restrict__ planes, int k_pad, int64_t plane_stride,
+__device__ __forceinline__ void split_one_row(const double* A, int64_t r, int64_t m, int k,
+                                              int64_t lda, int s_arg, int32_t* exps,
+                                              void* planes, int k_pad, int64_t plane_stride,
                                               int* flag) {
   constexpr bool kNearest = BETA != 7;
   constexpr int kSweep = 2 * kPairs * THREADS;
@@ -379,9 +379,11 @@ __device__ __forceinline__ void split_one_row(const double* __restrict__ A, int6
 // 128; n = 2048 with difference planes 33 and 21).
 template <int KIND, int BETA, int S, bool DIFF, int THREADS>
 __global__ void __launch_bounds__(THREADS, 1024 / THREADS)
-split_rows_kernel(const double* __restrict__ A, int64_t m, int64_t k, int64_t lda, int s,
-                  int32_t* __restrict__ exps, void* __restrict__ planes, int64_t k_pad,
+split_rows_kernel(const double* A, int64_t m, int64_t k, int64_t lda, int s,
+                  int32_t* exps, void* planes, int64_t k_pad,
                   int64_t plane_stride, int* flag, const int* done) {
+  chain_wait();
+  chain_next();
   if (done != nullptr && *done) return;
   split_one_row<KIND, BETA, S, THREADS, DIFF>(A, blockIdx.x, m, static_cast<int>(k), lda, s, exps, planes,
                                               static_cast<int>(k_pad), plane_stride, flag);
@@ -395,8 +397,8 @@ void launch_split_s(dim3 grid, cudaStream_t st, const double* A, int64_t m, int6
                     int32_t* exps, void* planes, int64_t k_pad, int64_t plane_stride, int* flag, const int* done) {
   auto launch = [&](auto threads) {
     constexpr int T = decltype(threads)::value;
-    split_rows_kernel<KIND, BETA, S, DIFF, T><<<grid, T, 0, st>>>(A, m, k, lda, s, exps, planes, k_pad, plane_stride,
-                                                                  flag, done);
+    launch_chained(split_rows_kernel<KIND, BETA, S, DIFF, T>, grid, T, st, A, m, k, lda, s, exps, planes, k_pad,
+                   plane_stride, flag, done);
   };
   if (k_pad <= 2 * kPairs * 128) {
     launch(std::integral_constant<int, 128>());
@@ -450,8 +452,10 @@ split_grouped_kernel(const BatchMat* __restrict__ mats, const int64_t* __restric
                                                      static_cast<int>(M.k_pad), M.n_pad * M.k_pad, nullptr);
 }
 
-__global__ void transpose_kernel(const double* __restrict__ A, int64_t m, int64_t n, int64_t lda,
-                                 double* __restrict__ At) {
+__global__ void transpose_kernel(const double* A, int64_t m, int64_t n, int64_t lda,
+                                 double* At) {
+  chain_wait();
+  chain_next();
   __shared__ double tile[32][33];
   const int64_t bx = static_cast<int64_t>(blockIdx.x) * 32;  // column block of A
   const int64_t by = static_cast<int64_t>(blockIdx.y) * 32;  // row block of A
@@ -500,7 +504,7 @@ cudaError_t launch_transpose(const double* A, int64_t m, int64_t n, int64_t lda,
   if (m <= 0 || n <= 0) return cudaSuccess;
   dim3 grid(static_cast<unsigned>((n + 31) / 32), static_cast<unsigned>((m + 31) / 32));
   ProfScope prof(DMP_PROF_OTHER, st);
-  transpose_kernel<<<grid, dim3(32, 8), 0, st>>>(A, m, n, lda, At);
+  launch_chained(transpose_kernel, grid, dim3(32, 8), st, A, m, n, lda, At);
   count_launch();
   return cudaGetLastError();
 }
