@@ -165,7 +165,7 @@ int64_t row_pad(int executor) { return executor == DMP_EXEC_TC ? 256 : kTileM; }
 size_t area_bytes(const Opts& o) {
   return o.mode != DMP_FP64 && o.executor == DMP_EXEC_TC ? tc_area_bytes() : 0;
 }
-TcArea area_at(const Opts& o, void* ws, size_t off) { return TcArea{static_cast<char*>(ws) + off, area_bytes(o), 0}; }
+TcArea area_at(const Opts& o, void* ws, size_t off) { return TcArea{static_cast<char*>(ws) + off, area_bytes(o), 0, 0}; }
 
 // ---------------------------------------------------------------- dm_purify layout
 struct PurifyLayout {
@@ -501,11 +501,10 @@ int dm_purify(const double* H, int64_t n, int64_t ldh, int64_t n_occ, const dmp_
     DMP_CUDA(reader.mark());
     PurifyState now;
     if (o.method != DMP_METHOD_PM) {
-      // SP2 / TRS4 (the step's kind and weights are on the device): elementwise, in place
-      DMP_CUDA(launch_axpby(cur, ldcur, X2, n, n, state, st));
+      // SP2 / TRS4 (the step's kind and weights are on the device): elementwise, in
+      // place, or X' = X2 Z: Z into alt, then the symmetric product written over X
+      DMP_CUDA(launch_variant_step(cur, ldcur, X2, n, alt, ldalt, n, state, st));
       if (o.method == DMP_METHOD_TRS4) {
-        // or X' = X2 Z: Z into alt, then the symmetric product written over X
-        DMP_CUDA(launch_trs4_z(cur, ldcur, X2, n, alt, ldalt, n, state, st));
         const int* skip = &state->no_product;
         EpiArgs ez{};
         ez.kind = EPI_SYM_STORE;
@@ -718,10 +717,10 @@ GemmLayout gemm_layout(int64_t m, int64_t n, int64_t k, const Opts& o) {
   const size_t planes = static_cast<size_t>(planes_of(o, o.s));
   G.ea = c.take(G.m_pad * sizeof(int32_t));
   G.eb = c.take(G.n_pad * sizeof(int32_t));
-  G.err = c.take(sizeof(int32_t));
   G.pa = c.take(planes * G.m_pad * G.k_pad * elem_bytes(o));
   G.pb = c.take(planes * G.n_pad * G.k_pad * elem_bytes(o));
   G.Bt = c.take(static_cast<size_t>(n) * k * sizeof(double));
+  G.err = c.take(sizeof(int32_t));  // directly before the area: cleared with it
   G.area = c.take(area_bytes(o));
   G.total = c.cur;
   return G;
@@ -795,7 +794,7 @@ static int ozaki_common(int64_t m, int64_t n, int64_t k, const double* A, int64_
   DMP_CUDA(launch_transpose(B, k, n, ldb, Bt, st));
   DMP_CUDA(launch_split_rows(Bt, n, k, k, o.s, o.beta, eb, pb, G.n_pad, G.k_pad, elem_kind(o), diff, nullptr,
                              nullptr, st));
-  if (o.executor == DMP_EXEC_TC) DMP_CUDA(cudaMemsetAsync(err, 0, sizeof(int), st));
+  area.front = G.area - G.err;
   DMP_CUDA(launch_product(o, pa, pb, ea, eb, m, n, k, G.m_pad, G.n_pad, G.k_pad, 0, epi, nullptr, err, area, st));
   if (o.executor == DMP_EXEC_TC) {
     // report an expired device wait; skipped while the stream is being captured

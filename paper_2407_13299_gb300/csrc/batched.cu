@@ -355,7 +355,7 @@ int dm_purify_batched(int32_t batch, const double* const* H, const int64_t* n, c
   double* dpart = reinterpret_cast<double*>(at(ws, L.partials));
   int* derr = reinterpret_cast<int*>(at(ws, L.err));
   int* dcounter = reinterpret_cast<int*>(at(ws, L.counter));
-  TcArea area{at(ws, L.area), tc_area_bytes(), 0};
+  TcArea area{at(ws, L.area), tc_area_bytes(), 0, 0};
   const int64_t nmax_idx = std::max_element(n, n + batch) - n;
   const int64_t nmax = n[nmax_idx];
 

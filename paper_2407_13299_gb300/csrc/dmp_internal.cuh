@@ -198,6 +198,7 @@ constexpr int kTcMaxCtas = 160;
 struct TcArea {
   void* ptr;
   size_t bytes, clean;
+  size_t front;  // bytes before ptr that the first clearing takes along
 };
 size_t tc_area_bytes();
 // zeroes the first `bytes` of the area as far as they are not known to be zero
@@ -233,15 +234,13 @@ cudaError_t launch_refine_weights(PurifyState* state, cudaStream_t st);
 cudaError_t launch_energy(const double* P, int64_t ldp, const double* H, int64_t ldh, int64_t n, double* partials,
                           PurifyState* state, cudaStream_t st);
 // SP2 / TRS4: measures with tr X^4 and variant_decide; the elementwise step
-// X <- alpha X + b2 X2 (a step of kind 0, else nothing); the TRS4 factor
-// Z = zd I + zx X + zx2 X2 (a step of kind 1, else nothing); weights from the
-// state; full n x n, so the results are exactly symmetric as X and X2 are).
+// X <- alpha X + b2 X2 (a step of kind 0), or the TRS4 factor Z = zd I + zx X +
+// zx2 X2 (kind 1); weights from the state; full n x n, so the results are
+// exactly symmetric as X and X2 are.
 cudaError_t launch_measure_variant(const double* X, int64_t ldx, const double* X2, int64_t ldx2, const double* H,
                                    int64_t ldh, int64_t n, double* partials, PurifyState* state, cudaStream_t st);
-cudaError_t launch_axpby(double* X, int64_t ldx, const double* X2, int64_t ldx2, int64_t n, const PurifyState* state,
-                         cudaStream_t st);
-cudaError_t launch_trs4_z(const double* X, int64_t ldx, const double* X2, int64_t ldx2, double* out, int64_t ldo,
-                          int64_t n, const PurifyState* state, cudaStream_t st);
+cudaError_t launch_variant_step(double* X, int64_t ldx, const double* X2, int64_t ldx2, double* Z, int64_t ldz,
+                                int64_t n, const PurifyState* state, cudaStream_t st);
 cudaError_t launch_measure(const double* P, int64_t ldp, const double* X2, int64_t ldx,
                            const double* H, int64_t ldh, int64_t n, double* partials,
                            PurifyState* state, cudaStream_t st);

@@ -1593,7 +1593,8 @@ int set_tc_split_tiles(int enable) {
 // to them: cleared here once per call, by the finish kernel after that.
 cudaError_t tc_area_clear(TcArea& a, size_t bytes, cudaStream_t st) {
   if (bytes <= a.clean) return cudaSuccess;
-  const cudaError_t e = cudaMemsetAsync(static_cast<char*>(a.ptr) + a.clean, 0, bytes - a.clean, st);
+  const size_t front = a.clean == 0 ? a.front : 0;
+  const cudaError_t e = cudaMemsetAsync(static_cast<char*>(a.ptr) + a.clean - front, 0, bytes - a.clean + front, st);
   if (e == cudaSuccess) a.clean = bytes;
   return e;
 }

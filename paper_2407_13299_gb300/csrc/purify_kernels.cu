@@ -305,22 +305,28 @@ measure_kernel(const double* P, int64_t ldp, const double* X2, int64_t ldx,
   }
 }
 
-// The elementwise steps below return at once unless the measured state asks for
-// them: both are enqueued before the host knows which it is. A block holds up to
-// 1024 entries of a row, four per thread, whose loads do not wait for one another.
+// The elementwise half of an SP2 / TRS4 step, enqueued before the host knows the
+// step's kind: X <- alpha X + b2 X2 in place (kind 0), or the TRS4 factor
+// Z = zd I + zx X + zx2 X2 of F + gamma G = X2 Z (kind 1), over the full n x n. A
+// block holds up to 1024 entries of a row, four per thread, whose loads do not
+// wait for one another (n = 999: 11 us; 20 with a loop over rows and entries, and
+// 4 more for a second kernel that finds that the step is of the other kind).
 constexpr int kElemCols = 1024;
 
 dim3 elem_grid(int64_t n) {
   return dim3(static_cast<unsigned>((n + kElemCols - 1) / kElemCols), static_cast<unsigned>(std::min<int64_t>(n, 65535)));
 }
 
-// X <- alpha X + b2 X2 (step_kind 0), over the full n x n
 __global__ void __launch_bounds__(256)
-axpby_kernel(double* X, int64_t ldx, const double* X2, int64_t ldx2, int64_t n, const PurifyState* st) {
+variant_step_kernel(double* X, int64_t ldx, const double* X2, int64_t ldx2, double* Z, int64_t ldz, int64_t n,
+                    const PurifyState* st) {
   chain_wait();
   chain_next();
-  if (st->done != 0 || st->step_kind != 0) return;
-  const double a = st->alpha, b = st->b2;
+  if (st->done != 0) return;
+  const bool product = st->step_kind != 0;
+  const double a = product ? st->zx : st->alpha, b = product ? st->zx2 : st->b2, d = st->zd;
+  double* out = product ? Z : X;
+  const int64_t ldo = product ? ldz : ldx;
   const bool r32 = st->store32 != 0;
   const int64_t j0 = static_cast<int64_t>(blockIdx.x) * kElemCols + threadIdx.x;
   for (int64_t i = blockIdx.y; i < n; i += gridDim.y) {
@@ -334,34 +340,9 @@ axpby_kernel(double* X, int64_t ldx, const double* X2, int64_t ldx2, int64_t n, 
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       const int64_t j = j0 + 256 * u;
-      if (j < n) X[i * ldx + j] = stored_value(a * x[u] + b * y[u], r32);
-    }
-  }
-}
-
-// Z = zd I + zx X + zx2 X2 (the TRS4 factor with F + gamma G = X2 Z; step_kind 1)
-__global__ void __launch_bounds__(256)
-trs4_z_kernel(const double* X, int64_t ldx, const double* X2, int64_t ldx2,
-              double* out, int64_t ldo, int64_t n, const PurifyState* st) {
-  chain_wait();
-  chain_next();
-  if (st->no_product != 0) return;
-  const double zd = st->zd, zx = st->zx, zx2 = st->zx2;
-  const bool r32 = st->store32 != 0;
-  const int64_t j0 = static_cast<int64_t>(blockIdx.x) * kElemCols + threadIdx.x;
-  for (int64_t i = blockIdx.y; i < n; i += gridDim.y) {
-    double x[4], y[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int64_t j = j0 + 256 * u;
-      x[u] = j < n ? X[i * ldx + j] : 0.0;
-      y[u] = j < n ? X2[i * ldx2 + j] : 0.0;
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int64_t j = j0 + 256 * u;
-      const double v = zx * x[u] + zx2 * y[u];
-      if (j < n) out[i * ldo + j] = stored_value(j == i ? v + zd : v, r32);
+      double v = a * x[u] + b * y[u];
+      if (product && j == i) v += d;
+      if (j < n) out[i * ldo + j] = stored_value(v, r32);
     }
   }
 }
@@ -437,18 +418,10 @@ cudaError_t launch_measure_variant(const double* X, int64_t ldx, const double* X
   return cudaGetLastError();
 }
 
-cudaError_t launch_axpby(double* X, int64_t ldx, const double* X2, int64_t ldx2, int64_t n, const PurifyState* state,
-                         cudaStream_t st) {
+cudaError_t launch_variant_step(double* X, int64_t ldx, const double* X2, int64_t ldx2, double* Z, int64_t ldz,
+                                int64_t n, const PurifyState* state, cudaStream_t st) {
   ProfScope prof(DMP_PROF_OTHER, st);
-  launch_chained(axpby_kernel, elem_grid(n), 256, st, X, ldx, X2, ldx2, n, state);
-  count_launch();
-  return cudaGetLastError();
-}
-
-cudaError_t launch_trs4_z(const double* X, int64_t ldx, const double* X2, int64_t ldx2, double* out, int64_t ldo,
-                          int64_t n, const PurifyState* state, cudaStream_t st) {
-  ProfScope prof(DMP_PROF_OTHER, st);
-  launch_chained(trs4_z_kernel, elem_grid(n), 256, st, X, ldx, X2, ldx2, out, ldo, n, state);
+  launch_chained(variant_step_kernel, elem_grid(n), 256, st, X, ldx, X2, ldx2, Z, ldz, n, state);
   count_launch();
   return cudaGetLastError();
 }
