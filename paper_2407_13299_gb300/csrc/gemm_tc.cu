@@ -1762,12 +1762,18 @@ cudaError_t launch_ozaki_tc(const void* A, const void* B, const int32_t* ea, con
   // product, INT8 s = 5, pair / 128 x 128 / 128 x 64 tiles: n = 256 22.9 / 18.1 /
   // 16.1 us, n = 384 25.1 / 19.5 / 19.0, n = 512 27.7 / 21.5 / 25.5, n = 768 34.5 /
   // 30.4 / 34.4, n = 1024 41.0 / 42.7 / 52.2; the other modes alike.
+  // With a short K the adds outweigh the products on larger outputs as well, as
+  // long as the 128 x 128 tiles are one wave. 128 x 128 against pair tiles, us: 1000
+  // x 333 x 257 BF16 s = 6 31.6 / 43.6, 2000 x 700 x 128 INT8 s = 7 48 / 58, 1000 x
+  // 500 x 257 E4M3 s = 8 35.6 / 44; level at 1000 x 1000 x 257 INT8 52 / 50, behind
+  // at 900 x 900 x 300 E4M3 54 / 46 and 2500 x 1000 x 96 INT8 (160 tiles) 61 / 58.
   const int64_t tm = (m + 255) / 256, tn = (n + 255) / 256;
   const int64_t big_tiles = sym ? tn * (tn + 1) / 2 : tm * tn;
   if (pair && big_tiles <= 1)
     return f8 ? run_product<64, false, true>(A, B, k_pad, planes, p, area, st)
               : run_product<64, false, false>(A, B, k_pad, planes, p, area, st);
-  if (pair && big_tiles <= 6)
+  const bool short_k = !sym && big_tiles * k <= 4096 && ((m + 127) / 128) * ((n + 127) / 128) <= tc_max_ctas();
+  if (pair && (big_tiles <= 6 || short_k))
     return f8 ? run_product<128, false, true>(A, B, k_pad, planes, p, area, st)
               : run_product<128, false, false>(A, B, k_pad, planes, p, area, st);
   if (pair)
