@@ -506,18 +506,16 @@ const char* dmp_version(void);
  * counterpart in the paper. */
 int dmp_set_tc_pairing(int enable);
 
-/* Whether single-matrix DMP_EXEC_TC products split their output tiles when
- * they fill at most half a wave of the persistent kernel (one CTA, or CTA
- * pair, per SM): the tiles are then cut into units of one exact fp32 chunk and
- * shared out evenly over every CTA, so the idle part of the GPU works too
- * (n <= 2048 in the purification on GB300: 25-40 % less product time). The
- * partial level sums are
- * integers added at L2, so any split gives the same exact sums and the result
- * is bit-for-bit that of whole tiles. Used by dm_purify, dm_purify_backward and
- * dm_foe (their workspaces include the room it needs), with at most two level
- * groups (s <= 8 for beta 7 and 5, s <= 6 for beta 8); ozaki_gemm runs whole
- * tiles. On by default. Process-wide, read at each launch; returns the
- * previous setting. A performance knob with no counterpart in the paper. */
+/* Whether single-matrix DMP_EXEC_TC products split the output tiles of their
+ * last, partial wave (one CTA, or CTA pair, per SM): the tiles are cut into
+ * units of one exact fp32 chunk that all CTAs share, so no part of the GPU is
+ * idle while a few tiles are left (n = 256 in the purification on GB300: all
+ * of the product; n = 3000, 78 tiles on 76 pairs: half of it). The partial sums
+ * are integers added at L2, so any split gives the same exact sums and the
+ * result is bit-for-bit that of whole tiles. Used by every single-matrix call
+ * (their workspaces include the room it needs). On by default. Process-wide,
+ * read at each launch; returns the previous setting. A performance knob with
+ * no counterpart in the paper. */
 int dmp_set_tc_split_tiles(int enable);
 
 /* Tile shape of dm_purify_batched's grouped product: 0 (the default) lets the

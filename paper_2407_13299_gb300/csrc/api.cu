@@ -237,7 +237,7 @@ TapeLayout tape_layout(int64_t n, const Opts& o) {
 
 inline char* at(void* base, size_t off) { return static_cast<char*>(base) + off; }
 
-// dm_purify_backward workspace: six n x n matrices (G, G', Y, Z, YP, ZP), the
+// dm_purify_backward workspace: six n x n matrices (G, G', Y, W, V, U), the
 // recomputed iterates and squares of one checkpoint segment, and the split
 // buffers of one product.
 struct BackwardLayout {

@@ -14,8 +14,8 @@
 // Slice modes: INT8, BF16 (nearest 8-bit digits) and E4M3 (nearest 5-bit
 // digits, one-byte planes, 256-column tiles only).
 //
-// The autotuner picks the tile width (128 or 256 columns) by timing the P^2
-// product of the batch with both, and, when opts->slices is 0, the slice count:
+// The autotuner picks the tile shape (128 x 128 or 128 x 256 single CTAs, 256 x
+// 256 CTA pairs) by timing the P^2 product of the batch with each, and, when opts->slices is 0, the slice count:
 // the smallest s whose band energy on the largest matrix agrees with that of
 // s + 2 to the target (1e-8 relative, or opts->energy_tol when set). Choices are
 // cached per batch shape for the life of the process.

@@ -10,8 +10,9 @@
 // of such products is exact while every partial sum stays at most 2^24 in
 // magnitude; the K loop is therefore cut into chunks of 1024 (beta = 7 and 8:
 // 1024 * 128^2 = 2^24) or 8192 (beta = 5, where 65536 * 16^2 = 2^24 would do) K
-// elements. Each chunk lands in one of two TMEM accumulators; while the tensor core fills the other, eight epilogue warps
-// drain the finished one into exact int32 sums in registers.
+// elements. Each chunk lands in one of two TMEM accumulators; while the tensor
+// core fills the other, eight epilogue warps drain the finished one into exact
+// int32 sums in registers.
 //
 // A product runs as two kernels:
 //   ozaki_tc_kernel      the integer part. A program of slice-pair steps, cut
@@ -1708,7 +1709,8 @@ cudaError_t run_product(const void* A, const void* B, int64_t k_pad, int planes,
 
 cudaError_t launch_ozaki_tc(const void* A, const void* B, const int32_t* ea, const int32_t* eb, int64_t m,
                             int64_t n, int64_t k, int64_t rows_a, int64_t rows_b, int64_t k_pad, int s, int beta,
-                            bool diff, int sym, const EpiArgs& epi, const int* done, int* err, TcArea& area, cudaStream_t st) {
+                            bool diff, int sym, const EpiArgs& epi, const int* done, int* err, TcArea& area,
+                            cudaStream_t st) {
   if (m <= 0 || n <= 0) return cudaSuccess;
   const bool f8 = beta == 5;  // E4M3 nearest digits
   const int atom_k = f8 ? 128 : TC_BK;

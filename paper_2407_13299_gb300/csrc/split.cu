@@ -21,8 +21,9 @@
 // bfloat16 (beta 8).
 //
 // One CTA per row. Each thread loads pairs of adjacent entries (16-byte loads,
-// 512 contiguous bytes per warp) and keeps up to 8192 entries of the row in
-// registers, so the row is read from memory once: a max-reduction, then the
+// 512 contiguous bytes per warp) and keeps 16 entries of the row in registers
+// (128 to 512 threads by the row's length: rows of up to 8192 entries whole), so
+// the row is read from memory once: a max-reduction, then the
 // digits of the same registers go to every plane (4-byte stores of two bf16 or
 // 2-byte stores of two int8 digits per plane; nearest digits: four entries per
 // thread). Longer rows take further sweeps that read the rest of the row again.
@@ -44,7 +45,7 @@ constexpr int64_t kMaxRow = (int64_t{1} << 31) - 1 - kSweep;     // in-row offse
 
 // U = floor(|a| 2^(96 - e_row)) as w0 (bits 64..95), w1 (32..63), w2 (0..31).
 // |a| < 2^e_row for every finite entry, so U < 2^96; a row holding NaN/Inf has
-// e_row = 0 and its digits are never used (the epilogue writes NaN). With
+// e_row = 0 and its digits are never used (the product's output step writes NaN). With
 // m = mh 2^32 + ml the significand, U = m 2^t, t = E - 1075 - e_row + 96: word
 // i of U is the funnel shift by t mod 32 of words i - floor(t/32) - 1 and
 // i - floor(t/32) of m. Only 32-bit integer operations are used (64-bit integer
