@@ -502,16 +502,24 @@ def run_ours(args):
 
     # ---- roofline of the dominant kernel (the tcgen05 slice-pair product)
     peaks, peak_src = load_peaks()
-    # per product launch: p n^2 (n + 1) flops with p = s(s+1)/2 kept pairs (upper
-    # triangle with the diagonal, 2 k flops per output and pair). A purification
-    # of `iters` updates launches 2 iters + 1 loop products with s slices, and the
+    # per product: p n^2 (n + 1) flops (upper triangle with the diagonal, 2 k flops
+    # per output and plane product), p the products of digit planes that the
+    # tensor cores really form: the s(s+1)/2 kept pairs, or, where the INT8 mode
+    # multiplies digit differences (csrc/api.cu: has_diff), s - 1 squares, the two
+    # pairs with slice s and one product per difference. A purification of
+    # `iters` updates forms 2 iters + 1 loop products with s slices, and the
     # refinement step 2 more with its own slice count.
     def pairs(k):
         return k * (k + 1) // 2
+
+    def plane_products(k, md=mode):
+        if md != "int8" or args.executor != "tc" or not 4 <= k <= 9 or n < (1920 if k <= 6 else 2560):
+            return pairs(k)
+        return (k - 1) + 2 + sum(1 for i in range(1, k) for j in range(i + 1, k) if i + j <= k + 1)
     unit_flops = n * n * (n + 1)
     refined = bool(info.get("refined", 0))
-    per_step_flops = ((2 * info["iters"] + 1) * pairs(s) + (2 * pairs(refine) if refined and refine > 0 else 0)) * \
-        unit_flops
+    per_step_flops = ((2 * info["iters"] + 1) * plane_products(s) +
+                      (2 * plane_products(refine) if refined and refine > 0 else 0)) * unit_flops
     flops_per_launch = per_step_flops * args.steps / max(prod_n, 1)
     avg_launch_s = (prod_ms / 1e3) / max(prod_n, 1)
     achieved = flops_per_launch / avg_launch_s / 1e12
@@ -532,7 +540,9 @@ def run_ours(args):
                 "ozaki_imma_kernel",
                 "peak_source": (f"{peak_src} bf16 sustained x 2 (nominal fp8/bf16 ratio)" if f8 else
                                 f"{peak_src} bf16 sustained") + " (kernel timed inside a long step)",
-                "flops_per_launch": flops_per_launch, "avg_launch_ms": avg_launch_s * 1e3,
+                "flops_per_launch": flops_per_launch,
+                "plane_products": {str(k): plane_products(k) for k in mix},
+                "slice_pairs": {str(k): pairs(k) for k in mix}, "avg_launch_ms": avg_launch_s * 1e3,
                 "launches": prod_n,
                 "launch_mix": f"{2 * info['iters'] + 1} x s={s}" + (f" + 2 x s={refine}" if refined else "") +
                               " per purification"}
@@ -602,9 +612,9 @@ def run_ours(args):
         out = {"method": method, "mode": f"ozaki-{mode}", "target": target, "slices": cs, "refine_slices": cr,
                "value": a.elapsed_time(b) / 2e3, "unit": UNIT, "rel_energy_error": trel, "iters": ti["iters"]}
         if method == "pm" and args.executor == "tc" and t_n > 0:
-            # slice-pair flops of the two timed runs over their product launches
-            t_flops = 2 * ((2 * ti["iters"] + 1) * pairs(cs) + (2 * pairs(cr) if ti.get("refined") else 0)) * \
-                unit_flops
+            # flops of the two timed runs over their product launches
+            t_flops = 2 * ((2 * ti["iters"] + 1) * plane_products(cs, mode) +
+                           (2 * plane_products(cr, mode) if ti.get("refined") else 0)) * unit_flops
             rate = t_flops / (t_ms / 1e3) / 1e12
             tpeak = peak * (2.0 if mode == "e4m3" else 1.0)
             out["products"] = {"ms_per_purification": t_ms / 2, "launches": t_n, "achieved_tflops": rate,
@@ -704,7 +714,7 @@ def run_ours(args):
             occ_exact = fermi_occupations(h.e, fi["mu"], f_kT)
             E_f = float(np.sum(occ_exact * h.e))
             exact_rows = (Q_d[rows] * torch.as_tensor(occ_exact, device=dev)[None, :]) @ Q_d.T
-            f_flops = fi["products"] * pairs(f_slices) * unit_flops
+            f_flops = fi["products"] * plane_products(f_slices, "int8") * unit_flops
             return {"scheme": scheme, "value": a.elapsed_time(b) / 1e3, "unit": UNIT, "mu": fi["mu"],
                     "products": fi["products"], "tail": fi["tail"],
                     "trace_error": abs(fi["trace"] - float(np.sum(occ_exact))),
