@@ -12,8 +12,7 @@
 // the place of G P^2 and P G P. The result moves by 1 to 2 % of the products' own
 // error (which the forward's exceeds by far: the gradient's error stays the same
 // to three digits). For digits of fewer than 42 bits (E4M3 below 9 slices, INT8
-// below 6) that is over 1e-9 of the gradient, and the two products stay apart:
-// V = Y P and U = Y^T P, with V + U / 2 where V stands.
+// below 6) that is over 1e-9 of the gradient, and the two products stay apart.
 // and the new G is the symmetric part of g (the loss sees P only through
 // symmetric matrices, so the symmetric part carries every directional
 // derivative along symmetric perturbations).
@@ -153,7 +152,7 @@ adj_half_kernel(const double* Y, int64_t n, double* W, int T) {
 // is cp P + cx X2 + ci I. n = 1024: 20 us.
 __global__ void __launch_bounds__(256)
 adj_step_kernel(const double* G, const double* Y, const double* V,
-                const double* U, const double* P, const double* X2, int64_t n,
+                const double* P, const double* X2, int64_t n,
                 const AdjScalars* sc, double* Gn, int T) {
   chain_wait();
   chain_next();
@@ -169,8 +168,7 @@ adj_step_kernel(const double* G, const double* Y, const double* V,
   for (int y = y0; y < 32; y += 8) {
     if (j0 + y < n && i0 + x < n) {
       const int64_t ji = (j0 + y) * n + i0 + x;
-      const double v = U ? __fma_rn(0.5, U[ji], V[ji]) : V[ji];
-      low[y][x] = __fma_rn(b3, v, __dmul_rn(b2, Y[ji]));
+      low[y][x] = __fma_rn(b3, V[ji], __dmul_rn(b2, Y[ji]));
     }
   }
   __syncthreads();
@@ -183,8 +181,7 @@ adj_step_kernel(const double* G, const double* Y, const double* V,
     // G, P, X2 are symmetric; Y and V are not
     const double dc = __fma_rn(cp, P[ij], cx * X2[ij]);
     // one rounding order for both elements of a pair: G_new is symmetric to the last bit
-    const double vij = U ? __fma_rn(0.5, U[ij], V[ij]) : V[ij];
-    const double yv = __dadd_rn(__fma_rn(b3, vij, __dmul_rn(b2, Y[ij])), low[x][y0 + 8 * u]);
+    const double yv = __dadd_rn(__fma_rn(b3, V[ij], __dmul_rn(b2, Y[ij])), low[x][y0 + 8 * u]);
     v[u] = __fma_rn(a, G[ij], __dadd_rn(yv, dc));
     if (i == j) v[u] += ci;
     Gn[ij] = v[u];
@@ -197,6 +194,79 @@ adj_step_kernel(const double* G, const double* Y, const double* V,
 #pragma unroll
   for (int y = y0; y < 32; y += 8)
     if (j0 + y < n && i0 + x < n) Gn[(j0 + y) * n + i0 + x] = low[x][y];
+}
+
+// ---- the step with the two products apart (YP = G P^2, ZP = P G P, Z = Y^T).
+// With so few digits a last-bit difference in a step moves digits of the next
+// one, and the gradient by more than 1e-9: the sums and the terms keep one order.
+
+// Partial sums over all elements, rows i = blockIdx.x + k gridDim.x:
+//   0: tr P   1: tr X2   2: <G, P>   3: <G, X2>   4: <Z, X2>
+__global__ void __launch_bounds__(256)
+adj_reduce_apart_kernel(const double* __restrict__ P, const double* __restrict__ X2, const double* __restrict__ G,
+                  const double* __restrict__ Z, int64_t n, double* __restrict__ part) {
+  double v[5] = {0, 0, 0, 0, 0};
+  for (int64_t i = blockIdx.x; i < n; i += gridDim.x) {
+    const int64_t o = i * n;
+    if (threadIdx.x == 0) {
+      v[0] += P[o + i];
+      v[1] += X2[o + i];
+    }
+    for (int64_t j = threadIdx.x; j < n; j += blockDim.x) {
+      const double p = P[o + j], x = X2[o + j];
+      v[2] += G[o + j] * p;
+      v[3] += G[o + j] * x;
+      v[4] += Z[o + j] * x;
+    }
+  }
+  __shared__ double red[8][5];
+#pragma unroll
+  for (int q = 0; q < 5; ++q) v[q] = warp_sum(v[q]);
+  if ((threadIdx.x & 31) == 0)
+#pragma unroll
+    for (int q = 0; q < 5; ++q) red[threadIdx.x >> 5][q] = v[q];
+  __syncthreads();
+  if (threadIdx.x < 5) {
+    double t = 0.0;
+    for (int w = 0; w < 8; ++w) t += red[w][threadIdx.x];
+    part[static_cast<int64_t>(blockIdx.x) * 5 + threadIdx.x] = t;
+  }
+}
+
+// The sums in block order, one thread each, and the step's scalars.
+__global__ void adj_scalars_kernel(const double* __restrict__ part, int nblocks, double c,
+                                   AdjScalars* __restrict__ out) {
+  __shared__ double s[5];
+  if (threadIdx.x < 5) {
+    double t = 0.0;
+#pragma unroll 8
+    for (int b = 0; b < nblocks; ++b) t += part[static_cast<int64_t>(b) * 5 + threadIdx.x];
+    s[threadIdx.x] = t;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) step_scalars(s, c, out);
+}
+
+// G_new = sym(g), one thread per element pair on the upper triangle.
+__global__ void adj_step_apart_kernel(const double* __restrict__ G, const double* __restrict__ Y,
+                                const double* __restrict__ YP, const double* __restrict__ ZP,
+                                const double* __restrict__ P, const double* __restrict__ X2, int64_t n,
+                                const AdjScalars* __restrict__ sc, double* __restrict__ Gn) {
+  const int64_t j = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+  const int64_t i = blockIdx.y;
+  if (j < i || j >= n) return;
+  const double a = sc->alpha, b2 = sc->b2, b3 = sc->b3;
+  const double td = sc->td, tn = sc->tn, k = sc->dLdc / (td * td);
+  const int64_t ij = i * n + j, ji = j * n + i;
+  const double dij = (i == j) ? 1.0 : 0.0;
+  // G, P, X2 are symmetric; Y, YP, ZP are not
+  const double dc = ((2.0 * P[ij] - 3.0 * X2[ij]) * td - tn * (dij - 2.0 * P[ij])) * k;
+  const double yy = Y[ij] + Y[ji];
+  const double gij = a * G[ij] + b2 * yy + b3 * (YP[ij] + ZP[ij] + YP[ji]) + dc;
+  const double gji = a * G[ij] + b2 * yy + b3 * (YP[ji] + ZP[ji] + YP[ij]) + dc;
+  const double v = 0.5 * (gij + gji);
+  Gn[ij] = v;
+  Gn[ji] = v;
 }
 
 // Symmetric part of a general n x n matrix (leading dimension ld) into dense out.
@@ -295,12 +365,27 @@ cudaError_t launch_adj_reduce(const double* P, const double* X2, const double* G
   return cudaGetLastError();
 }
 
-cudaError_t launch_adj_step(const double* G, const double* Y, const double* V, const double* U, const double* P,
-                            const double* X2, int64_t n, const AdjScalars* sc, double* Gn, cudaStream_t st) {
+cudaError_t launch_adj_step(const double* G, const double* Y, const double* V, const double* P, const double* X2,
+                            int64_t n, const AdjScalars* sc, double* Gn, cudaStream_t st) {
   ProfScope prof(DMP_PROF_OTHER, st);
   const int T = static_cast<int>((n + 31) / 32);
-  launch_chained(adj_step_kernel, T * (T + 1) / 2, 256, st, G, Y, V, U, P, X2, n, sc, Gn, T);
+  launch_chained(adj_step_kernel, T * (T + 1) / 2, 256, st, G, Y, V, P, X2, n, sc, Gn, T);
   count_launch();
+  return cudaGetLastError();
+}
+
+cudaError_t launch_adj_apart(const double* G, const double* Y, const double* Z, const double* YP, const double* ZP,
+                             const double* P, const double* X2, int64_t n, double* part, double c, AdjScalars* sc,
+                             double* Gn, cudaStream_t st) {
+  {
+    ProfScope prof(DMP_PROF_MEASURE, st);
+    adj_reduce_apart_kernel<<<kAdjBlocks, 256, 0, st>>>(P, X2, G, Z, n, part);
+    adj_scalars_kernel<<<1, 32, 0, st>>>(part, kAdjBlocks, c, sc);
+  }
+  ProfScope prof(DMP_PROF_OTHER, st);
+  dim3 grid(static_cast<unsigned>((n + 255) / 256), static_cast<unsigned>(n));
+  adj_step_apart_kernel<<<grid, 256, 0, st>>>(G, Y, YP, ZP, P, X2, n, sc, Gn);
+  count_launch(3);
   return cudaGetLastError();
 }
 

@@ -1012,13 +1012,14 @@ int dm_purify_backward(const double* H, int64_t n, int64_t n_occ, const dmp_opts
       if (merged) {
         DMP_CUDA(launch_adj_half(Y, n, W, st));
         DMP_CUDA(times_P(W, Pk, V));
+        DMP_CUDA(launch_adj_reduce(Pk, Xk, G, Y, n, part, ticket, cs[k], sc, st));
+        DMP_CUDA(launch_adj_step(G, Y, V, Pk, Xk, n, sc, Gn, st));
       } else {
-        DMP_CUDA(times_P(Y, Pk, V));
         DMP_CUDA(launch_transpose(Y, n, n, n, W, st));
-        DMP_CUDA(times_P(W, Pk, U));
+        DMP_CUDA(times_P(Y, Pk, V));  // G P^2
+        DMP_CUDA(times_P(W, Pk, U));  // P G P
+        DMP_CUDA(launch_adj_apart(G, Y, W, V, U, Pk, Xk, n, part, cs[k], sc, Gn, st));
       }
-      DMP_CUDA(launch_adj_reduce(Pk, Xk, G, Y, n, part, ticket, cs[k], sc, st));
-      DMP_CUDA(launch_adj_step(G, Y, V, merged ? nullptr : U, Pk, Xk, n, sc, Gn, st));
       std::swap(G, Gn);
     }
     int flag = 0;

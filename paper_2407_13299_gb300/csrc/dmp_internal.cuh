@@ -424,9 +424,12 @@ cudaError_t launch_adj_half(const double* Y, int64_t n, double* W, cudaStream_t 
 // *ticket is 0 between kernels.
 cudaError_t launch_adj_reduce(const double* P, const double* X2, const double* G, const double* Y, int64_t n,
                               double* part, int32_t* ticket, double c, AdjScalars* sc, cudaStream_t st);
-// U nullable: V + U / 2 in the place of V.
-cudaError_t launch_adj_step(const double* G, const double* Y, const double* V, const double* U, const double* P,
-                            const double* X2, int64_t n, const AdjScalars* sc, double* Gn, cudaStream_t st);
+cudaError_t launch_adj_step(const double* G, const double* Y, const double* V, const double* P, const double* X2,
+                            int64_t n, const AdjScalars* sc, double* Gn, cudaStream_t st);
+// The sums and the step with G P^2 and P G P apart (Z = Y^T).
+cudaError_t launch_adj_apart(const double* G, const double* Y, const double* Z, const double* YP, const double* ZP,
+                             const double* P, const double* X2, int64_t n, double* part, double c, AdjScalars* sc,
+                             double* Gn, cudaStream_t st);
 cudaError_t launch_sym_part(const double* A, int64_t ld, int64_t n, double* out, cudaStream_t st);
 cudaError_t launch_p0_adjoint(const double* G0, const double* H, int64_t ldh, int64_t n, double* part,
                               int32_t* ticket, P0Adjoint* s, double* out, int64_t ldo, cudaStream_t st);
