@@ -57,9 +57,9 @@
 #include <atomic>
 #include <cmath>
 #include <cstring>
-#include <vector>
 
 #include "dmp_internal.cuh"
+#include "tile_order.h"
 
 namespace dmp {
 
@@ -119,10 +119,6 @@ struct TcProgram {
   int ng;       // group sums per element
   TcSeg seg[kMaxSegs];
   unsigned char pa[kMaxSteps], pb[kMaxSteps];  // plane indices of the steps
-};
-
-struct TileAt {
-  unsigned short bi, bj;
 };
 
 struct TcParams {
@@ -1602,28 +1598,6 @@ cudaError_t tc_area_clear(TcArea& a, size_t bytes, cudaStream_t st) {
 
 namespace {
 
-// The output tiles of an m x n product in the order they are walked: bands of
-// column blocks, each cut into groups of row blocks, about as many tiles per
-// block as run at once (`units`) and near-square in elements, so that the tiles
-// in flight together share their operand panels in L2.
-template <int BN, int BM>
-std::vector<TileAt> tile_order(int64_t m, int64_t n, int sym, int units) {
-  const int tm = static_cast<int>((m + BM - 1) / BM), tn = static_cast<int>((n + BN - 1) / BN);
-  const int w = std::max(1, std::min(static_cast<int>(std::lround(std::sqrt(static_cast<double>(units) * BM / BN))), tn));
-  const int hgt = std::max(1, units / w);
-  // row blocks of column block c that hold tiles (symmetric: some element with row <= column)
-  auto rows_of = [&](int c) { return sym ? std::min(tm, (BN * (c + 1) + BM - 1) / BM) : tm; };
-  std::vector<TileAt> t;
-  for (int c0 = 0; c0 < tn; c0 += w) {
-    const int c1 = std::min(tn, c0 + w);
-    for (int r0 = 0; r0 < rows_of(c1 - 1); r0 += hgt)
-      for (int c = c0; c < c1; ++c)
-        for (int r = r0; r < std::min(rows_of(c), r0 + hgt); ++r)
-          t.push_back({static_cast<unsigned short>(r), static_cast<unsigned short>(c)});
-  }
-  return t;
-}
-
 // Length of the equal parts of a split tile's `units` (TcParams::head_len): the
 // one for which the longest share is shortest, the rest of the nsplit tiles
 // going to `extra` CTAs (none: the parts cover the tile).
@@ -1654,8 +1628,8 @@ cudaError_t run_product(const void* A, const void* B, int64_t k_pad, int planes,
   if (!make_plane_map(&ta, A, k_pad, planes * p.rows_a, TC_BM, F8)) return cudaErrorInvalidValue;
   if (!make_plane_map(&tb, B, k_pad, planes * p.rows_b, PAIR ? BN / 2 : BN, F8)) return cudaErrorInvalidValue;
   const int units = PAIR ? tc_max_pairs() : tc_max_ctas();
-  const std::vector<TileAt> tiles = tile_order<BN, Cfg::BM>(p.m, p.n, p.sym, units);
-  const int ntiles = static_cast<int>(tiles.size());
+  TileOrder order(p.m, p.n, Cfg::BM, BN, p.sym != 0, units);
+  const int64_t ntiles = order.count();
   // While there are fewer tiles than CTAs, chunks no longer than a CTA's share of
   // the K atoms (half of it on 256-column tiles, where an added chunk costs less
   // than an uneven share: n = 1024, E4M3, s = 9 62 -> 58 us).
@@ -1671,14 +1645,13 @@ cudaError_t run_product(const void* A, const void* B, int64_t k_pad, int planes,
 
   // rounds of as many tiles as the area holds group sums for, in whole waves
   const size_t tile_bytes = static_cast<size_t>(Cfg::RANKS) * p.prog.ng * Cfg::PART * sizeof(long long);
-  int per = static_cast<int>(std::min<size_t>(std::min(ntiles, kMaxLaunchTiles), area.bytes / tile_bytes));
+  int per = static_cast<int>(std::min<int64_t>(std::min<int64_t>(ntiles, kMaxLaunchTiles), area.bytes / tile_bytes));
   if (per <= 0) return cudaErrorInvalidValue;
   if (per < ntiles && per > units) per = per / units * units;
   cudaError_t e = tc_area_clear(area, per * tile_bytes, st);
-  for (int t0 = 0; t0 < ntiles && e == cudaSuccess; t0 += per) {
-    p.tile0 = t0;
-    p.ntiles = std::min(per, ntiles - t0);
-    std::copy(tiles.begin() + t0, tiles.begin() + t0 + p.ntiles, p.at);
+  for (int64_t t0 = 0; t0 < ntiles && e == cudaSuccess; t0 += per) {
+    p.ntiles = static_cast<int>(std::min<int64_t>(per, ntiles - t0));
+    for (int t = 0; t < p.ntiles; ++t) p.at[t] = order.next();
     p.nwhole = g_split_tiles ? p.ntiles / units * units : p.ntiles;
     const int nsplit = p.ntiles - p.nwhole;
     // The tiles of a partial wave are shared by all CTAs. While the planes stay
