@@ -452,6 +452,8 @@ int dm_purify(const double* H, int64_t n, int64_t ldh, int64_t n_occ, const dmp_
   init.status = DMP_NOT_CONVERGED;
   init.method = o.method;
   init.store32 = o.store32 ? 1 : 0;
+  // until a measure says otherwise: none runs for an H that the set-up rejects
+  init.no_product = 1;
   DMP_CUDA(cudaMemcpyAsync(state, &init, sizeof(init), cudaMemcpyHostToDevice, st));
   DMP_CUDA(launch_gershgorin_init(H, n, ldh, n_occ, rowbuf, state, P, ldp, st));
 
