@@ -21,6 +21,15 @@
  *     buffer `ws` of `ws_bytes`, sized by the matching *_workspace_size call;
  *     the library allocates no device memory of its own (the one exception
  *     is the fixed array behind ozaki_gemm_noalloc).
+ *     That size is the one the call runs fastest in. The matching
+ *     *_least_workspace_size call gives the size it needs at the least, below
+ *     which it returns DMP_ERR_WORKSPACE; any size from there on is accepted
+ *     and gives the same results. The two differ where the call multiplies
+ *     digit differences (DMP_OZAKI_INT8 on DMP_EXEC_TC, 4 to 9 slices, smallest
+ *     dimension from 1920 on, from 2560 on above 6 slices): their planes raise
+ *     the planes' part of the workspace 1.75 times at 4 slices, 2 times at 5,
+ *     2.9 at 8 and 3.1 at 9. No workspace grows past 128 GiB for them: above,
+ *     both calls give the least size.
  *   - Return value: 0 (DMP_OK) or a positive numerical status for purification
  *     (see below), or a negative error. No C++ exception crosses this ABI.
  *   - Thread safety: calls on different streams with different workspaces may
@@ -167,6 +176,7 @@ typedef struct {
 
 /* Bytes of workspace dm_purify needs for this n and these options. */
 int dmp_workspace_size(int64_t n, const dmp_opts* opts, size_t* bytes);
+int dmp_least_workspace_size(int64_t n, const dmp_opts* opts, size_t* bytes);
 
 /* Bytes of the adjoint tape dm_purify writes when given one (checkpoints every
  * opts->checkpoint_every iterates plus per-step scalars). */
@@ -218,6 +228,7 @@ int dm_purify(const double* H, int64_t n, int64_t ldh, int64_t n_occ, const dmp_
  * options: room for device copies of H and P (2 n^2 doubles) followed by
  * dm_purify's workspace. */
 int dmp_host_workspace_size(int64_t n, const dmp_opts* opts, size_t* bytes);
+int dmp_host_least_workspace_size(int64_t n, const dmp_opts* opts, size_t* bytes);
 
 /*
  * dm_purify_host: dm_purify with H and P in HOST memory -- the problem as Sec.
@@ -243,6 +254,8 @@ int dm_purify_host(const double* H_host, int64_t n, int64_t ldh, int64_t n_occ, 
 /* Bytes of workspace ozaki_gemm needs. */
 int ozaki_gemm_workspace_size(int64_t m, int64_t n, int64_t k, int32_t mode, int32_t slices,
                               int32_t executor, size_t* bytes);
+int ozaki_gemm_least_workspace_size(int64_t m, int64_t n, int64_t k, int32_t mode, int32_t slices,
+                                    int32_t executor, size_t* bytes);
 
 /*
  * ozaki_gemm: C = A B, m x k times k x n, through the Ozaki scheme
@@ -287,8 +300,8 @@ int ozaki_gemm(int64_t m, int64_t n, int64_t k, const double* A, int64_t lda, co
  *   - All calls share the one array, so calls that overlap on the GPU (on
  *     different streams, or from several threads) race and give undefined
  *     results. Serialise them.
- *   - Problems whose scratch (as ozaki_gemm_workspace_size reports it) exceeds
- *     128 MiB are rejected with DMP_ERR_WORKSPACE before any work is enqueued.
+ *   - Problems whose scratch (as ozaki_gemm_least_workspace_size reports it)
+ *     exceeds 128 MiB are rejected with DMP_ERR_WORKSPACE before any work is enqueued.
  *     At s = 7 square problems fit up to m = n = k = 1056 in the INT8 and BF16
  *     modes on the tcgen05 executor (two-byte digits and an 80 MiB partial-sum
  *     area), 1440 in the E4M3 mode and 2432 on the int8 mma executor.
@@ -303,7 +316,8 @@ int ozaki_gemm_noalloc(int64_t m, int64_t n, int64_t k, const double* A, int64_t
  * ozaki_level_sums: the exact integer slice-pair products of ozaki_gemm,
  * S[L-2][i][j] = (sum_{a+b=L} A_a B_b)[i][j] as int32, L = 2..s+1, written to
  * S (s x m x n, row-major, leading dimension n). Exposed so that the integer
- * part of the scheme can be compared bit for bit. Same workspace as ozaki_gemm.
+ * part of the scheme can be compared bit for bit. Runs in ozaki_gemm's least
+ * workspace.
  */
 int ozaki_level_sums(int64_t m, int64_t n, int64_t k, const double* A, int64_t lda,
                      const double* B, int64_t ldb, int32_t* S, int32_t mode, int32_t slices,
@@ -356,6 +370,7 @@ int dm_purify_batched(int32_t batch, const double* const* H, const int64_t* n,
 
 /* Workspace for the backward call below. */
 int dmp_backward_workspace_size(int64_t n, const dmp_opts* opts, size_t* bytes);
+int dmp_backward_least_workspace_size(int64_t n, const dmp_opts* opts, size_t* bytes);
 
 /*
  * dm_purify_backward: reverse mode through the purification that dm_purify
@@ -438,6 +453,7 @@ typedef struct {
 /* Bytes of workspace dm_foe needs for this n, these parameters (only n_terms
  * and scheme matter) and these options. */
 int dm_foe_workspace_size(int64_t n, const dmp_foe_params* params, const dmp_opts* opts, size_t* bytes);
+int dm_foe_least_workspace_size(int64_t n, const dmp_foe_params* params, const dmp_opts* opts, size_t* bytes);
 
 /*
  * dm_foe: P = f(H), f(e) = 1 / (1 + exp((e - mu) / kT)) (occupations in [0, 1];

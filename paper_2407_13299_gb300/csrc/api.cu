@@ -68,7 +68,7 @@ struct Opts {
   bool store32;  // DMP_FLAG_FP32_STORAGE
   int late_s;    // late-slice schedule: 0 off, else the slice count after the switch
   double late_idem;
-  int64_t diff_n;  // the size that decides on difference products (they take more planes); 0: none
+  int64_t diff_n;  // the size that decides on difference products (they take more planes; take_room); 0: none
 };
 
 int normalize(const dmp_opts* o, Opts& out) {
@@ -166,6 +166,21 @@ size_t area_bytes(const Opts& o) {
   return o.mode != DMP_FP64 && o.executor == DMP_EXEC_TC ? tc_area_bytes() : 0;
 }
 TcArea area_at(const Opts& o, void* ws, size_t off) { return TcArea{static_cast<char*>(ws) + off, area_bytes(o), 0, 0}; }
+
+// A call runs in the least workspace, pair by pair, and takes the difference
+// planes where `room` bytes hold them too; total() is the call's layout for the
+// options as they stand. The size calls pass room without limit, or none for the
+// least size. With the planes a workspace is at most 128 GiB: they are more than
+// half of one (s = 5 with an 8-slice refinement: 108 n^2 bytes against 48), and a
+// problem that fills the GPU without them still has to fit.
+constexpr size_t kAnyRoom = ~size_t{0};
+constexpr size_t kDiffRoom = size_t{128} << 30;
+
+template <typename Total>
+void take_room(Opts& o, int64_t m, int64_t n, int64_t k, size_t room, const Total& total) {
+  o.diff_n = diff_size(o, m, n, k);
+  if (o.diff_n != 0 && total() > std::min(room, kDiffRoom)) o.diff_n = 0;
+}
 
 // ---------------------------------------------------------------- dm_purify layout
 struct PurifyLayout {
@@ -385,14 +400,20 @@ const char* dmp_status_str(int code) {
   }
 }
 
-int dmp_workspace_size(int64_t n, const dmp_opts* opts, size_t* bytes) {
+static int purify_bytes(int64_t n, const dmp_opts* opts, size_t room, size_t* bytes) {
   Opts o;
   const int rc = normalize(opts, o);
   if (rc != DMP_OK) return rc;
   if (n < 2 || bytes == nullptr) return DMP_ERR_INVALID_ARG;
-  o.diff_n = diff_size(o, n, n, n);
+  take_room(o, n, n, n, room, [&] { return purify_layout(n, o).total; });
   *bytes = purify_layout(n, o).total;
   return DMP_OK;
+}
+int dmp_workspace_size(int64_t n, const dmp_opts* opts, size_t* bytes) {
+  return purify_bytes(n, opts, kAnyRoom, bytes);
+}
+int dmp_least_workspace_size(int64_t n, const dmp_opts* opts, size_t* bytes) {
+  return purify_bytes(n, opts, 0, bytes);
 }
 
 int dmp_tape_size(int64_t n, const dmp_opts* opts, size_t* bytes) {
@@ -420,9 +441,7 @@ int dm_purify(const double* H, int64_t n, int64_t ldh, int64_t n_occ, const dmp_
     return DMP_ERR_UNSUPPORTED;
   if ((o.refine != 0 || o.method != DMP_METHOD_PM || o.store32 || o.late_s > 0) && tape != nullptr)
     return DMP_ERR_UNSUPPORTED;
-  // a workspace without room for the difference planes runs the pairs one by one
-  o.diff_n = diff_size(o, n, n, n);
-  if (ws_bytes < purify_layout(n, o).total) o.diff_n = 0;
+  take_room(o, n, n, n, ws_bytes, [&] { return purify_layout(n, o).total; });
   const PurifyLayout L = purify_layout(n, o);
   if (ws_bytes < L.total) return DMP_ERR_WORKSPACE;
   TapeLayout TL{};
@@ -663,12 +682,18 @@ static size_t host_front_bytes(int64_t n) {
   return 2 * ((nn + 255) / 256 * 256);
 }
 
-int dmp_host_workspace_size(int64_t n, const dmp_opts* opts, size_t* bytes) {
+static int host_bytes(int64_t n, const dmp_opts* opts, size_t room, size_t* bytes) {
   size_t inner = 0;
-  const int rc = dmp_workspace_size(n, opts, &inner);
+  const int rc = purify_bytes(n, opts, room, &inner);
   if (rc != DMP_OK) return rc;
   *bytes = host_front_bytes(n) + inner;
   return DMP_OK;
+}
+int dmp_host_workspace_size(int64_t n, const dmp_opts* opts, size_t* bytes) {
+  return host_bytes(n, opts, kAnyRoom, bytes);
+}
+int dmp_host_least_workspace_size(int64_t n, const dmp_opts* opts, size_t* bytes) {
+  return host_bytes(n, opts, 0, bytes);
 }
 
 int dm_purify_host(const double* H_host, int64_t n, int64_t ldh, int64_t n_occ, const dmp_opts* opts,
@@ -736,30 +761,27 @@ int gemm_opts(int32_t mode, int32_t slices, int32_t executor, Opts& o) {
   return normalize(&d, o);
 }
 }  // namespace
-
-int gemm_least_bytes(int64_t m, int64_t n, int64_t k, int32_t mode, int32_t slices, int32_t executor,
-                     size_t* bytes) {
-  Opts o;
-  const int rc = gemm_opts(mode, slices, executor, o);
-  if (rc != DMP_OK) return rc;
-  if (m < 0 || n < 0 || k < 0 || bytes == nullptr) return DMP_ERR_INVALID_ARG;
-  *bytes = o.mode == DMP_FP64 ? 0 : gemm_layout(m, n, k, o).total;
-  return DMP_OK;
-}
-
 }  // namespace dmp
 
 extern "C" {
 
-int ozaki_gemm_workspace_size(int64_t m, int64_t n, int64_t k, int32_t mode, int32_t slices,
-                              int32_t executor, size_t* bytes) {
+static int gemm_bytes(int64_t m, int64_t n, int64_t k, int32_t mode, int32_t slices, int32_t executor, size_t room,
+                      size_t* bytes) {
   Opts o;
   const int rc = gemm_opts(mode, slices, executor, o);
   if (rc != DMP_OK) return rc;
   if (m < 0 || n < 0 || k < 0 || bytes == nullptr) return DMP_ERR_INVALID_ARG;
-  o.diff_n = diff_size(o, m, n, k);
+  take_room(o, m, n, k, room, [&] { return gemm_layout(m, n, k, o).total; });
   *bytes = o.mode == DMP_FP64 ? 0 : gemm_layout(m, n, k, o).total;
   return DMP_OK;
+}
+int ozaki_gemm_workspace_size(int64_t m, int64_t n, int64_t k, int32_t mode, int32_t slices,
+                              int32_t executor, size_t* bytes) {
+  return gemm_bytes(m, n, k, mode, slices, executor, kAnyRoom, bytes);
+}
+int ozaki_gemm_least_workspace_size(int64_t m, int64_t n, int64_t k, int32_t mode, int32_t slices,
+                                    int32_t executor, size_t* bytes) {
+  return gemm_bytes(m, n, k, mode, slices, executor, 0, bytes);
 }
 
 static int ozaki_common(int64_t m, int64_t n, int64_t k, const double* A, int64_t lda, const double* B,
@@ -779,8 +801,9 @@ static int ozaki_common(int64_t m, int64_t n, int64_t k, const double* A, int64_
   }
   if (!levels_fit_int32(k, o.s, o.mode))
     return DMP_ERR_UNSUPPORTED;
-  if (epi.kind != EPI_LEVELS) o.diff_n = diff_size(o, m, n, k);
-  if (ws_bytes < gemm_layout(m, n, k, o).total) o.diff_n = 0;
+  // (the level sums are formed pair by pair, s of them per element)
+  if (epi.kind != EPI_LEVELS)
+    take_room(o, m, n, k, ws_bytes, [&] { return gemm_layout(m, n, k, o).total; });
   const GemmLayout G = gemm_layout(m, n, k, o);
   if (ws == nullptr || ws_bytes < G.total) return DMP_ERR_WORKSPACE;
   const bool diff = has_diff(o, o.s);
@@ -859,14 +882,20 @@ int ozaki_split(int64_t m, int64_t k, const double* A, int64_t lda, int32_t mode
   return DMP_OK;
 }
 
-int dmp_backward_workspace_size(int64_t n, const dmp_opts* opts, size_t* bytes) {
+static int backward_bytes(int64_t n, const dmp_opts* opts, size_t room, size_t* bytes) {
   Opts o;
   const int rc = normalize(opts, o);
   if (rc != DMP_OK) return rc;
   if (n < 2 || bytes == nullptr) return DMP_ERR_INVALID_ARG;
-  o.diff_n = diff_size(o, n, n, n);
+  take_room(o, n, n, n, room, [&] { return backward_layout(n, o).total; });
   *bytes = backward_layout(n, o).total;
   return DMP_OK;
+}
+int dmp_backward_workspace_size(int64_t n, const dmp_opts* opts, size_t* bytes) {
+  return backward_bytes(n, opts, kAnyRoom, bytes);
+}
+int dmp_backward_least_workspace_size(int64_t n, const dmp_opts* opts, size_t* bytes) {
+  return backward_bytes(n, opts, 0, bytes);
 }
 
 int dm_purify_backward(const double* H, int64_t n, int64_t n_occ, const dmp_opts* opts, const void* tape,
@@ -881,8 +910,7 @@ int dm_purify_backward(const double* H, int64_t n, int64_t n_occ, const dmp_opts
   if (n < 2 || n_occ <= 0 || n_occ >= n) return DMP_ERR_INVALID_ARG;
   const TapeLayout TL = tape_layout(n, o);
   if (tape_bytes < TL.total) return DMP_ERR_WORKSPACE;
-  o.diff_n = diff_size(o, n, n, n);
-  if (ws_bytes < backward_layout(n, o).total) o.diff_n = 0;
+  take_room(o, n, n, n, ws_bytes, [&] { return backward_layout(n, o).total; });
   const BackwardLayout B = backward_layout(n, o);
   if (ws_bytes < B.total) return DMP_ERR_WORKSPACE;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
@@ -1048,7 +1076,7 @@ int dm_purify_backward(const double* H, int64_t n, int64_t n_occ, const dmp_opts
   return DMP_OK;
 }
 
-int dm_foe_workspace_size(int64_t n, const dmp_foe_params* params, const dmp_opts* opts, size_t* bytes) {
+static int foe_bytes(int64_t n, const dmp_foe_params* params, const dmp_opts* opts, size_t room, size_t* bytes) {
   Opts o;
   const int rc = foe_opts(opts, o);
   if (rc != DMP_OK) return rc;
@@ -1057,9 +1085,15 @@ int dm_foe_workspace_size(int64_t n, const dmp_foe_params* params, const dmp_opt
   const int scheme = params->scheme;
   if (M < 2 || M > kFoeMaxTerms) return DMP_ERR_INVALID_ARG;
   if (scheme != DMP_FOE_RECURRENCE && scheme != DMP_FOE_PATERSON_STOCKMEYER) return DMP_ERR_INVALID_ARG;
-  o.diff_n = diff_size(o, n, n, n);
+  take_room(o, n, n, n, room, [&] { return foe_layout(n, o, scheme, M).total; });
   *bytes = foe_layout(n, o, scheme, M).total;
   return DMP_OK;
+}
+int dm_foe_workspace_size(int64_t n, const dmp_foe_params* params, const dmp_opts* opts, size_t* bytes) {
+  return foe_bytes(n, params, opts, kAnyRoom, bytes);
+}
+int dm_foe_least_workspace_size(int64_t n, const dmp_foe_params* params, const dmp_opts* opts, size_t* bytes) {
+  return foe_bytes(n, params, opts, 0, bytes);
 }
 
 int dm_foe(const double* H, int64_t n, int64_t ldh, const dmp_foe_params* params, const dmp_opts* opts,
@@ -1080,8 +1114,7 @@ int dm_foe(const double* H, int64_t n, int64_t ldh, const dmp_foe_params* params
   if (fp.scheme != DMP_FOE_RECURRENCE && !ps) return DMP_ERR_INVALID_ARG;
   if (!std::isfinite(fp.e_min) || !std::isfinite(fp.e_max)) return DMP_ERR_INVALID_ARG;
   if (o.mode != DMP_FP64 && !levels_fit_int32(n, o.s, o.mode)) return DMP_ERR_UNSUPPORTED;
-  o.diff_n = diff_size(o, n, n, n);
-  if (ws_bytes < foe_layout(n, o, fp.scheme, M).total) o.diff_n = 0;
+  take_room(o, n, n, n, ws_bytes, [&] { return foe_layout(n, o, fp.scheme, M).total; });
   const FoeLayout L = foe_layout(n, o, fp.scheme, M);
   if (ws_bytes < L.total) return DMP_ERR_WORKSPACE;
   cudaStream_t st = static_cast<cudaStream_t>(stream);

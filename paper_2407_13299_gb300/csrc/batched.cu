@@ -255,7 +255,7 @@ BatchLayout batch_layout(int batch, const int64_t* n, int s_max, int beta) {
   t.slices = max_slices(t.mode);
   t.executor = DMP_EXEC_TC;
   size_t tb = 0;
-  dmp_workspace_size(nmax, &t, &tb);
+  dmp_least_workspace_size(nmax, &t, &tb);
   L.tune_bytes = tb;
   L.tune_ws = c.take(tb);
   L.total = c.cur;

@@ -150,9 +150,6 @@ cudaError_t launch_split_rows(const double* A, int64_t m, int64_t k, int64_t lda
                               int32_t* exps, void* planes, int64_t m_pad, int64_t k_pad,
                               int elem_kind, bool diff, int* flag, const int* done, cudaStream_t st);
 
-// The smallest workspace ozaki_gemm accepts (without difference planes).
-int gemm_least_bytes(int64_t m, int64_t n, int64_t k, int32_t mode, int32_t slices, int32_t executor, size_t* bytes);
-
 // Out-of-place transpose (m x n, lda) -> (n x m, leading dimension m).
 cudaError_t launch_transpose(const double* A, int64_t m, int64_t n, int64_t lda, double* At,
                              cudaStream_t st);

@@ -41,8 +41,7 @@ int ozaki_gemm_noalloc(int64_t m, int64_t n, int64_t k, const double* A, int64_t
                        int64_t ldb, double* C, int64_t ldc, int32_t mode, int32_t slices, int32_t executor,
                        void* stream) {
   size_t need = 0;
-  // the least ozaki_gemm can run in (it takes difference planes when they fit the array too)
-  const int rc = dmp::gemm_least_bytes(m, n, k, mode, slices, executor, &need);
+  const int rc = ozaki_gemm_least_workspace_size(m, n, k, mode, slices, executor, &need);
   if (rc != DMP_OK) return rc;
   if (need > dmp::kNoAllocBytes) return DMP_ERR_WORKSPACE;  // problem too large for the fixed array
   void* scratch = nullptr;

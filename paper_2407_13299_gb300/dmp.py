@@ -10,6 +10,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+from functools import partial
 
 import torch
 
@@ -80,13 +81,16 @@ _szp = ctypes.POINTER(ctypes.c_size_t)
 # exported symbol -> (restype, argtypes); the test suite checks this list against include/dmp.h
 SIGNATURES = {
     "dmp_workspace_size": (ctypes.c_int, [_i64, ctypes.POINTER(Opts), _szp]),
+    "dmp_least_workspace_size": (ctypes.c_int, [_i64, ctypes.POINTER(Opts), _szp]),
     "dmp_tape_size": (ctypes.c_int, [_i64, ctypes.POINTER(Opts), _szp]),
     "dm_purify": (ctypes.c_int, [_vp, _i64, _i64, _i64, ctypes.POINTER(Opts), _vp, _i64,
                                  ctypes.POINTER(Info), _vp, _sz, _vp, _sz, _vp]),
     "dmp_host_workspace_size": (ctypes.c_int, [_i64, ctypes.POINTER(Opts), _szp]),
+    "dmp_host_least_workspace_size": (ctypes.c_int, [_i64, ctypes.POINTER(Opts), _szp]),
     "dm_purify_host": (ctypes.c_int, [_vp, _i64, _i64, _i64, ctypes.POINTER(Opts), _vp, _i64,
                                       ctypes.POINTER(Info), _vp, _sz, _vp]),
     "ozaki_gemm_workspace_size": (ctypes.c_int, [_i64, _i64, _i64, _i32, _i32, _i32, _szp]),
+    "ozaki_gemm_least_workspace_size": (ctypes.c_int, [_i64, _i64, _i64, _i32, _i32, _i32, _szp]),
     "ozaki_gemm": (ctypes.c_int, [_i64, _i64, _i64, _vp, _i64, _vp, _i64, _vp, _i64, _i32, _i32, _i32,
                                   _vp, _sz, _vp]),
     "ozaki_gemm_noalloc": (ctypes.c_int, [_i64, _i64, _i64, _vp, _i64, _vp, _i64, _vp, _i64, _i32, _i32, _i32,
@@ -99,9 +103,11 @@ SIGNATURES = {
                                          ctypes.POINTER(_vp), ctypes.POINTER(Opts), ctypes.POINTER(Info), _vp,
                                          _sz, _vp]),
     "dmp_backward_workspace_size": (ctypes.c_int, [_i64, ctypes.POINTER(Opts), _szp]),
+    "dmp_backward_least_workspace_size": (ctypes.c_int, [_i64, ctypes.POINTER(Opts), _szp]),
     "dm_purify_backward": (ctypes.c_int, [_vp, _i64, _i64, ctypes.POINTER(Opts), _vp, _sz, _vp, _vp, _vp,
                                           _sz, _vp]),
     "dm_foe_workspace_size": (ctypes.c_int, [_i64, ctypes.POINTER(FoeParams), ctypes.POINTER(Opts), _szp]),
+    "dm_foe_least_workspace_size": (ctypes.c_int, [_i64, ctypes.POINTER(FoeParams), ctypes.POINTER(Opts), _szp]),
     "dm_foe": (ctypes.c_int, [_vp, _i64, _i64, ctypes.POINTER(FoeParams), ctypes.POINTER(Opts), _vp, _i64,
                               ctypes.POINTER(FoeInfo), _vp, _sz, _vp]),
     "dmp_profile_enable": (ctypes.c_int, [ctypes.c_int]),
@@ -230,10 +236,30 @@ def workspace(nbytes: int, device=None) -> torch.Tensor:
     return torch.empty(max(int(nbytes), 256), dtype=torch.uint8, device=device or "cuda")
 
 
-def purify_workspace_bytes(n: int, opts: Opts) -> int:
+def _bytes(name: str, least: bool, *args) -> int:
+    """A size call of the library: `name`_workspace_size, or with `least`
+    `name`_least_workspace_size."""
+    name += "_least_workspace_size" if least else "_workspace_size"
     b = ctypes.c_size_t(0)
-    _check(lib().dmp_workspace_size(n, ctypes.byref(opts), ctypes.byref(b)), "dmp_workspace_size")
+    _check(getattr(lib(), name)(*args, ctypes.byref(b)), name)
     return b.value
+
+
+def _fitting_workspace(size, device=None) -> torch.Tensor:
+    """A workspace of size(least=False) bytes, in which the call runs fastest, or,
+    where the GPU's memory has no room for that, of size(least=True)."""
+    nbytes = size(least=False)
+    try:
+        return workspace(nbytes, device)
+    except torch.cuda.OutOfMemoryError:
+        least = size(least=True)
+        if least >= nbytes:
+            raise
+    return workspace(least, device)
+
+
+def purify_workspace_bytes(n: int, opts: Opts, least: bool = False) -> int:
+    return _bytes("dmp", least, n, ctypes.byref(opts))
 
 
 def tape_bytes(n: int, opts: Opts) -> int:
@@ -260,7 +286,7 @@ def purify(H: torch.Tensor, n_occ: int, mode="int8", slices=7, executor="auto", 
     if P is None:
         P = torch.empty_like(H)
     if ws is None:
-        ws = workspace(purify_workspace_bytes(n, opts), H.device)
+        ws = _fitting_workspace(partial(purify_workspace_bytes, n, opts), H.device)
     info = Info()
     tp = tape.data_ptr() if tape is not None else None
     tb = tape.numel() if tape is not None else 0
@@ -271,10 +297,8 @@ def purify(H: torch.Tensor, n_occ: int, mode="int8", slices=7, executor="auto", 
     return P, info.as_dict()
 
 
-def host_workspace_bytes(n: int, opts: Opts) -> int:
-    b = ctypes.c_size_t(0)
-    _check(lib().dmp_host_workspace_size(n, ctypes.byref(opts), ctypes.byref(b)), "dmp_host_workspace_size")
-    return b.value
+def host_workspace_bytes(n: int, opts: Opts, least: bool = False) -> int:
+    return _bytes("dmp_host", least, n, ctypes.byref(opts))
 
 
 def purify_host(H_host: torch.Tensor, n_occ: int, out: torch.Tensor | None = None, ws=None, stream=None,
@@ -298,7 +322,7 @@ def purify_host(H_host: torch.Tensor, n_occ: int, out: torch.Tensor | None = Non
     if out.is_cuda or out.dtype != torch.float64 or out.stride(1) != 1 or tuple(out.shape) != (n, n):
         raise ValueError("out must be an n x n row-major float64 host tensor")
     if ws is None:
-        ws = workspace(host_workspace_bytes(n, opts))
+        ws = _fitting_workspace(partial(host_workspace_bytes, n, opts))
     info = Info()
     code = lib().dm_purify_host(H_host.data_ptr(), n, H_host.stride(0), int(n_occ), ctypes.byref(opts),
                                 out.data_ptr(), out.stride(0), ctypes.byref(info), ws.data_ptr(), ws.numel(),
@@ -314,11 +338,8 @@ def foe_params(kT: float, n_terms: int, mu: float | None = None, n_occ: int | No
                      int(n_terms), FOE_SCHEMES[scheme], lo, hi)
 
 
-def foe_workspace_bytes(n: int, params: FoeParams, opts: Opts) -> int:
-    b = ctypes.c_size_t(0)
-    _check(lib().dm_foe_workspace_size(n, ctypes.byref(params), ctypes.byref(opts), ctypes.byref(b)),
-           "dm_foe_workspace_size")
-    return b.value
+def foe_workspace_bytes(n: int, params: FoeParams, opts: Opts, least: bool = False) -> int:
+    return _bytes("dm_foe", least, n, ctypes.byref(params), ctypes.byref(opts))
 
 
 def foe(H: torch.Tensor, kT: float, n_terms: int, mu: float | None = None, n_occ: int | None = None,
@@ -339,7 +360,7 @@ def foe(H: torch.Tensor, kT: float, n_terms: int, mu: float | None = None, n_occ
     if P is None:
         P = torch.empty_like(H)
     if ws is None:
-        ws = workspace(foe_workspace_bytes(n, params, opts), H.device)
+        ws = _fitting_workspace(partial(foe_workspace_bytes, n, params, opts), H.device)
     info = FoeInfo()
     code = lib().dm_foe(H.data_ptr(), n, H.stride(0), ctypes.byref(params), ctypes.byref(opts), P.data_ptr(),
                         P.stride(0), ctypes.byref(info), ws.data_ptr(), ws.numel(), _stream_ptr(stream))
@@ -347,11 +368,8 @@ def foe(H: torch.Tensor, kT: float, n_terms: int, mu: float | None = None, n_occ
     return P, info.as_dict()
 
 
-def gemm_workspace_bytes(m, n, k, mode="int8", slices=7, executor="auto") -> int:
-    b = ctypes.c_size_t(0)
-    _check(lib().ozaki_gemm_workspace_size(m, n, k, MODES[mode], slices, EXECUTORS[executor],
-                                           ctypes.byref(b)), "ozaki_gemm_workspace_size")
-    return b.value
+def gemm_workspace_bytes(m, n, k, mode="int8", slices=7, executor="auto", least=False) -> int:
+    return _bytes("ozaki_gemm", least, m, n, k, MODES[mode], slices, EXECUTORS[executor])
 
 
 def ozaki_gemm(A: torch.Tensor, B: torch.Tensor, mode="int8", slices=7, executor="auto", C=None, ws=None,
@@ -364,7 +382,7 @@ def ozaki_gemm(A: torch.Tensor, B: torch.Tensor, mode="int8", slices=7, executor
     if C is None:
         C = torch.empty((m, n), dtype=torch.float64, device=A.device)
     if ws is None:
-        ws = workspace(gemm_workspace_bytes(m, n, k, mode, slices, executor), A.device)
+        ws = _fitting_workspace(partial(gemm_workspace_bytes, m, n, k, mode, slices, executor), A.device)
     code = lib().ozaki_gemm(m, n, k, A.data_ptr(), A.stride(0), B.data_ptr(), B.stride(0), C.data_ptr(),
                             C.stride(0), MODES[mode], slices, EXECUTORS[executor], ws.data_ptr(), ws.numel(),
                             _stream_ptr(stream))
@@ -379,7 +397,7 @@ def ozaki_level_sums(A: torch.Tensor, B: torch.Tensor, mode="int8", slices=7, ex
     m, k = A.shape
     n = B.shape[1]
     S = torch.zeros((slices, m, n), dtype=torch.int32, device=A.device)
-    ws = workspace(gemm_workspace_bytes(m, n, k, mode, slices, executor), A.device)
+    ws = workspace(gemm_workspace_bytes(m, n, k, mode, slices, executor, least=True), A.device)
     code = lib().ozaki_level_sums(m, n, k, A.data_ptr(), A.stride(0), B.data_ptr(), B.stride(0), S.data_ptr(),
                                   MODES[mode], slices, EXECUTORS[executor], ws.data_ptr(), ws.numel(),
                                   _stream_ptr(stream))
@@ -404,10 +422,8 @@ def ozaki_split(A: torch.Tensor, mode="int8", slices=7, executor="auto", stream=
     return exps, digits
 
 
-def backward_workspace_bytes(n: int, opts: Opts) -> int:
-    b = ctypes.c_size_t(0)
-    _check(lib().dmp_backward_workspace_size(n, ctypes.byref(opts), ctypes.byref(b)), "dmp_backward_workspace_size")
-    return b.value
+def backward_workspace_bytes(n: int, opts: Opts, least: bool = False) -> int:
+    return _bytes("dmp_backward", least, n, ctypes.byref(opts))
 
 
 def purify_backward(H: torch.Tensor, n_occ: int, tape: torch.Tensor, G: torch.Tensor, mode="int8", slices=7,
@@ -423,7 +439,7 @@ def purify_backward(H: torch.Tensor, n_occ: int, tape: torch.Tensor, G: torch.Te
     G = G.contiguous()
     out = torch.empty_like(H)
     if ws is None:
-        ws = workspace(backward_workspace_bytes(n, opts), H.device)
+        ws = _fitting_workspace(partial(backward_workspace_bytes, n, opts), H.device)
     code = lib().dm_purify_backward(H.data_ptr(), n, int(n_occ), ctypes.byref(opts), tape.data_ptr(), tape.numel(),
                                     G.data_ptr(), out.data_ptr(), ws.data_ptr(), ws.numel(), _stream_ptr(stream))
     _check(code, "dm_purify_backward")
