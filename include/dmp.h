@@ -24,12 +24,16 @@
  *     That size is the one the call runs fastest in. The matching
  *     *_least_workspace_size call gives the size it needs at the least, below
  *     which it returns DMP_ERR_WORKSPACE; any size from there on is accepted
- *     and gives the same results. The two differ where the call multiplies
- *     digit differences (DMP_OZAKI_INT8 on DMP_EXEC_TC, 4 to 9 slices, smallest
- *     dimension from 1920 on, from 2560 on above 6 slices): their planes raise
- *     the planes' part of the workspace 1.75 times at 4 slices, 2 times at 5,
- *     2.9 at 8 and 3.1 at 9. No workspace grows past 128 GiB for them: above,
- *     both calls give the least size.
+ *     and gives the same results. The two differ
+ *       by 40 MiB in calls with three group sums per element (above 8 slices
+ *         for beta 7 and 5, 6 for beta 8) and many output tiles of 256 x 256
+ *         (more than 53 in a batch; elsewhere from 152 on, with k >= 2048, or
+ *         4096 for DMP_OZAKI_E4M3);
+ *       where the call multiplies digit differences (DMP_OZAKI_INT8 on
+ *         DMP_EXEC_TC, 4 to 9 slices, smallest dimension from 1920 on, from
+ *         2560 on above 6 slices): their planes raise the planes' part of the
+ *         workspace 1.75 times at 4 slices, 2 times at 5, 2.9 at 8 and 3.1 at
+ *         9. No workspace grows past 128 GiB for them.
  *   - Return value: 0 (DMP_OK) or a positive numerical status for purification
  *     (see below), or a negative error. No C++ exception crosses this ABI.
  *   - Thread safety: calls on different streams with different workspaces may
@@ -343,6 +347,7 @@ int ozaki_split(int64_t m, int64_t k, const double* A, int64_t lda, int32_t mode
 
 /* Workspace for the batched call below. */
 int dmp_batched_workspace_size(int32_t batch, const int64_t* n, const dmp_opts* opts, size_t* bytes);
+int dmp_batched_least_workspace_size(int32_t batch, const int64_t* n, const dmp_opts* opts, size_t* bytes);
 
 /*
  * dm_purify_batched: purify `batch` independent Hamiltonians of possibly

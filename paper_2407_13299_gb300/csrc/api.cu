@@ -68,7 +68,9 @@ struct Opts {
   bool store32;  // DMP_FLAG_FP32_STORAGE
   int late_s;    // late-slice schedule: 0 off, else the slice count after the switch
   double late_idem;
-  int64_t diff_n;  // the size that decides on difference products (they take more planes; take_room); 0: none
+  // taken where the workspace has room for them (take_room)
+  int64_t diff_n;  // the size that decides on difference products (they take more planes); 0: none
+  bool wave;       // group sums of a whole wave of tiles, with three per element too
 };
 
 int normalize(const dmp_opts* o, Opts& out) {
@@ -106,6 +108,7 @@ int normalize(const dmp_opts* o, Opts& out) {
   if (out.refine != 0 && out.mode == DMP_FP64) out.refine = -1;
   if (out.refine < -1 || out.refine > smax) return DMP_ERR_INVALID_ARG;
   out.diff_n = 0;
+  out.wave = false;
   out.late_s = out.mode == DMP_FP64 ? 0 : o->late_slices;
   out.late_idem = o->late_idem;
   if (out.late_s < 0 || out.late_s > smax || !(out.late_idem >= 0.0)) return DMP_ERR_INVALID_ARG;
@@ -163,23 +166,44 @@ int64_t row_pad(int executor) { return executor == DMP_EXEC_TC ? 256 : kTileM; }
 
 // The tcgen05 executor's group sums in a workspace (empty for the other executors).
 size_t area_bytes(const Opts& o) {
-  return o.mode != DMP_FP64 && o.executor == DMP_EXEC_TC ? tc_area_bytes() : 0;
+  return o.mode != DMP_FP64 && o.executor == DMP_EXEC_TC ? tc_area_bytes(o.wave) : 0;
 }
 TcArea area_at(const Opts& o, void* ws, size_t off) { return TcArea{static_cast<char*>(ws) + off, area_bytes(o), 0, 0}; }
 
-// A call runs in the least workspace, pair by pair, and takes the difference
-// planes where `room` bytes hold them too; total() is the call's layout for the
-// options as they stand. The size calls pass room without limit, or none for the
-// least size. With the planes a workspace is at most 128 GiB: they are more than
+// Whether some product of the call wants tc_area_bytes(true): an m x n output
+// (sym: its upper triangle). A single matrix shares the tiles of a partial wave
+// out over all CTA pairs, so the larger area pays for several waves of long
+// products only. Least area against the larger one, us: E4M3 s = 9, n = 5000
+// 4531 / 4243, s = 12, n = 6000 12500 / 11740, but n = 2304 (81 tiles) 525 / 559;
+// BF16 s = 7, 4000 x 4000 x 300 (256 tiles) 640 / 670, its 40 MiB to clear among it.
+// At two waves and k = 2100 (4700 x 2000) BF16 s = 7 983 / 945, INT8 s = 9 1371 /
+// 1281, E4M3 s = 9, whose products take half the time, 910 / 928.
+constexpr int64_t kWaveTiles = 152;  // two waves of the 76 pairs
+constexpr int64_t kWaveK = 2048, kWaveK8 = 4096;
+
+bool wants_wave(const Opts& o, int64_t m, int64_t n, int64_t k, bool sym) {
+  if (o.mode == DMP_FP64 || o.executor != DMP_EXEC_TC) return false;
+  if (k < (o.mode == DMP_OZAKI_E4M3 ? kWaveK8 : kWaveK)) return false;
+  const int64_t tm = (m + 255) / 256, tn = (n + 255) / 256;
+  const int64_t tiles = sym ? tn * (tn + 1) / 2 : tm * tn;
+  return tiles >= kWaveTiles && tc_wants_wave(std::max(o.s, std::max(o.refine, o.late_s)), o.beta, tiles);
+}
+
+// A call runs in the least workspace, and takes the difference planes and the
+// larger area where `room` bytes hold them too; total() is the call's layout for
+// the options as they stand. The size calls pass room without limit, or none for
+// the least size. With the planes a workspace is at most 128 GiB: they are more than
 // half of one (s = 5 with an 8-slice refinement: 108 n^2 bytes against 48), and a
 // problem that fills the GPU without them still has to fit.
 constexpr size_t kAnyRoom = ~size_t{0};
 constexpr size_t kDiffRoom = size_t{128} << 30;
 
 template <typename Total>
-void take_room(Opts& o, int64_t m, int64_t n, int64_t k, size_t room, const Total& total) {
+void take_room(Opts& o, int64_t m, int64_t n, int64_t k, bool sym, size_t room, const Total& total) {
   o.diff_n = diff_size(o, m, n, k);
+  o.wave = wants_wave(o, m, n, k, sym);
   if (o.diff_n != 0 && total() > std::min(room, kDiffRoom)) o.diff_n = 0;
+  if (o.wave && total() > room) o.wave = false;
 }
 
 // ---------------------------------------------------------------- dm_purify layout
@@ -405,7 +429,7 @@ static int purify_bytes(int64_t n, const dmp_opts* opts, size_t room, size_t* by
   const int rc = normalize(opts, o);
   if (rc != DMP_OK) return rc;
   if (n < 2 || bytes == nullptr) return DMP_ERR_INVALID_ARG;
-  take_room(o, n, n, n, room, [&] { return purify_layout(n, o).total; });
+  take_room(o, n, n, n, true, room, [&] { return purify_layout(n, o).total; });
   *bytes = purify_layout(n, o).total;
   return DMP_OK;
 }
@@ -441,7 +465,7 @@ int dm_purify(const double* H, int64_t n, int64_t ldh, int64_t n_occ, const dmp_
     return DMP_ERR_UNSUPPORTED;
   if ((o.refine != 0 || o.method != DMP_METHOD_PM || o.store32 || o.late_s > 0) && tape != nullptr)
     return DMP_ERR_UNSUPPORTED;
-  take_room(o, n, n, n, ws_bytes, [&] { return purify_layout(n, o).total; });
+  take_room(o, n, n, n, true, ws_bytes, [&] { return purify_layout(n, o).total; });
   const PurifyLayout L = purify_layout(n, o);
   if (ws_bytes < L.total) return DMP_ERR_WORKSPACE;
   TapeLayout TL{};
@@ -771,7 +795,7 @@ static int gemm_bytes(int64_t m, int64_t n, int64_t k, int32_t mode, int32_t sli
   const int rc = gemm_opts(mode, slices, executor, o);
   if (rc != DMP_OK) return rc;
   if (m < 0 || n < 0 || k < 0 || bytes == nullptr) return DMP_ERR_INVALID_ARG;
-  take_room(o, m, n, k, room, [&] { return gemm_layout(m, n, k, o).total; });
+  take_room(o, m, n, k, false, room, [&] { return gemm_layout(m, n, k, o).total; });
   *bytes = o.mode == DMP_FP64 ? 0 : gemm_layout(m, n, k, o).total;
   return DMP_OK;
 }
@@ -803,7 +827,7 @@ static int ozaki_common(int64_t m, int64_t n, int64_t k, const double* A, int64_
     return DMP_ERR_UNSUPPORTED;
   // (the level sums are formed pair by pair, s of them per element)
   if (epi.kind != EPI_LEVELS)
-    take_room(o, m, n, k, ws_bytes, [&] { return gemm_layout(m, n, k, o).total; });
+    take_room(o, m, n, k, false, ws_bytes, [&] { return gemm_layout(m, n, k, o).total; });
   const GemmLayout G = gemm_layout(m, n, k, o);
   if (ws == nullptr || ws_bytes < G.total) return DMP_ERR_WORKSPACE;
   const bool diff = has_diff(o, o.s);
@@ -887,7 +911,7 @@ static int backward_bytes(int64_t n, const dmp_opts* opts, size_t room, size_t* 
   const int rc = normalize(opts, o);
   if (rc != DMP_OK) return rc;
   if (n < 2 || bytes == nullptr) return DMP_ERR_INVALID_ARG;
-  take_room(o, n, n, n, room, [&] { return backward_layout(n, o).total; });
+  take_room(o, n, n, n, false, room, [&] { return backward_layout(n, o).total; });
   *bytes = backward_layout(n, o).total;
   return DMP_OK;
 }
@@ -910,7 +934,7 @@ int dm_purify_backward(const double* H, int64_t n, int64_t n_occ, const dmp_opts
   if (n < 2 || n_occ <= 0 || n_occ >= n) return DMP_ERR_INVALID_ARG;
   const TapeLayout TL = tape_layout(n, o);
   if (tape_bytes < TL.total) return DMP_ERR_WORKSPACE;
-  take_room(o, n, n, n, ws_bytes, [&] { return backward_layout(n, o).total; });
+  take_room(o, n, n, n, false, ws_bytes, [&] { return backward_layout(n, o).total; });
   const BackwardLayout B = backward_layout(n, o);
   if (ws_bytes < B.total) return DMP_ERR_WORKSPACE;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
@@ -1085,7 +1109,7 @@ static int foe_bytes(int64_t n, const dmp_foe_params* params, const dmp_opts* op
   const int scheme = params->scheme;
   if (M < 2 || M > kFoeMaxTerms) return DMP_ERR_INVALID_ARG;
   if (scheme != DMP_FOE_RECURRENCE && scheme != DMP_FOE_PATERSON_STOCKMEYER) return DMP_ERR_INVALID_ARG;
-  take_room(o, n, n, n, room, [&] { return foe_layout(n, o, scheme, M).total; });
+  take_room(o, n, n, n, true, room, [&] { return foe_layout(n, o, scheme, M).total; });
   *bytes = foe_layout(n, o, scheme, M).total;
   return DMP_OK;
 }
@@ -1114,7 +1138,7 @@ int dm_foe(const double* H, int64_t n, int64_t ldh, const dmp_foe_params* params
   if (fp.scheme != DMP_FOE_RECURRENCE && !ps) return DMP_ERR_INVALID_ARG;
   if (!std::isfinite(fp.e_min) || !std::isfinite(fp.e_max)) return DMP_ERR_INVALID_ARG;
   if (o.mode != DMP_FP64 && !levels_fit_int32(n, o.s, o.mode)) return DMP_ERR_UNSUPPORTED;
-  take_room(o, n, n, n, ws_bytes, [&] { return foe_layout(n, o, fp.scheme, M).total; });
+  take_room(o, n, n, n, true, ws_bytes, [&] { return foe_layout(n, o, fp.scheme, M).total; });
   const FoeLayout L = foe_layout(n, o, fp.scheme, M);
   if (ws_bytes < L.total) return DMP_ERR_WORKSPACE;
   cudaStream_t st = static_cast<cudaStream_t>(stream);

@@ -195,7 +195,7 @@ __global__ void refine_end_kernel(const BatchMat* __restrict__ mats, int nmats, 
 
 // ---------------------------------------------------------------- host side
 struct BatchLayout {
-  size_t mats, tiles, row_start, partials, err, counter, active, area, tune_ws, total;
+  size_t mats, tiles, row_start, partials, err, counter, active, area, area_bytes, tune_ws, total;
   std::vector<size_t> state, rowbuf, expsP, expsX, buf1, X2, planesP, planesX;
   std::vector<int64_t> n_pad, k_pad;
   int ntiles;
@@ -219,7 +219,8 @@ int tiles_of(int64_t n_pad, int bn) {
   return cnt;
 }
 
-BatchLayout batch_layout(int batch, const int64_t* n, int s_max, int beta) {
+// wave: the larger area of group sums (tc_area_bytes)
+BatchLayout batch_layout(int batch, const int64_t* n, int s_max, int beta, bool wave) {
   BatchLayout L;
   Carve c;
   const int eb = beta == 5 ? 1 : 2;  // E4M3 bytes or bf16 planes (tcgen05 executor)
@@ -233,7 +234,8 @@ BatchLayout batch_layout(int batch, const int64_t* n, int s_max, int beta) {
   L.err = c.take(sizeof(int));
   L.counter = c.take(sizeof(int));
   L.active = c.take(sizeof(int));
-  L.area = c.take(tc_area_bytes());
+  L.area = c.take(tc_area_bytes(wave));
+  L.area_bytes = tc_area_bytes(wave);
   int64_t nmax = 2;
   for (int b = 0; b < batch; ++b) {
     const int64_t np = round_up(n[b], 256), kp = round_up(n[b], kq);
@@ -260,6 +262,17 @@ BatchLayout batch_layout(int batch, const int64_t* n, int s_max, int beta) {
   L.tune_ws = c.take(tb);
   L.total = c.cur;
   return L;
+}
+
+// Whether the batch's products want the larger area: the tiles of all its members
+// are one list.
+bool batch_wants_wave(int batch, const int64_t* n, int s_max, int beta) {
+  int64_t tiles = 0;
+  for (int b = 0; b < batch; ++b) {
+    const int64_t t = (n[b] + 255) / 256;
+    tiles += t * (t + 1) / 2;
+  }
+  return tc_wants_wave(s_max, beta, tiles);
 }
 
 struct TuneKey {
@@ -305,7 +318,7 @@ using namespace dmp;
 
 extern "C" {
 
-int dmp_batched_workspace_size(int32_t batch, const int64_t* n, const dmp_opts* opts, size_t* bytes) {
+static int batched_bytes(int32_t batch, const int64_t* n, const dmp_opts* opts, bool least, size_t* bytes) {
   if (batch <= 0 || n == nullptr || opts == nullptr || bytes == nullptr) return DMP_ERR_INVALID_ARG;
   for (int b = 0; b < batch; ++b)
     if (n[b] < 2) return DMP_ERR_INVALID_ARG;
@@ -313,8 +326,14 @@ int dmp_batched_workspace_size(int32_t batch, const int64_t* n, const dmp_opts* 
   const int beta = beta_of(opts->mode);
   const int s_max =
       std::max(opts->slices > 0 ? opts->slices : max_slices(opts->mode), std::max(opts->refine_slices, 0));
-  *bytes = batch_layout(batch, n, s_max, beta).total;
+  *bytes = batch_layout(batch, n, s_max, beta, !least && batch_wants_wave(batch, n, s_max, beta)).total;
   return DMP_OK;
+}
+int dmp_batched_workspace_size(int32_t batch, const int64_t* n, const dmp_opts* opts, size_t* bytes) {
+  return batched_bytes(batch, n, opts, false, bytes);
+}
+int dmp_batched_least_workspace_size(int32_t batch, const int64_t* n, const dmp_opts* opts, size_t* bytes) {
+  return batched_bytes(batch, n, opts, true, bytes);
 }
 
 int dm_purify_batched(int32_t batch, const double* const* H, const int64_t* n, const int64_t* n_occ,
@@ -343,7 +362,8 @@ int dm_purify_batched(int32_t batch, const double* const* H, const int64_t* n, c
     if (static_cast<double>(smax_mode) * n[b] * dmax * dmax >= 2147483648.0) return DMP_ERR_UNSUPPORTED;
   }
   const int s_cap = std::max(opts->slices > 0 ? opts->slices : smax_mode, refine);
-  const BatchLayout L = batch_layout(batch, n, s_cap, beta);
+  BatchLayout L = batch_layout(batch, n, s_cap, beta, batch_wants_wave(batch, n, s_cap, beta));
+  if (ws_bytes < L.total) L = batch_layout(batch, n, s_cap, beta, false);
   if (ws_bytes < L.total) return DMP_ERR_WORKSPACE;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const int max_iter = opts->max_iter == 0 ? 100 : opts->max_iter;
@@ -355,7 +375,7 @@ int dm_purify_batched(int32_t batch, const double* const* H, const int64_t* n, c
   double* dpart = reinterpret_cast<double*>(at(ws, L.partials));
   int* derr = reinterpret_cast<int*>(at(ws, L.err));
   int* dcounter = reinterpret_cast<int*>(at(ws, L.counter));
-  TcArea area{at(ws, L.area), tc_area_bytes(), 0, 0};
+  TcArea area{at(ws, L.area), L.area_bytes, 0, 0};
   const int64_t nmax_idx = std::max_element(n, n + batch) - n;
   const int64_t nmax = n[nmax_idx];
 
@@ -554,6 +574,7 @@ int dm_purify_batched(int32_t batch, const double* const* H, const int64_t* n, c
   std::string gkey(reinterpret_cast<const char*>(hm.data()), sizeof(BatchMat) * batch);
   gkey.append(reinterpret_cast<const char*>(&ws), sizeof(ws));
   gkey.append(reinterpret_cast<const char*>(&cfg), sizeof(cfg));
+  gkey.append(reinterpret_cast<const char*>(&area.bytes), sizeof(area.bytes));  // the rounds of a launch
   gkey.append(reinterpret_cast<const char*>(&tbeta), sizeof(tbeta));  // the digit rule picks the kernels
   cudaGraphExec_t exec = nullptr;
   if (!stream_mode) {

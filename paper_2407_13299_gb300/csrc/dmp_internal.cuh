@@ -197,7 +197,10 @@ struct TcArea {
   size_t bytes, clean;
   size_t front;  // bytes before ptr that the first clearing takes along
 };
-size_t tc_area_bytes();
+// 80 MiB; `wave`: 120, for which products with three group sums per element ask
+// (tc_wants_wave: s slices, an output of `tiles` 256 x 256 tiles) and run without
+size_t tc_area_bytes(bool wave);
+bool tc_wants_wave(int s, int beta, int64_t tiles);
 // zeroes the first `bytes` of the area as far as they are not known to be zero
 cudaError_t tc_area_clear(TcArea& a, size_t bytes, cudaStream_t st);
 // whether the last partial wave of a single-matrix tcgen05 product's tiles is cut

@@ -1575,8 +1575,18 @@ int tc_max_ctas() {
 }
 
 // 80 MiB: 160 pair tiles of one group sum per element, two waves of the pair
-// kernel, which stay in the 129 MB L2 between the product and its output step.
-size_t tc_area_bytes() { return static_cast<size_t>(kTcMaxCtas) * 2 * TC_BM * 256 * sizeof(long long); }
+// kernel, which stay in the 129 MB L2 between the product and its output step, or
+// 80 of two. With three that is 53 tiles: 23 of the 76 pairs of every launch have
+// none of their own, and a batch's tiles are walked whole. 120 MiB hold a whole
+// wave. Batch of two matrices of n = 4096 (272 tiles, 8 iterations), 80 against 120
+// MiB: 9 and 11 E4M3 slices 57.9 / 45.3 and 77.5 / 59.7 ms, 9 INT8 slices 97.2 /
+// 72.6. (For single matrices see wants_wave in api.cu.)
+size_t tc_area_bytes(bool wave) {
+  return static_cast<size_t>(kTcMaxCtas) * (wave ? 3 : 2) * TC_BM * 256 * sizeof(long long);
+}
+bool tc_wants_wave(int s, int beta, int64_t tiles) {
+  return s > 2 * (beta == 8 ? 3 : 4) && tiles * 3 * (2 * TC_BM) * 256 * sizeof(long long) > tc_area_bytes(false);
+}
 
 bool g_split_tiles = true;
 
@@ -1616,6 +1626,10 @@ int head_length(int units, int nsplit, int heads, int extra) {
   return best;
 }
 
+// The part of the area that a launch fills: with one or two group sums the 80 MiB
+// that stay in L2.
+size_t area_room(const TcArea& a, int ng) { return ng > 2 ? a.bytes : std::min(a.bytes, tc_area_bytes(false)); }
+
 // Operand planes up to this size stay in L2 while a product runs.
 constexpr double kL2Planes = 70e6;
 
@@ -1645,7 +1659,8 @@ cudaError_t run_product(const void* A, const void* B, int64_t k_pad, int planes,
 
   // rounds of as many tiles as the area holds group sums for, in whole waves
   const size_t tile_bytes = static_cast<size_t>(Cfg::RANKS) * p.prog.ng * Cfg::PART * sizeof(long long);
-  int per = static_cast<int>(std::min<int64_t>(std::min<int64_t>(ntiles, kMaxLaunchTiles), area.bytes / tile_bytes));
+  int per = static_cast<int>(
+      std::min<int64_t>(std::min<int64_t>(ntiles, kMaxLaunchTiles), area_room(area, p.prog.ng) / tile_bytes));
   if (per <= 0) return cudaErrorInvalidValue;
   if (per < ntiles && per > units) per = per / units * units;
   cudaError_t e = tc_area_clear(area, per * tile_bytes, st);
@@ -1786,7 +1801,7 @@ cudaError_t launch_ozaki_tc_grouped(const BatchMat* mats, const int4* tiles, int
   std::memset(&unused, 0, sizeof(unused));
   const int units = pair ? tc_max_pairs() : tc_max_ctas();
   const size_t tile_bytes = static_cast<size_t>(pair ? 2 : 1) * p.prog.ng * TC_BM * bn * sizeof(long long);
-  int per = static_cast<int>(std::min<size_t>(ntiles, area.bytes / tile_bytes));
+  int per = static_cast<int>(std::min<size_t>(ntiles, area_room(area, p.prog.ng) / tile_bytes));
   if (per <= 0) return cudaErrorInvalidValue;
   if (pair && per < ntiles && per > units) per = per / units * units;
   ProfScope prof(DMP_PROF_PRODUCT, st);

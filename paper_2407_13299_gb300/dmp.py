@@ -99,6 +99,7 @@ SIGNATURES = {
                                         _vp, _sz, _vp]),
     "ozaki_split": (ctypes.c_int, [_i64, _i64, _vp, _i64, _i32, _i32, _i32, _vp, _vp, _vp, _sz, _vp]),
     "dmp_batched_workspace_size": (ctypes.c_int, [_i32, ctypes.POINTER(_i64), ctypes.POINTER(Opts), _szp]),
+    "dmp_batched_least_workspace_size": (ctypes.c_int, [_i32, ctypes.POINTER(_i64), ctypes.POINTER(Opts), _szp]),
     "dm_purify_batched": (ctypes.c_int, [_i32, ctypes.POINTER(_vp), ctypes.POINTER(_i64), ctypes.POINTER(_i64),
                                          ctypes.POINTER(_vp), ctypes.POINTER(Opts), ctypes.POINTER(Info), _vp,
                                          _sz, _vp]),
@@ -481,12 +482,9 @@ def purify_autograd(H, n_occ, mode="int8", slices=7, executor="auto", tol=1e-10,
     return PurifyFunction.apply(H, n_occ, mode, slices, executor, tol, max_iter, checkpoint_every, bounds_constant)
 
 
-def batched_workspace_bytes(ns, opts: Opts) -> int:
+def batched_workspace_bytes(ns, opts: Opts, least: bool = False) -> int:
     arr = (ctypes.c_int64 * len(ns))(*[int(x) for x in ns])
-    b = ctypes.c_size_t(0)
-    _check(lib().dmp_batched_workspace_size(len(ns), arr, ctypes.byref(opts), ctypes.byref(b)),
-           "dmp_batched_workspace_size")
-    return b.value
+    return _bytes("dmp_batched", least, len(ns), arr, ctypes.byref(opts))
 
 
 def purify_batched(Hs, n_occs, mode="int8", slices=0, executor="tc", tol=1e-10, energy_tol=0.0, max_iter=100,
@@ -510,7 +508,7 @@ def purify_batched(Hs, n_occs, mode="int8", slices=0, executor="tc", tol=1e-10, 
     if Ps is None:
         Ps = [torch.empty_like(H) for H in Hs]
     if ws is None:
-        ws = workspace(batched_workspace_bytes(ns, opts), Hs[0].device)
+        ws = _fitting_workspace(partial(batched_workspace_bytes, ns, opts), Hs[0].device)
     Hp = (ctypes.c_void_p * B)(*[H.data_ptr() for H in Hs])
     Pp = (ctypes.c_void_p * B)(*[P.data_ptr() for P in Ps])
     na = (ctypes.c_int64 * B)(*ns)

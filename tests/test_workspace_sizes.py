@@ -63,3 +63,23 @@ def test_a_purification_that_fills_the_gpu_still_fits(dmp):
     n = 65000
     most, least = _sizes(dmp, "purify", n, 5, refine=8)
     assert most == least and most + 2 * 8 * n * n < 284208 << 20
+
+
+@pytest.mark.parametrize("mode,s,three", [("int8", 8, False), ("int8", 9, True), ("bf16", 6, False),
+                                          ("bf16", 7, True), ("e4m3", 8, False), ("e4m3", 9, True)])
+def test_three_group_sums_have_room_for_a_wave_of_tiles(dmp, mode, s, three):
+    """Three sums per element of a 256 x 256 tile are 1.5 MiB, so 80 MiB hold the
+    tiles of 53 of the GPU's 76 CTA pairs; 40 more hold a whole wave. A batch's
+    tiles are walked whole, and it runs a quarter slower without."""
+    wave = lambda size: size(False) - size(True)
+    batch = lambda ns: wave(lambda least: dmp.batched_workspace_bytes(ns, dmp.make_opts(mode, s, "tc"), least))
+    assert batch([4096, 4096]) == (three << 20) * 40
+    assert batch([1024] * 5) == 0  # 50 tiles
+    assert batch([1024] * 6) == (three << 20) * 40
+    gemm = lambda m, n, k: wave(lambda least: dmp.gemm_workspace_bytes(m, n, k, mode, s, "tc", least))
+    if mode == "int8":  # (beside the difference planes)
+        return
+    k = 4096 if mode == "e4m3" else 2048
+    assert gemm(256 * 8, 256 * 19, k) == (three << 20) * 40
+    assert gemm(256 * 8, 256 * 19, k - 1) == 0
+    assert gemm(256 * 8, 256 * 18, k) == 0
