@@ -16,7 +16,10 @@
  *   - Matrices are row-major float64 in DEVICE memory owned by the caller,
  *     element (i, j) at ptr[i * ld + j], ld >= number of columns.
  *   - `stream` is a cudaStream_t (NULL = the legacy default stream). All work is
- *     enqueued on it.
+ *     enqueued on it, but for one copy: dm_purify (and dm_purify_host and the
+ *     slice tuner of dm_purify_batched, which run it) reads its state on a
+ *     private stream that waits for the state at an event of `stream`. The
+ *     private stream and the event live as long as the call.
  *   - Workspace: every call that needs scratch takes a caller-allocated device
  *     buffer `ws` of `ws_bytes`, sized by the matching *_workspace_size call;
  *     the library allocates no device memory of its own (the one exception
@@ -218,8 +221,10 @@ int dmp_tape_size(int64_t n, const dmp_opts* opts, size_t* bytes);
  *          lower triangle is taken as its mirror.
  *   P      n x n output, leading dimension ldp (may not alias H).
  *   info   host pointer or NULL (then nothing is reported).
- *          The call synchronises `stream` once per iteration to read the
- *          device-side stopping decision, and before it returns.
+ *          The host waits once per iteration for the device-side stopping
+ *          decision, on the private stream (see above), while `stream` goes on
+ *          with the step enqueued behind it; the call synchronises `stream`
+ *          before it returns.
  *   tape   NULL, or a device buffer of dmp_tape_size bytes that receives what
  *          dm_purify_backward needs.
  * Returns the status (>= 0) or a negative error.

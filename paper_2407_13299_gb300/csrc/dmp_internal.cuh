@@ -15,8 +15,8 @@ namespace dmp {
 constexpr int kMaxSlices = 12;   // beta 7: up to 10 (70 bits); beta 8: 9 (72); beta 5 nearest: 12 (60)
 constexpr int kTileM = 128;      // output tile rows of the slice-pair GEMMs
 constexpr int kTileN = 128;      // output tile columns
-constexpr int kPadK = 128;       // digit planes are padded to a multiple of this along K (two
-                                 // 64-element swizzle atoms: the paired tcgen05 kernel stages 128)
+constexpr int kPadK = 128;       // digit planes are padded to a multiple of this along K: two
+                                 // 64-element swizzle atoms (the product kernels walk K atom by atom)
 constexpr int kPadK8 = 256;      // the same for one-byte E4M3 digits (two 128-element atoms)
 constexpr int32_t kBadExp = 0x7fffffff;  // row exponent of a row holding NaN/Inf
 

@@ -27,9 +27,9 @@
 //                        definition, unscaled, the update applied and both
 //                        triangles written in full lines; the area is zeroed
 //                        behind the reads for the next product.
-// The output step used to run in the product kernel's epilogue, where one CTA
-// wrote its 128 x 256 part of a tile alone in 60-75 us while its tensor core
-// waited: at n = 256 (one tile) a product took 95 us, 85 of them in that step.
+// In the product kernel's epilogue the output step would leave one CTA alone with
+// its 128 x 256 part of a tile for 60-75 us while its tensor core waits: at n =
+// 256 (one tile) 85 of a product's 95 us, where the two kernels take 16.
 // Up to G consecutive levels (G = 4 for beta 7 and 5, 3 for beta 8) form an
 // exact group; one or two groups are one exact integer, rounded once, and
 // three or more are added in float64 from L = s+1 down to 2 -- the operation
@@ -79,10 +79,10 @@ constexpr int kTileRing = 4;  // WALK 2: tile indices the producer may announce 
 // A stage holds one K atom (a 128-byte row) of each operand. The copies into the
 // SM bound the kernel: an atom of the pair kernel takes 646 clocks (51 bytes per
 // clock and SM, at any size and hit rate) against 512 of its MMAs. The ring is
-// cut fine so that most of it is in flight (with two atoms per stage and three
-// stages a product of n = 8192, s = 5 took 3.88 ms, now 3.69). Sharing the A
-// rows of two pairs by TMA multicast (a quarter fewer bytes from L2, the same
-// into the SMs) left the clocks per atom as they are.
+// cut fine so that most of it is in flight (seven stages of one atom: a product
+// of n = 8192, s = 5, pairs one by one, 3.69 ms; three of two atoms 3.88). Sharing
+// the A rows of two pairs by TMA multicast (a quarter fewer bytes from L2, the
+// same into the SMs) leaves the clocks per atom as they are.
 template <int BN, bool PAIR = false, bool F8 = false>
 struct TcCfg {
   static constexpr int ATOM_K = F8 ? 128 : TC_BK;  // K elements per atom
@@ -101,15 +101,13 @@ struct TcCfg {
 
 // The program of one output tile: steps (the product of plane a of A with
 // plane b of B over the whole K) in segments. A segment's exact sum goes, times
-// w[i], into the group sums g0 + i; consecutive segments with fold = 0 share
-// the weights of the next one and are folded together.
+// w[i], into the group sums g0 + i.
 constexpr int kMaxSegs = 32;
 constexpr int kMaxSteps = 96;
 constexpr int kMaxLaunchTiles = 160;  // single-matrix launches
 
 struct TcSeg {
   int step0, nsteps;
-  int fold;  // the segment's sum (and those of the unfolded ones before it) is added to the groups
   int g0;
   long long w[3];
 };
@@ -526,9 +524,9 @@ __device__ __forceinline__ void store4(double* a, const double (&v)[4], bool vec
 // accesses; the row-major elements go through shared memory for the same
 // reason. n = 4096: 40 us (with the update 60, 45 of them the FP64 pipe's)
 // beside 470 of products, n = 1024: 6 (9) beside 29.
-// (Done instead by two further warps of the next wave's product kernel it cost
-// 3 % of the whole: 200 us per wave of 76 tiles on so few threads, and the
-// shared memory of a seventh stage.)
+// (On two further warps of the next wave's product kernel it costs 3 % of the
+// whole: 200 us per wave of 76 tiles on so few threads, and the shared memory of
+// a seventh stage.)
 // OUT: what becomes of an element. NG: group sums per element (0: EPI_LEVELS).
 constexpr int FIN_THREADS = 128;
 enum { OUT_STORE = 0, OUT_UPDATE = 1, OUT_CHEB = 2 };  // EPI_STORE and EPI_SYM_STORE, EPI_PM_UPDATE, EPI_CHEB
@@ -1288,7 +1286,6 @@ ozaki_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
         if (lo >= hi) continue;
         for (int ch = lo; ch < hi && ok; ++ch) ok = drain_chunk();
         if (!ok) break;
-        if (!seg.fold && u1 > base) continue;  // folded with the next segment
         // ---- add the exact sum to the tile's groups at L2 (red: nothing comes
         // back, so the adds cost no round trip)
         for (int i = 0; i < 3; ++i) {
@@ -1383,7 +1380,6 @@ void direct_program(int s, int beta, int group, int64_t k, bool levels, TcProgra
       ++step;
     }
     g.nsteps = step - g.step0;
-    g.fold = 1;
     g.g0 = levels ? L - 2 : (one ? 0 : pos / group);
     g.w[0] = levels ? 1 : 1ll << (beta * (one ? pos : pos % group));
   }
@@ -1408,7 +1404,6 @@ void diff_program(int s, int beta, int group, int64_t k, TcProgram& pr) {
   auto open = [&]() -> TcSeg& {
     TcSeg& g = pr.seg[pr.nsegs++];
     g.step0 = step;
-    g.fold = 1;
     return g;
   };
   auto weigh = [&](TcSeg& g, int L, int sign) {
