@@ -324,6 +324,19 @@ def run_reference(args):
 
 
 # ---------------------------------------------------------------- our arm
+def pairs(k):
+    return k * (k + 1) // 2
+
+
+def plane_products_of(k, mode, executor, n):
+    """Products of digit planes per emulated n x n product at k slices: the
+    library's rule for difference products, which tests/test_plane_products.py
+    holds against its workspace sizes."""
+    if mode != "int8" or executor != "tc" or not 4 <= k <= 9 or n < (1920 if k <= 6 else 2560):
+        return pairs(k)
+    return (k - 1) + 2 + sum(1 for i in range(1, k) for j in range(i + 1, k) if i + j <= k + 1)
+
+
 def run_ours(args):
     import numpy as np
     import torch
@@ -509,13 +522,8 @@ def run_ours(args):
     # pairs with slice s and one product per difference. A purification of
     # `iters` updates forms 2 iters + 1 loop products with s slices, and the
     # refinement step 2 more with its own slice count.
-    def pairs(k):
-        return k * (k + 1) // 2
-
     def plane_products(k, md=mode):
-        if md != "int8" or args.executor != "tc" or not 4 <= k <= 9 or n < (1920 if k <= 6 else 2560):
-            return pairs(k)
-        return (k - 1) + 2 + sum(1 for i in range(1, k) for j in range(i + 1, k) if i + j <= k + 1)
+        return plane_products_of(k, md, args.executor, n)
     unit_flops = n * n * (n + 1)
     refined = bool(info.get("refined", 0))
     per_step_flops = ((2 * info["iters"] + 1) * plane_products(s) +
