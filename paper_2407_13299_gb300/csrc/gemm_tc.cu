@@ -133,6 +133,7 @@ struct TcParams {
   int64_t m, n;
   int64_t rows_a, rows_b;  // padded rows per digit plane
   int sym;
+  int column_bits;  // of the words in `at`
   const int32_t* ea;
   const int32_t* eb;
   EpiArgs epi;
@@ -149,8 +150,8 @@ struct TcParams {
   TcProgram prog;
   // single-matrix launches: row and column block of each of the launch's tiles
   // (a table: finding a tile's place in the order by counting took the finish
-  // kernel a thousand instructions per warp)
-  TileAt at[kMaxLaunchTiles];
+  // kernel a thousand instructions per warp), packed with column_bits bits
+  uint32_t at[kMaxLaunchTiles];
 };
 
 // ---------------------------------------------------------------- PTX wrappers
@@ -475,8 +476,9 @@ __device__ __forceinline__ Job job_of(const TcParams& p, const CUtensorMap* tmA,
   if (p.mats == nullptr) {
     j.ta = tmA;
     j.tb = tmB;
-    j.m0 = static_cast<int64_t>(p.at[tile].bi) * BM + TC_BM * static_cast<int64_t>(rank);
-    j.n0 = static_cast<int64_t>(p.at[tile].bj) * BN;
+    const TileAt at = unpack_tile(p.at[tile], p.column_bits);
+    j.m0 = static_cast<int64_t>(at.bi) * BM + TC_BM * static_cast<int64_t>(rank);
+    j.n0 = static_cast<int64_t>(at.bj) * BN;
     j.rows_a = p.rows_a;
     j.rows_b = p.rows_b;
     j.KT = p.KT;
@@ -577,8 +579,9 @@ ozaki_finish_kernel(const __grid_constant__ TcParams p) {
   const int32_t* eb = p.eb;
   EpiArgs epi = p.epi;
   if (p.mats == nullptr) {
-    m0 = p.at[tile].bi * Cfg::BM;
-    n0 = p.at[tile].bj * BN;
+    const TileAt at = unpack_tile(p.at[tile], p.column_bits);
+    m0 = at.bi * Cfg::BM;
+    n0 = at.bj * BN;
   } else {
     const int4 t = p.tiles[p.tile0 + tile];
     const BatchMat& M = p.mats[t.x];
@@ -1639,6 +1642,8 @@ cudaError_t run_product(const void* A, const void* B, int64_t k_pad, int planes,
   const int units = PAIR ? tc_max_pairs() : tc_max_ctas();
   TileOrder order(p.m, p.n, Cfg::BM, BN, p.sym != 0, units);
   const int64_t ntiles = order.count();
+  p.column_bits = order.column_bits();
+  if (p.column_bits < 0) return cudaErrorInvalidValue;
   // While there are fewer tiles than CTAs, chunks no longer than a CTA's share of
   // the K atoms (half of it on 256-column tiles, where an added chunk costs less
   // than an uneven share: n = 1024, E4M3, s = 9 62 -> 58 us).
@@ -1661,7 +1666,7 @@ cudaError_t run_product(const void* A, const void* B, int64_t k_pad, int planes,
   cudaError_t e = tc_area_clear(area, per * tile_bytes, st);
   for (int64_t t0 = 0; t0 < ntiles && e == cudaSuccess; t0 += per) {
     p.ntiles = static_cast<int>(std::min<int64_t>(per, ntiles - t0));
-    for (int t = 0; t < p.ntiles; ++t) p.at[t] = order.next();
+    for (int t = 0; t < p.ntiles; ++t) p.at[t] = pack_tile(order.next(), p.column_bits);
     p.nwhole = g_split_tiles ? p.ntiles / units * units : p.ntiles;
     const int nsplit = p.ntiles - p.nwhole;
     // The tiles of a partial wave are shared by all CTAs. While the planes stay

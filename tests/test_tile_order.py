@@ -1,6 +1,6 @@
 """The walk over a product's output tiles (csrc/tile_order.h, host code): every
 tile once, in the order of the bands and groups, for every tile shape, and for
-products of more than 65536 row or column blocks."""
+products of more than 65536 row or column blocks; the word that holds a tile."""
 
 import os
 import subprocess
@@ -22,7 +22,8 @@ int main(int, char** v) {
   std::vector<unsigned char> seen(tm * tn, 0);
   long long distinct = 0, outside = 0;
   for (long long i = 0; i < count; ++i) {
-    const dmp::TileAt t = order.next();
+    // as the kernels get it
+    const dmp::TileAt t = dmp::unpack_tile(dmp::pack_tile(order.next(), order.column_bits()), order.column_bits());
     if (print) printf("%d %d\n", (int)t.bi, (int)t.bj);
     const long long r = t.bi, c = t.bj;
     // symmetric: only tiles holding some element with row <= column
@@ -88,3 +89,10 @@ def _bands(m, n, bm, bn, sym, units):
 def test_order_of_the_walk(walk, bm, bn, m, n, sym):
     got = [tuple(map(int, l.split())) for l in walk(m, n, bm, bn, sym, 76, 1).splitlines()]
     assert got == _bands(m, n, bm, bn, sym, 76)
+
+
+@pytest.mark.parametrize("m,n,sym", [(256 * 3_000_000, 1, 0), (1, 256 * 3_000_000, 0), (2_000_000, 40_000, 0)])
+def test_words_of_the_largest_products(walk, m, n, sym):
+    """Products whose operands or result fill the GPU's memory."""
+    count, distinct, outside, want = map(int, walk(m, n, 256, 256, sym, 76, 0).split())
+    assert (count, distinct, outside) == (want, want, 0)
